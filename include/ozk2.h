@@ -54,12 +54,16 @@ typedef enum {
  *
  * The operation of Sec. II (C ~ AB via A' = trunc(diag(mu) A), B' = trunc(B diag(nu)),
  * residues modulo p_1..p_N, CRT, inverse scaling) with the FP8 construction of
- * Sec. III: hybrid moduli (Sec. III-D), square moduli by Eq. 3matmult-notKaratsuba,
- * the rest by the Karatsuba split (Sec. III-B), accurate-mode scaling by an FP8
- * bound product (Sec. III-E).  3N + 1 FP8 products run on the tensor cores.
+ * Sec. III: the exponents take their budget P from the first N hybrid moduli
+ * (Sec. III-D), accurate-mode scaling by an FP8 bound product (Sec. III-E).  A'B' itself is
+ * computed in another set of pairwise coprime moduli with a product of at least P, chosen
+ * for fewer FP8 products than the hybrid list's 3N (ozk2_product_count): single-digit
+ * moduli up to 49 and Karatsuba moduli (Eq. C'-Karatsuba) up to 1283.  |A'B'| < P / 2, so
+ * the integers and C are the ones the hybrid list gives, bit for bit.
  *
  * m, n, k >= 0.  If m == 0 or n == 0 nothing is written; if k == 0, C is set to 0.
- * k is unrestricted: reductions longer than 2^16 are split into exact blocks.
+ * k is unrestricted: reductions longer than 2^14 (for digits up to 32) to 2^16 are split
+ * into exact blocks.
  * C must not overlap A or B.  Uses a workspace owned by the library (one per
  * device, grown on demand with cudaMalloc, which synchronises the device when it
  * grows; see ozk2_workspace_size for its size).  Each output entry is the
@@ -74,8 +78,9 @@ ozk2_status ozk2_dgemm(int64_t m, int64_t n, int64_t k,
 
 /*
  * ozk2_workspace_size - bytes of device workspace one call with these sizes needs:
- * the FP8 bound operands, M_N digit planes per operand (Sec. IV-B Eq. M), N int16
- * residue-product matrices and the scale vectors.  Returns 0 on invalid arguments.
+ * the FP8 bound operands, room for M_N digit planes per operand (Sec. IV-B Eq. M) and N
+ * int16 residue-product matrices (the residue system in use needs a little less), and the
+ * scale vectors.  Returns 0 on invalid arguments.
  */
 size_t ozk2_workspace_size(int64_t m, int64_t n, int64_t k, int num_moduli);
 
@@ -135,10 +140,10 @@ ozk2_status ozk2_noalloc_device_status(ozk2_stream_t stream);
 /* Operand form and scaling mode of ozk2_dgemm_ex. */
 typedef enum { OZK2_OP_N = 0, OZK2_OP_T = 1 } ozk2_op;
 typedef enum {
-  OZK2_MODE_ACCURATE = 0, /* bound from an FP8 product of |A| and |B| (Sec. III-E); 3N + 1
-                             FP8 products                                              */
+  OZK2_MODE_ACCURATE = 0, /* bound from an FP8 product of |A| and |B| (Sec. III-E); one
+                             FP8 product more than fast mode                           */
   OZK2_MODE_FAST = 1      /* Cauchy-Schwarz bound from row / column norms (Sec. III-E,
-                             "fast mode"); 3N FP8 products, a few bits less accuracy     */
+                             "fast mode"); a few bits less accuracy                      */
 } ozk2_mode;
 
 /*
@@ -308,6 +313,13 @@ ozk2_status ozk2_device_status(void *workspace, ozk2_stream_t stream);
 int ozk2_moduli(int num_moduli, int32_t *p_out);
 
 /*
+ * ozk2_product_count - FP8 products of one emulated product with N moduli, without the
+ * bound product of accurate mode (the hybrid list needs 3N; 27 at N = 12).  Returns -1 if
+ * N is outside 1..20.
+ */
+int ozk2_product_count(int num_moduli);
+
+/*
  * ozk2_set_timing / ozk2_get_timing - per-phase timing of the next ozk2_dgemm calls
  * with CUDA events recorded on the call's stream (enable = 1 turns it on).
  * ozk2_get_timing waits for the last timed call and writes up to `max` phase times
@@ -352,14 +364,9 @@ int ozk2_set_tile_n(int tile_n);
 int ozk2_batch_plan_tile_n(ozk2_batch_plan plan);
 
 /*
- * ozk2_set_square_split - the residue products of a square modulus p = s^2 (Eq.
- * 3matmult-notKaratsuba: X = A1 B2 + A2 B1, Z = A2 B2, C' = mod(s X + Z, p)) run as one
- * pass over both tensor-memory accumulators, or, for reductions of at most kmax terms, as
- * two single-slot passes (X, whose residue is kept, then Z), which lets the epilogue of
- * one pass overlap the next when k is short.  Applies to calls and batch plans made
- * after it; results are bit-identical either way.  Default 0 (never split: measured
- * neutral or slower on this GPU); a negative kmax only queries.  Returns the previous (or
- * current) setting.
+ * ozk2_set_square_split - a setting without effect on the products, whose residue system
+ * has no square moduli (it chose how those ran; results never depended on it).  Stores
+ * kmax; a negative kmax only queries.  Returns the previous (or current) setting.
  */
 int64_t ozk2_set_square_split(int64_t kmax);
 
@@ -404,7 +411,7 @@ int ozk2_debug_timeline(float *ms, int max);
  *   dB: H'_ij = trunc(2^(h_j - e_i) dC_ij) with A' fixed, dB_hj = 2^-h_j (A'^T H')_hj;
  * g and h take the whole budget of P (Eq. condition: 2 sum |G'||B'| < P) from FP8 bound
  * products of |dC| with |B| and of |A| with |dC| (as accurate mode, Sec. III-E), so
- * 3N + 1 FP8 products run per gradient, as in a fresh emulation, but A and B are not
+ * as many FP8 products run per gradient as in a fresh emulation, but A and B are not
  * converted again (their planes are transposed), and one kernel converts dC for both.
  *   forward_workspace  device memory of the current device, the workspace of the
  *                      ozk2_dgemm_ws / ozk2_dgemm_ex call (accurate mode, no blocking,
@@ -484,7 +491,7 @@ ozk2_status ozk2_debug_scales_ex(ozk2_op transa, ozk2_op transb,
                                  ozk2_stream_t stream);
 
 /*
- * ozk2_debug_residue_planes - FP8 digit planes of A' = trunc(diag(2^e) A) and
+ * ozk2_debug_residue_planes - FP8 digit planes, in the hybrid list, of A' = trunc(diag(2^e) A) and
  * B' = trunc(B diag(2^f)) for the given exponents (Eqs. def:A', def:B'; digit splits
  * of Sec. III-B and III-D).  planesA: M_N x m x kp bytes, planesB: M_N x n x kp bytes
  * (B transposed, K-major).  Square modulus l < 6 owns planes 2l, 2l+1 (d1, d2);

@@ -23,6 +23,7 @@ from .ozk2 import (  # noqa: F401
     get_timing,
     last_launch_count,
     moduli,
+    product_count,
     residue_planes,
     residue_products,
     scales,

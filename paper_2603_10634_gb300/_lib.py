@@ -57,6 +57,7 @@ SIGNATURES = {
     "ozk2_status_string": (ctypes.c_char_p, [c_int]),
     "ozk2_device_status": (c_int, [c_void_p, c_void_p]),
     "ozk2_moduli": (c_int, [c_int, ctypes.POINTER(ctypes.c_int32)]),
+    "ozk2_product_count": (c_int, [c_int]),
     "ozk2_set_timing": (None, [c_int]),
     "ozk2_get_timing": (c_int, [ctypes.POINTER(ctypes.c_float), c_int]),
     "ozk2_last_launch_count": (c_int, []),

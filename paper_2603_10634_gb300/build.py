@@ -24,7 +24,7 @@ LIB = os.path.join(PKG, "libozk2.so")
 BUILD_DEBUG = os.path.join(PKG, "_build_debug")
 LIB_DEBUG = os.path.join(PKG, "libozk2_debug.so")
 SOURCES = ["api.cu", "scale.cu", "resid.cu", "gemm.cu", "crt.cu", "noalloc.cu", "moduli.cpp"]
-HEADERS = ["internal.h", "device.cuh"]
+HEADERS = ["internal.h", "device.cuh", "rns.h"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),

@@ -5,9 +5,12 @@
 //   bound product Abar Bbar -> row / column maxima               (Eq. barCupper)
 //   exponents e, f                                                (Eq. mu-computation)
 //   residues and FP8 digits of A' and B'                          (Sec. III-B..III-D)
-//   3N digit products + mod-reduce -> C'_l                        (Eqs. 3matmult, C'-Karatsuba)
+//   digit products + mod-reduce -> C'_l                           (Eqs. 3matmult, C'-Karatsuba)
 //   CRT + inverse scaling -> C                                    (Eqs. CRT_finalreduction,
 //                                                                  inversescaling)
+// The exponents use the hybrid list's P for the caller's N; the products run in the
+// residue system of rns.h, whose product of moduli is at least P (the same integers A'B',
+// hence the same C, from fewer FP8 products).
 // All kernels are launched on the caller's stream (a host-buffer call moves its data on
 // a library copy stream); nothing here runs on the CPU except bookkeeping.
 #include <algorithm>
@@ -110,11 +113,8 @@ int64_t padded(int64_t n, int64_t t) { return ((n + t - 1) / t) * t; }
 
 int tile_rule(int64_t padded256, int64_t padded128) { return 4 * padded256 >= 5 * padded128 ? 128 : 256; }
 
-// Square moduli run as two single-slot passes (X, then Z) when the reduction is at most
-// this long (ozk2_set_square_split).  Off by default: measured on the 512-product batch,
-// the 65536 x 1024 x 1024 product and square sizes 1024-8192, the split was neutral or
-// slower (the drain of both slots after a one-pass square modulus is not what limits
-// short reductions).
+// ozk2_set_square_split: kept for callers; the product path has no square moduli, and
+// results never depended on it.
 std::atomic<int64_t> g_split_kmax{0};
 
 int tile_for(int64_t n) {
@@ -140,7 +140,11 @@ bool device_memory_here(const void* p) {
 // ------------------------------------------------------------------ constant tables
 struct Tables {
   bool built = false;
-  ModTable mt;
+  RnsTable rt;       // the product path
+  GemmMods gm;
+  RnsCrt rc;
+  ModTable mt;       // the hybrid list (parity hooks)
+  GemmMods paper_gm;
   CrtTable ct;
   float pprime;
 };
@@ -151,7 +155,9 @@ const Tables* tables_for(int N) {
   std::lock_guard<std::mutex> lk(g_tab_mutex);
   Tables& t = g_tables[N];
   if (!t.built) {
-    if (!build_mod_table(N, &t.mt) || !build_crt_table(N, &t.ct)) return nullptr;
+    if (!build_mod_table(N, &t.mt) || !build_crt_table(N, &t.ct) || !build_rns_table(N, &t.rt) ||
+        !build_gemm_mods(N, &t.gm) || !build_paper_mods(N, &t.paper_gm) || !build_rns_crt(N, &t.rc))
+      return nullptr;
     t.pprime = p_prime_f32(N);
     t.built = true;
   }
@@ -184,8 +190,26 @@ struct Layout {
   int planes;
   size_t flags, R, S, colmaxA, colbadA, colmaxB, colbadB, zero_end;
   size_t eprime, fprime, e, f, rowstat, colstat;
-  size_t Abar, BbarT, partA, partB, planesA, planesB, cres, total;
+  size_t Abar, BbarT, partA, partB, planesA, planesB, cres, cres8, total;
 };
+
+// Residue rows hold a multiple of 16 columns (16-byte stores of 8-bit residues).
+int64_t residue_pitch(int64_t n) { return ((n + 15) / 16) * 16; }
+
+// Bytes of the residue region: the Karatsuba moduli's 16-bit planes, then the single
+// moduli's 8-bit planes.  Sized for at least N 16-bit planes with rows of a multiple of 8
+// columns, and the digit-plane regions for the hybrid list's M_N planes (which the parity
+// hooks write): the documented workspace, a few percent more than the product path uses.
+size_t residue_bytes(int64_t m, int64_t n, int N) {
+  const size_t own = size_t(kRnsSingles[N] + 2 * kRnsKars[N]) * size_t(m) * size_t(residue_pitch(n));
+  const size_t hybrid = 2 * size_t(N) * size_t(m) * size_t(((n + 7) / 8) * 8);
+  return std::max(own, hybrid);
+}
+// Offset of the 8-bit planes within it.
+size_t residue8_offset(int64_t m, int64_t n, int N) { return 2 * size_t(kRnsKars[N]) * size_t(m) * size_t(residue_pitch(n)); }
+
+// N 16-bit residue planes of the hybrid list (parity hooks, after the layout).
+size_t paper_residue_bytes(int64_t m, int64_t n, int N) { return 2 * size_t(N) * size_t(m) * size_t(residue_pitch(n)); }
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -193,7 +217,7 @@ Layout make_layout(int64_t m, int64_t n, int64_t k, int N, bool fast) {
   Layout L;
   L.kp = ((k + 31) / 32) * 32;
   L.ldp = plane_pitch(L.kp);
-  L.ldr = ((n + 7) / 8) * 8;
+  L.ldr = residue_pitch(n);
   L.planes = (N <= kNumSquares) ? 2 * N : 3 * N - kNumSquares;
   size_t o = 0;
   auto take = [&o](size_t bytes) {
@@ -221,7 +245,8 @@ Layout make_layout(int64_t m, int64_t n, int64_t k, int N, bool fast) {
   L.partB = fast ? take(4 * size_t(n) * (L.kp / 32)) : o;
   L.planesA = take(size_t(L.planes) * m * L.ldp);
   L.planesB = take(size_t(L.planes) * n * L.ldp);
-  L.cres = take(2 * size_t(N) * m * L.ldr);
+  L.cres = take(residue_bytes(m, n, N));
+  L.cres8 = L.cres + residue8_offset(m, n, N);
   L.total = o;
   return L;
 }
@@ -430,46 +455,46 @@ ozk2_status phase_scales(Ctx& c, const Operand& a, const Operand& b, bool clear_
 // plane_stride: bytes between the planes (0: lines * pitch; the whole operand's when
 // `op`, `ex` and `planes` point at a slice of its lines).
 cudaError_t residues_operand(Ctx& c, const Operand& op, int lines, const int32_t* ex, uint8_t* planes,
-                             int64_t pitch, int64_t plane_stride = 0) {
+                             int64_t plane_stride = 0) {
   if (op.kcontig)
-    return launch_residues_rows(op.ptr, op.ld, lines, c.k, int(c.L.kp), pitch, ex, c.tab->mt, planes,
+    return launch_residues_rows(op.ptr, op.ld, lines, c.k, int(c.L.kp), c.L.ldp, ex, c.tab->rt, planes,
                                 c.at<uint32_t>(c.L.flags), c.st, plane_stride);
-  return launch_residues_cols(op.ptr, op.ld, c.k, lines, int(c.L.kp), pitch, ex, c.tab->mt, planes,
+  return launch_residues_cols(op.ptr, op.ld, c.k, lines, int(c.L.kp), c.L.ldp, ex, c.tab->rt, planes,
                               c.at<uint32_t>(c.L.flags), c.st, plane_stride);
 }
 
-// pitch: row pitch of the destination planes (0: the workspace pitch L.ldp).
-ozk2_status phase_residues(Ctx& c, const Operand& a, const Operand& b, const int32_t* e, const int32_t* f,
-                           uint8_t* planesA, uint8_t* planesB, int64_t pitch = 0) {
-  if (pitch == 0) pitch = c.L.ldp;
-  OZK2_TRY(residues_operand(c, a, c.m, e, planesA, pitch));
-  OZK2_TRY(residues_operand(c, b, c.n, f, planesB, pitch));
+// The hybrid list's digit planes of row-major A and B (parity hooks), packed.
+ozk2_status paper_planes(Ctx& c, const double* A, int64_t lda, const double* B, int64_t ldb, const int32_t* e,
+                         const int32_t* f, uint8_t* planesA, uint8_t* planesB) {
+  uint32_t* flags = c.at<uint32_t>(c.L.flags);
+  OZK2_TRY(launch_paper_planes_rows(A, lda, c.m, c.k, int(c.L.kp), e, c.tab->mt, planesA, flags, c.st));
+  OZK2_TRY(launch_paper_planes_cols(B, ldb, c.k, c.n, int(c.L.kp), f, c.tab->mt, planesB, flags, c.st));
   t_launches += 2;
-  mark(c, 4);
   return OZK2_OK;
 }
 
-// Residue products C'_l for output rows [i0, i0 + rows), on stream `st`.
-ozk2_status products_rows(Ctx& c, int64_t i0, int rows, cudaStream_t st) {
+// Residue products C'_l for output rows [i0, i0 + rows), on stream `st`.  `mode`:
+// kModeResidue, or kModePaper (the hybrid list, from packed planes of its digits).
+ozk2_status products_rows(Ctx& c, int64_t i0, int rows, cudaStream_t st, int mode = kModeResidue) {
   const Layout& L = c.L;
   GemmArgs g{};
-  g.mode = kModeResidue;
+  g.mode = mode;
   g.m = rows;
   g.n = c.n;
   g.k = c.k;
   g.num_sms = c.num_sms;
   g.cres = c.at<int16_t>(L.cres) + i0 * L.ldr;
+  g.cres8 = c.at<int8_t>(L.cres8) + i0 * L.ldr;
   g.ldr = L.ldr;
   g.res_stride = int64_t(c.m) * L.ldr;
-  g.mt = &c.tab->mt;
+  g.mods = mode == kModePaper ? &c.tab->paper_gm : &c.tab->gm;
   g.flags = c.at<uint32_t>(L.flags);
   g.plane_stride_a = int64_t(c.m) * L.ldp;
   g.plane_stride_b = int64_t(c.n) * L.ldp;
   g.tile_n = tile_for(c.n);
-  g.split_squares = c.k <= g_split_kmax.load();
   if (!launch_controls(g)) return OZK2_ERR_CUDA;
-  OZK2_TRY(launch_fp8_gemm(g, c.at<uint8_t>(L.planesA) + i0 * L.ldp, L.ldp, L.planes, c.at<uint8_t>(L.planesB),
-                           L.ldp, L.planes, st));
+  OZK2_TRY(launch_fp8_gemm(g, c.at<uint8_t>(L.planesA) + i0 * L.ldp, L.ldp, g.mods->planes,
+                           c.at<uint8_t>(L.planesB), L.ldp, g.mods->planes, st));
   t_launches += 1;
   return OZK2_OK;
 }
@@ -485,8 +510,8 @@ ozk2_status phase_products(Ctx& c) {
 ozk2_status crt_rows(Ctx& c, int64_t i0, int rows, const int32_t* e, const int32_t* f, const uint8_t* rowstat,
                      const uint8_t* colstat, double* C, int64_t ldc, cudaStream_t st) {
   const Layout& L = c.L;
-  OZK2_TRY(launch_crt(c.at<int16_t>(L.cres) + i0 * L.ldr, L.ldr, int64_t(c.m) * L.ldr, rows, c.n, e + i0, f,
-                      rowstat ? rowstat + i0 : nullptr, colstat, C, ldc, c.tab->ct, st));
+  OZK2_TRY(launch_crt(c.at<int16_t>(L.cres) + i0 * L.ldr, c.at<int8_t>(L.cres8) + i0 * L.ldr, L.ldr,
+                      int64_t(c.m) * L.ldr, rows, c.n, e + i0, f, rowstat + i0, colstat, C, ldc, c.tab->rc, st));
   t_launches += 1;
   return OZK2_OK;
 }
@@ -572,7 +597,7 @@ struct CopyBack {
 // after the last CRT is a quarter of a block.  Returns the count; first[b] is the first
 // row of block b, first[count] = m.
 int row_blocks(const Ctx& c, int64_t (&first)[kMaxRowBlocks + 1]) {
-  const int64_t units = ((int64_t(c.m) + 127) / 128) * ((int64_t(c.n) + 255) / 256) * c.N;
+  const int64_t units = ((int64_t(c.m) + 127) / 128) * ((int64_t(c.n) + 255) / 256) * rns_moduli(c.N);
   const int64_t nb = std::max<int64_t>(1, std::min<int64_t>(4, units / (16 * int64_t(c.num_sms))));
   const int64_t rb = ((c.m + nb - 1) / nb + 127) / 128 * 128;
   int count = 0;
@@ -599,7 +624,7 @@ ozk2_status products_and_crt(Ctx& c, const Operand* a, double* C, int64_t ldc, c
   const uint8_t* rs = c.at<uint8_t>(L.rowstat);
   const uint8_t* cs = c.at<uint8_t>(L.colstat);
   if (a) {
-    OZK2_TRY(residues_operand(c, *a, c.m, e, c.at<uint8_t>(L.planesA), L.ldp));
+    OZK2_TRY(residues_operand(c, *a, c.m, e, c.at<uint8_t>(L.planesA)));
     t_launches += 1;
   }
   mark(c, 4);
@@ -633,7 +658,7 @@ ozk2_status run_one(const Operand& a, const Operand& b, int64_t m, int64_t n, in
   mark(c, 0);
   const Layout& L = c.L;
   if ((s = phase_scales(c, a, b, first)) != OZK2_OK) return s;
-  OZK2_TRY(residues_operand(c, b, c.n, c.at<int32_t>(L.f), c.at<uint8_t>(L.planesB), L.ldp));
+  OZK2_TRY(residues_operand(c, b, c.n, c.at<int32_t>(L.f), c.at<uint8_t>(L.planesB)));
   t_launches += 1;
   return products_and_crt(c, &a, C, ldc, nullptr);
 }
@@ -810,7 +835,7 @@ ozk2_status run_host(ozk2_op transa, ozk2_op transb, int64_t m, int64_t n, int64
   // bound), so B's residues need not wait for A
   auto residues_b = [&]() -> ozk2_status {
     OZK2_TRY(exponents_of(c, 0, 0, true));
-    OZK2_TRY(residues_operand(c, b, int(n), c.at<int32_t>(L.f), c.at<uint8_t>(L.planesB), L.ldp));
+    OZK2_TRY(residues_operand(c, b, int(n), c.at<int32_t>(L.f), c.at<uint8_t>(L.planesB)));
     t_launches += 1;
     return OZK2_OK;
   };
@@ -829,7 +854,7 @@ ozk2_status run_host(ozk2_op transa, ozk2_op transb, int64_t m, int64_t n, int64
       if (last) mark(c, 2);
       OZK2_TRY(exponents_of(c, i0, rows, false));
       OZK2_TRY(residues_operand(c, ai, rows, c.at<int32_t>(L.e) + i0, c.at<uint8_t>(L.planesA) + i0 * L.ldp,
-                                L.ldp, planes_a_stride));
+                                planes_a_stride));
       t_launches += 1;
     } else if (last) {
       mark(c, 1);
@@ -872,15 +897,15 @@ struct BwLayout {
   int planes;
   size_t flags, R, S, Rk, Sk, colmaxA, colbadA, colmaxC, colbadC, zk, zero_end;
   size_t gp, hp, g, h, t, tA, rstatC, cstatC, rstatB, cstatA;
-  size_t Gbar, Bhat, AhatT, HhatT, planesG, planesBT, planesAT, planesH, cresA, cresB, total;
+  size_t Gbar, Bhat, AhatT, HhatT, planesG, planesBT, planesAT, planesH, cresA, cresA8, cresB, cresB8, total;
 };
 
 BwLayout make_bw_layout(int64_t m, int64_t n, int64_t k, int N) {
   BwLayout L;
   L.np = ((n + 31) / 32) * 32;
   L.mp = ((m + 31) / 32) * 32;
-  L.ldrk = ((k + 7) / 8) * 8;
-  L.ldrn = ((n + 7) / 8) * 8;
+  L.ldrk = residue_pitch(k);
+  L.ldrn = residue_pitch(n);
   L.planes = (N <= kNumSquares) ? 2 * N : 3 * N - kNumSquares;
   size_t o = 0;
   auto take = [&o](size_t bytes) {
@@ -917,8 +942,10 @@ BwLayout make_bw_layout(int64_t m, int64_t n, int64_t k, int N) {
   L.planesBT = take(size_t(L.planes) * k * L.np);
   L.planesAT = take(size_t(L.planes) * k * L.mp);
   L.planesH = take(size_t(L.planes) * n * L.mp);
-  L.cresA = take(2 * size_t(N) * m * L.ldrk);
-  L.cresB = take(2 * size_t(N) * k * L.ldrn);
+  L.cresA = take(residue_bytes(m, k, N));
+  L.cresA8 = L.cresA + residue8_offset(m, k, N);
+  L.cresB = take(residue_bytes(k, n, N));
+  L.cresB8 = L.cresB + residue8_offset(k, n, N);
   L.total = o;
   return L;
 }
@@ -945,27 +972,27 @@ cudaError_t bw_bound(const Ctx& c, const uint8_t* a, const uint8_t* b, int64_t p
 }
 
 // Residue products of one gradient: `planes` planes of a (rows lines) and b (cols lines),
-// contraction len, row pitch `pitch`, into cres (N x rows x ldr).
+// contraction len, row pitch `pitch`, into the residue region at cres (8-bit planes at cres8).
 cudaError_t bw_products(const Ctx& c, const uint8_t* a, const uint8_t* b, int64_t pitch, int rows, int cols, int len,
-                        int16_t* cres, int64_t ldr, uint32_t* flags) {
+                        uint8_t* cres, uint8_t* cres8, int64_t ldr, uint32_t* flags) {
   GemmArgs g{};
   g.mode = kModeResidue;
   g.m = rows;
   g.n = cols;
   g.k = len;
   g.num_sms = c.num_sms;
-  g.cres = cres;
+  g.cres = reinterpret_cast<int16_t*>(cres);
+  g.cres8 = reinterpret_cast<int8_t*>(cres8);
   g.ldr = ldr;
   g.res_stride = int64_t(rows) * ldr;
-  g.mt = &c.tab->mt;
+  g.mods = &c.tab->gm;
   g.flags = flags;
   g.plane_stride_a = int64_t(rows) * pitch;
   g.plane_stride_b = int64_t(cols) * pitch;
   g.tile_n = tile_for(cols);
-  g.split_squares = len <= g_split_kmax.load();
   if (!launch_controls(g)) return cudaErrorLaunchFailure;
   t_launches += 1;
-  return launch_fp8_gemm(g, a, pitch, c.tab->mt.num_planes, b, pitch, c.tab->mt.num_planes, c.st);
+  return launch_fp8_gemm(g, a, pitch, g.mods->planes, b, pitch, g.mods->planes, c.st);
 }
 
 ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
@@ -1003,7 +1030,7 @@ ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64
   const uint8_t* planesA = f8 + FL.planesA;
   const uint8_t* planesB = f8 + FL.planesB;
   uint32_t* flags = reinterpret_cast<uint32_t*>(at(L.flags));
-  const int P = L.planes;
+  const int P = rns_planes(N);
   int32_t* gp = reinterpret_cast<int32_t*>(at(L.gp));
   int32_t* hp = reinterpret_cast<int32_t*>(at(L.hp));
   int32_t* g = reinterpret_cast<int32_t*>(at(L.g));
@@ -1040,24 +1067,24 @@ ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64
                                   reuse_budget_f32(N), flags, st));
   // dC's two integer matrices from one read of dC; the forward's planes transposed
   OZK2_TRY(launch_grad_residues(dC, lddc, c.m, c.n, g, f, h, e, wantA ? at(L.planesG) : nullptr, L.np,
-                                wantB ? at(L.planesH) : nullptr, L.mp, c.tab->mt, flags, st));
+                                wantB ? at(L.planesH) : nullptr, L.mp, c.tab->rt, flags, st));
   t_launches += 2;
   if (wantA) {
     OZK2_TRY(launch_transpose_planes(planesB, FL.ldp, int64_t(n) * FL.ldp, c.n, c.k, at(L.planesBT), L.np,
                                      int64_t(k) * L.np, P, st));
-    OZK2_TRY(bw_products(c, at(L.planesG), at(L.planesBT), L.np, c.m, c.k, c.n,
-                         reinterpret_cast<int16_t*>(at(L.cresA)), L.ldrk, flags));
-    OZK2_TRY(launch_crt(reinterpret_cast<int16_t*>(at(L.cresA)), L.ldrk, int64_t(m) * L.ldrk, c.m, c.k, g, zk,
-                        at(L.rstatC), at(L.rstatB), dA, ldda, c.tab->ct, st));
+    OZK2_TRY(bw_products(c, at(L.planesG), at(L.planesBT), L.np, c.m, c.k, c.n, at(L.cresA), at(L.cresA8), L.ldrk,
+                         flags));
+    OZK2_TRY(launch_crt(reinterpret_cast<int16_t*>(at(L.cresA)), reinterpret_cast<int8_t*>(at(L.cresA8)), L.ldrk,
+                        int64_t(m) * L.ldrk, c.m, c.k, g, zk, at(L.rstatC), at(L.rstatB), dA, ldda, c.tab->rc, st));
     t_launches += 2;
   }
   if (wantB) {
     OZK2_TRY(launch_transpose_planes(planesA, FL.ldp, int64_t(m) * FL.ldp, c.m, c.k, at(L.planesAT), L.mp,
                                      int64_t(k) * L.mp, P, st));
-    OZK2_TRY(bw_products(c, at(L.planesAT), at(L.planesH), L.mp, c.k, c.n, c.m,
-                         reinterpret_cast<int16_t*>(at(L.cresB)), L.ldrn, flags));
-    OZK2_TRY(launch_crt(reinterpret_cast<int16_t*>(at(L.cresB)), L.ldrn, int64_t(k) * L.ldrn, c.k, c.n, zk, h,
-                        at(L.cstatA), at(L.cstatC), dB, lddb, c.tab->ct, st));
+    OZK2_TRY(bw_products(c, at(L.planesAT), at(L.planesH), L.mp, c.k, c.n, c.m, at(L.cresB), at(L.cresB8), L.ldrn,
+                         flags));
+    OZK2_TRY(launch_crt(reinterpret_cast<int16_t*>(at(L.cresB)), reinterpret_cast<int8_t*>(at(L.cresB8)), L.ldrn,
+                        int64_t(k) * L.ldrn, c.k, c.n, zk, h, at(L.cstatA), at(L.cstatC), dB, lddb, c.tab->rc, st));
     t_launches += 2;
   }
   return OZK2_OK;
@@ -1164,14 +1191,13 @@ BatchLayout batch_layout(int count, const int64_t* m, const int64_t* n, const in
   L.zero_end = o;
   for (int i = 0, j = 0; i < count; ++i) {
     if (!active_problem(m[i], n[i], k[i])) continue;
-    const int64_t mi = m[i], ni = n[i], kp = ((k[i] + 31) / 32) * 32, ldp = plane_pitch(kp),
-                  ldr = ((ni + 7) / 8) * 8;
+    const int64_t mi = m[i], ni = n[i], kp = ((k[i] + 31) / 32) * 32, ldp = plane_pitch(kp), ldr = residue_pitch(ni);
     const size_t ep = take(4 * size_t(mi)), fp = take(4 * size_t(ni)), e = take(4 * size_t(mi)),
                  f = take(4 * size_t(ni)), rs = take(size_t(mi)), cs = take(size_t(ni));
     const size_t abar = fast ? 0 : take(size_t(mi) * kp), bbar = fast ? 0 : take(size_t(ni) * kp);
     const size_t part = fast ? take(4 * size_t(ni) * size_t(kp / 32)) : 0;
     const size_t pa = take(size_t(planes) * mi * ldp), pb = take(size_t(planes) * ni * ldp);
-    const size_t cres = take(2 * size_t(N) * mi * ldr);
+    const size_t cres = take(residue_bytes(mi, ni, N));
     if (probs) {
       BatchProblem& q = P(j);
       q.m = int(mi);
@@ -1192,6 +1218,7 @@ BatchLayout batch_layout(int count, const int64_t* m, const int64_t* n, const in
       q.planesA = at(pa);
       q.planesB = at(pb);
       q.cres = reinterpret_cast<int16_t*>(at(cres));
+      q.cres8 = reinterpret_cast<int8_t*>(at(cres + residue8_offset(mi, ni, N)));
     }
     ++j;
   }
@@ -1299,6 +1326,7 @@ ozk2_status create_plan(ozk2_batch_plan* out, int count, const int64_t* m, const
     q.planesA = rebase(q.planesA, base);
     q.planesB = rebase(q.planesB, base);
     q.cres = rebase(q.cres, base);
+    q.cres8 = rebase(q.cres8, base);
     batch_block_counts(q.m, q.n, q.k, q.kp, fast, q.nblocks);
     for (int w = 0; w < kBatchKernels; ++w) {
       q.first_block[w] = running[w];
@@ -1331,7 +1359,6 @@ ozk2_status create_plan(ozk2_batch_plan* out, int count, const int64_t* m, const
     return narrow[a] != narrow[b] ? narrow[a] < narrow[b] : probs[a].k > probs[b].k;
   });
   std::vector<GemmProblem> gres(probs.size()), gbound(fast ? 0 : probs.size());
-  const int64_t split_kmax = g_split_kmax.load();
   int64_t ubound = 0;
   for (size_t r = 0; r < order.size(); ++r) {
     const BatchProblem& q = probs[size_t(order[r])];
@@ -1339,15 +1366,15 @@ ozk2_status create_plan(ozk2_batch_plan* out, int count, const int64_t* m, const
     const int tile = grp ? 128 : 256;
     GemmProblem& g = gres[r];
     std::memset(&g, 0, sizeof(g));
-    if (!encode_gemm_problem(&g, q.planesA, q.planesB, q.ldp, tab->mt.num_planes, q.m, q.n, q.k, tile)) {
+    if (!encode_gemm_problem(&g, q.planesA, q.planesB, q.ldp, tab->gm.planes, q.m, q.n, q.k, tile)) {
       destroy_plan(plan);
       return OZK2_ERR_INTERNAL;
     }
     // the products of one problem are addressed like those of a single call, but the
     // planes of the B operand have n rows: the map was encoded with the packed strides
     g.unit_start = plan->res_units[grp];  // units are numbered within each grouped launch
-    g.split = q.k <= split_kmax ? 1 : 0;
     g.cres = q.cres;
+    g.cres8 = q.cres8;
     g.ldr = q.ldr;
     g.res_stride = int64_t(q.m) * q.ldr;
     plan->res_units[grp] += fp8_gemm_units(kModeResidue, q.m, q.n, N, tile);
@@ -1447,11 +1474,11 @@ ozk2_status execute_plan(ozk2_batch_plan plan, cudaStream_t st) {
   }
   OZK2_TRY(launch_exponents_batch(probs, plan->cnt, plan->totals[kBkExponents], tab->pprime, delta_f32(), st));
   OZK2_TRY(fork());
-  OZK2_TRY(launch_residues_batch(probs, plan->cnt, plan->totals[kBkResidRows], plan->totals[kBkResidCols], tab->mt,
+  OZK2_TRY(launch_residues_batch(probs, plan->cnt, plan->totals[kBkResidRows], plan->totals[kBkResidCols], tab->rt,
                                  flags, st, plan->side));
   OZK2_TRY(join());
   g.mode = kModeResidue;
-  g.mt = &tab->mt;
+  g.mods = &tab->gm;
   const GemmProblem* gres = reinterpret_cast<const GemmProblem*>(ws + L.gres);
   for (int grp = 0, first = 0; grp < 2; first += plan->res_cnt[grp], ++grp) {
     if (plan->res_cnt[grp] == 0) continue;
@@ -1460,7 +1487,7 @@ ozk2_status execute_plan(ozk2_batch_plan plan, cudaStream_t st) {
     OZK2_TRY(launch_fp8_gemm_grouped(g, gres + first, plan->res_cnt[grp], plan->res_units[grp], st));
     t_launches += 1;
   }
-  OZK2_TRY(launch_crt_batch(probs, plan->cnt, plan->totals[kBkCrt], tab->ct, st));
+  OZK2_TRY(launch_crt_batch(probs, plan->cnt, plan->totals[kBkCrt], tab->rc, st));
   t_launches += 4;
   return OZK2_OK;
 }
@@ -1663,6 +1690,10 @@ int ozk2_moduli(int num_moduli, int32_t* p_out) {
   return num_moduli;
 }
 
+int ozk2_product_count(int num_moduli) {
+  return num_moduli < 1 || num_moduli > kMaxModuli ? -1 : rns_planes(num_moduli);
+}
+
 void ozk2_set_timing(int enable) {
   std::lock_guard<std::mutex> lk(g_timing_mutex);
   g_timing.enabled = enable != 0;
@@ -1839,8 +1870,7 @@ ozk2_status ozk2_debug_residue_planes(int64_t m, int64_t n, int64_t k, const dou
     return OZK2_ERR_INVALID_VALUE;
   Ctx c;
   if ((s = setup(c, m, n, k, num_moduli, false, nullptr, 0, st)) != OZK2_OK) return s;
-  return phase_residues(c, operand_a(OZK2_OP_N, A, lda), operand_b(OZK2_OP_N, B, ldb), e, f, planesA, planesB,
-                        c.L.kp);  // the caller's planes are packed (pitch kp)
+  return paper_planes(c, A, lda, B, ldb, e, f, planesA, planesB);
 }
 
 ozk2_status ozk2_debug_residue_products(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda,
@@ -1852,12 +1882,13 @@ ozk2_status ozk2_debug_residue_products(int64_t m, int64_t n, int64_t k, const d
   if (m == 0 || n == 0 || k == 0 || !A || !B || !e || !f || !Cres || lda < k || ldb < n)
     return OZK2_ERR_INVALID_VALUE;
   Ctx c;
-  if ((s = setup(c, m, n, k, num_moduli, false, nullptr, 0, st)) != OZK2_OK) return s;
-  const Layout& L = c.L;
-  if ((s = phase_residues(c, operand_a(OZK2_OP_N, A, lda), operand_b(OZK2_OP_N, B, ldb), e, f,
-                          c.at<uint8_t>(L.planesA), c.at<uint8_t>(L.planesB))) != OZK2_OK)
+  if ((s = setup(c, m, n, k, num_moduli, false, nullptr, 0, st, paper_residue_bytes(m, n, num_moduli))) != OZK2_OK)
     return s;
-  if ((s = phase_products(c)) != OZK2_OK) return s;
+  c.L.cres = c.L.total;
+  const Layout& L = c.L;
+  if ((s = paper_planes(c, A, lda, B, ldb, e, f, c.at<uint8_t>(L.planesA), c.at<uint8_t>(L.planesB))) != OZK2_OK)
+    return s;
+  if ((s = products_rows(c, 0, c.m, c.st, kModePaper)) != OZK2_OK) return s;
   OZK2_TRY(cudaMemcpy2DAsync(Cres, size_t(n) * 2, c.ws + L.cres, size_t(L.ldr) * 2, size_t(n) * 2,
                              size_t(num_moduli) * size_t(m), cudaMemcpyDeviceToDevice, st));
   return OZK2_OK;
@@ -1871,11 +1902,15 @@ ozk2_status ozk2_debug_crt(int64_t m, int64_t n, int num_moduli, const int16_t* 
   if (m == 0 || n == 0) return OZK2_OK;
   if (!Cres || !e || !f || !C || ldc < n) return OZK2_ERR_INVALID_VALUE;
   Ctx c;
-  if ((s = setup(c, m, n, 1, num_moduli, false, nullptr, 0, st)) != OZK2_OK) return s;
+  if ((s = setup(c, m, n, 1, num_moduli, false, nullptr, 0, st, paper_residue_bytes(m, n, num_moduli))) != OZK2_OK)
+    return s;
+  c.L.cres = c.L.total;
   const Layout& L = c.L;
   OZK2_TRY(cudaMemcpy2DAsync(c.ws + L.cres, size_t(L.ldr) * 2, Cres, size_t(n) * 2, size_t(n) * 2,
                              size_t(num_moduli) * size_t(m), cudaMemcpyDeviceToDevice, st));
-  return phase_crt(c, e, f, nullptr, nullptr, C, ldc);
+  OZK2_TRY(launch_paper_crt(c.at<int16_t>(L.cres), L.ldr, int64_t(m) * L.ldr, c.m, c.n, e, f, C, ldc, c.tab->ct, st));
+  t_launches += 1;
+  return OZK2_OK;
 }
 
 }  // extern "C"

@@ -1,35 +1,36 @@
 // FP8 tensor-core products of the method on tcgen05 (sm_103a): one persistent kernel,
-// three epilogues.
+// four epilogues.
 //
-//   residue : C'_l = mod(A'_l B'_l, p_l) for an output tile, from digit-plane products
-//             held in TMEM and reduced mod p in registers:
-//               square p = s^2 : X = A1 B2 + A2 B1 (one accumulator), Z = A2 B2,
-//                                C'_l = mod(s X + Z, p)           [Eq. 3matmult-notKaratsuba]
-//               Karatsuba      : Dx = Ax Bx, x = 1, 2, 3,
-//                                256 D1 + D2 + 16 (D3 - D1 - D2) = 16 (15 D1 - D2 + D3) + D2
-//                                                                  [Eq. C'-Karatsuba]
+//   residue : C'_l = mod(A'_l B'_l, p_l) for an output tile and one modulus of the
+//             product path's residue system (rns.h), from digit-plane products held in
+//             TMEM and reduced mod p in registers:
+//               single    : D = A1 B1, C'_l = D mod p (int8)
+//               Karatsuba : Dx = Ax Bx, x = 1, 2, 3, C'_l = mod(c1 D1 + c2 D2 + c3 D3, p)
+//                           (int16; Eq. C'-Karatsuba for a general base)
+//   paper   : the same for the hybrid list (the residue-product parity hook, int16):
+//               square p = s^2 : X = A1 B2 + A2 B1, Z = A2 B2, C'_l = mod(s X + Z, p)
+//                                                                  [Eq. 3matmult-notKaratsuba]
+//               Karatsuba      : c1, c2, c3 = 240, -15, 16 (256 D1 + D2 + 16 (D3 - D1 - D2))
 //             Every FP32 accumulator is an exact integer of magnitude <= 2^24
-//             (Eq. error-free-FP8-matmult): a Karatsuba product over at most 2^16
-//             terms of digits |d| <= 16, or the shared square accumulator over at most
-//             2^15.  Longer reductions run in blocks whose residues are added mod p.
+//             (Eq. error-free-FP8-matmult); a modulus's `chunk` bounds the terms of one
+//             block accordingly, and longer reductions run in blocks whose residues are
+//             added mod p.
 //   bound   : Cbar = RU((1 + k 2^-24) Abar Bbar) folded into row / column maxima
 //             (Eq. barCupper); Cbar itself is never stored.
 //   raw     : D = A B^T in FP32 (a parity hook for the tensor-core path).
 //
 // Tiles are 128 x 256 (M x N); TMEM holds two 256-column FP32 accumulator slots (the
 // whole 512 columns).  A unit (one tile of one modulus) is a sequence of passes over
-// the k-block:
-//   square p = s^2 : one pass over BOTH slots, the products interleaved per k-step,
-//                    X = A1 B2 + A2 B1 -> slot 0, Z = A2 B2 -> slot 1 (A2 and B2 are
-//                    loaded while still in L2), C'_l = mod(s X + Z, p);
-//   Karatsuba      : three passes over ONE slot each, alternating slots, so the
-//                    epilogue drains one slot while the tensor cores fill the other:
-//                    D1, park d1 = mod(D1, p); D2, park v = mod(240 d1 - 15 D2, p);
-//                    D3, C'_l = mod(v + 16 D3, p)  (256 D1 + D2 + 16 (D3 - D1 - D2)
-//                    = 240 D1 - 15 D2 + 16 D3; every operand of mod is below 2^28).
+// the k-block, each filling one slot; passes alternate slots, so the epilogue drains one
+// while the tensor cores fill the other:
+//   single         one pass;
+//   Karatsuba      three passes: D1, park d1 = D1 mod p; D2, park v = mod(c1 d1 + c2 D2, p);
+//                  D3, C'_l = mod(v + c3 D3, p);
+//   paper squares  two passes: X (two products per k-step), park x = X mod p; Z.
 // Parked values are int16 pairs in the epilogue threads' registers (every pass of a
-// unit gives a thread the same row and columns).  The bound and raw products are one single-slot pass per unit.  The wide tile halves the
-// operand bytes each SM pulls per flop compared with 128 x 128.
+// unit gives a thread the same row and columns).  The bound and raw products are one pass
+// per unit.  The wide tile halves the operand bytes each SM pulls per flop compared with
+// 128 x 128.
 //
 // Roles (320 threads for single problems, 576 for grouped launches; one persistent CTA
 // per SM):
@@ -69,8 +70,6 @@ struct Epi {
   static constexpr int kThreads = 64 + 32 * kWarps;
   static constexpr int kCW = GROUPED ? 16 : 32;  // columns per TMEM load of the residue epilogue
 };
-constexpr int kChunkKaratsuba = 65536;  // 2^16 * 16 * 16 = 2^24
-constexpr int kChunkSquare = 32768;     // shared accumulator: 2 * 2^15 * 16 * 16 = 2^24
 constexpr int kGroupM = 16;             // tile rasterisation: bands of 16 tile rows (2048 rows of A)
 
 // Tile shapes: 128 x 256 (the default) or 128 x 128 (narrow or ragged products, where a
@@ -86,22 +85,16 @@ struct Tile {
   static constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(kStages) * kStageBytes + 256;
 };
 
-struct EpiMod {
-  int p[kMaxModuli];
-  int half[kMaxModuli];
-  int s[kMaxModuli];
-  float inv_p[kMaxModuli];
-};
-
 struct GemmParams {
   int mode;
   int m, n, k;
   int tiles_m, tiles_n, tiles;
   int num_units;
-  int16_t* cres;
+  int16_t* cres;   // 16-bit residues (Karatsuba moduli; all of the paper mode)
+  int8_t* cres8;   // 8-bit residues (single moduli)
   int64_t ldr;
   int64_t res_stride;
-  EpiMod mod;
+  GemmMods mods;
   float factor;
   float* R;
   float* S;
@@ -114,7 +107,6 @@ struct GemmParams {
   const int32_t* rowshift;
   unsigned long long wait_ns;  // limit of every device wait (the drains of an abort use the default)
   int stall;                   // fault injection: the MMA thread's first wait never completes
-  int split_squares;           // single problems: square moduli in two single-slot passes
 };
 
 __device__ __forceinline__ void decode_unit(int tiles_m, int tiles_n, int tiles, int u, int& mod, int& tm,
@@ -142,11 +134,11 @@ struct UnitCtx {
   int tiles_m, tiles_n, tiles;
   int64_t unit_start, next_start;  // grouped: units [unit_start, next_start) are this problem's
   int16_t* cres;
+  int8_t* cres8;
   int64_t ldr, res_stride;
   float factor;
   float* R;
   float* S;
-  bool split;  // square moduli in two single-slot passes
 };
 
 template <bool GROUPED>
@@ -161,12 +153,12 @@ __device__ __forceinline__ void resolve_unit(const GemmParams& P, const CUtensor
     c.prob = 0;
     decode_unit(P.tiles_m, P.tiles_n, P.tiles, u, c.mod, c.tm, c.tn);
     c.cres = P.cres;
+    c.cres8 = P.cres8;
     c.ldr = P.ldr;
     c.res_stride = P.res_stride;
     c.factor = P.factor;
     c.R = P.R;
     c.S = P.S;
-    c.split = P.split_squares != 0;
   } else {
     if (c.prob < 0 || u >= c.next_start) {
       // the last problem starting at or before u, searched above the current one
@@ -189,12 +181,12 @@ __device__ __forceinline__ void resolve_unit(const GemmParams& P, const CUtensor
       c.unit_start = G.unit_start;
       c.next_start = lo + 1 < nprobs ? probs[lo + 1].unit_start : 0x7FFFFFFFFFFFFFFFll;
       c.cres = G.cres;
+      c.cres8 = G.cres8;
       c.ldr = G.ldr;
       c.res_stride = G.res_stride;
       c.factor = G.factor;
       c.R = G.R;
       c.S = G.S;
-      c.split = G.split != 0;
     }
     decode_unit(c.tiles_m, c.tiles_n, c.tiles, static_cast<int>(u - c.unit_start), c.mod, c.tm, c.tn);
   }
@@ -213,68 +205,51 @@ struct UnitPlan {
   int npasses;    // passes per block
 };
 
-// split: a square modulus runs as two single-slot passes, X = A1 B2 + A2 B1 (its residue
-// parked) and then Z = A2 B2, instead of one pass over both slots; chosen for short
-// reductions, where the drain of both slots after a pair pass would leave the tensor
-// cores idle.
 template <int MODE>
-__device__ __forceinline__ UnitPlan plan_of(int k, int mod, bool split) {
+__device__ __forceinline__ UnitPlan plan_of(const GemmParams& P, int k, int mod) {
   UnitPlan u;
-  if (MODE == kModeResidue) {
-    const bool square = mod < kNumSquares;
-    u.chunk_len = square ? kChunkSquare : kChunkKaratsuba;
-    u.npasses = square ? (split ? 2 : 1) : 3;
+  if constexpr (MODE == kModeResidue || MODE == kModePaper) {
+    u.chunk_len = P.mods.m[mod].chunk;
+    if constexpr (MODE == kModeResidue) u.npasses = mod < P.mods.kars ? 3 : 1;
+    else u.npasses = mod < kNumSquares ? 2 : 3;
+    u.nchunks = (k + u.chunk_len - 1) / u.chunk_len;
   } else {
     u.chunk_len = ((k + BK - 1) / BK) * BK;
     u.npasses = 1;
+    u.nchunks = 1;
   }
-  u.nchunks = (k + u.chunk_len - 1) / u.chunk_len;
   return u;
 }
 
-// A pass uses both slots (a square modulus in one pass) or one.
+// Products of one pass per k-step, and the digit planes (pa, pb) of product x.
 template <int MODE>
-__device__ __forceinline__ bool pair_pass(int mod, bool split) {
-  return MODE == kModeResidue && mod < kNumSquares && !split;
-}
-
-// Products of one pass per k-step, the digit planes (pa, pb) of product x and the
-// accumulator (0: the pass's first slot, 1: slot 1 of a pair pass) it adds to.
-template <int MODE>
-__device__ __forceinline__ int num_products(int mod, int pass, bool split) {
-  if (pair_pass<MODE>(mod, split)) return 3;
-  if (MODE == kModeResidue && mod < kNumSquares) return pass == 0 ? 2 : 1;  // split square: X, then Z
-  return 1;
+__device__ __forceinline__ int num_products(int mod, int pass) {
+  return MODE == kModePaper && mod < kNumSquares && pass == 0 ? 2 : 1;
 }
 
 template <int MODE>
-__device__ __forceinline__ void product_of(int mod, int pass, int x, bool split, int& pa, int& pb, int& acc) {
-  if (MODE != kModeResidue) {
-    pa = pb = 0;
-    acc = 0;
-  } else if (mod < kNumSquares) {
-    const int a0 = 2 * mod;  // (A1, B2) -> X, (A2, B1) -> X, (A2, B2) -> Z
-    const int xs = split ? (pass == 0 ? x : 2) : x;
-    pa = (xs == 0) ? a0 : a0 + 1;
-    pb = (xs == 1) ? a0 : a0 + 1;
-    acc = (!split && xs == 2) ? 1 : 0;
+__device__ __forceinline__ void product_of(const GemmParams& P, int mod, int pass, int x, int& pa, int& pb) {
+  if constexpr (MODE == kModeResidue) {
+    pa = pb = mod < P.mods.kars ? 3 * mod + pass : 2 * P.mods.kars + mod;
+  } else if constexpr (MODE == kModePaper) {
+    if (mod < kNumSquares) {  // (A1, B2) + (A2, B1), then (A2, B2)
+      const int a0 = 2 * mod;
+      pa = (pass == 0 && x == 0) ? a0 : a0 + 1;
+      pb = (pass == 0 && x == 1) ? a0 : a0 + 1;
+    } else {
+      pa = pb = 2 * kNumSquares + 3 * (mod - kNumSquares) + pass;
+    }
   } else {
-    pa = pb = 2 * kNumSquares + 3 * (mod - kNumSquares) + pass;  // (Ax, Bx) -> Dx
-    acc = 0;
+    pa = pb = 0;
   }
 }
 
 // Slot bookkeeping shared by the MMA thread and the epilogue, which walk the same pass
-// sequence: a single-slot pass takes slot `next` and flips it; a pair pass takes both
-// (X in slot 0, Z in slot 1).  uses[j] counts the passes that used slot j before.
+// sequence: pass t of this CTA uses slot t mod 2, for the (t / 2)-th time.
 struct Slots {
-  uint32_t u0 = 0u, u1 = 0u;  // passes that used slot 0 / slot 1
-  uint32_t next = 0u;
-  __device__ __forceinline__ uint32_t uses(uint32_t j) const { return j ? u1 : u0; }
-  __device__ __forceinline__ void bump(uint32_t j) {
-    u0 += (j == 0u) ? 1u : 0u;
-    u1 += (j == 1u) ? 1u : 0u;
-  }
+  uint32_t t = 0u;
+  __device__ __forceinline__ uint32_t slot() const { return t & 1u; }
+  __device__ __forceinline__ uint32_t uses() const { return t >> 1; }
 };
 
 // Lane l of the warp ends with the maximum of column l over the 32 lanes.
@@ -339,39 +314,77 @@ __device__ __forceinline__ float2 unpack2(uint32_t w) {
   return make_float2(static_cast<float>(static_cast<int16_t>(w & 0xFFFFu)), static_cast<float>(static_cast<int16_t>(w >> 16)));
 }
 
-// Store 8 int16 residues of one row at columns gc .. gc + 7, packed two per word (adding
-// the previous block's residues when `accumulate`), as one 16-byte store when the 8
-// columns are all inside the matrix.  The debug build checks that every residue lies in
-// the symmetric range [-h, p - 1 - h].
-__device__ __forceinline__ void store_residues8(int16_t* dst, int gc, int n, uint32_t (&pk)[4], bool accumulate,
-                                                int p, int h, uint32_t* flags) {
+// Store 8 int16 residues of one row at columns gc .. gc + 7 (gc < n), packed two per word,
+// as one 16-byte store (adding the previous block's residues when `accumulate`): rows are
+// padded to 16 columns, so the store stays inside the row.  The debug build checks that
+// every residue lies in [-h - 1, p - h] (paper mode: the symmetric range [-h, p - 1 - h]).
+template <bool EXACT>
+__device__ __forceinline__ void store_residues8(int16_t* dst, int gc, uint32_t (&pk)[4], bool accumulate, int p, int h,
+                                                uint32_t* flags) {
+  uint4* out = reinterpret_cast<uint4*>(dst + gc);
   if (accumulate) {
+    const uint4 prev = *out;
+    const uint32_t pw[4] = {prev.x, prev.y, prev.z, prev.w};
 #pragma unroll
     for (int z = 0; z < 4; ++z) {
-      const int j = gc + 2 * z;
-      const int a = smod_small(static_cast<int16_t>(pk[z] & 0xFFFFu) + (j < n ? dst[j] : 0), p, h);
-      const int b = smod_small(static_cast<int16_t>(pk[z] >> 16) + (j + 1 < n ? dst[j + 1] : 0), p, h);
+      const int a = smod_small(static_cast<int16_t>(pk[z] & 0xFFFFu) + static_cast<int16_t>(pw[z] & 0xFFFFu), p, h);
+      const int b = smod_small(static_cast<int16_t>(pk[z] >> 16) + static_cast<int16_t>(pw[z] >> 16), p, h);
       pk[z] = (static_cast<uint32_t>(a) & 0xFFFFu) | (static_cast<uint32_t>(b) << 16);
     }
   }
 #ifdef OZK2_DEBUG
+  constexpr int kSlack = EXACT ? 0 : 1;
   bool in_range = true;
 #pragma unroll
   for (int z = 0; z < 4; ++z) {
     const int a = static_cast<int16_t>(pk[z] & 0xFFFFu), b = static_cast<int16_t>(pk[z] >> 16);
-    in_range = in_range && a >= -h && a <= p - 1 - h && b >= -h && b <= p - 1 - h;
+    in_range = in_range && a >= -h - kSlack && a <= p - 1 - h + kSlack && b >= -h - kSlack && b <= p - 1 - h + kSlack;
   }
   OZK2_DCHECK(in_range, flags);
 #else
   (void)flags;
 #endif
-  if (gc + 8 <= n) {
-    *reinterpret_cast<uint4*>(dst + gc) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-  } else {
+  *out = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+}
+
+// The same for 16 int8 residues, packed four per word.
+__device__ __forceinline__ void store_residues16(int8_t* dst, int gc, uint32_t (&pk)[4], bool accumulate, int p, int h,
+                                                 uint32_t* flags) {
+  uint4* out = reinterpret_cast<uint4*>(dst + gc);
+  if (accumulate) {
+    const uint4 prev = *out;
+    const uint32_t pw[4] = {prev.x, prev.y, prev.z, prev.w};
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (gc + j < n) dst[gc + j] = static_cast<int16_t>((j & 1) ? (pk[j >> 1] >> 16) : (pk[j >> 1] & 0xFFFFu));
+    for (int z = 0; z < 4; ++z) {
+      uint32_t r = 0;
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const int x = smod_small(static_cast<int8_t>(pk[z] >> (8 * b)) + static_cast<int8_t>(pw[z] >> (8 * b)), p, h);
+        r |= (static_cast<uint32_t>(x) & 0xFFu) << (8 * b);
+      }
+      pk[z] = r;
+    }
   }
+#ifdef OZK2_DEBUG
+  bool in_range = true;
+#pragma unroll
+  for (int z = 0; z < 16; ++z) {
+    const int a = static_cast<int8_t>(pk[z >> 2] >> (8 * (z & 3)));
+    in_range = in_range && a >= -h - 1 && a <= p - h;
+  }
+  OZK2_DCHECK(in_range, flags);
+#else
+  (void)flags;
+#endif
+  *out = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+}
+
+// Four exact-integer floats |r| < 2^7 as four int8 of one word, in order (the low bytes
+// of r + 1.5 2^23).
+__device__ __forceinline__ uint32_t pack4(float2 a, float2 b) {
+  const float2 x = __fadd2_rn(a, dup2(kMagic)), y = __fadd2_rn(b, dup2(kMagic));
+  return __byte_perm(__byte_perm(__float_as_uint(x.x), __float_as_uint(x.y), 0x0040),
+                     __byte_perm(__float_as_uint(y.x), __float_as_uint(y.y), 0x0040), 0x5410);
 }
 
 // GROUPED: the units of all `nprobs` problems of `probs` (tmA, tmB unused).  TN: tile width.
@@ -445,20 +458,20 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
           last_prob = uc.prob;
         }
         const int mod = uc.mod;
-        const UnitPlan up = plan_of<MODE>(uc.k, mod, uc.split);
+        const UnitPlan up = plan_of<MODE>(prm, uc.k, mod);
         for (int c = 0; ok && c < up.nchunks; ++c) {
           const int k0 = c * up.chunk_len;
           const int ksteps = (min(uc.k, k0 + up.chunk_len) - k0 + BK - 1) / BK;
           for (int ps = 0; ok && ps < up.npasses; ++ps) {
-            const int np = num_products<MODE>(mod, ps, uc.split);
+            const int np = num_products<MODE>(mod, ps);
             for (int s = 0; ok && s < ksteps; ++s) {
               for (int x = 0; x < np; ++x) {
                 if (!mbar_wait_bounded(empty + stage, phase ^ 1u, abort_flag, wait_ns)) {
                   ok = false;
                   break;
                 }
-                int pa, pb, acc;
-                product_of<MODE>(mod, ps, x, uc.split, pa, pb, acc);
+                int pa, pb;
+                product_of<MODE>(prm, mod, ps, x, pa, pb);
                 uint8_t* dst = tiles + stage * kStageBytes;
                 mbar_arrive_expect_tx(full + stage, kStageBytes);
                 tma_load_3d(dst, uc.ta, full + stage, k0 + s * BK, uc.tm * BM, pa);
@@ -496,56 +509,37 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
       for (int u = u_first; ok && u < prm.num_units; u += u_step) {
         resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
         const int mod = uc.mod;
-        const UnitPlan up = plan_of<MODE>(uc.k, mod, uc.split);
+        const UnitPlan up = plan_of<MODE>(prm, uc.k, mod);
         for (int c = 0; ok && c < up.nchunks; ++c) {
           const int k0 = c * up.chunk_len;
           const int ksteps = (min(uc.k, k0 + up.chunk_len) - k0 + BK - 1) / BK;
           for (int ps = 0; ok && ps < up.npasses; ++ps) {
-            const bool pair = pair_pass<MODE>(mod, uc.split);
-            const uint32_t first_slot = pair ? 0u : sl.next;
-            for (uint32_t j = 0; j < 2 && ok; ++j) {
-              if (!pair && j != first_slot) continue;
-              ok = mbar_wait_bounded(tempty + j, (sl.uses(j) & 1u) ^ 1u, abort_flag, wait_ns);
-            }
+            const uint32_t slot = sl.slot();
+            ok = mbar_wait_bounded(tempty + slot, (sl.uses() & 1u) ^ 1u, abort_flag, wait_ns);
             if (!ok) break;
             tc_fence_after();
-            const int np = num_products<MODE>(mod, ps, uc.split);
-            for (int s = 0; ok && s < ksteps; ++s) {
-              for (int x = 0; x < np; ++x) {
-                if (!mbar_wait_bounded(full + stage, phase, abort_flag, wait_ns)) {
-                  ok = false;
-                  break;
-                }
-                tc_fence_after();
-                int pa, pb, acc;
-                product_of<MODE>(mod, ps, x, uc.split, pa, pb, acc);
-                const bool first = s == 0 && (pair ? (x == 0 || x == 2) : x == 0);  // first into its slot
-                const uint32_t dtm = tmem_base + (first_slot + static_cast<uint32_t>(acc)) * static_cast<uint32_t>(BN);
-                const uint32_t sa = smem_addr(tiles + stage * kStageBytes);
-                const uint64_t adesc = sw128_kmajor_desc(sa);
-                const uint64_t bdesc = sw128_kmajor_desc(sa + kATileBytes);
+            const uint32_t dtm = tmem_base + slot * static_cast<uint32_t>(BN);
+            const int steps = ksteps * num_products<MODE>(mod, ps);
+            for (int s = 0; s < steps; ++s) {
+              if (!mbar_wait_bounded(full + stage, phase, abort_flag, wait_ns)) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+              const uint32_t sa = smem_addr(tiles + stage * kStageBytes);
+              const uint64_t adesc = sw128_kmajor_desc(sa);
+              const uint64_t bdesc = sw128_kmajor_desc(sa + kATileBytes);
 #pragma unroll
-                for (int kk = 0; kk < BK / 32; ++kk)
-                  mma_fp8(dtm, adesc + 2ull * kk, bdesc + 2ull * kk, idesc, (first && kk == 0) ? 0u : 1u);
-                mma_commit(empty + stage);
-                if (++stage == kStages) {
-                  stage = 0;
-                  phase ^= 1u;
-                }
+              for (int kk = 0; kk < BK / 32; ++kk)
+                mma_fp8(dtm, adesc + 2ull * kk, bdesc + 2ull * kk, idesc, (s == 0 && kk == 0) ? 0u : 1u);
+              mma_commit(empty + stage);
+              if (++stage == kStages) {
+                stage = 0;
+                phase ^= 1u;
               }
             }
-            if (pair) {
-              if (ok) {
-                mma_commit(tfull + 0);
-                mma_commit(tfull + 1);
-              }
-              sl.bump(0u);
-              sl.bump(1u);
-            } else {
-              if (ok) mma_commit(tfull + first_slot);
-              sl.bump(first_slot);
-              sl.next ^= 1u;
-            }
+            if (ok) mma_commit(tfull + slot);
+            ++sl.t;
           }
         }
       }
@@ -572,32 +566,28 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
     // stay in registers (the chunk loop unrolled).  An earlier form parked them in a
     // CTA-private scratch tile in L2; its round trips made short reductions up to 14%
     // slower.
-    uint32_t park[MODE == kModeResidue ? kChunks : 1][kCW / 2];
+    constexpr bool kResidues = MODE == kModeResidue || MODE == kModePaper;
+    uint32_t park[kResidues ? kChunks : 1][kCW / 2];
     Slots sl;  // the MMA thread's pass sequence, replayed
     bool ok = true;
     UnitCtx uc;
     for (int u = u_first; ok && u < prm.num_units; u += u_step) {
       resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
       const int mod = uc.mod, tn = uc.tn;
-      const UnitPlan up = plan_of<MODE>(uc.k, mod, uc.split);
+      const UnitPlan up = plan_of<MODE>(prm, uc.k, mod);
       const int gi = uc.tm * BM + row;
       for (int c = 0; ok && c < up.nchunks; ++c) {
         for (int ps = 0; ok && ps < up.npasses; ++ps) {
-          const bool pair = pair_pass<MODE>(mod, uc.split);
-          const uint32_t slot = pair ? 0u : sl.next;
-          for (uint32_t j = 0; j < 2 && ok; ++j) {
-            if (!pair && j != slot) continue;
-            ok = mbar_wait_bounded(tfull + j, sl.uses(j) & 1u, abort_flag, wait_ns);
-          }
+          const uint32_t slot = sl.slot();
+          ok = mbar_wait_bounded(tfull + slot, sl.uses() & 1u, abort_flag, wait_ns);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
           const uint32_t ts = tq + slot * static_cast<uint32_t>(BN);
-          if constexpr (MODE == kModeResidue) {
-            const int p = prm.mod.p[mod], h = prm.mod.half[mod], sq = prm.mod.s[mod];
-            const ModPair mp{dup2(-static_cast<float>(p)), dup2(prm.mod.inv_p[mod]), p == 1024};
-            const bool last = ps == up.npasses - 1;
-            int16_t* dst = uc.cres + static_cast<int64_t>(mod) * uc.res_stride + static_cast<int64_t>(gi) * uc.ldr;
+          if constexpr (kResidues) {
+            const GemmMod& gm = prm.mods.m[mod];
+            const int p = gm.p, h = gm.half;
+            const ModPair mp{dup2(-static_cast<float>(p)), dup2(gm.inv_p), MODE == kModePaper && p == 1024};
             // one chunk of kCW columns; sp: this thread's kCW parked int16 of the chunk, two per
             // word (registers: every index below is known at compile time)
             auto store4 = [](uint32_t* sp, int w, const uint32_t (&pk)[4]) {
@@ -608,50 +598,51 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
 #pragma unroll
               for (int z = 0; z < 4; ++z) pr[z] = sp[4 * w + z];
             };
-            // single problems: the pass's slot(s) go back to the MMA thread as soon as the last
+            // single problems: the pass's slot goes back to the MMA thread as soon as the last
             // chunk has been read from TMEM, before that chunk's arithmetic and stores (in the
             // grouped kernel the extra live state made it spill, and the release stays at the
             // end of the pass)
             auto release = [&]() {
               tc_fence_before();
-              if (pair) {
-                mbar_arrive(tempty + 0);
-                mbar_arrive(tempty + 1);
-              } else {
-                mbar_arrive(tempty + slot);
-              }
+              mbar_arrive(tempty + slot);
             };
-            auto chunk = [&](int cb, uint32_t* sp) {
-              const int gc = tn * BN + cgrp * kCols + cb * kCW;
-              const bool keep = gi < uc.m;  // this thread's row is inside the matrix
-              if (pair) {  // square modulus: X in slot 0, Z in slot 1
-                uint32_t vx[kCW], vz[kCW];
-                tmem_ld_cols(tq + cb * kCW, vx);
-                tmem_ld_cols(tq + BN + cb * kCW, vz);
-                tmem_ld_wait();
-                if (!GROUPED && cb == kChunks - 1) release();
-                // mod(s X + Z, p): X mod p first keeps s (X mod p) + Z below 2^24 (|X| <= 2^24,
-                // |Z| <= 2^23), so every step is exact
-#pragma unroll
-                for (int w = 0; w < kCW / 8; ++w) {
-                  uint32_t pk[4];
-#pragma unroll
-                  for (int z = 0; z < 4; ++z) {
-                    const int j = 8 * w + 2 * z;
-                    const float2 xr = mod_near2(bits2(vx[j], vx[j + 1]), mp);
-                    const float2 y = __ffma2_rn(dup2(static_cast<float>(sq)), xr, bits2(vz[j], vz[j + 1]));
-                    pk[z] = pack2(smod2(y, mp));
-                  }
-                  if (keep) store_residues8(dst, gc + 8 * w, uc.n, pk, c > 0, p, h, prm.flags);
-                }
-                return;
-              }
-              uint32_t v[kCW];
+            auto load = [&](int cb, uint32_t (&v)[kCW]) {
               tmem_ld_cols(ts + cb * kCW, v);
               tmem_ld_wait();
               if (!GROUPED && cb == kChunks - 1) release();
-              if (mod < kNumSquares) {  // square modulus in two passes
-                if (ps == 0) {  // park x = X mod p (|x| < 0.51 p)
+            };
+            const bool keep_row = gi < uc.m;  // this thread's row is inside the matrix
+            const int gc0 = tn * BN + cgrp * kCols;
+            const int64_t off = static_cast<int64_t>(gi) * uc.ldr;
+            if (MODE == kModeResidue && mod >= prm.mods.kars) {  // single modulus
+              int8_t* dst = uc.cres8 + static_cast<int64_t>(mod - prm.mods.kars) * uc.res_stride + off;
+#pragma unroll
+              for (int cb = 0; cb < kChunks; ++cb) {
+                uint32_t v[kCW];
+                load(cb, v);
+#pragma unroll
+                for (int w = 0; w < kCW / 16; ++w) {
+                  uint32_t pk[4];
+#pragma unroll
+                  for (int z = 0; z < 4; ++z) {
+                    const int j = 16 * w + 4 * z;
+                    pk[z] = pack4(mod_near2(bits2(v[j], v[j + 1]), mp), mod_near2(bits2(v[j + 2], v[j + 3]), mp));
+                  }
+                  const int gc = gc0 + cb * kCW + 16 * w;
+                  if (keep_row && gc < uc.n) store_residues16(dst, gc, pk, c > 0, p, h, prm.flags);
+                }
+              }
+            } else {
+              int16_t* dst = uc.cres + static_cast<int64_t>(mod) * uc.res_stride + off;
+              const bool square = MODE == kModePaper && mod < kNumSquares;
+              const bool last = ps == up.npasses - 1;
+              const float c1 = gm.c1, c2 = gm.c2, c3 = gm.c3;
+#pragma unroll
+              for (int cb = 0; cb < kChunks; ++cb) {
+                uint32_t* sp = park[cb];
+                uint32_t v[kCW];
+                load(cb, v);
+                if (ps == 0) {  // park x = X mod p or d1 = D1 mod p (|.| < 0.51 p)
 #pragma unroll
                   for (int w = 0; w < kCW / 8; ++w) {
                     uint32_t pk[4];
@@ -659,69 +650,43 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
                     for (int z = 0; z < 4; ++z) pk[z] = pack2(mod_near2(bits2(v[8 * w + 2 * z], v[8 * w + 2 * z + 1]), mp));
                     store4(sp, w, pk);
                   }
-                  return;
-                }
-                // C' = mod(s x + Z, p), as the one-pass form computes it
+                } else if (!last) {  // Karatsuba pass 2: park v = mod(c1 d1 + c2 D2, p); D2 mod p first
+                                     // keeps the sum below 2^21
 #pragma unroll
-                for (int w = 0; w < kCW / 8; ++w) {
-                  uint32_t pr[4];
-                  load4(sp, w, pr);
-                  uint32_t pk[4];
+                  for (int w = 0; w < kCW / 8; ++w) {
+                    uint32_t pr[4];
+                    load4(sp, w, pr);
+                    uint32_t pk[4];
 #pragma unroll
-                  for (int z = 0; z < 4; ++z) {
-                    const int j = 8 * w + 2 * z;
-                    const float2 y = __ffma2_rn(dup2(static_cast<float>(sq)), unpack2(pr[z]), bits2(v[j], v[j + 1]));
-                    pk[z] = pack2(smod2(y, mp));
+                    for (int z = 0; z < 4; ++z) {
+                      const int j = 8 * w + 2 * z;
+                      const float2 d2 = mod_near2(bits2(v[j], v[j + 1]), mp);
+                      const float2 y = __ffma2_rn(dup2(c2), d2, __fmul2_rn(dup2(c1), unpack2(pr[z])));
+                      pk[z] = pack2(mod_near2(y, mp));
+                    }
+                    store4(sp, w, pk);
                   }
-                  if (keep) store_residues8(dst, gc + 8 * w, uc.n, pk, c > 0, p, h, prm.flags);
-                }
-                return;
-              }
-              if (ps == 0) {  // Karatsuba pass 1: park d1 = mod(D1, p)
+                } else {
+                  // Karatsuba pass 3: C' = mod(v + c3 D3, p); D3 mod p first.  Square pass 2:
+                  // C' = mod(s x + Z, p), |s x| < 2^23 and |Z| <= 2^23
 #pragma unroll
-                for (int w = 0; w < kCW / 8; ++w) {
-                  uint32_t pk[4];
+                  for (int w = 0; w < kCW / 8; ++w) {
+                    uint32_t pr[4];
+                    load4(sp, w, pr);
+                    uint32_t pk[4];
 #pragma unroll
-                  for (int z = 0; z < 4; ++z) pk[z] = pack2(smod2(bits2(v[8 * w + 2 * z], v[8 * w + 2 * z + 1]), mp));
-                  store4(sp, w, pk);
-                }
-                return;
-              }
-              if (!last) {  // Karatsuba pass 2: park v = mod(240 d1 - 15 D2, p); D2 mod p first
-                            // keeps |240 d1 - 15 (D2 mod p)| below 2^17
-#pragma unroll
-                for (int w = 0; w < kCW / 8; ++w) {
-                  uint32_t pr[4];
-                  load4(sp, w, pr);
-                  uint32_t pk[4];
-#pragma unroll
-                  for (int z = 0; z < 4; ++z) {
-                    const int j = 8 * w + 2 * z;
-                    const float2 d2 = mod_near2(bits2(v[j], v[j + 1]), mp);
-                    const float2 y = __ffma2_rn(dup2(-15.0f), d2, __fmul2_rn(dup2(240.0f), unpack2(pr[z])));
-                    pk[z] = pack2(smod_small2(y, mp));
+                    for (int z = 0; z < 4; ++z) {
+                      const int j = 8 * w + 2 * z;
+                      const float2 d = bits2(v[j], v[j + 1]);
+                      if (square) pk[z] = pack2(smod2(__ffma2_rn(dup2(c1), unpack2(pr[z]), d), mp));
+                      else pk[z] = pack2(mod_near2(__ffma2_rn(dup2(c3), mod_near2(d, mp), unpack2(pr[z])), mp));
+                    }
+                    const int gc = gc0 + cb * kCW + 8 * w;
+                    if (keep_row && gc < uc.n) store_residues8<MODE == kModePaper>(dst, gc, pk, c > 0, p, h, prm.flags);
                   }
-                  store4(sp, w, pk);
                 }
-                return;
               }
-              // Karatsuba pass 3: C' = mod(v + 16 D3, p); D3 mod p first (|v + 16 (D3 mod p)| < 2^14)
-#pragma unroll
-              for (int w = 0; w < kCW / 8; ++w) {
-                uint32_t pr[4];
-                load4(sp, w, pr);
-                uint32_t pk[4];
-#pragma unroll
-                for (int z = 0; z < 4; ++z) {
-                  const int j = 8 * w + 2 * z;
-                  const float2 d3 = mod_near2(bits2(v[j], v[j + 1]), mp);
-                  pk[z] = pack2(smod_small2(__ffma2_rn(dup2(16.0f), d3, unpack2(pr[z])), mp));
-                }
-                if (keep) store_residues8(dst, gc + 8 * w, uc.n, pk, c > 0, p, h, prm.flags);
-              }
-            };
-#pragma unroll
-            for (int cb = 0; cb < kChunks; ++cb) chunk(cb, park[cb]);
+            }
           } else if constexpr (MODE == kModeBound) {
             float rmax = 0.0f;
             // 2^-s for an integer s clamped to [-126, 126] (an upper bound of 2^-s for
@@ -769,22 +734,11 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
               }
             }
           }
-          if constexpr (MODE != kModeResidue || GROUPED) {  // else the epilogue released the slot(s) itself
+          if constexpr (!kResidues || GROUPED) {  // else the epilogue released the slot itself
             tc_fence_before();
-            if (pair) {
-              mbar_arrive(tempty + 0);
-              mbar_arrive(tempty + 1);
-            } else {
-              mbar_arrive(tempty + slot);
-            }
+            mbar_arrive(tempty + slot);
           }
-          if (pair) {
-            sl.bump(0u);
-            sl.bump(1u);
-          } else {
-            sl.bump(slot);
-            sl.next ^= 1u;
-          }
+          ++sl.t;
         }
       }
     }
@@ -828,15 +782,6 @@ cudaError_t launch_tile(int tn, const GemmParams& prm, const CUtensorMap& ta, co
 
 int tile_width(int tile_n) { return tile_n == 128 ? 128 : 256; }
 
-void fill_mod(GemmParams& prm, const ModTable& mt) {
-  for (int l = 0; l < mt.N; ++l) {
-    prm.mod.p[l] = mt.p[l];
-    prm.mod.half[l] = mt.half[l];
-    prm.mod.s[l] = mt.s[l];
-    prm.mod.inv_p[l] = mt.inv_p[l];
-  }
-}
-
 }  // namespace
 
 cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, int planes_a, const uint8_t* b,
@@ -846,16 +791,17 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
   prm.m = g.m;
   prm.n = g.n;
   prm.k = g.k;
-  const int BN = tile_width(g.tile_n);
+  const int BN = g.mode == kModePaper ? 256 : tile_width(g.tile_n);
   prm.tiles_m = (g.m + BM - 1) / BM;
   prm.tiles_n = (g.n + BN - 1) / BN;
   prm.tiles = prm.tiles_m * prm.tiles_n;
-  const int nmod = (g.mode == kModeResidue) ? g.mt->N : 1;
-  prm.num_units = prm.tiles * nmod;
+  const bool residues = g.mode == kModeResidue || g.mode == kModePaper;
+  if (residues) prm.mods = *g.mods;
+  prm.num_units = prm.tiles * (residues ? prm.mods.count : 1);
   prm.cres = g.cres;
+  prm.cres8 = g.cres8;
   prm.ldr = g.ldr;
   prm.res_stride = g.res_stride;
-  if (g.mode == kModeResidue) fill_mod(prm, *g.mt);
   prm.factor = g.factor;
   prm.R = g.R;
   prm.S = g.S;
@@ -866,7 +812,6 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
   prm.rowshift = g.rowshift;
   prm.wait_ns = g.wait_ns;
   prm.stall = g.stall ? 1 : 0;
-  prm.split_squares = g.split_squares ? 1 : 0;
 
   CUtensorMap ta, tb;
   if (!encode_fp8_map(&ta, a, g.k, g.m, planes_a, lda8, g.plane_stride_a, BM, BK)) return cudaErrorInvalidValue;
@@ -876,6 +821,8 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
   switch (g.mode) {
     case kModeResidue:
       return launch_tile<kModeResidue, false>(BN, prm, ta, tb, grid, nullptr, 0, st);
+    case kModePaper:
+      return launch_mode<kModePaper, false, 256>(prm, ta, tb, grid, nullptr, 0, st);
     case kModeBound:
       return launch_tile<kModeBound, false>(BN, prm, ta, tb, grid, nullptr, 0, st);
     default:
@@ -886,7 +833,7 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
 int64_t fp8_gemm_units(int mode, int m, int n, int N, int tile_n) {
   const int BN = tile_width(tile_n);
   const int64_t tiles = static_cast<int64_t>((m + BM - 1) / BM) * ((n + BN - 1) / BN);
-  return tiles * (mode == kModeResidue ? N : 1);
+  return tiles * (mode == kModeResidue ? rns_moduli(N) : 1);
 }
 
 bool encode_gemm_problem(GemmProblem* gp, const uint8_t* a, const uint8_t* b, int64_t ld8, int planes, int m, int n,
@@ -913,7 +860,7 @@ cudaError_t launch_fp8_gemm_grouped(const GemmArgs& g, const GemmProblem* probs,
   prm.flags = g.flags;
   prm.wait_ns = g.wait_ns;
   prm.stall = g.stall ? 1 : 0;
-  if (g.mode == kModeResidue) fill_mod(prm, *g.mt);
+  if (g.mode == kModeResidue) prm.mods = *g.mods;
   CUtensorMap unused;
   std::memset(&unused, 0, sizeof(unused));
   const int ctas = g.num_sms < kMaxGemmCtas ? g.num_sms : kMaxGemmCtas;

@@ -9,6 +9,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "rns.h"
+
 namespace ozk2 {
 
 constexpr int kMaxModuli = 20;
@@ -44,6 +46,55 @@ struct ModTable {
   float2 w2[kMaxModuli][5];
 };
 
+// The product path's residue system (rns.h): constants of the residue kernels, per
+// remainder taken (pairs of single moduli, then Karatsuba moduli).  FP32 constants are
+// duplicated pairs, as above.
+struct RnsTable {
+  int N;
+  int singles, pairs, kars;
+  int pair_words, lut_words;                // 16-byte words of the pairs' digit tables, of all
+  float2 neg_m2[kMaxVirtual], inv_m2[kMaxVirtual];
+  float2 w2[kMaxVirtual][5];                // 2^(11 j) mod M, symmetric
+  int16_t pow2[kMaxVirtual][kPow2Table];    // 2^t mod M, symmetric
+  int32_t lut_bias[kMaxVirtual];            // byte offset of remainder 0 in the block's digit
+                                            // tables, minus the bits of 1.5 2^23
+};
+
+// One modulus of the FP8 products' epilogue.
+struct GemmMod {
+  int p, half;
+  float inv_p;
+  float c1, c2, c3;  // Karatsuba: r r' = c1 D1 + c2 D2 + c3 D3 (mod p); a square s^2: c1 = s
+  int chunk;         // terms per exactness block
+};
+struct GemmMods {
+  int count;  // moduli
+  int kars;   // product path: moduli [0, kars) are Karatsuba, the rest single
+  int planes;
+  GemmMod m[kMaxRns];
+};
+
+// CRT of the product path: sum_l c_l w_l with w_l = y_l P2 / p_l is formed as
+// sum_g t_g P2 / P_g, t_g = sum_{l in g} c_l u_l an int32 (u_l = y_l P_g / p_l), over small
+// groups g of moduli with product P_g.
+constexpr int kCrtSingleGroup = 4;  // single moduli per group
+OZK2_HD constexpr int crt_kar_group(int N) { return kRnsKars[N] <= 6 ? 2 : 1; }  // 64-bit limb sums bound it
+OZK2_HD constexpr int crt_groups(int N) {
+  return (kRnsSingles[N] + kCrtSingleGroup - 1) / kCrtSingleGroup + (kRnsKars[N] + crt_kar_group(N) - 1) / crt_kar_group(N);
+}
+constexpr int kMaxCrtGroups = 16;
+// Bits of P2 for N (checked by build_rns_crt).
+constexpr int kRnsBits[21] = {0,  12,  22,  33,  42,  52,  61,  68,  77,  87, 96,
+                              106, 113, 122, 132, 140, 149, 157, 167, 175, 183};
+OZK2_HD constexpr int rns_limbs(int N) { return kRnsBits[N] <= 95 ? 3 : (kRnsBits[N] + 1 + 31) / 32; }  // signed |x| < P2
+struct RnsCrt {
+  int N;
+  int32_t u[kMaxRns];                          // Karatsuba moduli first, as in the products
+  int32_t wb[kMaxCrtGroups][kMaxLimbs];        // P2 / P_g in balanced 32-bit limbs; Karatsuba groups first
+  uint32_t P[kMaxLimbs];
+  float est_hi, est_lo;                        // V / P2 from V's limbs (crt.cu)
+};
+
 struct CrtTable {
   int N;
   int limbs;                               // L, 32-bit limbs of the signed result
@@ -74,10 +125,15 @@ int validate_dgemm(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda
 int dgemm_library_ws(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,
                      double* C, int64_t ldc, int N, void* ws, size_t ws_bytes, cudaStream_t st);
 
-// Host-side constant generation (moduli.cpp)
+// Host-side constant generation (moduli.cpp).  The hybrid list's residues, digits and CRT
+// (ModTable, CrtTable) serve the parity hooks; the product path uses rns.h's system.
 bool build_mod_table(int N, ModTable* mt);
 bool build_crt_table(int N, CrtTable* ct);
 int hybrid_moduli(int N, int* out);  // returns N or -1
+bool build_rns_table(int N, RnsTable* rt);
+bool build_gemm_mods(int N, GemmMods* gm);    // the product path
+bool build_paper_mods(int N, GemmMods* gm);   // the hybrid list (parity hook)
+bool build_rns_crt(int N, RnsCrt* rc);
 float p_prime_f32(int N);            // RD_fp32((log2(P - 1) - 1) / 2)
 float delta_f32();                   // RD_fp32(-1 / (2 - 2^-21))
 float reuse_budget_f32(int N);       // RD_fp32(log2(P - 1) - 1), the budget of one side
@@ -110,39 +166,46 @@ cudaError_t launch_reuse_exponents(int m, const int32_t* gp, const uint8_t* rsta
                                    const int32_t* hp, const uint8_t* cstat, const float* S, int32_t* h, float q,
                                    uint32_t* flags, cudaStream_t st);
 
-// resid.cu.  Planes: M_N planes of lines x kp bytes, row pitch ldp bytes (>= kp, a
+// resid.cu.  Planes: rns_planes(N) planes of lines x kp bytes, row pitch ldp bytes (>= kp, a
 // multiple of 16), plane stride plane_stride bytes (0: lines * ldp; larger when the
 // lines converted are a slice of a taller operand).
 cudaError_t launch_residues_rows(const double* A, int64_t lda, int m, int k, int kp, int64_t ldp,
-                                 const int32_t* e, const ModTable& mt, uint8_t* planes,
+                                 const int32_t* e, const RnsTable& rt, uint8_t* planes,
                                  uint32_t* flags, cudaStream_t st, int64_t plane_stride = 0);
 cudaError_t launch_residues_cols(const double* B, int64_t ldb, int k, int n, int kp, int64_t ldp,
-                                 const int32_t* f, const ModTable& mt, uint8_t* planes,
+                                 const int32_t* f, const RnsTable& rt, uint8_t* planes,
                                  uint32_t* flags, cudaStream_t st, int64_t plane_stride = 0);
+// The hybrid list's digit planes (parity hooks), packed.
+cudaError_t launch_paper_planes_rows(const double* A, int64_t lda, int m, int k, int kp, const int32_t* e,
+                                     const ModTable& mt, uint8_t* planes, uint32_t* flags, cudaStream_t st);
+cudaError_t launch_paper_planes_cols(const double* B, int64_t ldb, int k, int n, int kp, const int32_t* f,
+                                     const ModTable& mt, uint8_t* planes, uint32_t* flags, cudaStream_t st);
 
 // Gradient operands (resid.cu): the digit planes of G'_ij = trunc(2^(g_i - f_j) dC_ij)
 // (m lines along j, pitch ldg) and of H'_ij = trunc(2^(h_j - e_i) dC_ij) (n lines along i,
 // pitch ldh) from one read of dC; a null plane pointer skips that output.
 cudaError_t launch_grad_residues(const double* dC, int64_t lddc, int m, int n, const int32_t* g, const int32_t* f,
                                  const int32_t* h, const int32_t* e, uint8_t* planesG, int64_t ldg, uint8_t* planesH,
-                                 int64_t ldh, const ModTable& mt, uint32_t* flags, cudaStream_t st);
+                                 int64_t ldh, const RnsTable& rt, uint32_t* flags, cudaStream_t st);
 // dst[p][x][y] = src[p][y][x], y < lines, x < len (pitches and strides multiples of 16;
 // src_pitch >= len and dst_pitch >= lines, both rounded up to 16).
 cudaError_t launch_transpose_planes(const uint8_t* src, int64_t src_pitch, int64_t src_stride, int lines, int len,
                                     uint8_t* dst, int64_t dst_pitch, int64_t dst_stride, int planes, cudaStream_t st);
 
 // gemm.cu
-enum GemmMode { kModeResidue = 0, kModeBound = 1, kModeRaw = 2 };
+enum GemmMode { kModeResidue = 0, kModeBound = 1, kModeRaw = 2, kModePaper = 3 };
 
 struct GemmArgs {
   int mode;
   int m, n, k;
   int num_sms;
-  // residue products
+  // residue products (kModeResidue: `cres` the Karatsuba moduli's planes, `cres8` the single
+  // moduli's; kModePaper: `cres` only)
   int16_t* cres;
-  int64_t ldr;          // int16 elements per row of a residue plane
+  int8_t* cres8;
+  int64_t ldr;          // elements per row of a residue plane (a multiple of 16)
   int64_t res_stride;   // elements between residue planes
-  const ModTable* mt;
+  const GemmMods* mods;
   // bound product
   float factor;
   float* R;
@@ -160,7 +223,6 @@ struct GemmArgs {
   unsigned long long wait_ns;  // limit of each device wait (wait_limit_ns())
   bool stall;                  // fault injection: the kernel's first MMA wait never completes
   int tile_n;                  // output tile width: 128, or 256 (any other value)
-  bool split_squares;          // residue products: square moduli in two single-slot passes
 };
 // A operand: `planes_a` digit planes (K-major, m x k bytes, row stride lda8 bytes, plane
 // stride plane_stride_a); B operand the same with n rows.
@@ -169,10 +231,12 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
                             const uint8_t* b, int64_t ldb8, int planes_b, cudaStream_t st);
 
 // crt.cu
-cudaError_t launch_crt(const int16_t* cres, int64_t ldr, int64_t res_stride, int m, int n,
-                       const int32_t* e, const int32_t* f, const uint8_t* rowstat,
-                       const uint8_t* colstat, double* C, int64_t ldc, const CrtTable& ct,
-                       cudaStream_t st);
+cudaError_t launch_crt(const int16_t* cres, const int8_t* cres8, int64_t ldr, int64_t res_stride, int m, int n,
+                       const int32_t* e, const int32_t* f, const uint8_t* rowstat, const uint8_t* colstat, double* C,
+                       int64_t ldc, const RnsCrt& ct, cudaStream_t st);
+// From the hybrid list's residues (parity hook).
+cudaError_t launch_paper_crt(const int16_t* cres, int64_t ldr, int64_t res_stride, int m, int n, const int32_t* e,
+                             const int32_t* f, double* C, int64_t ldc, const CrtTable& ct, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Grouped launches: one launch of a kernel serves every problem of a batch.  Problem p
@@ -217,13 +281,14 @@ struct BatchProblem {
   uint8_t* planesA;
   uint8_t* planesB;
   int16_t* cres;
+  int8_t* cres8;
   int64_t first_block[kBatchKernels];
   int64_t nblocks[kBatchKernels];
 };
 
 // Tile of the column residue kernel: kResidTileCols columns x kResidTileK k per block
 // (one block per tile in a grouped launch).
-constexpr int kResidTileCols = 64, kResidTileK = 128;
+constexpr int kResidTileCols = 32, kResidTileK = 128;
 
 // Items of the row residue kernel: a warp covers 2^s lanes x 8 k of 32 / 2^s rows, s = 4
 // (128 consecutive k of two rows) for kp > 64, else the smallest s with 2^s 8 >= kp (kp is
@@ -256,9 +321,9 @@ cudaError_t launch_scale_batch(const BatchProblem* probs, int count, const int64
 cudaError_t launch_exponents_batch(const BatchProblem* probs, int count, int64_t total_blocks, float pprime,
                                    float delta, cudaStream_t st);
 cudaError_t launch_residues_batch(const BatchProblem* probs, int count, int64_t rows_blocks,
-                                  int64_t cols_blocks, const ModTable& mt, uint32_t* flags, cudaStream_t st,
+                                  int64_t cols_blocks, const RnsTable& rt, uint32_t* flags, cudaStream_t st,
                                   cudaStream_t st_cols);
-cudaError_t launch_crt_batch(const BatchProblem* probs, int count, int64_t total_blocks, const CrtTable& ct,
+cudaError_t launch_crt_batch(const BatchProblem* probs, int count, int64_t total_blocks, const RnsCrt& ct,
                              cudaStream_t st);
 
 // One problem of a grouped GEMM launch: its operand maps and outputs.  Units (tile x
@@ -270,16 +335,16 @@ struct GemmProblem {  // CUtensorMap carries the 64-byte alignment TMA needs
   int tiles_m, tiles_n, tiles;
   int64_t unit_start;
   int16_t* cres;
+  int8_t* cres8;
   int64_t ldr;
   int64_t res_stride;
   float factor;
   float* R;
   float* S;
-  int split;  // residue products: square moduli in two single-slot passes
 };
 // Units of one problem in a GEMM of mode `mode` with N moduli and tiles of width tile_n.
 int64_t fp8_gemm_units(int mode, int m, int n, int N, int tile_n);
-// g supplies mode, num_sms, mt and flags; the problems (device memory, built on
+// g supplies mode, num_sms, mods and flags; the problems (device memory, built on
 // the host with encode_gemm_problem) supply everything else.
 cudaError_t launch_fp8_gemm_grouped(const GemmArgs& g, const GemmProblem* probs, int count, int64_t total_units,
                                     cudaStream_t st);

@@ -224,6 +224,175 @@ bool build_crt_table(int N, CrtTable* ct) {
   return true;
 }
 
+namespace {
+
+// the product path's moduli in product order: Karatsuba, then single
+std::vector<int> rns_list(int N) {
+  std::vector<int> p;
+  for (int j = 0; j < kRnsKars[N]; ++j) p.push_back(kKarP[j]);
+  for (int i = 0; i < kRnsSingles[N]; ++i) p.push_back(kSingleP[i]);
+  return p;
+}
+
+Big rns_product(int N) {
+  Big P{1u};
+  for (int p : rns_list(N)) P = mul_small(P, static_cast<uint32_t>(p));
+  return P;
+}
+
+int symmetric(int v, int p) { return v > p / 2 ? v - p : v; }  // of v in [0, p)
+
+// balanced 32-bit limbs of x >= 0; false if they do not fit
+bool balanced_limbs(const Big& x, int limbs, int32_t* out) {
+  int64_t carry = 0;
+  for (int t = 0; t < limbs; ++t) {
+    int64_t u = (t < static_cast<int>(x.size()) ? static_cast<int64_t>(x[t]) : 0) + carry;
+    carry = u >= (int64_t(1) << 31) ? 1 : 0;
+    out[t] = static_cast<int32_t>(u - (carry << 32));
+  }
+  return carry == 0 && static_cast<int>(x.size()) <= limbs;
+}
+
+}  // namespace
+
+bool build_rns_table(int N, RnsTable* rt) {
+  if (N < 1 || N > kMaxModuli) return false;
+  std::memset(rt, 0, sizeof(*rt));
+  rt->N = N;
+  rt->singles = kRnsSingles[N];
+  rt->pairs = rns_pairs(N);
+  rt->kars = kRnsKars[N];
+  rt->pair_words = pair_lut_offset(rt->pairs) / 16;
+  rt->lut_words = rns_lut_bytes(N) / 16;
+  for (int v = 0; v < rns_virtual(N); ++v) {
+    const bool kar = v >= rt->pairs;
+    const int M = kar ? kKarP[v - rt->pairs] : pair_modulus(v);
+    rt->neg_m2[v] = make_float2(-static_cast<float>(M), -static_cast<float>(M));
+    const float inv = static_cast<float>(1.0 / M);
+    rt->inv_m2[v] = make_float2(inv, inv);
+    int x = 1;
+    for (int t = 0; t < kPow2Table; ++t) {
+      rt->pow2[v][t] = static_cast<int16_t>(symmetric(x, M));
+      if (t % 11 == 0 && t / 11 < 5) {
+        const float w = static_cast<float>(symmetric(x, M));
+        rt->w2[v][t / 11] = make_float2(w, w);
+      }
+      x = 2 * x % M;
+    }
+    const int entry = kar ? 4 : 2;
+    const int base = kar ? pair_lut_offset(rt->pairs) + kar_lut_offset(v - rt->pairs) : pair_lut_offset(v);
+    rt->lut_bias[v] = base + entry * (M / 2 + 1) - 0x4B400000;
+  }
+  return true;
+}
+
+bool build_gemm_mods(int N, GemmMods* gm) {
+  if (N < 1 || N > kMaxModuli) return false;
+  std::memset(gm, 0, sizeof(*gm));
+  gm->count = rns_moduli(N);
+  gm->kars = kRnsKars[N];
+  gm->planes = rns_planes(N);
+  // the workspace's plane regions hold the hybrid list's M_N planes
+  if (gm->planes > ((N <= kNumSquares) ? 2 * N : 3 * N - kNumSquares)) return false;
+  const std::vector<int> mods = rns_list(N);
+  for (int l = 0; l < gm->count; ++l) {
+    GemmMod& m = gm->m[l];
+    const int p = mods[static_cast<size_t>(l)];
+    m.p = p;
+    m.half = p / 2;
+    m.inv_p = static_cast<float>(1.0 / p);
+    if (l < gm->kars) {
+      const int b = kKarBeta[l];
+      m.c1 = static_cast<float>(symmetric(((1 - b) % p + p) % p, p));
+      m.c2 = static_cast<float>(symmetric(static_cast<int>((static_cast<int64_t>(b) * b - b) % p), p));
+      m.c3 = static_cast<float>(symmetric(b, p));
+      m.chunk = chunk_terms(kDigitMax);
+    } else {
+      m.chunk = chunk_terms(single_digit_max(p));
+    }
+  }
+  return true;
+}
+
+bool build_paper_mods(int N, GemmMods* gm) {
+  int mods[kMaxModuli];
+  if (hybrid_moduli(N, mods) != N) return false;
+  std::memset(gm, 0, sizeof(*gm));
+  gm->count = N;
+  gm->planes = (N <= kNumSquares) ? 2 * N : 3 * N - kNumSquares;
+  for (int l = 0; l < N; ++l) {
+    GemmMod& m = gm->m[l];
+    m.p = mods[l];
+    m.half = m.p / 2;
+    m.inv_p = static_cast<float>(1.0 / m.p);
+    if (l < kNumSquares) {
+      m.c1 = static_cast<float>(std::lround(std::sqrt(static_cast<double>(m.p))));
+      m.chunk = 32768;  // X accumulates two products: 2 2^15 16 16 = 2^24
+    } else {
+      m.c1 = 240.0f;  // 256 D1 + D2 + 16 (D3 - D1 - D2)
+      m.c2 = -15.0f;
+      m.c3 = 16.0f;
+      m.chunk = 65536;  // 2^16 16 16 = 2^24
+    }
+  }
+  return true;
+}
+
+bool build_rns_crt(int N, RnsCrt* rc) {
+  if (N < 1 || N > kMaxModuli) return false;
+  std::memset(rc, 0, sizeof(*rc));
+  rc->N = N;
+  const std::vector<int> mods = rns_list(N);
+  const Big P = rns_product(N);
+  if (bit_length(P) != kRnsBits[N]) return false;
+  {  // the slack the rounded quotient relies on: 10 P2 >= 11 P
+    int mp[kMaxModuli];
+    if (hybrid_moduli(N, mp) != N) return false;
+    int e2, e1;
+    const double p2 = top_as_double(P, &e2), p1 = top_as_double(product_of(N), &e1);
+    if (std::ldexp(p2, e2 - e1) < 1.1 * p1) return false;
+  }
+  const int L = rns_limbs(N), kars = kRnsKars[N], total = rns_moduli(N);
+  auto big_div_mod = [](const Big& x, int p, Big* q) {
+    uint32_t rem = 0;
+    Big d = div_small(x, static_cast<uint32_t>(p), &rem);
+    if (q) *q = d;
+    return static_cast<int>(rem);
+  };
+  int g = 0;
+  for (int l0 = 0; l0 < total; ++g) {
+    const int size = l0 < kars ? crt_kar_group(N) : kCrtSingleGroup;
+    const int l1 = l0 < kars ? (l0 + size < kars ? l0 + size : kars) : (l0 + size < total ? l0 + size : total);
+    int64_t Pg = 1;
+    Big rest = P;
+    for (int l = l0; l < l1; ++l) {
+      Pg *= mods[static_cast<size_t>(l)];
+      big_div_mod(rest, mods[static_cast<size_t>(l)], &rest);
+    }
+    int64_t tmax = 0;
+    for (int l = l0; l < l1; ++l) {
+      const int p = mods[static_cast<size_t>(l)];
+      Big pl;
+      big_div_mod(P, p, &pl);  // P2 / p
+      const int y = symmetric(modinv(big_div_mod(pl, p, nullptr), p), p);
+      const int64_t u = static_cast<int64_t>(y) * (Pg / p);
+      rc->u[l] = static_cast<int32_t>(u);
+      tmax += (p / 2 + 1) * (u < 0 ? -u : u);  // residues |c| <= p / 2 + 1
+    }
+    if (tmax >= (int64_t(1) << 31) || g >= kMaxCrtGroups || !balanced_limbs(rest, L, rc->wb[g])) return false;
+    l0 = l1;
+  }
+  if (g != crt_groups(N)) return false;
+  for (size_t t = 0; t < P.size(); ++t) rc->P[t] = P[t];
+  // quotient estimate: see crt.cu; scale of one unit of limb TL (or of 2^13 of them) in P2s
+  int eP;
+  const double Pt = top_as_double(P, &eP);
+  const int TL = (kRnsBits[N] - 1) / 32, tb = kRnsBits[N] - 32 * TL;
+  rc->est_hi = static_cast<float>(std::ldexp(1.0 / Pt, 32 * TL + (tb <= 18 ? 0 : 13) - eP));
+  rc->est_lo = static_cast<float>(std::ldexp(1.0 / Pt, 32 * (TL - 1) - eP));
+  return true;
+}
+
 float p_prime_f32(int N) {
   int mods[kMaxModuli];
   if (hybrid_moduli(N, mods) != N) return NAN;

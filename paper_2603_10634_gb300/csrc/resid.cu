@@ -8,11 +8,16 @@
 //                    d3 = d1 + d2                                (Sec. III-B)
 // and each digit (|d| <= 16, exact in E4M3) is stored as an E4M3 byte in its plane.
 //
+// Those are the digits of the hybrid list; the parity hooks return them (PaperSys below).
+// The product path converts to the residue system of rns.h instead (RnsSys): remainders
+// mod 11 to 20 moduli of at most 2303, each looked up in a table of digit bytes.
+//
 // a' is never formed as a wide integer or a double.  With a = M 2^E (M the 53-bit
 // significand) and t = E + e: a' = M' 2^t', where M' = M >> -t, t' = 0 if t < 0 and
 // M' = M, t' = t otherwise.  M' is split once into five signed 11-bit pieces c_j
 // (exact floats), and for each modulus
 //   x = sum_j c_j w_j,   w_j = 2^(11j) mod p in [-p/2, p/2],   |x| <= 5 (2^11 - 1) 544 < 2^23
+// (RnsSys: |w_j| <= 1151, |x| < 2^24)
 // is formed with exact FP32 fused multiply-adds.  For odd p the exact product x (1/p)
 // rounded once (see reduce) differs from x / p by at most |x| 2^-24 / p < 1/(2p), less
 // than the distance from x / p to any half-integer, so q is the nearest integer to x / p
@@ -25,6 +30,7 @@
 // (plane rows are columns of B), so both operands of the tensor-core products are
 // K-major.  Each thread owns 8 elements.
 #include <algorithm>
+#include <atomic>
 
 #include <cuda_fp8.h>
 
@@ -318,6 +324,197 @@ __device__ __forceinline__ void task_planes(int N, const Tables& tb, const f2 (&
   else all_planes<false>(N, tb, c, tp, st, flags);
 }
 
+// ------------------------------------------------------------------ residue systems
+// What the kernels below are templated on: the constants a block stages in shared memory
+// and the conversion of a task's 8 elements to every plane.
+struct PaperSys {  // the hybrid list's digits (parity hooks)
+  using Table = ModTable;
+  static size_t smem_bytes(const Table&) { return sizeof(Tables); }
+  static __device__ __forceinline__ void load(const Table& mt, unsigned char* smem) {
+    load_tables(mt, *reinterpret_cast<Tables*>(smem));
+  }
+  static __device__ __forceinline__ void planes(const Table& mt, const unsigned char* smem,
+                                                const f2 (&c)[kPairs][kPieces], const TpPack& tp, int any_tp,
+                                                const PlaneStore& st, uint32_t* flags) {
+    task_planes(mt.N, *reinterpret_cast<const Tables*>(smem), c, tp, any_tp, st, flags);
+  }
+};
+
+// Digit tables of rns.h, indexed by the remainder: the digit bytes of both single moduli
+// of a pair (16-bit entries), and of u, v, w of a Karatsuba modulus (32-bit entries).
+struct alignas(16) PairLut {
+  uint16_t v[kPairLutBytes / 2];
+};
+struct alignas(16) KarLut {
+  uint32_t v[kKarLutBytes / 4];
+};
+constexpr PairLut make_pair_lut() {
+  PairLut t{};
+  for (int q = 0; q < kPairs1; ++q) {
+    const int M = pair_modulus(q), h1 = M / 2 + 1, o = pair_lut_offset(q) / 2;
+    const int p0 = kSingleP[2 * q], p1 = 2 * q + 1 < kSingles ? kSingleP[2 * q + 1] : 1;
+    for (int r = -h1; r <= h1; ++r)
+      t.v[o + r + h1] = static_cast<uint16_t>(e4m3_of_digit(single_digit(r, p0)) | (e4m3_of_digit(single_digit(r, p1)) << 8));
+  }
+  return t;
+}
+constexpr KarLut make_kar_lut() {
+  KarLut t{};
+  for (int j = 0; j < kKars; ++j) {
+    const int p = kKarP[j], b = kKarBeta[j], h1 = p / 2 + 1, o = kar_lut_offset(j) / 4;
+    bool seen[1300] = {};
+    // smallest digits first
+    for (int mx = 0; mx <= kDigitMax; ++mx) {
+      if (!digit_ok(mx)) continue;
+      for (int a = -mx; a <= mx; ++a) {
+        if (!digit_ok(a)) continue;
+        for (int side = 0; side < 4; ++side) {
+          const int u = side == 0 ? mx : side == 1 ? -mx : a, v = side == 2 ? mx : side == 3 ? -mx : a;
+          const int w = u + v;
+          if ((w < 0 ? -w : w) > kDigitMax || !digit_ok(w)) continue;
+          const int r = symmetric_mod(u + b * v, p);
+          if (seen[r + h1]) continue;
+          seen[r + h1] = true;
+          t.v[o + r + h1] = e4m3_of_digit(u) | (e4m3_of_digit(v) << 8) | (e4m3_of_digit(w) << 16);
+        }
+      }
+    }
+    // the slack entries repeat the residue they stand for
+    t.v[o] = t.v[o + p];
+    t.v[o + 2 * h1] = t.v[o + 2 * h1 - p];
+  }
+  return t;
+}
+__device__ const PairLut g_pair_lut = make_pair_lut();
+__device__ const KarLut g_kar_lut = make_kar_lut();
+
+struct __align__(16) RnsConsts {
+  f2 neg_m, inv_m;
+  f2 w[kPieces];
+  int bias, pad;  // byte offset of remainder 0's entry, minus the bits of 1.5 2^23
+};
+
+struct RnsSys {  // the product path's digits
+  using Table = RnsTable;
+  // shared memory: constants, 2^t mod M (64 floats each), digit tables
+  static constexpr int kPerModulus = static_cast<int>(sizeof(RnsConsts)) + 4 * kPow2Table;
+  static size_t smem_bytes(const Table& rt) {
+    return static_cast<size_t>(rns_virtual(rt.N)) * kPerModulus + static_cast<size_t>(rns_lut_bytes(rt.N));
+  }
+  static __device__ __forceinline__ void load(const Table& rt, unsigned char* smem) {
+    const int nv = rt.pairs + rt.kars;
+    RnsConsts* cs = reinterpret_cast<RnsConsts*>(smem);
+    float* pow2 = reinterpret_cast<float*>(smem + nv * sizeof(RnsConsts));
+    uint4* lut = reinterpret_cast<uint4*>(smem + nv * kPerModulus);
+    const uint4* pl = reinterpret_cast<const uint4*>(&g_pair_lut);
+    const uint4* kl = reinterpret_cast<const uint4*>(&g_kar_lut);
+    for (int i = threadIdx.x; i < rt.lut_words; i += blockDim.x)
+      lut[i] = __ldg(i < rt.pair_words ? pl + i : kl + (i - rt.pair_words));
+    for (int i = threadIdx.x; i < nv * kPow2Table; i += blockDim.x)
+      pow2[i] = static_cast<float>(rt.pow2[i / kPow2Table][i % kPow2Table]);
+    for (int v = threadIdx.x; v < nv; v += blockDim.x) {
+      RnsConsts& c = cs[v];
+      c.neg_m = rt.neg_m2[v];
+      c.inv_m = rt.inv_m2[v];
+#pragma unroll
+      for (int j = 0; j < kPieces; ++j) c.w[j] = rt.w2[v][j];
+      c.bias = rt.lut_bias[v];
+      c.pad = 0;
+    }
+    __syncthreads();
+  }
+
+  // Table entries (byte offsets scaled by 4 or 2: entry size) of an element pair's
+  // remainders.  x = sum_j c_j w_j is an exact integer below 2^24; the rounded quotient
+  // is within 1/2 + 1/M of x / M, so the remainder lies within the table's slack.
+  template <bool P2>
+  static __device__ __forceinline__ int2 entry(const f2 (&c)[kPieces], int tp0, int tp1, const RnsConsts& k,
+                                               const float* pow2, float scale) {
+    f2 x = c[0];
+#pragma unroll
+    for (int j = 1; j < kPieces; ++j) x = __ffma2_rn(c[j], k.w[j], x);
+    f2 r = __ffma2_rn(k.neg_m, round_magic(__ffma2_rn(x, k.inv_m, dup(kMagic))), x);
+    if constexpr (P2) {
+      x = __fmul2_rn(r, make_float2(pow2[tp0], pow2[tp1]));  // below 2^21
+      r = __ffma2_rn(k.neg_m, round_magic(__ffma2_rn(x, k.inv_m, dup(kMagic))), x);
+    }
+    const f2 y = __ffma2_rn(r, dup(scale), dup(kMagic));  // bits: those of 1.5 2^23, plus scale r
+    return make_int2(__float_as_int(y.x) + k.bias, __float_as_int(y.y) + k.bias);
+  }
+
+  static __device__ __forceinline__ void check(const uint32_t (&w)[2], uint32_t* flags) {
+    // every digit |d| <= 32: E4M3 magnitude code at most 0x60 (= 32)
+    OZK2_DCHECK(__vcmpgtu4(w[0] & 0x7F7F7F7Fu, 0x60606060u) == 0u && __vcmpgtu4(w[1] & 0x7F7F7F7Fu, 0x60606060u) == 0u,
+                flags);
+  }
+
+  // Every plane of a task, one remainder at a time (rolled loops: see all_planes).
+  template <bool P2>
+  static __device__ __forceinline__ void all(const Table& rt, const unsigned char* smem,
+                                             const f2 (&c)[kPairs][kPieces], const TpPack& tp, PlaneStore st,
+                                             uint32_t* flags) {
+    const int nv = rt.pairs + rt.kars;
+    const RnsConsts* cs = reinterpret_cast<const RnsConsts*>(smem);
+    const float* pow2 = reinterpret_cast<const float*>(smem + nv * sizeof(RnsConsts));
+    const unsigned char* lut = smem + nv * kPerModulus;
+#pragma unroll 1
+    for (int v = rt.pairs; v < nv; ++v) {
+      uint32_t w[3][2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        uint32_t e[4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int pr = 2 * q + u;
+          const int2 i = entry<P2>(c[pr], tp_of(tp, 2 * pr), tp_of(tp, 2 * pr + 1), cs[v], pow2 + v * kPow2Table, 4.0f);
+          e[2 * u] = *reinterpret_cast<const uint32_t*>(lut + i.x);
+          e[2 * u + 1] = *reinterpret_cast<const uint32_t*>(lut + i.y);
+        }
+        const uint32_t a = __byte_perm(e[0], e[1], 0x5140), b = __byte_perm(e[2], e[3], 0x5140);  // u u v v
+        w[0][q] = __byte_perm(a, b, 0x5410);
+        w[1][q] = __byte_perm(a, b, 0x7632);
+        w[2][q] = __byte_perm(__byte_perm(e[0], e[1], 0x0062), __byte_perm(e[2], e[3], 0x0062), 0x5410);
+      }
+#pragma unroll
+      for (int x = 0; x < 3; ++x) {
+        check(w[x], flags);
+        st.put(w[x]);
+      }
+    }
+#pragma unroll 1
+    for (int v = 0; v < rt.pairs; ++v) {
+      uint32_t w[2][2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        uint32_t e[4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int pr = 2 * q + u;
+          const int2 i = entry<P2>(c[pr], tp_of(tp, 2 * pr), tp_of(tp, 2 * pr + 1), cs[v], pow2 + v * kPow2Table, 2.0f);
+          e[2 * u] = *reinterpret_cast<const uint16_t*>(lut + i.x);
+          e[2 * u + 1] = *reinterpret_cast<const uint16_t*>(lut + i.y);
+        }
+        const uint32_t a = __byte_perm(e[0], e[1], 0x5410), b = __byte_perm(e[2], e[3], 0x5410);
+        w[0][q] = __byte_perm(a, b, 0x6420);
+        w[1][q] = __byte_perm(a, b, 0x7531);
+      }
+      check(w[0], flags);
+      st.put(w[0]);
+      if (2 * v + 1 < rt.singles) {
+        check(w[1], flags);
+        st.put(w[1]);
+      }
+    }
+  }
+
+  static __device__ __forceinline__ void planes(const Table& rt, const unsigned char* smem,
+                                                const f2 (&c)[kPairs][kPieces], const TpPack& tp, int any_tp,
+                                                const PlaneStore& st, uint32_t* flags) {
+    if (__any_sync(0xffffffffu, any_tp != 0)) all<true>(rt, smem, c, tp, st, flags);
+    else all<false>(rt, smem, c, tp, st, flags);
+  }
+};
+
 // Rows of A.  A warp item covers 2^s lanes x 8 k of 32 / 2^s rows (16 lanes on 128
 // consecutive k of two rows, or 4 or 8 lanes per row for rows of at most 64 k; see
 // resid_rows_lane_log), so short rows and the ends of rows leave few lanes idle.  Lane
@@ -327,8 +524,9 @@ static_assert(kElems == 8, "the row kernel's item shapes assume 8 elements per l
 
 // vblock / vgrid: the block's index among, and the number of, the blocks serving this
 // operand (the warps stride over its items).
-__device__ __forceinline__ void residues_rows_body(const ResidArgs& a, int N, const Tables& tb, int64_t vblock,
-                                                   int64_t vgrid) {
+template <class Sys>
+__device__ __forceinline__ void residues_rows_body(const ResidArgs& a, const typename Sys::Table& mt,
+                                                   const unsigned char* tb, int64_t vblock, int64_t vgrid) {
   const int lane = threadIdx.x & 31;
   const int warps_per_block = blockDim.x >> 5;
   const int ls = resid_rows_lane_log(a.kp);
@@ -377,7 +575,7 @@ __device__ __forceinline__ void residues_rows_body(const ResidArgs& a, int N, co
     for (int t = 0; t < kElems; ++t) decode_into(c, t, v[t], e, tp, any_tp, range_err);
     const PlaneStore st{a.planes + static_cast<int64_t>(row_ok ? row : 0) * a.ldp + h0, a.plane_stride,
                         row_ok && h0 < a.kp};
-    task_planes(N, tb, c, tp, any_tp, st, a.flags);
+    Sys::planes(mt, tb, c, tp, any_tp, st, a.flags);
   }
   if (range_err) atomicOr(a.flags, kFlagRange);
 }
@@ -401,8 +599,10 @@ __device__ __forceinline__ int tile_slot(int h) {  // position of k offset h wit
 
 // Tiles t0, t0 + tstride, ... of the operand (tiles numbered with the column tile
 // fastest).
-__device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, int N, const Tables& tb,
-                                                         unsigned long long* tile, int64_t t0, int64_t tstride) {
+template <class Sys>
+__device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, const typename Sys::Table& mt,
+                                                         const unsigned char* tb, unsigned long long* tile, int64_t t0,
+                                                         int64_t tstride) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tiles_n = (a.lines + kTileCols - 1) / kTileCols, tiles_k = (a.kp + kTileK - 1) / kTileK;
   const int64_t tiles = static_cast<int64_t>(tiles_n) * tiles_k;
@@ -410,19 +610,19 @@ __device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, int
   for (int64_t t = t0; t < tiles; t += tstride) {
     const int j0 = static_cast<int>(t % tiles_n) * kTileCols;
     const int k0 = static_cast<int>(t / tiles_n) * kTileK;
-    // load: warp w reads rows w, w + 8, ...; lane l takes columns l and l + 32
-#pragma unroll 4
+    // load: warp w reads rows w, w + 8, ...; lane l takes columns l, l + 32, ...
+#pragma unroll 8
     for (int r = warp; r < kTileK; r += 8) {
       const int h = k0 + r;
       const unsigned long long* row = reinterpret_cast<const unsigned long long*>(a.X + static_cast<int64_t>(h) * a.ldx);
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < kTileCols / 32; ++u) {
         const int c = lane + 32 * u, j = j0 + c;
         tile[c * kTilePitch + tile_slot(r)] = (h < a.k && j < a.lines) ? __ldg(row + j) : 0ull;
       }
     }
     __syncthreads();
-    // convert: 4 rounds of 256 (column, 8-k chunk) tasks; a half-warp per column
+    // convert: rounds of 256 (column, 8-k chunk) tasks; a half-warp per column
 #pragma unroll 1
     for (int round = 0; round < kTileCols * kTileK / (8 * 256); ++round) {
       const int q = round * 256 + tid;
@@ -440,53 +640,55 @@ __device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, int
       }
       const PlaneStore st{a.planes + static_cast<int64_t>(j < a.lines ? j : 0) * a.ldp + (h0 < a.kp ? h0 : 0),
                           a.plane_stride, active};
-      task_planes(N, tb, cc, tp, any_tp, st, a.flags);
+      Sys::planes(mt, tb, cc, tp, any_tp, st, a.flags);
     }
     __syncthreads();  // the tile is reloaded
   }
   if (range_err) atomicOr(a.flags, kFlagRange);
 }
 
+// Both kernels stage the system's constants behind the column kernel's tile (rows: alone).
+template <class Sys>
 __global__ void __launch_bounds__(256, 3) residues_cols_tiled_kernel(ResidArgs a,
-                                                                    const __grid_constant__ ModTable mt) {
+                                                                    const __grid_constant__ typename Sys::Table mt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  Tables& tb = *reinterpret_cast<Tables*>(smem_raw + kTileBytes);
-  load_tables(mt, tb);
-  residues_cols_tiled_body(a, mt.N, tb, reinterpret_cast<unsigned long long*>(smem_raw), blockIdx.x, gridDim.x);
+  Sys::load(mt, smem_raw + kTileBytes);
+  residues_cols_tiled_body<Sys>(a, mt, smem_raw + kTileBytes, reinterpret_cast<unsigned long long*>(smem_raw),
+                                blockIdx.x, gridDim.x);
 }
 
-__global__ void __launch_bounds__(256, 3) residues_rows_kernel(ResidArgs a, const __grid_constant__ ModTable mt) {
-  __shared__ Tables tb;
-  load_tables(mt, tb);
-  residues_rows_body(a, mt.N, tb, blockIdx.x, gridDim.x);
+template <class Sys>
+__global__ void __launch_bounds__(256, 3) residues_rows_kernel(ResidArgs a,
+                                                              const __grid_constant__ typename Sys::Table mt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Sys::load(mt, smem_raw);
+  residues_rows_body<Sys>(a, mt, smem_raw, blockIdx.x, gridDim.x);
 }
 
 // Grouped: rows of every A; columns of every B (one virtual block per tile).
 __global__ void __launch_bounds__(256, 2) residues_rows_batch(const BatchProblem* __restrict__ probs, int count,
                                                            int64_t total, uint32_t* flags,
-                                                           const __grid_constant__ ModTable mt) {
-  __shared__ Tables tb;
-  load_tables(mt, tb);
+                                                           const __grid_constant__ RnsTable mt) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  RnsSys::load(mt, smem_raw);
   for_each_vblock(probs, count, kBkResidRows, total, [&](const BatchProblem& P, int64_t v) {
     const ResidArgs a{P.A, P.lda, P.m, P.k, P.kp, P.ldp, P.e, P.planesA, static_cast<int64_t>(P.m) * P.ldp, flags};
-    residues_rows_body(a, mt.N, tb, v, P.nblocks[kBkResidRows]);
+    residues_rows_body<RnsSys>(a, mt, smem_raw, v, P.nblocks[kBkResidRows]);
   });
 }
 
 __global__ void __launch_bounds__(256, 3) residues_cols_batch(const BatchProblem* __restrict__ probs, int count,
                                                            int64_t total, uint32_t* flags,
-                                                           const __grid_constant__ ModTable mt) {
+                                                           const __grid_constant__ RnsTable mt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  Tables& tb = *reinterpret_cast<Tables*>(smem_raw + kTileBytes);
-  load_tables(mt, tb);
+  RnsSys::load(mt, smem_raw + kTileBytes);
   for_each_vblock(probs, count, kBkResidCols, total, [&](const BatchProblem& P, int64_t v) {
     const ResidArgs a{P.B, P.ldb, P.n, P.k, P.kp, P.ldp, P.f, P.planesB, static_cast<int64_t>(P.n) * P.ldp, flags};
-    residues_cols_tiled_body(a, mt.N, tb, reinterpret_cast<unsigned long long*>(smem_raw), v,
-                             P.nblocks[kBkResidCols]);
+    residues_cols_tiled_body<RnsSys>(a, mt, smem_raw + kTileBytes, reinterpret_cast<unsigned long long*>(smem_raw), v,
+                                     P.nblocks[kBkResidCols]);
   });
 }
 
-constexpr size_t kColsSmem = kTileBytes + sizeof(Tables);
 static_assert(kTileBytes % 16 == 0, "the tables follow the tile on a 16-byte boundary");
 
 // ------------------------------------------------------------------ gradient operands
@@ -497,8 +699,8 @@ static_assert(kTileBytes % 16 == 0, "the tables follow the tile on a 16-byte bou
 // One kernel reads each kTileK x kTileCols tile of dC once into shared memory (the
 // layout of the column kernel above: tile rows are rows i of dC, tile columns are
 // columns j) and converts it twice: the column pass writes H' exactly as the column
-// kernel writes B's planes; the row pass writes G' with 8 consecutive j per task, a
-// warp covering 4 rows x 64 columns (64-byte plane pieces).
+// kernel writes B's planes; the row pass writes G' with 8 consecutive j per task (plane
+// pieces of kTileCols bytes).
 struct GradArgs {
   const double* dC;
   int64_t lddc;
@@ -515,12 +717,11 @@ struct GradArgs {
   bool do_g, do_h;  // which of the two outputs to write
 };
 
-__global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const __grid_constant__ ModTable mt) {
+__global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const __grid_constant__ RnsTable mt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned long long* tile = reinterpret_cast<unsigned long long*>(smem_raw);
-  Tables& tb = *reinterpret_cast<Tables*>(smem_raw + kTileBytes);
-  load_tables(mt, tb);
-  const int N = mt.N;
+  const unsigned char* tb = smem_raw + kTileBytes;
+  RnsSys::load(mt, smem_raw + kTileBytes);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tiles_n = (a.n + kTileCols - 1) / kTileCols, tiles_m = (a.m + kTileK - 1) / kTileK;
   const int64_t tiles = static_cast<int64_t>(tiles_n) * tiles_m;
@@ -528,12 +729,12 @@ __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
     const int j0 = static_cast<int>(t % tiles_n) * kTileCols;
     const int i0 = static_cast<int>(t / tiles_n) * kTileK;
-#pragma unroll 4
+#pragma unroll 8
     for (int r = warp; r < kTileK; r += 8) {
       const int i = i0 + r;
       const unsigned long long* row = reinterpret_cast<const unsigned long long*>(a.dC + static_cast<int64_t>(i) * a.lddc);
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < kTileCols / 32; ++u) {
         const int c = lane + 32 * u, j = j0 + c;
         tile[c * kTilePitch + tile_slot(r)] = (i < a.m && j < a.n) ? __ldg(row + j) : 0ull;
       }
@@ -559,12 +760,14 @@ __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const
       }
       const PlaneStore st{a.planesH + static_cast<int64_t>(j < a.n ? j : 0) * a.ldh + (ib < a.m ? ib : 0),
                           static_cast<int64_t>(a.n) * a.ldh, active};
-      task_planes(N, tb, cc, tp, any_tp, st, a.flags);
+      RnsSys::planes(mt, tb, cc, tp, any_tp, st, a.flags);
     }
-    // row pass: G' (lines i, positions j); warp w, round s: rows 4 (8 s + w) + lane / 8
+    // row pass: G' (lines i, positions j): kTileCols / 8 chunks per row
 #pragma unroll 1
     for (int round = 0; a.do_g && round < kTileK * kTileCols / (8 * 256); ++round) {
-      const int r = 4 * (8 * round + warp) + (lane >> 3), chunk = lane & 7;
+      constexpr int kChunks = kTileCols / 8;
+      const int q = round * 256 + tid;
+      const int r = q / kChunks, chunk = q % kChunks;
       const int i = i0 + r, jb = j0 + chunk * 8;
       const bool active = i < a.m && jb < a.n;
       const int gi = i < a.m ? a.g[i] : 0;
@@ -579,7 +782,7 @@ __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const
       }
       const PlaneStore st{a.planesG + static_cast<int64_t>(i < a.m ? i : 0) * a.ldg + (jb < a.n ? jb : 0),
                           static_cast<int64_t>(a.m) * a.ldg, active};
-      task_planes(N, tb, cc, tp, any_tp, st, a.flags);
+      RnsSys::planes(mt, tb, cc, tp, any_tp, st, a.flags);
     }
     __syncthreads();  // the tile is reloaded
   }
@@ -654,75 +857,106 @@ __global__ void __launch_bounds__(256) transpose_planes_kernel(const uint8_t* __
   }
 }
 
-// Opt a column kernel into kColsSmem bytes of dynamic shared memory, once per device
-// (a launch on a device where this failed reports the error itself).
+// Opt a kernel into `bytes` of dynamic shared memory, raised when a later call needs more
+// (per device; a launch on a device where this failed reports the error itself).
 template <class K>
-void allow_cols_smem(K* kernel, bool (&done)[64]) {
+void allow_smem(K* kernel, std::atomic<int> (&allowed)[64], size_t bytes) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
-  if (!done[dev] && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kColsSmem)) == cudaSuccess)
-    done[dev] = true;
+  const int want = static_cast<int>(bytes);
+  if (allowed[dev].load() >= want) return;
+  // every thread asks for the same largest size, so the order of concurrent first calls
+  // does not matter
+  constexpr int kMost = 227 * 1024;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) == cudaSuccess)
+    allowed[dev].store(kMost);
 }
 
-int grid_for(int64_t warps) {
+int sm_count() {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t want = (warps + 7) / 8;
-  const int64_t cap = static_cast<int64_t>(sms) * 16;
-  return static_cast<int>(want < cap ? (want > 0 ? want : 1) : cap);
+  return sms;
+}
+
+// Blocks of a conversion kernel: one per 8 warps of work, at most the resident ones (each
+// stages the tables once and strides over the work).
+int resident_grid(int64_t blocks, size_t smem) {
+  const int per_sm = static_cast<int>(std::max<size_t>(1, std::min<size_t>(3, (226 * 1024) / (smem + 1024))));
+  const int64_t cap = static_cast<int64_t>(sm_count()) * per_sm;
+  return static_cast<int>(std::max<int64_t>(1, std::min(blocks, cap)));
+}
+
+template <class Sys>
+cudaError_t run_rows(const ResidArgs& a, const typename Sys::Table& t, cudaStream_t st) {
+  const size_t smem = Sys::smem_bytes(t);
+  static std::atomic<int> allowed[64];
+  allow_smem(residues_rows_kernel<Sys>, allowed, smem);
+  const int64_t items = resid_rows_items(a.lines, a.kp);
+  residues_rows_kernel<Sys><<<resident_grid((items + 7) / 8, smem), 256, smem, st>>>(a, t);
+  return cudaGetLastError();
+}
+
+template <class Sys>
+cudaError_t run_cols(const ResidArgs& a, const typename Sys::Table& t, cudaStream_t st) {
+  const size_t smem = kTileBytes + Sys::smem_bytes(t);
+  static std::atomic<int> allowed[64];
+  allow_smem(residues_cols_tiled_kernel<Sys>, allowed, smem);
+  const int64_t tiles = static_cast<int64_t>((a.lines + kTileCols - 1) / kTileCols) * ((a.kp + kTileK - 1) / kTileK);
+  residues_cols_tiled_kernel<Sys><<<resident_grid(tiles, smem), 256, smem, st>>>(a, t);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_residues_rows(const double* A, int64_t lda, int m, int k, int kp, int64_t ldp, const int32_t* e,
-                                 const ModTable& mt, uint8_t* planes, uint32_t* flags, cudaStream_t st,
+                                 const RnsTable& rt, uint8_t* planes, uint32_t* flags, cudaStream_t st,
                                  int64_t plane_stride) {
-  ResidArgs a{A, lda, m, k, kp, ldp, e, planes, plane_stride ? plane_stride : static_cast<int64_t>(m) * ldp, flags};
-  residues_rows_kernel<<<grid_for(resid_rows_items(m, kp)), 256, 0, st>>>(a, mt);
-  return cudaGetLastError();
+  return run_rows<RnsSys>(
+      ResidArgs{A, lda, m, k, kp, ldp, e, planes, plane_stride ? plane_stride : static_cast<int64_t>(m) * ldp, flags},
+      rt, st);
 }
 
 cudaError_t launch_residues_cols(const double* B, int64_t ldb, int k, int n, int kp, int64_t ldp, const int32_t* f,
-                                 const ModTable& mt, uint8_t* planes, uint32_t* flags, cudaStream_t st,
+                                 const RnsTable& rt, uint8_t* planes, uint32_t* flags, cudaStream_t st,
                                  int64_t plane_stride) {
-  ResidArgs a{B, ldb, n, k, kp, ldp, f, planes, plane_stride ? plane_stride : static_cast<int64_t>(n) * ldp, flags};
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t tiles = static_cast<int64_t>((n + kTileCols - 1) / kTileCols) * ((kp + kTileK - 1) / kTileK);
-  const int grid = static_cast<int>(std::min<int64_t>(tiles, 3 * static_cast<int64_t>(sms)));
-  static bool done[64] = {};  // per device
-  allow_cols_smem(residues_cols_tiled_kernel, done);
-  residues_cols_tiled_kernel<<<grid, 256, kColsSmem, st>>>(a, mt);
-  return cudaGetLastError();
+  return run_cols<RnsSys>(
+      ResidArgs{B, ldb, n, k, kp, ldp, f, planes, plane_stride ? plane_stride : static_cast<int64_t>(n) * ldp, flags},
+      rt, st);
+}
+
+cudaError_t launch_paper_planes_rows(const double* A, int64_t lda, int m, int k, int kp, const int32_t* e,
+                                     const ModTable& mt, uint8_t* planes, uint32_t* flags, cudaStream_t st) {
+  return run_rows<PaperSys>(ResidArgs{A, lda, m, k, kp, kp, e, planes, static_cast<int64_t>(m) * kp, flags}, mt, st);
+}
+
+cudaError_t launch_paper_planes_cols(const double* B, int64_t ldb, int k, int n, int kp, const int32_t* f,
+                                     const ModTable& mt, uint8_t* planes, uint32_t* flags, cudaStream_t st) {
+  return run_cols<PaperSys>(ResidArgs{B, ldb, n, k, kp, kp, f, planes, static_cast<int64_t>(n) * kp, flags}, mt, st);
 }
 
 cudaError_t launch_residues_batch(const BatchProblem* probs, int count, int64_t rows_blocks, int64_t cols_blocks,
-                                  const ModTable& mt, uint32_t* flags, cudaStream_t st, cudaStream_t st_cols) {
+                                  const RnsTable& rt, uint32_t* flags, cudaStream_t st, cudaStream_t st_cols) {
   if (rows_blocks < 1 || cols_blocks < 1 || rows_blocks > 0x7FFFFFFFll || cols_blocks > 0x7FFFFFFFll)
     return cudaErrorInvalidValue;
-  static bool done[64] = {};
-  allow_cols_smem(residues_cols_batch, done);
-  residues_rows_batch<<<grouped_grid(rows_blocks, 3), 256, 0, st>>>(probs, count, rows_blocks, flags, mt);
-  residues_cols_batch<<<grouped_grid(cols_blocks, 3), 256, kColsSmem, st_cols>>>(probs, count, cols_blocks, flags,
-                                                                                mt);
+  const size_t rows_smem = RnsSys::smem_bytes(rt), cols_smem = kTileBytes + rows_smem;
+  static std::atomic<int> allowed_rows[64], allowed_cols[64];
+  allow_smem(residues_rows_batch, allowed_rows, rows_smem);
+  allow_smem(residues_cols_batch, allowed_cols, cols_smem);
+  residues_rows_batch<<<grouped_grid(rows_blocks, 2), 256, rows_smem, st>>>(probs, count, rows_blocks, flags, rt);
+  residues_cols_batch<<<grouped_grid(cols_blocks, 2), 256, cols_smem, st_cols>>>(probs, count, cols_blocks, flags, rt);
   return cudaGetLastError();
 }
 
 cudaError_t launch_grad_residues(const double* dC, int64_t lddc, int m, int n, const int32_t* g, const int32_t* f,
                                  const int32_t* h, const int32_t* e, uint8_t* planesG, int64_t ldg, uint8_t* planesH,
-                                 int64_t ldh, const ModTable& mt, uint32_t* flags, cudaStream_t st) {
+                                 int64_t ldh, const RnsTable& rt, uint32_t* flags, cudaStream_t st) {
   GradArgs a{dC, lddc, m, n, g, f, h, e, planesG, ldg, planesH, ldh, flags, planesG != nullptr, planesH != nullptr};
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const size_t smem = kTileBytes + RnsSys::smem_bytes(rt);
+  static std::atomic<int> allowed[64];
+  allow_smem(grad_residues_kernel, allowed, smem);
   const int64_t tiles = static_cast<int64_t>((n + kTileCols - 1) / kTileCols) * ((m + kTileK - 1) / kTileK);
-  const int grid = static_cast<int>(std::min<int64_t>(tiles, 3 * static_cast<int64_t>(sms)));
-  static bool done[64] = {};  // per device
-  allow_cols_smem(grad_residues_kernel, done);
-  grad_residues_kernel<<<grid, 256, kColsSmem, st>>>(a, mt);
+  grad_residues_kernel<<<resident_grid(tiles, smem), 256, smem, st>>>(a, rt);
   return cudaGetLastError();
 }
 

@@ -105,6 +105,14 @@ def moduli(num_moduli=12):
     return list(buf)
 
 
+def product_count(num_moduli=12):
+    """FP8 products of one emulated product, without accurate mode's bound product."""
+    n = int(_lib.load().ozk2_product_count(num_moduli))
+    if n < 0:
+        raise ValueError("num_moduli must be in 1..20")
+    return n
+
+
 def workspace_size(m, n, k, num_moduli=12, mode="accurate", block=None):
     bm, bn = _block(block)
     return int(_lib.load().ozk2_workspace_size_ex(m, n, k, num_moduli, _mode(mode), bm, bn))
