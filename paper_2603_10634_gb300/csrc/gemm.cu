@@ -32,14 +32,23 @@
 // per unit.  The wide tile halves the operand bytes each SM pulls per flop compared with
 // 128 x 128.
 //
+// Large single problems run in CTA pairs (PAIR): clusters of two CTAs share 256 x 256 tiles
+// through tcgen05.mma.cta_group::2.  Per k-step each SM then receives 32 KiB instead of 48
+// and its tensor core reads 8 KiB per instruction instead of 12, and the shared-memory
+// bandwidth these take is what bounds the single-CTA kernel (75% of the tensor rate; pairs
+// reach 91% at 8192^3: 13.0 M cycles instead of 15.6 M).  Every cross-CTA signal of the k
+// loop is asynchronous: both CTAs' TMA loads count their bytes on the leader's full
+// barrier, and the leader's commits arrive on both CTAs' empty and tfull barriers; only
+// the release of an accumulator slot is a (relaxed) remote arrival, one per warp and pass.
+//
 // Roles (320 threads for single problems, 576 for grouped launches; one persistent CTA
 // per SM):
-//   warp 0      TMA producer: 128-row A and 256-row B^T boxes of 128 bytes along K
-//               (K-major, 128-byte swizzle, zero fill past m, n, k) into a 4-stage
-//               ring of 48 KiB stages, mbarrier complete_tx.
-//   warp 1      TMEM allocation and the single MMA-issuing thread:
-//               tcgen05.mma.cta_group::1.kind::f8f6f4, M = 128, N = 256, K = 32; a pass
-//               starts once the epilogue has released the slot(s) it writes.
+//   warp 0      TMA producer: 128-row A and 256-row B^T boxes (pairs: 128 rows) of 128
+//               bytes along K (K-major, 128-byte swizzle, zero fill past m, n, k) into a
+//               ring of 4 48-KiB stages (pairs: 6 of 32 KiB), mbarrier complete_tx.
+//   warp 1      TMEM allocation and the single MMA-issuing thread (pairs: the leader's):
+//               tcgen05.mma.kind::f8f6f4, M = 128 (256), N = 256, K = 32; a pass starts
+//               once the epilogue has released the slot it writes.
 //   warps 2-9   epilogue (warps 2-17 in grouped launches): warp w reads TMEM lane
 //               quadrant w % 4, column half (quarter) (w - 2) / 4, with tcgen05.ld;
 //               FP32 math; global stores.
@@ -47,6 +56,7 @@
 // up raises a CTA-wide abort flag and the global timeout flag, drains the copies and
 // products this CTA has in flight, frees TMEM and returns.  Operands are read only with
 // plain (non-multicast) TMA loads of this CTA's own tiles.
+#include <algorithm>
 #include <cstring>
 
 #include "device.cuh"
@@ -75,11 +85,16 @@ constexpr int kGroupM = 16;             // tile rasterisation: bands of 16 tile 
 // Tile shapes: 128 x 256 (the default) or 128 x 128 (narrow or ragged products, where a
 // 256-wide tile would spend much of its tensor work on padding).  Both keep two TMEM
 // accumulator slots of TN columns and fill about 192 KiB of shared memory with stages.
-template <int TN>
+// PAIR: two CTAs share a 256 x 256 tile; each stages its own 128 rows of A and half the rows
+// of B (32 KiB a stage instead of 48), and holds its 128 rows of the accumulators.  (256 x
+// 128 pair tiles for narrow products were no faster than single CTAs: 8192 x 100 x 4096
+// streams A's planes from HBM either way.)
+template <int TN, bool PAIR>
 struct Tile {
-  static_assert(TN == 256 || TN == 128, "tile widths 256 and 128");
-  static constexpr int kStages = TN == 256 ? 4 : 6;
-  static constexpr int kBTileBytes = TN * BK;
+  static_assert(TN == 256 || (TN == 128 && !PAIR), "tile widths 256 and 128, pairs 256 only");
+  static constexpr int kStages = PAIR || TN == 128 ? 6 : 4;
+  static constexpr int kBRows = PAIR ? TN / 2 : TN;
+  static constexpr int kBTileBytes = kBRows * BK;
   static constexpr int kStageBytes = kATileBytes + kBTileBytes;
   static constexpr uint32_t kTmemCols = 2 * TN;
   static constexpr size_t kSmemBytes = 1024 + static_cast<size_t>(kStages) * kStageBytes + 256;
@@ -107,16 +122,18 @@ struct GemmParams {
   const int32_t* rowshift;
   unsigned long long wait_ns;  // limit of every device wait (the drains of an abort use the default)
   int stall;                   // fault injection: the MMA thread's first wait never completes
+  uint32_t* pace;              // two zeroed words for the pacing of long reductions (Pace), or null
 };
 
+template <int GROUP_M>
 __device__ __forceinline__ void decode_unit(int tiles_m, int tiles_n, int tiles, int u, int& mod, int& tm,
                                             int& tn) {
   mod = u / tiles;
   const int t = u - mod * tiles;
-  const int per_group = kGroupM * tiles_n;
+  const int per_group = GROUP_M * tiles_n;
   const int g = t / per_group;
-  const int first_m = g * kGroupM;
-  const int gsz = min(tiles_m - first_m, kGroupM);
+  const int first_m = g * GROUP_M;
+  const int gsz = min(tiles_m - first_m, GROUP_M);
   const int r = t - g * per_group;
   tm = first_m + r % gsz;
   tn = r / gsz;
@@ -141,7 +158,7 @@ struct UnitCtx {
   float* S;
 };
 
-template <bool GROUPED>
+template <bool GROUPED, bool PAIR>
 __device__ __forceinline__ void resolve_unit(const GemmParams& P, const CUtensorMap* tmA, const CUtensorMap* tmB,
                                              const GemmProblem* __restrict__ probs, int nprobs, int u, UnitCtx& c) {
   if constexpr (!GROUPED) {
@@ -151,7 +168,7 @@ __device__ __forceinline__ void resolve_unit(const GemmParams& P, const CUtensor
     c.n = P.n;
     c.k = P.k;
     c.prob = 0;
-    decode_unit(P.tiles_m, P.tiles_n, P.tiles, u, c.mod, c.tm, c.tn);
+    decode_unit<PAIR ? kGroupM / 2 : kGroupM>(P.tiles_m, P.tiles_n, P.tiles, u, c.mod, c.tm, c.tn);
     c.cres = P.cres;
     c.cres8 = P.cres8;
     c.ldr = P.ldr;
@@ -188,7 +205,8 @@ __device__ __forceinline__ void resolve_unit(const GemmParams& P, const CUtensor
       c.R = G.R;
       c.S = G.S;
     }
-    decode_unit(c.tiles_m, c.tiles_n, c.tiles, static_cast<int>(u - c.unit_start), c.mod, c.tm, c.tn);
+    decode_unit<PAIR ? kGroupM / 2 : kGroupM>(c.tiles_m, c.tiles_n, c.tiles, static_cast<int>(u - c.unit_start), c.mod,
+                                              c.tm, c.tn);
   }
 }
 
@@ -250,6 +268,60 @@ struct Slots {
   uint32_t t = 0u;
   __device__ __forceinline__ uint32_t slot() const { return t & 1u; }
   __device__ __forceinline__ uint32_t uses() const { return t >> 1; }
+};
+
+// Pacing.  CTA pairs keep their tensor cores busy whatever the L2 does, so nothing holds
+// their places in the k loop together, and once they have drifted apart each reads operand
+// tiles from DRAM that its neighbours have already pulled through the L2.  Each pair
+// therefore reports every kPaceSteps k-steps (about 30 us of products) and waits, its ring
+// still full, until all pairs have reported as often; a pair that is done reports for good.
+// Only a hint: a wait that takes longer than kPaceNs (the launch does not have the GPU to
+// itself, or the last round) ends the pacing for this pair.  words[0]: reports, words[1]:
+// pairs done; the last one zeroes both.  DRAM reads of a 16384^3 launch 331 -> 123 GB (the
+// single-CTA kernel, which the operand ring slowed into step: 128 GB), and with them the
+// power that the cap turns into clock: 72.4 -> 64.5 ms; 8192^3 8.55 -> 7.75 ms.  Waiting every
+// 16 steps, or letting a pair run one round ahead, was slower (66.2, 66.9 ms).
+constexpr int kPaceSteps = 64;
+constexpr unsigned long long kPaceNs = 20000ull;
+constexpr uint32_t kPaceDone = 0x10000u;  // more reports than a launch's rounds that still wait
+struct Pace {
+  uint32_t* words;
+  uint32_t round = 0u;
+  int steps = 0;  // k-steps since the last report
+  bool on;
+  __device__ __forceinline__ explicit Pace(uint32_t* w) : words(w), on(w != nullptr) {}
+  __device__ __forceinline__ void k_step(uint32_t pairs) {
+    if (words == nullptr) return;
+    if (steps != 0) {
+      steps = steps + 1 < kPaceSteps ? steps + 1 : 0;
+      return;
+    }
+    steps = 1;
+    atomicAdd(words, 1u);
+    ++round;
+    if (!on) return;
+    const uint32_t want = pairs * round;
+    const unsigned long long t0 = global_ns();
+    while (load_relaxed(words) < want) {
+      if (global_ns() - t0 > kPaceNs) {
+        on = false;
+        break;
+      }
+    }
+  }
+  __device__ __forceinline__ void finish(uint32_t pairs) {
+    if (words == nullptr) return;
+    atomicAdd(words, kPaceDone);
+    if (atomicAdd(words + 1, 1u) == pairs - 1u) {
+      words[0] = 0u;
+      words[1] = 0u;
+    }
+  }
+  static __device__ __forceinline__ uint32_t load_relaxed(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+  }
 };
 
 // Lane l of the warp ends with the maximum of column l over the 32 lanes.
@@ -388,14 +460,17 @@ __device__ __forceinline__ uint32_t pack4(float2 a, float2 b) {
 }
 
 // GROUPED: the units of all `nprobs` problems of `probs` (tmA, tmB unused).  TN: tile width.
-template <int MODE, bool GROUPED, int TN>
+// PAIR: launched in clusters of two CTAs.
+template <int MODE, bool GROUPED, int TN, bool PAIR>
 __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
     fp8_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ GemmParams prm, const GemmProblem* __restrict__ probs, int nprobs) {
   constexpr int BN = TN;
-  constexpr int kStages = Tile<TN>::kStages;
-  constexpr int kStageBytes = Tile<TN>::kStageBytes;
-  constexpr uint32_t kTmemCols = Tile<TN>::kTmemCols;
+  using T = Tile<TN, PAIR>;
+  constexpr int G = PAIR ? 2 : 1;  // CTAs per tile
+  constexpr int kStages = T::kStages;
+  constexpr int kStageBytes = T::kStageBytes;
+  constexpr uint32_t kTmemCols = T::kTmemCols;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* tiles = smem;
@@ -410,8 +485,10 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int u_first = static_cast<int>(blockIdx.x);
-  const int u_step = static_cast<int>(gridDim.x);
+  const uint32_t rank = PAIR ? cluster_rank() : 0u;
+  const bool leader = rank == 0u;
+  const int u_first = static_cast<int>(blockIdx.x) / G;
+  const int u_step = static_cast<int>(gridDim.x) / G;
   const unsigned long long wait_ns = prm.wait_ns;
 
   if (threadIdx.x == 0) {
@@ -421,7 +498,7 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
     }
     for (int j = 0; j < 2; ++j) {
       mbar_init(tfull + j, 1);
-      mbar_init(tempty + j, 32 * Epi<GROUPED>::kWarps);
+      mbar_init(tempty + j, PAIR ? 2 * Epi<GROUPED>::kWarps : 32 * Epi<GROUPED>::kWarps);  // per warp / per thread
     }
     mbar_init(done, 1);
     mbar_init(never, 1);
@@ -433,11 +510,11 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
     tma_prefetch_map(&tmB);
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, kTmemCols);
-    tmem_relinquish();
+    tmem_alloc<G>(tmem_slot, kTmemCols);
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync();  // both CTAs' barriers are ready
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
@@ -450,8 +527,9 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
       bool ok = true;
       int last_prob = -1;
       UnitCtx uc;
+      Pace pace(PAIR && leader ? prm.pace : nullptr);
       for (int u = u_first; ok && u < prm.num_units; u += u_step) {
-        resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
+        resolve_unit<GROUPED, PAIR>(prm, &tmA, &tmB, probs, nprobs, u, uc);
         if (GROUPED && uc.prob != last_prob) {
           tensormap_acquire(uc.ta);
           tensormap_acquire(uc.tb);
@@ -465,6 +543,9 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
           for (int ps = 0; ok && ps < up.npasses; ++ps) {
             const int np = num_products<MODE>(mod, ps);
             for (int s = 0; ok && s < ksteps; ++s) {
+              if constexpr (PAIR) {
+                pace.k_step(static_cast<uint32_t>(u_step));
+              }
               for (int x = 0; x < np; ++x) {
                 if (!mbar_wait_bounded(empty + stage, phase ^ 1u, abort_flag, wait_ns)) {
                   ok = false;
@@ -473,9 +554,18 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
                 int pa, pb;
                 product_of<MODE>(prm, mod, ps, x, pa, pb);
                 uint8_t* dst = tiles + stage * kStageBytes;
-                mbar_arrive_expect_tx(full + stage, kStageBytes);
-                tma_load_3d(dst, uc.ta, full + stage, k0 + s * BK, uc.tm * BM, pa);
-                tma_load_3d(dst + kATileBytes, uc.tb, full + stage, k0 + s * BK, uc.tn * BN, pb);
+                if constexpr (PAIR) {
+                  // both CTAs' bytes count on the leader's barrier
+                  const uint32_t bar = leader_addr(full + stage);
+                  if (leader) mbar_arrive_expect_tx(full + stage, 2 * kStageBytes);
+                  tma_load_3d_pair(dst, uc.ta, bar, k0 + s * BK, (uc.tm * 2 + static_cast<int>(rank)) * BM, pa);
+                  tma_load_3d_pair(dst + kATileBytes, uc.tb, bar, k0 + s * BK,
+                                   uc.tn * BN + static_cast<int>(rank) * T::kBRows, pb);
+                } else {
+                  mbar_arrive_expect_tx(full + stage, kStageBytes);
+                  tma_load_3d(dst, uc.ta, full + stage, k0 + s * BK, uc.tm * BM, pa);
+                  tma_load_3d(dst + kATileBytes, uc.tb, full + stage, k0 + s * BK, uc.tn * BN, pb);
+                }
                 issued |= 1u << stage;
                 issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
                 if (++stage == kStages) {
@@ -487,18 +577,27 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
           }
         }
       }
+      if constexpr (PAIR) pace.finish(static_cast<uint32_t>(u_step));
       if (!ok) {
         *abort_flag = 1;
         atomicOr(prm.flags, kFlagTimeout);
         int no_abort = 0;  // let this thread's copies in flight land before exiting
-        for (int s = 0; s < kStages; ++s)
-          if (issued & (1u << s)) mbar_wait_bounded(full + s, (issued_phase >> s) & 1u, &no_abort, kWaitLimitNs);
+        if constexpr (PAIR) {
+          // the barriers count both CTAs' copies and the other CTA may have given up at
+          // another stage: wait a fixed time, thousands of times a copy's
+          const unsigned long long t0 = global_ns();
+          while (global_ns() - t0 < 5000000ull) {
+          }
+        } else {
+          for (int s = 0; s < kStages; ++s)
+            if (issued & (1u << s)) mbar_wait_bounded(full + s, (issued_phase >> s) & 1u, &no_abort, kWaitLimitNs);
+        }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = fp8_idesc(BM, BN);
+    if (lane == 0 && leader) {
+      constexpr uint32_t idesc = fp8_idesc(G * BM, BN);
       int stage = 0;
       uint32_t phase = 0;
       Slots sl;
@@ -507,7 +606,7 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
       bool ok = prm.stall ? mbar_wait_bounded(never, 0u, abort_flag, wait_ns) : true;
       UnitCtx uc;
       for (int u = u_first; ok && u < prm.num_units; u += u_step) {
-        resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
+        resolve_unit<GROUPED, PAIR>(prm, &tmA, &tmB, probs, nprobs, u, uc);
         const int mod = uc.mod;
         const UnitPlan up = plan_of<MODE>(prm, uc.k, mod);
         for (int c = 0; ok && c < up.nchunks; ++c) {
@@ -531,19 +630,19 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
               const uint64_t bdesc = sw128_kmajor_desc(sa + kATileBytes);
 #pragma unroll
               for (int kk = 0; kk < BK / 32; ++kk)
-                mma_fp8(dtm, adesc + 2ull * kk, bdesc + 2ull * kk, idesc, (s == 0 && kk == 0) ? 0u : 1u);
-              mma_commit(empty + stage);
+                mma_fp8<G>(dtm, adesc + 2ull * kk, bdesc + 2ull * kk, idesc, (s == 0 && kk == 0) ? 0u : 1u);
+              mma_commit<G>(empty + stage);
               if (++stage == kStages) {
                 stage = 0;
                 phase ^= 1u;
               }
             }
-            if (ok) mma_commit(tfull + slot);
+            if (ok) mma_commit<G>(tfull + slot);
             ++sl.t;
           }
         }
       }
-      mma_commit(done);  // every product issued here completes before TMEM is freed
+      mma_commit<G>(done);  // every product issued here completes before TMEM is freed
       int no_abort = 0;
       mbar_wait_bounded(done, 0, &no_abort, kWaitLimitNs);
       if (!ok) {
@@ -572,10 +671,10 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
     bool ok = true;
     UnitCtx uc;
     for (int u = u_first; ok && u < prm.num_units; u += u_step) {
-      resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
+      resolve_unit<GROUPED, PAIR>(prm, &tmA, &tmB, probs, nprobs, u, uc);
       const int mod = uc.mod, tn = uc.tn;
       const UnitPlan up = plan_of<MODE>(prm, uc.k, mod);
-      const int gi = uc.tm * BM + row;
+      const int gi = (uc.tm * G + static_cast<int>(rank)) * BM + row;
       for (int c = 0; ok && c < up.nchunks; ++c) {
         for (int ps = 0; ok && ps < up.npasses; ++ps) {
           const uint32_t slot = sl.slot();
@@ -584,6 +683,15 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
           if (!ok) break;
           tc_fence_after();
           const uint32_t ts = tq + slot * static_cast<uint32_t>(BN);
+          auto release = [&]() {
+            tc_fence_before();
+            if constexpr (PAIR) {
+              __syncwarp();
+              if (lane == 0) mbar_arrive_cluster(leader_addr(tempty + slot));
+            } else {
+              mbar_arrive(tempty + slot);
+            }
+          };
           if constexpr (kResidues) {
             const GemmMod& gm = prm.mods.m[mod];
             const int p = gm.p, h = gm.half;
@@ -602,10 +710,6 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
             // chunk has been read from TMEM, before that chunk's arithmetic and stores (in the
             // grouped kernel the extra live state made it spill, and the release stays at the
             // end of the pass)
-            auto release = [&]() {
-              tc_fence_before();
-              mbar_arrive(tempty + slot);
-            };
             auto load = [&](int cb, uint32_t (&v)[kCW]) {
               tmem_ld_cols(ts + cb * kCW, v);
               tmem_ld_wait();
@@ -734,10 +838,7 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
               }
             }
           }
-          if constexpr (!kResidues || GROUPED) {  // else the epilogue released the slot itself
-            tc_fence_before();
-            mbar_arrive(tempty + slot);
-          }
+          if constexpr (!kResidues || GROUPED) release();  // else the epilogue released the slot itself
           ++sl.t;
         }
       }
@@ -750,34 +851,75 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
 
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) {
+    // the leader has waited for its last commit; the other CTA waits for that commit's
+    // arrival here (no later signal follows), then neither CTA's shared or tensor memory is
+    // read or written by the other any more
+    if (!leader && threadIdx.x == 32) {
+      int no_abort = 0;
+      mbar_wait_bounded(done, 0, &no_abort, kWaitLimitNs);
+    }
+    cluster_sync();
+  }
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kTmemCols);
+    tmem_dealloc<G>(tmem_base, kTmemCols);
   }
 }
 
-template <int MODE, bool GROUPED, int TN>
+template <int MODE, bool GROUPED, int TN, bool PAIR>
 cudaError_t launch_mode(const GemmParams& prm, const CUtensorMap& ta, const CUtensorMap& tb, int grid,
                         const GemmProblem* probs, int nprobs, cudaStream_t st) {
   static bool configured[64] = {false};
-  constexpr size_t smem = Tile<TN>::kSmemBytes;
+  constexpr size_t smem = Tile<TN, PAIR>::kSmemBytes;
+  auto* kernel = fp8_gemm_kernel<MODE, GROUPED, TN, PAIR>;
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !configured[dev]) {
-    cudaError_t err = cudaFuncSetAttribute(fp8_gemm_kernel<MODE, GROUPED, TN>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
     configured[dev] = true;
   }
-  fp8_gemm_kernel<MODE, GROUPED, TN><<<grid, Epi<GROUPED>::kThreads, smem, st>>>(ta, tb, prm, probs, nprobs);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(Epi<GROUPED>::kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = PAIR ? 2 : 1;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = PAIR ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, ta, tb, prm, probs, nprobs);
 }
 
 template <int MODE, bool GROUPED>
 cudaError_t launch_tile(int tn, const GemmParams& prm, const CUtensorMap& ta, const CUtensorMap& tb, int grid,
                         const GemmProblem* probs, int nprobs, cudaStream_t st) {
-  if (tn == 128) return launch_mode<MODE, GROUPED, 128>(prm, ta, tb, grid, probs, nprobs, st);
-  return launch_mode<MODE, GROUPED, 256>(prm, ta, tb, grid, probs, nprobs, st);
+  if (tn == 128) return launch_mode<MODE, GROUPED, 128, false>(prm, ta, tb, grid, probs, nprobs, st);
+  return launch_mode<MODE, GROUPED, 256, false>(prm, ta, tb, grid, probs, nprobs, st);
+}
+
+// Single problems whose operand planes (one of A, one of B) exceed this are paced: smaller
+// ones stay in the L2 however the pairs drift (4096^3, 34 MB: no difference).
+constexpr int64_t kPaceBytes = int64_t(64) << 20;
+constexpr int kPaceWord = 32;  // offset of the pacing words in the zeroed 256-byte flag region
+
+// CTA pairs for the residue products of single problems in 256-wide tiles.  Their launch takes about 2 us longer
+// (clusters, the barriers between the CTAs) and their products 10-13% less time, so they
+// pay from about 16 us of products on: `rounds` (units per CTA, in passes) x k-steps of at
+// least 56 (single / pair: 512 x 512 x 4096 55 / 49 us, 1024^3 35 / 35, 768^3 27 / 29, 2048^3
+// 160 / 141, 4096^3 1067 / 956, 16384^3 70.9 / 64.5 ms).  A pair's tile is 256 rows high: not
+// where that pads the rows by over a third (384 x 4096 x 4096 145 / 137 us, 128 x 8192 x 4096
+// 160 / 166).  The bound product gains nothing (4096^3 55 / 55 us; at 16384^3 0.2 ms, which
+// the power cap takes back from the residue products).
+bool use_pairs(const GemmArgs& g, int BN) {
+  if (g.mode != kModeResidue || BN != 256 || g.num_sms % 2 != 0) return false;
+  const int64_t rows1 = (g.m + BM - 1) / BM, rows2 = (g.m + 2 * BM - 1) / (2 * BM);
+  if (6 * rows2 > 4 * rows1) return false;
+  const int64_t rounds = (g.mods->planes * rows1 * ((g.n + BN - 1) / BN) + g.num_sms - 1) / g.num_sms;
+  return rounds * ((g.k + BK - 1) / BK) >= 56;
 }
 
 int tile_width(int tile_n) { return tile_n == 128 ? 128 : 256; }
@@ -792,7 +934,8 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
   prm.n = g.n;
   prm.k = g.k;
   const int BN = g.mode == kModePaper ? 256 : tile_width(g.tile_n);
-  prm.tiles_m = (g.m + BM - 1) / BM;
+  const bool pair = use_pairs(g, BN);
+  prm.tiles_m = (g.m + (pair ? 2 : 1) * BM - 1) / ((pair ? 2 : 1) * BM);
   prm.tiles_n = (g.n + BN - 1) / BN;
   prm.tiles = prm.tiles_m * prm.tiles_n;
   const bool residues = g.mode == kModeResidue || g.mode == kModePaper;
@@ -812,17 +955,20 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
   prm.rowshift = g.rowshift;
   prm.wait_ns = g.wait_ns;
   prm.stall = g.stall ? 1 : 0;
+  prm.pace = pair && static_cast<int64_t>(g.m + g.n) * g.k >= kPaceBytes ? g.flags + kPaceWord : nullptr;
 
   CUtensorMap ta, tb;
   if (!encode_fp8_map(&ta, a, g.k, g.m, planes_a, lda8, g.plane_stride_a, BM, BK)) return cudaErrorInvalidValue;
-  if (!encode_fp8_map(&tb, b, g.k, g.n, planes_b, ldb8, g.plane_stride_b, BN, BK)) return cudaErrorInvalidValue;
+  if (!encode_fp8_map(&tb, b, g.k, g.n, planes_b, ldb8, g.plane_stride_b, pair ? BN / 2 : BN, BK))
+    return cudaErrorInvalidValue;
   const int ctas = g.num_sms < kMaxGemmCtas ? g.num_sms : kMaxGemmCtas;
-  const int grid = prm.num_units < ctas ? prm.num_units : ctas;
+  const int grid = pair ? 2 * std::min(prm.num_units, ctas / 2) : std::min(prm.num_units, ctas);
   switch (g.mode) {
     case kModeResidue:
-      return launch_tile<kModeResidue, false>(BN, prm, ta, tb, grid, nullptr, 0, st);
+      return pair ? launch_mode<kModeResidue, false, 256, true>(prm, ta, tb, grid, nullptr, 0, st)
+                  : launch_tile<kModeResidue, false>(BN, prm, ta, tb, grid, nullptr, 0, st);
     case kModePaper:
-      return launch_mode<kModePaper, false, 256>(prm, ta, tb, grid, nullptr, 0, st);
+      return launch_mode<kModePaper, false, 256, false>(prm, ta, tb, grid, nullptr, 0, st);
     case kModeBound:
       return launch_tile<kModeBound, false>(BN, prm, ta, tb, grid, nullptr, 0, st);
     default:
