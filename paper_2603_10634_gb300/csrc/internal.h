@@ -47,17 +47,17 @@ struct ModTable {
 };
 
 // The product path's residue system (rns.h): constants of the residue kernels, per
-// remainder taken (pairs of single moduli, then Karatsuba moduli).  FP32 constants are
-// duplicated pairs, as above.
+// remainder taken (groups of single moduli, then Karatsuba moduli).
 struct RnsTable {
   int N;
-  int singles, pairs, kars;
+  int singles, groups, kars;
   int pair_words, lut_words;                // 16-byte words of the pairs' digit tables, of all
-  float2 neg_m2[kMaxVirtual], inv_m2[kMaxVirtual];
-  float2 w2[kMaxVirtual][5];                // 2^(11 j) mod M, symmetric
+  float neg_m[kMaxVirtual], inv_m[kMaxVirtual];
+  float w[kMaxVirtual][kRnsPieces - 1];     // 2^22, 2^33, 2^44 mod M, symmetric
+  float neg_p[kMaxVirtual][kGroupMax];      // members of a group: -p, RN(1/p)
+  float inv_p[kMaxVirtual][kGroupMax];
   int16_t pow2[kMaxVirtual][kPow2Table];    // 2^t mod M, symmetric
-  int32_t lut_bias[kMaxVirtual];            // byte offset of remainder 0 in the block's digit
-                                            // tables, minus the bits of 1.5 2^23
+  int32_t lut_base[kMaxVirtual];            // byte offset of remainder 0 in the block's digit tables
 };
 
 // One modulus of the FP8 products' epilogue.

@@ -260,28 +260,33 @@ bool build_rns_table(int N, RnsTable* rt) {
   std::memset(rt, 0, sizeof(*rt));
   rt->N = N;
   rt->singles = kRnsSingles[N];
-  rt->pairs = rns_pairs(N);
+  rt->groups = rns_groups(N);
   rt->kars = kRnsKars[N];
-  rt->pair_words = pair_lut_offset(rt->pairs) / 16;
-  rt->lut_words = rns_lut_bytes(N) / 16;
-  for (int v = 0; v < rns_virtual(N); ++v) {
-    const bool kar = v >= rt->pairs;
-    const int M = kar ? kKarP[v - rt->pairs] : pair_modulus(v);
-    rt->neg_m2[v] = make_float2(-static_cast<float>(M), -static_cast<float>(M));
-    const float inv = static_cast<float>(1.0 / M);
-    rt->inv_m2[v] = make_float2(inv, inv);
+  const int pairs = rns_lut_pairs(N);
+  rt->pair_words = pair_lut_offset(pairs) / 16;
+  rt->lut_words = (pair_lut_offset(pairs) + kar_lut_offset(rt->kars)) / 16;
+  for (int v = 0; v < rt->groups + rt->kars; ++v) {
+    const bool kar = v >= rt->groups;
+    const int M = kar ? kKarP[v - rt->groups] : group_modulus(v);
+    rt->neg_m[v] = -static_cast<float>(M);
+    rt->inv_m[v] = static_cast<float>(1.0 / M);
     int x = 1;
     for (int t = 0; t < kPow2Table; ++t) {
       rt->pow2[v][t] = static_cast<int16_t>(symmetric(x, M));
-      if (t % 11 == 0 && t / 11 < 5) {
-        const float w = static_cast<float>(symmetric(x, M));
-        rt->w2[v][t / 11] = make_float2(w, w);
-      }
+      for (int j = 1; j < kRnsPieces; ++j)
+        if (t == kRnsPieceShift[j]) rt->w[v][j - 1] = static_cast<float>(symmetric(x, M));
       x = 2 * x % M;
     }
-    const int entry = kar ? 4 : 2;
-    const int base = kar ? pair_lut_offset(rt->pairs) + kar_lut_offset(v - rt->pairs) : pair_lut_offset(v);
-    rt->lut_bias[v] = base + entry * (M / 2 + 1) - 0x4B400000;
+    if (kar) {
+      rt->lut_base[v] = pair_lut_offset(pairs) + kar_lut_offset(v - rt->groups) + 4 * (M / 2 + 1);
+    } else if (v < kLutPairs) {
+      rt->lut_base[v] = pair_lut_offset(v) + 2 * (M / 2 + 1);
+    } else {
+      for (int j = 0; j < (v == kGroups1 - 1 ? 3 : 2); ++j) {
+        rt->neg_p[v][j] = -static_cast<float>(kSingleP[2 * v + j]);
+        rt->inv_p[v][j] = static_cast<float>(1.0 / kSingleP[2 * v + j]);
+      }
+    }
   }
   return true;
 }

@@ -10,14 +10,15 @@
 //
 // Those are the digits of the hybrid list; the parity hooks return them (PaperSys below).
 // The product path converts to the residue system of rns.h instead (RnsSys): remainders
-// mod 11 to 20 moduli of at most 2303, each looked up in a table of digit bytes.
+// mod groups of its moduli (products of at most 2431), whose digits come from a table or,
+// for single moduli up to 32, from a second reduction.
 //
 // a' is never formed as a wide integer or a double.  With a = M 2^E (M the 53-bit
 // significand) and t = E + e: a' = M' 2^t', where M' = M >> -t, t' = 0 if t < 0 and
 // M' = M, t' = t otherwise.  M' is split once into five signed 11-bit pieces c_j
 // (exact floats), and for each modulus
 //   x = sum_j c_j w_j,   w_j = 2^(11j) mod p in [-p/2, p/2],   |x| <= 5 (2^11 - 1) 544 < 2^23
-// (RnsSys: |w_j| <= 1151, |x| < 2^24)
+// (RnsSys: four pieces, |x| < 2^24)
 // is formed with exact FP32 fused multiply-adds.  For odd p the exact product x (1/p)
 // rounded once (see reduce) differs from x / p by at most |x| 2^-24 / p < 1/(2p), less
 // than the distance from x / p to any half-integer, so q is the nearest integer to x / p
@@ -326,16 +327,22 @@ __device__ __forceinline__ void task_planes(int N, const Tables& tb, const f2 (&
 
 // ------------------------------------------------------------------ residue systems
 // What the kernels below are templated on: the constants a block stages in shared memory
-// and the conversion of a task's 8 elements to every plane.
+// and the conversion of a task, 8 elements v[u] with exponents ex(u), to every plane.
 struct PaperSys {  // the hybrid list's digits (parity hooks)
   using Table = ModTable;
   static size_t smem_bytes(const Table&) { return sizeof(Tables); }
   static __device__ __forceinline__ void load(const Table& mt, unsigned char* smem) {
     load_tables(mt, *reinterpret_cast<Tables*>(smem));
   }
-  static __device__ __forceinline__ void planes(const Table& mt, const unsigned char* smem,
-                                                const f2 (&c)[kPairs][kPieces], const TpPack& tp, int any_tp,
-                                                const PlaneStore& st, uint32_t* flags) {
+  template <class Ex>
+  static __device__ __forceinline__ void task(const Table& mt, const unsigned char* smem,
+                                              const unsigned long long (&v)[kElems], Ex ex, const PlaneStore& st,
+                                              uint32_t* flags, bool& range_err) {
+    f2 c[kPairs][kPieces];
+    TpPack tp{};
+    int any_tp = 0;
+#pragma unroll
+    for (int u = 0; u < kElems; ++u) decode_into(c, u, v[u], ex(u), tp, any_tp, range_err);
     task_planes(mt.N, *reinterpret_cast<const Tables*>(smem), c, tp, any_tp, st, flags);
   }
 };
@@ -350,9 +357,9 @@ struct alignas(16) KarLut {
 };
 constexpr PairLut make_pair_lut() {
   PairLut t{};
-  for (int q = 0; q < kPairs1; ++q) {
-    const int M = pair_modulus(q), h1 = M / 2 + 1, o = pair_lut_offset(q) / 2;
-    const int p0 = kSingleP[2 * q], p1 = 2 * q + 1 < kSingles ? kSingleP[2 * q + 1] : 1;
+  for (int q = 0; q < kLutPairs; ++q) {
+    const int M = group_modulus(q), h1 = M / 2 + 1, o = pair_lut_offset(q) / 2;
+    const int p0 = kSingleP[2 * q], p1 = kSingleP[2 * q + 1];
     for (int r = -h1; r <= h1; ++r)
       t.v[o + r + h1] = static_cast<uint16_t>(e4m3_of_digit(single_digit(r, p0)) | (e4m3_of_digit(single_digit(r, p1)) << 8));
   }
@@ -388,21 +395,24 @@ constexpr KarLut make_kar_lut() {
 __device__ const PairLut g_pair_lut = make_pair_lut();
 __device__ const KarLut g_kar_lut = make_kar_lut();
 
+// Shared-memory constants of one remainder taken.
 struct __align__(16) RnsConsts {
   f2 neg_m, inv_m;
-  f2 w[kPieces];
-  int bias, pad;  // byte offset of remainder 0's entry, minus the bits of 1.5 2^23
+  f2 w[kRnsPieces - 1];
+  f2 scale, base;                                  // table address of a remainder (address())
+  f2 neg_p[kGroupMax], inv_p[kGroupMax];           // members of a group without a table
 };
+static_assert(sizeof(RnsConsts) % 16 == 0, "");
 
 struct RnsSys {  // the product path's digits
   using Table = RnsTable;
   // shared memory: constants, 2^t mod M (64 floats each), digit tables
   static constexpr int kPerModulus = static_cast<int>(sizeof(RnsConsts)) + 4 * kPow2Table;
   static size_t smem_bytes(const Table& rt) {
-    return static_cast<size_t>(rns_virtual(rt.N)) * kPerModulus + static_cast<size_t>(rns_lut_bytes(rt.N));
+    return static_cast<size_t>(rt.groups + rt.kars) * kPerModulus + 16 * static_cast<size_t>(rt.lut_words);
   }
   static __device__ __forceinline__ void load(const Table& rt, unsigned char* smem) {
-    const int nv = rt.pairs + rt.kars;
+    const int nv = rt.groups + rt.kars;
     RnsConsts* cs = reinterpret_cast<RnsConsts*>(smem);
     float* pow2 = reinterpret_cast<float*>(smem + nv * sizeof(RnsConsts));
     uint4* lut = reinterpret_cast<uint4*>(smem + nv * kPerModulus);
@@ -414,32 +424,100 @@ struct RnsSys {  // the product path's digits
       pow2[i] = static_cast<float>(rt.pow2[i / kPow2Table][i % kPow2Table]);
     for (int v = threadIdx.x; v < nv; v += blockDim.x) {
       RnsConsts& c = cs[v];
-      c.neg_m = rt.neg_m2[v];
-      c.inv_m = rt.inv_m2[v];
+      c.neg_m = dup(rt.neg_m[v]);
+      c.inv_m = dup(rt.inv_m[v]);
 #pragma unroll
-      for (int j = 0; j < kPieces; ++j) c.w[j] = rt.w2[v][j];
-      c.bias = rt.lut_bias[v];
-      c.pad = 0;
+      for (int j = 0; j < kRnsPieces - 1; ++j) c.w[j] = dup(rt.w[v][j]);
+      c.scale = dup(__int_as_float(v < rt.groups ? 2 : 4));
+      c.base = dup(__int_as_float(rt.lut_base[v]));
+#pragma unroll
+      for (int j = 0; j < kGroupMax; ++j) {
+        c.neg_p[j] = dup(rt.neg_p[v][j]);
+        c.inv_p[j] = dup(rt.inv_p[v][j]);
+      }
     }
     __syncthreads();
   }
 
-  // Table entries (byte offsets scaled by 4 or 2: entry size) of an element pair's
-  // remainders.  x = sum_j c_j w_j is an exact integer below 2^24; the rounded quotient
-  // is within 1/2 + 1/M of x / M, so the remainder lies within the table's slack.
+  // ---------------------------------------------------------------- elements
+  // |a'| = c_0 + c_1 2^22 + c_2 2^33 + c_3 2^44, pieces of 22, 11, 11 and 9 bits: the first
+  // has weight 1 mod every M, so it may be wide and x = sum_j c_j w_j still stays below
+  // 2^22 + 1216 (2^11 + 2^11 + 2^9) < 2^24.  piece b -> float via the bit pattern of
+  // 2^23 + b, the sign folded into one FMA: sg (2^23 + b) - sg 2^23 = sg b.
+  static __device__ __forceinline__ void pieces(uint32_t lo, uint32_t hi, uint32_t sign, float (&c)[kRnsPieces]) {
+    const float sg = __uint_as_float((sign & 0x80000000u) | 0x3F800000u);
+    const float off = __uint_as_float((sign & 0x80000000u) ^ 0xCB000000u);  // -sg 2^23
+    const uint32_t p[kRnsPieces] = {(lo & 0x3FFFFFu) | 0x4B000000u, (__funnelshift_r(lo, hi, 22) & 0x7FFu) | 0x4B000000u,
+                                    ((hi >> 1) & 0x7FFu) | 0x4B000000u, (hi >> 12) | 0x4B000000u};
+#pragma unroll
+    for (int j = 0; j < kRnsPieces; ++j) c[j] = fmaf(sg, __uint_as_float(p[j]), off);
+  }
+
+  // Elements the fast decoding does not cover: t > 0 (a' >= 2^53), subnormals, NaN and Inf.
+  static __device__ __forceinline__ bool rare(unsigned long long bits, int e) {
+    const uint32_t hi = static_cast<uint32_t>(bits >> 32), lo = static_cast<uint32_t>(bits);
+    const uint32_t h = hi & 0x7FFFFFFFu;
+    const int t = static_cast<int>(h >> 20) + e - 1075;
+    // h - 2^20 wraps for zero and subnormals, and reaches 0x7FE00000 for NaN and Inf
+    return t > 0 || (h - 0x00100000u >= 0x7FE00000u && (h | lo) != 0u);
+  }
+  static __device__ __forceinline__ void decode_fast(unsigned long long bits, int e, float (&c)[kRnsPieces]) {
+    const uint32_t hi = static_cast<uint32_t>(bits >> 32), lo = static_cast<uint32_t>(bits);
+    const uint32_t h = hi & 0x7FFFFFFFu;
+    const int be = static_cast<int>(h >> 20);
+    const int sh = be ? 1075 - be - e : 64;  // >= 0; zero shifts out
+    const uint32_t mh = (h & 0xFFFFFu) | 0x100000u;
+    // (mh : lo) >> sh
+    const int over = max(sh - 32, 0);
+    const uint32_t ml = over < 32 ? __funnelshift_rc(lo, mh, sh) >> over : 0u;
+    pieces(ml, sh < 32 ? mh >> sh : 0u, hi, c);
+  }
+  static __device__ __forceinline__ void decode_any(unsigned long long bits, int e, float (&c)[kRnsPieces], int& tp,
+                                                    bool& range_err) {
+    const unsigned long long mag = bits & kAbsMask;
+    unsigned long long Mp = 0;
+    tp = 0;
+    if (mag != 0 && mag < kInfBits) {
+      const int be = static_cast<int>(mag >> 52);
+      const unsigned long long M = be ? ((mag & ((1ull << 52) - 1)) | (1ull << 52)) : mag;
+      const int t = (be ? be - 1075 : -1074) + e;
+      if (t >= 0) {
+        Mp = M;
+        tp = t;
+      } else {
+        Mp = (t <= -64) ? 0ull : (M >> (-t));
+      }
+      if (tp >= kPow2Table) {
+        range_err = true;
+        Mp = 0;
+        tp = 0;
+      }
+    }
+    pieces(static_cast<uint32_t>(Mp), static_cast<uint32_t>(Mp >> 32), static_cast<uint32_t>(bits >> 32), c);
+  }
+
+  // ---------------------------------------------------------------- remainders
+  // Remainders of an element pair mod M.  x is an exact integer below 2^24; the rounded
+  // quotient is within 1/2 + 1/M of x / M, so the remainder lies within [-h - 1, h + 1].
+  static __device__ __forceinline__ f2 reduce_near(f2 x, f2 neg_m, f2 inv_m) {
+    return __ffma2_rn(neg_m, round_magic(__ffma2_rn(x, inv_m, dup(kMagic))), x);
+  }
   template <bool P2>
-  static __device__ __forceinline__ int2 entry(const f2 (&c)[kPieces], int tp0, int tp1, const RnsConsts& k,
-                                               const float* pow2, float scale) {
+  static __device__ __forceinline__ f2 remainder(const f2 (&c)[kRnsPieces], int tp0, int tp1, const RnsConsts& k,
+                                                 const float* pow2) {
     f2 x = c[0];
 #pragma unroll
-    for (int j = 1; j < kPieces; ++j) x = __ffma2_rn(c[j], k.w[j], x);
-    f2 r = __ffma2_rn(k.neg_m, round_magic(__ffma2_rn(x, k.inv_m, dup(kMagic))), x);
-    if constexpr (P2) {
-      x = __fmul2_rn(r, make_float2(pow2[tp0], pow2[tp1]));  // below 2^21
-      r = __ffma2_rn(k.neg_m, round_magic(__ffma2_rn(x, k.inv_m, dup(kMagic))), x);
-    }
-    const f2 y = __ffma2_rn(r, dup(scale), dup(kMagic));  // bits: those of 1.5 2^23, plus scale r
-    return make_int2(__float_as_int(y.x) + k.bias, __float_as_int(y.y) + k.bias);
+    for (int j = 1; j < kRnsPieces; ++j) x = __ffma2_rn(c[j], k.w[j - 1], x);
+    f2 r = reduce_near(x, k.neg_m, k.inv_m);
+    if constexpr (P2) r = reduce_near(__fmul2_rn(r, make_float2(pow2[tp0], pow2[tp1])), k.neg_m, k.inv_m);
+    return r;
+  }
+  // Byte offsets of the remainders' table entries: `scale` and `base` are the entry size
+  // and the offset of remainder 0 as multiples of 2^-149, and so is the result, a
+  // non-negative (sub)normal whose bit pattern is the integer.
+  static __device__ __forceinline__ int2 address(f2 r, const RnsConsts& k) {
+    const f2 y = __ffma2_rn(r, k.scale, k.base);
+    return make_int2(__float_as_int(y.x), __float_as_int(y.y));
   }
 
   static __device__ __forceinline__ void check(const uint32_t (&w)[2], uint32_t* flags) {
@@ -448,25 +526,33 @@ struct RnsSys {  // the product path's digits
                 flags);
   }
 
-  // Every plane of a task, one remainder at a time (rolled loops: see all_planes).
+  // Every plane of a task, one remainder at a time (rolled loops: see all_planes).  Of the
+  // single moduli, the three pairs above 32 go through a table (their digits need the
+  // r -+ p step); the others reduce the group's remainder once more and convert, which
+  // costs two instructions per element and pair more than a lookup but none of its bank
+  // conflicts (a lookup takes 4.1 shared-memory cycles a warp, and those bound the kernel:
+  // with every pair in a table the load/store pipe was 75% busy, 12 lookups an element;
+  // now 67%, 7 lookups).  4096 x 4096, N = 12: rows 149 -> 133 us, columns 174 -> 162 us.
   template <bool P2>
   static __device__ __forceinline__ void all(const Table& rt, const unsigned char* smem,
-                                             const f2 (&c)[kPairs][kPieces], const TpPack& tp, PlaneStore st,
+                                             const f2 (&c)[kPairs][kRnsPieces], const TpPack& tp, PlaneStore st,
                                              uint32_t* flags) {
-    const int nv = rt.pairs + rt.kars;
+    const int nv = rt.groups + rt.kars;
     const RnsConsts* cs = reinterpret_cast<const RnsConsts*>(smem);
     const float* pow2 = reinterpret_cast<const float*>(smem + nv * sizeof(RnsConsts));
     const unsigned char* lut = smem + nv * kPerModulus;
+    auto rem = [&](int v, int pr) {
+      return remainder<P2>(c[pr], tp_of(tp, 2 * pr), tp_of(tp, 2 * pr + 1), cs[v], pow2 + v * kPow2Table);
+    };
 #pragma unroll 1
-    for (int v = rt.pairs; v < nv; ++v) {
+    for (int v = rt.groups; v < nv; ++v) {
       uint32_t w[3][2];
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         uint32_t e[4];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const int pr = 2 * q + u;
-          const int2 i = entry<P2>(c[pr], tp_of(tp, 2 * pr), tp_of(tp, 2 * pr + 1), cs[v], pow2 + v * kPow2Table, 4.0f);
+          const int2 i = address(rem(v, 2 * q + u), cs[v]);
           e[2 * u] = *reinterpret_cast<const uint32_t*>(lut + i.x);
           e[2 * u + 1] = *reinterpret_cast<const uint32_t*>(lut + i.y);
         }
@@ -482,15 +568,14 @@ struct RnsSys {  // the product path's digits
       }
     }
 #pragma unroll 1
-    for (int v = 0; v < rt.pairs; ++v) {
+    for (int v = 0; v < rt.groups && v < kLutPairs; ++v) {
       uint32_t w[2][2];
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         uint32_t e[4];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const int pr = 2 * q + u;
-          const int2 i = entry<P2>(c[pr], tp_of(tp, 2 * pr), tp_of(tp, 2 * pr + 1), cs[v], pow2 + v * kPow2Table, 2.0f);
+          const int2 i = address(rem(v, 2 * q + u), cs[v]);
           e[2 * u] = *reinterpret_cast<const uint16_t*>(lut + i.x);
           e[2 * u + 1] = *reinterpret_cast<const uint16_t*>(lut + i.y);
         }
@@ -498,20 +583,68 @@ struct RnsSys {  // the product path's digits
         w[0][q] = __byte_perm(a, b, 0x6420);
         w[1][q] = __byte_perm(a, b, 0x7531);
       }
-      check(w[0], flags);
-      st.put(w[0]);
-      if (2 * v + 1 < rt.singles) {
-        check(w[1], flags);
-        st.put(w[1]);
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        check(w[x], flags);
+        st.put(w[x]);
+      }
+    }
+    int left = rt.singles - 2 * kLutPairs;
+#pragma unroll 1
+    for (int v = kLutPairs; v < rt.groups; ++v) {
+      f2 r[kPairs];
+#pragma unroll
+      for (int pr = 0; pr < kPairs; ++pr) r[pr] = rem(v, pr);
+      const int members = min(left, v == kGroups1 - 1 ? 3 : 2);
+      left -= members;
+#pragma unroll 1
+      for (int x = 0; x < members; ++x) {
+        const f2 neg_p = cs[v].neg_p[x], inv_p = cs[v].inv_p[x];
+        uint32_t w[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          w[q] = e4m3x4(reduce_near(r[2 * q], neg_p, inv_p), reduce_near(r[2 * q + 1], neg_p, inv_p));
+        check(w, flags);
+        st.put(w);
       }
     }
   }
 
-  static __device__ __forceinline__ void planes(const Table& rt, const unsigned char* smem,
-                                                const f2 (&c)[kPairs][kPieces], const TpPack& tp, int any_tp,
-                                                const PlaneStore& st, uint32_t* flags) {
-    if (__any_sync(0xffffffffu, any_tp != 0)) all<true>(rt, smem, c, tp, st, flags);
-    else all<false>(rt, smem, c, tp, st, flags);
+  template <class Ex>
+  static __device__ __forceinline__ void task(const Table& rt, const unsigned char* smem,
+                                              const unsigned long long (&v)[kElems], Ex ex, const PlaneStore& st,
+                                              uint32_t* flags, bool& range_err) {
+    bool any = false;
+#pragma unroll
+    for (int u = 0; u < kElems; ++u) any |= rare(v[u], ex(u));
+    f2 c[kPairs][kRnsPieces];
+    TpPack tp{};
+    auto put = [&](int u, const float (&x)[kRnsPieces]) {
+#pragma unroll
+      for (int j = 0; j < kRnsPieces; ++j) {
+        if (u & 1) c[u >> 1][j].y = x[j];
+        else c[u >> 1][j].x = x[j];
+      }
+    };
+    if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+      for (int u = 0; u < kElems; ++u) {
+        float x[kRnsPieces];
+        int t;
+        decode_any(v[u], ex(u), x, t, range_err);
+        tp.w[u >> 2] |= static_cast<uint32_t>(t) << (8 * (u & 3));
+        put(u, x);
+      }
+      all<true>(rt, smem, c, tp, st, flags);
+    } else {
+#pragma unroll
+      for (int u = 0; u < kElems; ++u) {
+        float x[kRnsPieces];
+        decode_fast(v[u], ex(u), x);
+        put(u, x);
+      }
+      all<false>(rt, smem, c, tp, st, flags);
+    }
   }
 };
 
@@ -568,14 +701,9 @@ __device__ __forceinline__ void residues_rows_body(const ResidArgs& a, const typ
 #pragma unroll
       for (int t = 0; t < kElems; ++t) v[t] = (row_ok && h0 + t < a.k) ? __ldg(x + t) : 0ull;
     }
-    f2 c[kPairs][kPieces];
-    TpPack tp{};
-    int any_tp = 0;
-#pragma unroll
-    for (int t = 0; t < kElems; ++t) decode_into(c, t, v[t], e, tp, any_tp, range_err);
     const PlaneStore st{a.planes + static_cast<int64_t>(row_ok ? row : 0) * a.ldp + h0, a.plane_stride,
                         row_ok && h0 < a.kp};
-    Sys::planes(mt, tb, c, tp, any_tp, st, a.flags);
+    Sys::task(mt, tb, v, [e](int) { return e; }, st, a.flags, range_err);
   }
   if (range_err) atomicOr(a.flags, kFlagRange);
 }
@@ -631,16 +759,12 @@ __device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, con
       const bool active = j < a.lines && h0 < a.kp;
       const int e = j < a.lines ? a.exps[j] : 0;
       const unsigned long long* src = tile + c * kTilePitch + chunk * 8;
-      f2 cc[kPairs][kPieces];
-      TpPack tp{};
-      int any_tp = 0;
+      unsigned long long v[kElems];
 #pragma unroll
-      for (int u = 0; u < kElems; ++u) {
-        decode_into(cc, u, src[u ^ ((chunk >> 1) & 7)], e, tp, any_tp, range_err);
-      }
+      for (int u = 0; u < kElems; ++u) v[u] = src[u ^ ((chunk >> 1) & 7)];
       const PlaneStore st{a.planes + static_cast<int64_t>(j < a.lines ? j : 0) * a.ldp + (h0 < a.kp ? h0 : 0),
                           a.plane_stride, active};
-      Sys::planes(mt, tb, cc, tp, any_tp, st, a.flags);
+      Sys::task(mt, tb, v, [e](int) { return e; }, st, a.flags, range_err);
     }
     __syncthreads();  // the tile is reloaded
   }
@@ -749,18 +873,17 @@ __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const
       const bool active = j < a.n && ib < a.m;
       const int hj = j < a.n ? a.h[j] : 0;
       const unsigned long long* src = tile + c * kTilePitch + chunk * 8;
-      f2 cc[kPairs][kPieces];
-      TpPack tp{};
-      int any_tp = 0;
+      unsigned long long v[kElems];
+      int ex[kElems];
 #pragma unroll
       for (int u = 0; u < kElems; ++u) {
         const int i = ib + u;
-        const int ex = hj - (i < a.m ? a.e[i] : 0);
-        decode_into(cc, u, src[u ^ ((chunk >> 1) & 7)], ex, tp, any_tp, range_err);
+        ex[u] = hj - (i < a.m ? a.e[i] : 0);
+        v[u] = src[u ^ ((chunk >> 1) & 7)];
       }
       const PlaneStore st{a.planesH + static_cast<int64_t>(j < a.n ? j : 0) * a.ldh + (ib < a.m ? ib : 0),
                           static_cast<int64_t>(a.n) * a.ldh, active};
-      RnsSys::planes(mt, tb, cc, tp, any_tp, st, a.flags);
+      RnsSys::task(mt, tb, v, [&ex](int u) { return ex[u]; }, st, a.flags, range_err);
     }
     // row pass: G' (lines i, positions j): kTileCols / 8 chunks per row
 #pragma unroll 1
@@ -771,18 +894,17 @@ __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const
       const int i = i0 + r, jb = j0 + chunk * 8;
       const bool active = i < a.m && jb < a.n;
       const int gi = i < a.m ? a.g[i] : 0;
-      f2 cc[kPairs][kPieces];
-      TpPack tp{};
-      int any_tp = 0;
+      unsigned long long v[kElems];
+      int ex[kElems];
 #pragma unroll
       for (int u = 0; u < kElems; ++u) {
         const int c = chunk * 8 + u, j = jb + u;
-        const int ex = gi - (j < a.n ? a.f[j] : 0);
-        decode_into(cc, u, tile[c * kTilePitch + tile_slot(r)], ex, tp, any_tp, range_err);
+        ex[u] = gi - (j < a.n ? a.f[j] : 0);
+        v[u] = tile[c * kTilePitch + tile_slot(r)];
       }
       const PlaneStore st{a.planesG + static_cast<int64_t>(i < a.m ? i : 0) * a.ldg + (jb < a.n ? jb : 0),
                           static_cast<int64_t>(a.m) * a.ldg, active};
-      RnsSys::planes(mt, tb, cc, tp, any_tp, st, a.flags);
+      RnsSys::task(mt, tb, v, [&ex](int u) { return ex[u]; }, st, a.flags, range_err);
     }
     __syncthreads();  // the tile is reloaded
   }

@@ -57,13 +57,19 @@ constexpr int rns_moduli(int N) { return kRnsSingles[N] + kRnsKars[N]; }
 constexpr int rns_planes(int N) { return kRnsSingles[N] + 3 * kRnsKars[N]; }  // = FP8 products
 // Plane order: three planes (u, v, w) per Karatsuba modulus, then one per single modulus.
 
-// The residue kernels reduce mod pairs of single moduli (49 47, 43 41, ..., 17 13, 11) and
-// mod each Karatsuba modulus, and look the digits up in a table indexed by the remainder.
-constexpr int kPairs1 = (kSingles + 1) / 2;  // pairs, the last one 11 alone
-constexpr int pair_modulus(int q) { return kSingleP[2 * q] * (2 * q + 1 < kSingles ? kSingleP[2 * q + 1] : 1); }
-constexpr int rns_pairs(int N) { return (kRnsSingles[N] + 1) / 2; }
-constexpr int rns_virtual(int N) { return rns_pairs(N) + kRnsKars[N]; }  // remainders taken per element
-constexpr int kMaxVirtual = kPairs1 + kKars;
+// The residue kernels take one remainder per group of single moduli (49 47, 43 41, 37 32,
+// 31 29, 27 25, 23 19, 17 13 11) and one per Karatsuba modulus.
+constexpr int kGroups1 = 7, kGroupMax = 3;
+constexpr int kLutPairs = 3;   // groups whose digits come from a table indexed by the remainder
+constexpr int kRnsPieces = 4;  // pieces of |a'|: 22, 11, 11 and 9 bits
+constexpr int kRnsPieceShift[kRnsPieces] = {0, 22, 33, 44};
+constexpr int group_modulus(int q) {
+  return kSingleP[2 * q] * kSingleP[2 * q + 1] * (q == kGroups1 - 1 ? kSingleP[2 * q + 2] : 1);
+}
+constexpr int rns_groups(int N) {
+  return kRnsSingles[N] > 2 * (kGroups1 - 1) ? kGroups1 : (kRnsSingles[N] + 1) / 2;
+}
+constexpr int kMaxVirtual = kGroups1 + kKars;
 
 // Table entries of a modulus M: remainders -(h + 1) .. h + 1, h = M / 2 (one of slack on
 // each side: the rounded quotient may leave a remainder just past +-M / 2).
@@ -72,7 +78,7 @@ OZK2_HD constexpr int round16(int bytes) { return (bytes + 15) / 16 * 16; }
 // Byte offsets: 16-bit entries for the pairs, then 32-bit entries for the Karatsuba moduli.
 constexpr int pair_lut_offset(int q) {
   int o = 0;
-  for (int i = 0; i < q; ++i) o += round16(2 * lut_entries(pair_modulus(i)));
+  for (int i = 0; i < q; ++i) o += round16(2 * lut_entries(group_modulus(i)));
   return o;
 }
 constexpr int kar_lut_offset(int j) {  // within the Karatsuba tables
@@ -80,9 +86,9 @@ constexpr int kar_lut_offset(int j) {  // within the Karatsuba tables
   for (int i = 0; i < j; ++i) o += round16(4 * lut_entries(kKarP[i]));
   return o;
 }
-constexpr int kPairLutBytes = pair_lut_offset(kPairs1);
+constexpr int kPairLutBytes = pair_lut_offset(kLutPairs);
 constexpr int kKarLutBytes = kar_lut_offset(kKars);
-constexpr int rns_lut_bytes(int N) { return pair_lut_offset(rns_pairs(N)) + kar_lut_offset(kRnsKars[N]); }
+constexpr int rns_lut_pairs(int N) { return rns_groups(N) < kLutPairs ? rns_groups(N) : kLutPairs; }
 
 // ------------------------------------------------------------------ digits
 constexpr int kDigitMax = 32;

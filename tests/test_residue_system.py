@@ -76,3 +76,37 @@ def test_constant_lines_have_exact_products(cuda, N, m, n, k):
     assert torch.equal(C[whole], (k * a * b)[whole])
     if N >= 12:
         assert bool(whole.all())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("N", [2, 9, 12, 17, 20])
+def test_unusual_elements_match_the_oracle(cuda, N):
+    """Zeros of both signs, subnormals, entries far below and far above their line's
+    neighbours (shifted out, or a' >= 2^53), in rows and in columns, bit for bit."""
+    import paper_2603_10634_gb300 as ozk
+
+    g = np.random.default_rng(N)
+    m, n, k = 21, 18, 45
+    special = np.array([0.0, -0.0, 5e-324, -3e-310, 2.0**-1022, 1.0, -2.0**-1000, 2.0**400, -1.5 * 2.0**60, 2.0**-60])
+    A = np.where(g.random((m, k)) < 0.3, special[g.integers(0, len(special), (m, k))], g.standard_normal((m, k)))
+    B = np.where(g.random((k, n)) < 0.3, special[g.integers(0, len(special), (k, n))], g.standard_normal((k, n)))
+    A[0], B[:, 0] = 5e-324 * g.integers(0, 9, k), 2.0**-1030 * g.integers(-9, 9, k)  # subnormal lines
+    A[1], B[:, 1] = 0.0, -0.0
+    A[2] *= 2.0**-300
+    Ad, Bd = torch.from_numpy(A).to(cuda), torch.from_numpy(B).to(cuda)
+    sc = ozk.scales(Ad, Bd, num_moduli=N)
+    C = ozk.dgemm(Ad, Bd, num_moduli=N).cpu().numpy()
+    status = ozk.device_status()
+    e, f = sc["e"].cpu().numpy(), sc["f"].cpu().numpy()
+    want = oz.ozk2_dgemm(A, B, N, e=e, f=f)["C"]
+
+    # an element whose significand would be scaled by 2^64 or more is out of the library's
+    # range (possible for subnormal lines at large N): flagged, its line not compared
+    def in_range(X, ex):
+        lsb = np.maximum(np.frexp(X)[1] - 53, -1074)
+        return ~((X != 0) & (lsb + ex[:, None] >= 64)).any(axis=1)
+
+    ok = np.outer(in_range(A, e), in_range(B.T, f))
+    assert status == ("OZK2_OK" if ok.all() else "OZK2_ERR_RANGE")
+    assert np.array_equal(C.view(np.uint64)[ok], want.view(np.uint64)[ok])
+    assert N > 12 or ok.all()
