@@ -11,12 +11,20 @@
 //   V = sum_l c_l w_l = sum_g t_g (P2 / P_g),   t_g = sum_{l in g} c_l y_l (P_g / p_l)
 //
 // over groups of up to four single or two Karatsuba moduli with product P_g: t_g is one
-// 32-bit integer (a 32-bit multiply-add per residue), and only the groups multiply the
-// wide weights, which are split into balanced 32-bit limbs accumulated in 64-bit integers
-// (N = 12: 6 x 4 wide multiply-adds per output instead of 12 x 4 one modulus at a time).
+// 32-bit integer, and only the groups multiply the wide weights, which are split into
+// balanced 32-bit limbs accumulated in 64-bit integers (N = 12: 19 wide multiply-adds per
+// output instead of 48 one modulus at a time).  The single moduli of a group come in two
+// pairs, t_g = d_0 P_1 + d_1 P_0 with d a two-way dot product of the pair's bytes (dp2a;
+// one byte permute interleaves the bytes of two planes for two outputs).
 // C' = V - round(V / P2) P2: V / P2 is C' / P2 (at most 0.455 in magnitude) away from an
-// integer, and the FP32 estimate from V's leading limbs is off by less than 0.04, so its
-// rounding is exact and no comparison with +-P2 / 2 follows.
+// integer, and the fixed-point estimate sum_g t_g round(2^35 / P_g) is off by little enough
+// (checked for each N when the table is built) that its rounding is exact and no comparison
+// with +-P2 / 2 follows.  The quotient is
+// known before the wide sums, which start from -Q P2: one carry pass is left.
+//
+// What bounds it: the integer pipes (31 bytes move per output at N = 12; HBM alone would take
+// 77 us for 4096^2 outputs).  One modulus at a time and a quotient from the normalised sum
+// took 232 instructions an output and 179 us; this form takes 168 and 133 us.
 //
 // The parity hook reconstructs from the hybrid list's residues one modulus at a time (the
 // quotient from 16-bit fractions, settled by one exact comparison when it is close).
@@ -72,19 +80,32 @@ __device__ __forceinline__ void into_symmetric_range(uint32_t (&v)[L], const Crt
 }
 
 // RN(v 2^-scale) of the two's complement integer v.
+// The double of (-1)^neg (top : mid : low : rest) 2^(32 (ti - 2) - scale), rounded to
+// nearest even, when it is a normal number or overflows and has more than 53 bits; ti is
+// the index of `top`, the leading nonzero limb, and `rest` is nonzero if any lower limb is.
+// The 96-bit window shifted left to its leading one holds the 53 significand bits, the
+// round bit and most of the sticky bits.  false: not covered.
+__device__ __forceinline__ bool finish_window(uint32_t top, uint32_t mid, uint32_t low, uint32_t rest, int ti,
+                                              bool neg, int scale, double& out) {
+  const int sh = __clz(top);
+  const int ebias = 32 * ti + 32 - sh - 53 - scale + 1074;  // exponent field before the implicit bit
+  if (32 * ti + 32 - sh <= 53 || ebias < 0) return false;
+  const uint32_t w2 = __funnelshift_l(mid, top, sh), w1 = __funnelshift_l(low, mid, sh), w0 = low << sh;
+  // round half to even: add 2^10 - 1 plus the last kept bit below it, with the bits under
+  // the window folded into its last one
+  const uint32_t b = w1 | ((w0 | rest) != 0u ? 1u : 0u);
+  uint64_t mant = (static_cast<uint64_t>(w2) << 21) | (w1 >> 11);
+  if ((b & 0x400u) && ((b & 0x3FFu) | (w1 & 0x800u))) mant += 1;
+  uint64_t bits = (static_cast<uint64_t>(static_cast<uint32_t>(ebias)) << 52) + mant;
+  if (ebias >= 2047 || (bits >> 52) >= 2047) bits = 0x7FF0000000000000ull;
+  if (neg) bits |= 0x8000000000000000ull;
+  out = __longlong_as_double(static_cast<long long>(bits));
+  return true;
+}
+
+// RN(|v| 2^-scale) with its sign for any v (magnitude limbs).
 template <int L>
-__device__ __forceinline__ double crt_finish(uint32_t (&v)[L], int scale, bool nan_out) {
-  if (nan_out) return __longlong_as_double(0x7FF8000000000000ll);
-  const bool neg = is_negative<L>(v);
-  if (neg) {  // magnitude
-    uint64_t c = 1;
-#pragma unroll
-    for (int t = 0; t < L; ++t) {
-      const uint64_t s = static_cast<uint64_t>(~v[t]) + c;
-      v[t] = static_cast<uint32_t>(s);
-      c = s >> 32;
-    }
-  }
+__device__ __noinline__ double finish_any(const uint32_t (&v)[L], bool neg, int scale) {
   // the top nonzero limb, the two below it and whether anything lies lower still
   uint32_t top = 0u, mid = 0u, low = 0u, rest = 0u, below = 0u;  // below: OR of v[0 .. t - 3]
   int ti = -1;
@@ -100,23 +121,9 @@ __device__ __forceinline__ double crt_finish(uint32_t (&v)[L], int scale, bool n
     if (t >= 2) below |= v[t >= 2 ? t - 2 : 0];
   }
   if (ti < 0) return 0.0;
+  double out;
+  if (finish_window(top, mid, low, rest, ti, neg, scale, out)) return out;
   const int nbits = 32 * ti + 32 - __clz(top);
-  if (nbits > 53 && nbits - 53 >= scale - 1074) {
-    // the common case, a normal result from more than 53 bits: the 96-bit window
-    // (top : mid : low) shifted left to its leading one holds the 53 significand bits,
-    // the round bit and most of the sticky bits
-    const int sh = __clz(top);
-    const uint32_t w2 = __funnelshift_l(mid, top, sh), w1 = __funnelshift_l(low, mid, sh), w0 = low << sh;
-    uint64_t mant = (static_cast<uint64_t>(w2) << 21) | (w1 >> 11);
-    const bool round_bit = (w1 >> 10) & 1u;
-    const bool sticky = ((w1 & 0x3FFu) | w0 | rest) != 0u;
-    if (round_bit && (sticky || (mant & 1ull))) mant += 1;
-    const int ebias = nbits - 53 - scale + 1074;  // exponent field before the implicit bit
-    uint64_t bits = (ebias >= 2047) ? 0x7FF0000000000000ull : (static_cast<uint64_t>(ebias) << 52) + mant;
-    if ((bits >> 52) >= 2047) bits = 0x7FF0000000000000ull;
-    if (neg) bits |= 0x8000000000000000ull;
-    return __longlong_as_double(static_cast<long long>(bits));
-  }
   // position (bit index of C') of the result's last significand bit
   const int rpos = max(nbits - 53, scale - 1074);
   uint64_t mant;
@@ -152,10 +159,47 @@ __device__ __forceinline__ double crt_finish(uint32_t (&v)[L], int scale, bool n
   return __longlong_as_double(static_cast<long long>(bits));
 }
 
+// RN(v 2^-scale) of the two's complement integer v, whose magnitude usually reaches limb
+// TL or TL - 1 (TL >= 1).
+template <int L, int TL>
+__device__ __forceinline__ double crt_finish(uint32_t (&v)[L], int scale) {
+  const bool neg = is_negative<L>(v);
+  const uint32_t m = neg ? 0xFFFFFFFFu : 0u;
+  uint32_t c = neg ? 1u : 0u;
+#pragma unroll
+  for (int t = 0; t < L; ++t) {  // magnitude
+    const uint64_t x = static_cast<uint64_t>(v[t] ^ m) + c;
+    v[t] = static_cast<uint32_t>(x);
+    c = static_cast<uint32_t>(x >> 32);
+  }
+  const bool high = v[TL] != 0u;
+  const uint32_t v1 = v[TL - 1], v2 = TL >= 2 ? v[TL >= 2 ? TL - 2 : 0] : 0u, v3 = TL >= 3 ? v[TL >= 3 ? TL - 3 : 0] : 0u;
+  uint32_t rest = 0u;
+#pragma unroll
+  for (int t = 0; t + 4 <= TL; ++t) rest |= v[t];
+  const uint32_t top = high ? v[TL] : v1, mid = high ? v1 : v2, low = high ? v2 : v3;
+  double out;
+  if (top != 0u && finish_window(top, mid, low, high ? v3 | rest : rest, high ? TL : TL - 1, neg, scale, out)) return out;
+  return finish_any<L>(v, neg, scale);
+}
+
 // ------------------------------------------------------------------ product path
-// 4 adjacent columns per thread: one 32-bit load per single modulus, one 64-bit load per
+// Adjacent columns per thread: 4 (2 for large N, whose residues would not fit the
+// registers): one 32-bit (16-bit) load per single modulus, one 64-bit (32-bit) load per
 // Karatsuba modulus, all issued together; one instance per N, so every loop unrolls.
-constexpr int kCrtCols = 4;
+OZK2_HD constexpr int crt_cols(int N) { return N <= 14 ? 4 : 2; }
+
+__device__ __forceinline__ int dp2a_lo(uint32_t w, uint32_t x, int c) {
+  return __dp2a_lo(static_cast<int>(w), static_cast<int>(x), c);
+}
+__device__ __forceinline__ int dp2a_hi(uint32_t w, uint32_t x, int c) {
+  return __dp2a_hi(static_cast<int>(w), static_cast<int>(x), c);
+}
+
+template <int N>
+struct CrtShape {
+  static constexpr uint64_t kLimbs = crt_limbs_packed(N);
+};
 
 template <int N>
 __device__ __forceinline__ void rns_crt_body(const int16_t* __restrict__ cres, const int8_t* __restrict__ cres8,
@@ -164,9 +208,11 @@ __device__ __forceinline__ void rns_crt_body(const int16_t* __restrict__ cres, c
                                              const uint8_t* __restrict__ rowstat, const uint8_t* __restrict__ colstat,
                                              double* __restrict__ C, int64_t ldc, const RnsCrt& ct, int64_t vblock,
                                              int64_t vgrid) {
-  constexpr int S = kRnsSingles[N], K = kRnsKars[N], L = rns_limbs(N), KG = crt_kar_group(N);
-  constexpr int TL = (kRnsBits[N] - 1) / 32, tb = kRnsBits[N] - 32 * TL;  // P2's leading limb and its bits
-  const int nq = (n + kCrtCols - 1) / kCrtCols;
+  constexpr int S = kRnsSingles[N], K = kRnsKars[N], L = rns_limbs(N), KG = kCrtKarGroup, W = crt_cols(N);
+  constexpr int TL = (kRnsBits[N] - 1) / 32 > 0 ? (kRnsBits[N] - 1) / 32 : 1;  // P2's leading limb
+  constexpr uint64_t kLimbs = CrtShape<N>::kLimbs;                // limbs of the groups' weights
+  constexpr int Q = (S + 3) / 4, GK = (K + KG - 1) / KG;  // groups of single and of Karatsuba moduli
+  const int nq = (n + W - 1) / W;
   const int64_t total = static_cast<int64_t>(m) * nq;
   const int64_t stride = vgrid * blockDim.x;
   const int64_t first = vblock * blockDim.x + threadIdx.x;
@@ -182,83 +228,101 @@ __device__ __forceinline__ void rns_crt_body(const int16_t* __restrict__ cres, c
       jq -= nq;
       if (++i >= m) break;
     }
-    const int j0 = jq * kCrtCols;
+    const int j0 = jq * W;
     const int64_t off = static_cast<int64_t>(i) * ldr + j0;
-    uint2 rk[K > 0 ? K : 1];
-    uint32_t rs[S];
+    uint32_t rk[K > 0 ? K : 1][W / 2];
+    uint32_t rs[4 * Q];
 #pragma unroll
-    for (int l = 0; l < K; ++l) rk[l] = __ldg(reinterpret_cast<const uint2*>(cres + off + l * rstride));
+    for (int l = 0; l < K; ++l) {
+      if constexpr (W == 4) {
+        const uint2 x = __ldg(reinterpret_cast<const uint2*>(cres + off + l * rstride));
+        rk[l][0] = x.x;
+        rk[l][W / 2 - 1] = x.y;
+      } else {
+        rk[l][0] = __ldg(reinterpret_cast<const unsigned int*>(cres + off + l * rstride));
+      }
+    }
 #pragma unroll
-    for (int l = 0; l < S; ++l) rs[l] = __ldg(reinterpret_cast<const unsigned int*>(cres8 + off + l * rstride));
+    for (int l = 0; l < 4 * Q; ++l) {
+      if (l >= S) rs[l] = 0u;
+      else if constexpr (W == 4) rs[l] = __ldg(reinterpret_cast<const unsigned int*>(cres8 + off + l * rstride));
+      else rs[l] = __ldg(reinterpret_cast<const unsigned short*>(cres8 + off + l * rstride));
+    }
+    // exponents and status of the columns: the arrays are padded to 256 bytes, so reading
+    // up to the group's end stays inside them
+    int fj[W];
+    uint32_t cst;
+    if constexpr (W == 4) {
+      const int4 x = __ldg(reinterpret_cast<const int4*>(f + j0));
+      fj[0] = x.x;
+      fj[1] = x.y;
+      fj[W - 2] = x.z;
+      fj[W - 1] = x.w;
+      cst = __ldg(reinterpret_cast<const unsigned int*>(colstat + j0));
+    } else {
+      const int2 x = __ldg(reinterpret_cast<const int2*>(f + j0));
+      fj[0] = x.x;
+      fj[1] = x.y;
+      cst = __ldg(reinterpret_cast<const unsigned short*>(colstat + j0));
+    }
     const int ei = e[i];
-    const bool rbad = rowstat != nullptr && (rowstat[i] & kLineNonfinite);
-    double out[kCrtCols];
+    if (rowstat[i] & kLineNonfinite) cst = 0x01010101u * kLineNonfinite;
+    // bytes of two planes interleaved: outputs 0, 1 (and 2, 3) of a pair of moduli
+    uint32_t rp[2 * Q][W / 2];
 #pragma unroll
-    for (int z = 0; z < kCrtCols; ++z) {
-      int64_t acc[L];
+    for (int x = 0; x < 2 * Q; ++x) {
+      rp[x][0] = __byte_perm(rs[2 * x], rs[2 * x + 1], 0x5140);
+      if constexpr (W == 4) rp[x][W / 2 - 1] = __byte_perm(rs[2 * x], rs[2 * x + 1], 0x7362);
+    }
+    double out[W];
 #pragma unroll
-      for (int t = 0; t < L; ++t) acc[t] = 0;
-      int g = 0;
+    for (int z = 0; z < W; ++z) {
+      int tg[GK + Q];
 #pragma unroll
-      for (int l0 = 0; l0 < K; l0 += KG) {
-        int t32 = 0;
+      for (int g = 0; g < GK; ++g) {
+        tg[g] = 0;
 #pragma unroll
-        for (int l = l0; l < l0 + KG && l < K; ++l) {
-          const uint32_t w = z < 2 ? rk[l].x : rk[l].y;
-          t32 += static_cast<int16_t>((z & 1) ? (w >> 16) : (w & 0xFFFFu)) * ct.u[l];
+        for (int l = g * KG; l < (g + 1) * KG && l < K; ++l) {
+          const uint32_t w = rk[l][z >> 1];
+          tg[g] += static_cast<int16_t>((z & 1) ? (w >> 16) : (w & 0xFFFFu)) * ct.u[l];
         }
-#pragma unroll
-        for (int t = 0; t < L; ++t) acc[t] += static_cast<int64_t>(t32) * ct.wb[g][t];
-        ++g;
       }
 #pragma unroll
-      for (int l0 = 0; l0 < S; l0 += kCrtSingleGroup) {
-        int t32 = 0;
+      for (int g = 0; g < Q; ++g) {
+        int d[2];
 #pragma unroll
-        for (int l = l0; l < l0 + kCrtSingleGroup && l < S; ++l)
-          t32 += static_cast<int8_t>(rs[l] >> (8 * z)) * ct.u[K + l];
-#pragma unroll
-        for (int t = 0; t < L; ++t) acc[t] += static_cast<int64_t>(t32) * ct.wb[g][t];
-        ++g;
+        for (int x = 0; x < 2; ++x) {
+          const uint32_t r = rp[2 * g + x][z >> 1];
+          d[x] = (z & 1) ? dp2a_hi(ct.pw[2 * g + x], r, 0) : dp2a_lo(ct.pw[2 * g + x], r, 0);
+        }
+        tg[GK + g] = d[0] * ct.pm[2 * g + 1] + d[1] * ct.pm[2 * g];
       }
-      // V in 32-bit limbs v[0 .. L-1] and a signed top
+      int64_t est = int64_t(1) << (kCrtFracBits - 1);
+#pragma unroll
+      for (int g = 0; g < GK + Q; ++g) est += static_cast<int64_t>(tg[g]) * ct.frac[g];
+      const int q = static_cast<int>(est >> kCrtFracBits);
+      // v = sum_g t_g W_g - Q P2, limb by limb
       uint32_t v[L];
       int64_t carry = 0;
 #pragma unroll
       for (int t = 0; t < L; ++t) {
-        const int64_t x = carry + acc[t];
-        v[t] = static_cast<uint32_t>(x);
-        carry = x >> 32;
-      }
-      // V / P2: |V| < 2^12 P2 < 2^(12 + tb + 32 TL).  tb <= 18: limb TL with its sign is an
-      // int32, limb TL - 1 refines it; else the 32-bit window 13 bits above limb TL's base
-      float est;
-      if constexpr (tb <= 18) {
-        est = static_cast<float>(static_cast<int32_t>(v[TL])) * ct.est_hi;
-        if constexpr (TL > 0) est = fmaf(static_cast<float>(v[TL > 0 ? TL - 1 : 0]), ct.est_lo, est);
-      } else {
-        const uint32_t above = TL + 1 < L ? v[TL + 1 < L ? TL + 1 : 0] : static_cast<uint32_t>(carry);
-        est = (static_cast<float>(static_cast<int32_t>(__funnelshift_r(v[TL], above, 13))) + 0.5f) * ct.est_hi;
-      }
-      const int q = __float2int_rn(est);
-      carry = 0;
+        int64_t x = carry - static_cast<int64_t>(q) * static_cast<int64_t>(ct.P[t]);
 #pragma unroll
-      for (int t = 0; t < L; ++t) {
-        const int64_t x = carry + v[t] - static_cast<int64_t>(q) * static_cast<int64_t>(ct.P[t]);
+        for (int g = 0; g < GK + Q; ++g)
+          if (t < static_cast<int>((kLimbs >> (4 * g)) & 15u)) x += static_cast<int64_t>(tg[g]) * ct.wb[g][t];
         v[t] = static_cast<uint32_t>(x);
-        carry = x >> 32;
+        carry = x >> 32;  // arithmetic: signed carry
       }
-      const int j = j0 + z < n ? j0 + z : n - 1;
-      const bool bad = rbad || (colstat != nullptr && (colstat[j] & kLineNonfinite));
-      out[z] = crt_finish<L>(v, ei + f[j], bad);
+      out[z] = crt_finish<L, TL>(v, ei + fj[z]);
+      if ((cst >> (8 * z)) & kLineNonfinite) out[z] = __longlong_as_double(0x7FF8000000000000ll);
     }
     double* dst = C + static_cast<int64_t>(i) * ldc + j0;
-    if (vec && j0 + kCrtCols <= n) {
-      reinterpret_cast<double2*>(dst)[0] = make_double2(out[0], out[1]);
-      reinterpret_cast<double2*>(dst)[1] = make_double2(out[2], out[3]);
+    if (vec && j0 + W <= n) {
+#pragma unroll
+      for (int z = 0; z < W; z += 2) reinterpret_cast<double2*>(dst)[z / 2] = make_double2(out[z], out[z + 1]);
     } else {
 #pragma unroll
-      for (int z = 0; z < kCrtCols; ++z)
+      for (int z = 0; z < W; ++z)
         if (j0 + z < n) dst[z] = out[z];
     }
   }
@@ -319,7 +383,7 @@ __global__ void __launch_bounds__(256)
       carry = y >> 32;  // arithmetic: signed carry
     }
     if (off > 19660 || off < -19660) into_symmetric_range<L>(v, ct);  // |est - Q| > 0.3
-    C[static_cast<int64_t>(i) * ldc + j] = crt_finish<L>(v, e[i] + f[j], false);
+    C[static_cast<int64_t>(i) * ldc + j] = crt_finish<L, L - 1>(v, e[i] + f[j]);
   }
 }
 
@@ -335,7 +399,7 @@ template <int N>
 cudaError_t launch_N(const int16_t* cres, const int8_t* cres8, int64_t ldr, int64_t rs, int m, int n, const int32_t* e,
                      const int32_t* f, const uint8_t* rowstat, const uint8_t* colstat, double* C, int64_t ldc,
                      const RnsCrt& ct, cudaStream_t st) {
-  const int grid = crt_grid(static_cast<int64_t>(m) * ((n + kCrtCols - 1) / kCrtCols));
+  const int grid = crt_grid(static_cast<int64_t>(m) * ((n + crt_cols(N) - 1) / crt_cols(N)));
   rns_crt_kernel<N><<<grid, 256, 0, st>>>(cres, cres8, ldr, rs, m, n, e, f, rowstat, colstat, C, ldc, ct);
   return cudaGetLastError();
 }

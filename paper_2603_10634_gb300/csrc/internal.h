@@ -75,24 +75,45 @@ struct GemmMods {
 };
 
 // CRT of the product path: sum_l c_l w_l with w_l = y_l P2 / p_l is formed as
-// sum_g t_g P2 / P_g, t_g = sum_{l in g} c_l u_l an int32 (u_l = y_l P_g / p_l), over small
-// groups g of moduli with product P_g.
+// sum_g t_g P2 / P_g, t_g = sum_{l in g} c_l y_l P_g / p_l an int32, over small groups g of
+// moduli with product P_g.
 constexpr int kCrtSingleGroup = 4;  // single moduli per group
-OZK2_HD constexpr int crt_kar_group(int N) { return kRnsKars[N] <= 6 ? 2 : 1; }  // 64-bit limb sums bound it
-OZK2_HD constexpr int crt_groups(int N) {
-  return (kRnsSingles[N] + kCrtSingleGroup - 1) / kCrtSingleGroup + (kRnsKars[N] + crt_kar_group(N) - 1) / crt_kar_group(N);
+constexpr int kCrtKarGroup = 2;     // Karatsuba moduli per group
+constexpr int crt_groups(int N) {
+  return (kRnsSingles[N] + kCrtSingleGroup - 1) / kCrtSingleGroup + (kRnsKars[N] + kCrtKarGroup - 1) / kCrtKarGroup;
 }
 constexpr int kMaxCrtGroups = 16;
+constexpr int kCrtFracBits = 35;  // fixed-point bits of the quotient estimate (2^35 / 17 fits an int32)
 // Bits of P2 for N (checked by build_rns_crt).
 constexpr int kRnsBits[21] = {0,  12,  22,  33,  42,  52,  61,  68,  77,  87, 96,
                               106, 113, 122, 132, 140, 149, 157, 167, 175, 183};
 OZK2_HD constexpr int rns_limbs(int N) { return kRnsBits[N] <= 95 ? 3 : (kRnsBits[N] + 1 + 31) / 32; }  // signed |x| < P2
+// Limbs of P2 / P_g (Karatsuba groups first): enough for its bits plus a sign.
+constexpr int crt_group_limbs(int N, int g) {
+  const int kg = kCrtKarGroup, gk = (kRnsKars[N] + kg - 1) / kg;
+  const int size = g < gk ? kg : kCrtSingleGroup, l0 = g < gk ? g * kg : (g - gk) * kCrtSingleGroup;
+  const int count = g < gk ? kRnsKars[N] : kRnsSingles[N];
+  long long pg = 1;
+  for (int l = l0; l < l0 + size && l < count; ++l) pg *= g < gk ? kKarP[l] : kSingleP[l];
+  int lg = 0;
+  while ((pg >> (lg + 1)) != 0) ++lg;
+  const int limbs = (kRnsBits[N] - lg + 1 + 31) / 32;
+  return limbs < rns_limbs(N) ? limbs : rns_limbs(N);
+}
+// All groups', 4 bits each.
+constexpr uint64_t crt_limbs_packed(int N) {
+  uint64_t x = 0;
+  for (int g = 0; g < crt_groups(N); ++g) x |= static_cast<uint64_t>(crt_group_limbs(N, g)) << (4 * g);
+  return x;
+}
 struct RnsCrt {
   int N;
-  int32_t u[kMaxRns];                          // Karatsuba moduli first, as in the products
+  int32_t u[kKars];                            // Karatsuba moduli: y_l P_g / p_l
+  uint32_t pw[kSingles + 1];                   // pairs of single moduli: y_0 p_1, y_1 p_0 (int16 each)
+  int32_t pm[kSingles + 1];                    // and their products p_0 p_1
+  int32_t frac[kMaxCrtGroups];                 // round(2^kCrtFracBits / P_g)
   int32_t wb[kMaxCrtGroups][kMaxLimbs];        // P2 / P_g in balanced 32-bit limbs; Karatsuba groups first
   uint32_t P[kMaxLimbs];
-  float est_hi, est_lo;                        // V / P2 from V's limbs (crt.cu)
 };
 
 struct CrtTable {

@@ -350,14 +350,14 @@ bool build_rns_crt(int N, RnsCrt* rc) {
   const std::vector<int> mods = rns_list(N);
   const Big P = rns_product(N);
   if (bit_length(P) != kRnsBits[N]) return false;
-  {  // the slack the rounded quotient relies on: 10 P2 >= 11 P
-    int mp[kMaxModuli];
-    if (hybrid_moduli(N, mp) != N) return false;
-    int e2, e1;
-    const double p2 = top_as_double(P, &e2), p1 = top_as_double(product_of(N), &e1);
-    if (std::ldexp(p2, e2 - e1) < 1.1 * p1) return false;
-  }
-  const int L = rns_limbs(N), kars = kRnsKars[N], total = rns_moduli(N);
+  int mp[kMaxModuli];
+  if (hybrid_moduli(N, mp) != N) return false;
+  int e2, e1;
+  const double p2 = top_as_double(P, &e2), p1 = top_as_double(product_of(N), &e1);
+  const double slack = std::ldexp(p2, e2 - e1) / p1;  // P2 / P
+  double est_err = 0.0;                               // of the quotient estimate
+  double limb_sum[kMaxLimbs] = {};
+  const int kars = kRnsKars[N], total = rns_moduli(N);
   auto big_div_mod = [](const Big& x, int p, Big* q) {
     uint32_t rem = 0;
     Big d = div_small(x, static_cast<uint32_t>(p), &rem);
@@ -366,8 +366,10 @@ bool build_rns_crt(int N, RnsCrt* rc) {
   };
   int g = 0;
   for (int l0 = 0; l0 < total; ++g) {
-    const int size = l0 < kars ? crt_kar_group(N) : kCrtSingleGroup;
-    const int l1 = l0 < kars ? (l0 + size < kars ? l0 + size : kars) : (l0 + size < total ? l0 + size : total);
+    const bool kar = l0 < kars;
+    const int size = kar ? kCrtKarGroup : kCrtSingleGroup;
+    const int end = kar ? kars : total;
+    const int l1 = l0 + size < end ? l0 + size : end;
     int64_t Pg = 1;
     Big rest = P;
     for (int l = l0; l < l1; ++l) {
@@ -381,21 +383,37 @@ bool build_rns_crt(int N, RnsCrt* rc) {
       big_div_mod(P, p, &pl);  // P2 / p
       const int y = symmetric(modinv(big_div_mod(pl, p, nullptr), p), p);
       const int64_t u = static_cast<int64_t>(y) * (Pg / p);
-      rc->u[l] = static_cast<int32_t>(u);
       tmax += (p / 2 + 1) * (u < 0 ? -u : u);  // residues |c| <= p / 2 + 1
+      if (kar) {
+        rc->u[l] = static_cast<int32_t>(u);
+      } else {
+        const int i = l - kars, other = (i ^ 1) + kars < total ? kSingleP[i ^ 1] : 1;
+        const int w = y * other;
+        if (w < -32768 || w > 32767) return false;
+        rc->pw[i / 2] |= (static_cast<uint32_t>(w) & 0xFFFFu) << (16 * (i & 1));
+      }
     }
-    if (tmax >= (int64_t(1) << 31) || g >= kMaxCrtGroups || !balanced_limbs(rest, L, rc->wb[g])) return false;
+    if (!kar)
+      for (int x = 0; x < 2; ++x) {  // products of the group's two pairs (1 for a missing modulus)
+        const int i = l0 - kars + 2 * x;
+        rc->pm[i / 2] = (i + kars < total ? kSingleP[i] : 1) * (i + 1 + kars < total ? kSingleP[i + 1] : 1);
+      }
+    const double fr = std::ldexp(1.0, kCrtFracBits) / static_cast<double>(Pg);
+    if (fr >= 2147483647.0) return false;
+    rc->frac[g] = static_cast<int32_t>(std::llround(fr));
+    est_err += std::ldexp(static_cast<double>(tmax), -kCrtFracBits) * std::fabs(fr - static_cast<double>(rc->frac[g]));
+    if (tmax >= (int64_t(1) << 31) || g >= kMaxCrtGroups || !balanced_limbs(rest, crt_group_limbs(N, g), rc->wb[g]))
+      return false;
+    for (int t = 0; t < kMaxLimbs; ++t)
+      limb_sum[t] += static_cast<double>(tmax) * std::fabs(static_cast<double>(rc->wb[g][t]));
     l0 = l1;
   }
+  for (double x : limb_sum)
+    if (x >= std::ldexp(1.0, 62)) return false;  // the 64-bit limb sums
   if (g != crt_groups(N)) return false;
   for (size_t t = 0; t < P.size(); ++t) rc->P[t] = P[t];
-  // quotient estimate: see crt.cu; scale of one unit of limb TL (or of 2^13 of them) in P2s
-  int eP;
-  const double Pt = top_as_double(P, &eP);
-  const int TL = (kRnsBits[N] - 1) / 32, tb = kRnsBits[N] - 32 * TL;
-  rc->est_hi = static_cast<float>(std::ldexp(1.0 / Pt, 32 * TL + (tb <= 18 ? 0 : 13) - eP));
-  rc->est_lo = static_cast<float>(std::ldexp(1.0 / Pt, 32 * (TL - 1) - eP));
-  return true;
+  // V / P2 is at most P / (2 P2) from an integer: the rounded estimate is that integer
+  return slack >= 1.1 && 0.5 / slack + est_err < 0.499;
 }
 
 float p_prime_f32(int N) {
