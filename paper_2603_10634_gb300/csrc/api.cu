@@ -188,7 +188,7 @@ Operand shift_lines(const Operand& o, int64_t first) {
 struct Layout {
   int64_t kp, ldp, ldr;  // kp: bytes of k per row; ldp: digit-plane row pitch
   int planes;
-  size_t flags, R, S, colmaxA, colbadA, colmaxB, colbadB, zero_end;
+  size_t flags, R, S, zero_end;
   size_t eprime, fprime, e, f, rowstat, colstat;
   size_t Abar, BbarT, partA, partB, planesA, planesB, cres, cres8, total;
 };
@@ -228,10 +228,6 @@ Layout make_layout(int64_t m, int64_t n, int64_t k, int N, bool fast) {
   L.flags = take(256);
   L.R = take(4 * size_t(m));
   L.S = take(4 * size_t(n));
-  L.colmaxA = take(4 * size_t(m));
-  L.colbadA = take(4 * size_t(m));
-  L.colmaxB = take(4 * size_t(n));
-  L.colbadB = take(4 * size_t(n));
   L.zero_end = o;
   L.eprime = take(4 * size_t(m));
   L.fprime = take(4 * size_t(n));
@@ -350,45 +346,56 @@ cudaError_t copy_2d(void* dst, size_t dpitch, const void* src, size_t spitch, si
 }
 
 // ------------------------------------------------------------------ phases
-// Zero the bound maxima and column reductions of a call (and its flag word when
-// clear_flags: the first block of a call; later blocks keep what earlier blocks
-// recorded).
-ozk2_status zero_scratch(Ctx& c, bool clear_flags) {
-  const Layout& L = c.L;
-  if (clear_flags)
-    OZK2_TRY(cudaMemsetAsync(c.ws, 0, L.zero_end, c.st));
-  else
-    OZK2_TRY(cudaMemsetAsync(c.ws + L.R, 0, L.zero_end - L.R, c.st));
-  return OZK2_OK;
+// Words a call's first scaling launch zeroes: the bound maxima and, with clear_flags (the
+// first block of a call; later blocks keep what earlier blocks recorded), the flag region.
+struct ZeroWords {
+  uint32_t* at = nullptr;
+  int64_t words = 0;
+};
+ZeroWords zero_words(const Ctx& c, bool clear_flags) {
+  const size_t from = clear_flags ? c.L.flags : c.L.R;
+  return ZeroWords{c.at<uint32_t>(from), int64_t(c.L.zero_end - from) / 4};
 }
 
 // Which operand a scaling launch serves.
 struct Side {
-  size_t eprime, stat, bar, sq, part, colmax, colbad;
+  size_t eprime, stat, bar, sq, part, planes;
 };
-Side side_a(const Layout& L) { return Side{L.eprime, L.rowstat, L.Abar, L.R, L.partA, L.colmaxA, L.colbadA}; }
-Side side_b(const Layout& L) { return Side{L.fprime, L.colstat, L.BbarT, L.S, L.partB, L.colmaxB, L.colbadB}; }
+Side side_a(const Layout& L) { return Side{L.eprime, L.rowstat, L.Abar, L.R, L.partA, L.planesA}; }
+Side side_b(const Layout& L) { return Side{L.fprime, L.colstat, L.BbarT, L.S, L.partB, L.planesB}; }
+
+// Lines [first, first + lines) of one operand (`op` points at line `first`).  The partial
+// column maxima live in the rows of the first digit plane that these lines' residues
+// overwrite later: ldp >= 32 bytes a line, of which ceil(k / 64) words are enough.
+ScaleJob scale_job(const Ctx& c, const Operand& op, int64_t first, int lines, const Side& sd) {
+  const Layout& L = c.L;
+  ScaleJob j{};
+  j.X = op.ptr;
+  j.ld = op.ld;
+  j.lines = lines;
+  j.kcontig = op.kcontig;
+  j.ep = c.at<int32_t>(sd.eprime) + first;
+  j.stat = c.at<uint8_t>(sd.stat) + first;
+  j.bar = c.at<uint8_t>(sd.bar) + first * L.kp;
+  j.sq = c.at<float>(sd.sq) + first;
+  j.part = c.at<float>(sd.part) + first * (L.kp / 32);
+  j.keys = reinterpret_cast<uint32_t*>(c.at<uint8_t>(sd.planes) + first * L.ldp);
+  return j;
+}
 
 // e'/status and either the E4M3 bound operand (accurate) or the sums of squares (fast)
-// of lines [first, first + lines) of one operand (`op` points at line `first`).
-ozk2_status scale_operand(Ctx& c, const Operand& op, int64_t first, int lines, const Side& sd) {
-  const Layout& L = c.L;
-  const int64_t kb = L.kp / 32;
-  int32_t* ep = c.at<int32_t>(sd.eprime) + first;
-  uint8_t* stat = c.at<uint8_t>(sd.stat) + first;
-  uint8_t* bar = c.at<uint8_t>(sd.bar) + first * L.kp;
-  float* sq = c.at<float>(sd.sq) + first;
-  if (op.kcontig) {
-    OZK2_TRY(launch_scale_rows(op.ptr, op.ld, lines, c.k, int(L.kp), ep, stat, bar, sq, c.fast,
-                               c.at<uint32_t>(L.flags), c.st));
-    t_launches += 1;
-  } else {
-    uint32_t* cm = c.at<uint32_t>(sd.colmax) + first;
-    uint32_t* cb = c.at<uint32_t>(sd.colbad) + first;
-    OZK2_TRY(launch_colmax(op.ptr, op.ld, c.k, lines, cm, cb, c.st));
-    OZK2_TRY(launch_scale_cols(op.ptr, op.ld, c.k, lines, int(L.kp), cm, cb, ep, stat, bar,
-                               c.at<float>(sd.part) + first * kb, sq, c.fast, c.at<uint32_t>(L.flags), c.st));
-    t_launches += c.fast ? 3 : 2;
+// of up to two operands.
+ozk2_status scale_operands(Ctx& c, const ScaleJob* jobs, int njobs, ZeroWords z) {
+  const int kp = int(c.L.kp);
+  OZK2_TRY(launch_scale_prep(jobs, njobs, c.k, kp, c.fast, z.at, z.words, c.st));
+  t_launches += 1;
+  ScaleJob cols[2];
+  int ncols = 0;
+  for (int i = 0; i < njobs; ++i)
+    if (!jobs[i].kcontig) cols[ncols++] = jobs[i];
+  if (ncols > 0) {
+    OZK2_TRY(launch_scale_cols(cols, ncols, c.k, kp, c.fast, c.st));
+    t_launches += c.fast ? 1 + ncols : 1;
   }
   return OZK2_OK;
 }
@@ -431,7 +438,7 @@ cudaError_t exponents_of(Ctx& c, int64_t i0, int rows, bool cols) {
   return launch_exponents(rows, cols ? c.n : 0, c.at<int32_t>(L.eprime) + i0, c.at<int32_t>(L.fprime),
                           c.at<uint8_t>(L.rowstat) + i0, c.at<uint8_t>(L.colstat), c.at<float>(L.R) + i0,
                           c.at<float>(L.S), c.tab->pprime, delta_f32(), c.at<int32_t>(L.e) + i0,
-                          c.at<int32_t>(L.f), c.st);
+                          c.at<int32_t>(L.f), c.at<uint32_t>(L.flags), c.st);
 }
 
 // Bound product (accurate mode) and the exponents e, f.
@@ -445,10 +452,9 @@ ozk2_status bound_and_exponents(Ctx& c) {
 }
 
 ozk2_status phase_scales(Ctx& c, const Operand& a, const Operand& b, bool clear_flags) {
-  ozk2_status s;
-  if ((s = zero_scratch(c, clear_flags)) != OZK2_OK) return s;
-  if ((s = scale_operand(c, a, 0, c.m, side_a(c.L))) != OZK2_OK) return s;
-  if ((s = scale_operand(c, b, 0, c.n, side_b(c.L))) != OZK2_OK) return s;
+  const ScaleJob jobs[2] = {scale_job(c, a, 0, c.m, side_a(c.L)), scale_job(c, b, 0, c.n, side_b(c.L))};
+  const ozk2_status s = scale_operands(c, jobs, 2, zero_words(c, clear_flags));
+  if (s != OZK2_OK) return s;
   return bound_and_exponents(c);
 }
 
@@ -828,9 +834,9 @@ ozk2_status run_host(ozk2_op transa, ozk2_op transb, int64_t m, int64_t n, int64
     OZK2_TRY(cudaEventRecord(ev_a[q], up));
   }
 
-  if ((s = zero_scratch(c, true)) != OZK2_OK) return s;
   OZK2_TRY(cudaStreamWaitEvent(st, ev_b, 0));
-  if ((s = scale_operand(c, b, 0, int(n), side_b(L))) != OZK2_OK) return s;
+  const ScaleJob job_b = scale_job(c, b, 0, int(n), side_b(L));
+  if ((s = scale_operands(c, &job_b, 1, zero_words(c, true))) != OZK2_OK) return s;
   // fast mode: f_j depends on column j of B alone (Sec. III-E with the Cauchy-Schwarz
   // bound), so B's residues need not wait for A
   auto residues_b = [&]() -> ozk2_status {
@@ -848,7 +854,8 @@ ozk2_status run_host(ozk2_op transa, ozk2_op transb, int64_t m, int64_t n, int64
     if (i1 > i0) {
       const int rows = int(i1 - i0);
       const Operand ai = shift_lines(a, i0);
-      if ((s = scale_operand(c, ai, i0, rows, side_a(L))) != OZK2_OK) return s;
+      const ScaleJob job_a = scale_job(c, ai, i0, rows, side_a(L));
+      if ((s = scale_operands(c, &job_a, 1, ZeroWords{})) != OZK2_OK) return s;
       if (last) mark(c, 1);
       if (!fast) OZK2_TRY(bound_rows(c, i0, rows));
       if (last) mark(c, 2);
@@ -895,7 +902,7 @@ size_t host_workspace_bytes(int64_t m, int64_t n, int64_t k, int N, bool fast) {
 struct BwLayout {
   int64_t np, mp, ldrk, ldrn;
   int planes;
-  size_t flags, R, S, Rk, Sk, colmaxA, colbadA, colmaxC, colbadC, zk, zero_end;
+  size_t flags, R, S, Rk, Sk, zk, zero_end;
   size_t gp, hp, g, h, t, tA, rstatC, cstatC, rstatB, cstatA;
   size_t Gbar, Bhat, AhatT, HhatT, planesG, planesBT, planesAT, planesH, cresA, cresA8, cresB, cresB8, total;
 };
@@ -918,10 +925,6 @@ BwLayout make_bw_layout(int64_t m, int64_t n, int64_t k, int N) {
   L.S = take(4 * size_t(n));
   L.Rk = take(4 * size_t(k));
   L.Sk = take(4 * size_t(k));
-  L.colmaxA = take(4 * size_t(k));
-  L.colbadA = take(4 * size_t(k));
-  L.colmaxC = take(4 * size_t(n));
-  L.colbadC = take(4 * size_t(n));
   L.zk = take(4 * size_t(k));
   L.zero_end = o;
   L.gp = take(4 * size_t(m));
@@ -1039,32 +1042,40 @@ ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64
   OZK2_TRY(cudaMemsetAsync(w, 0, L.zero_end, st));
   const bool wantA = dA != nullptr, wantB = dB != nullptr;
   // bounds and exponents of dC's rows (dA) and columns (dB)
+  auto job = [&](const double* X, int64_t ld, int lines, bool kc, int32_t* ep, size_t stat, size_t bar, uint8_t* keys) {
+    ScaleJob q{};
+    q.X = X;
+    q.ld = ld;
+    q.lines = lines;
+    q.kcontig = kc;
+    q.ep = ep;
+    q.stat = at(stat);
+    q.bar = at(bar);
+    q.keys = reinterpret_cast<uint32_t*>(keys);
+    return q;
+  };
   if (wantA) {
-    OZK2_TRY(launch_scale_rows(dC, lddc, c.m, c.n, int(L.np), gp, at(L.rstatC), at(L.Gbar), nullptr, false, flags, st));
-    OZK2_TRY(launch_scale_rows(B, ldb, c.k, c.n, int(L.np), reinterpret_cast<int32_t*>(at(L.t)), at(L.rstatB),
-                               at(L.Bhat), nullptr, false, flags, st));
+    const ScaleJob rows[2] = {job(dC, lddc, c.m, true, gp, L.rstatC, L.Gbar, nullptr),
+                              job(B, ldb, c.k, true, reinterpret_cast<int32_t*>(at(L.t)), L.rstatB, L.Bhat, nullptr)};
+    OZK2_TRY(launch_scale_prep(rows, 2, c.n, int(L.np), false, nullptr, 0, st));
     OZK2_TRY(bw_bound(c, at(L.Gbar), at(L.Bhat), L.np, c.m, c.k, c.n, reinterpret_cast<float*>(at(L.R)),
                       reinterpret_cast<float*>(at(L.Sk)), reinterpret_cast<const int32_t*>(at(L.t)), nullptr, flags));
-    t_launches += 2;
+    t_launches += 1;
   }
   if (wantB) {
-    uint32_t* cmC = reinterpret_cast<uint32_t*>(at(L.colmaxC));
-    uint32_t* cbC = reinterpret_cast<uint32_t*>(at(L.colbadC));
-    OZK2_TRY(launch_colmax(dC, lddc, c.m, c.n, cmC, cbC, st));
-    OZK2_TRY(launch_scale_cols(dC, lddc, c.m, c.n, int(L.mp), cmC, cbC, hp, at(L.cstatC), at(L.HhatT), nullptr,
-                               nullptr, false, flags, st));
-    uint32_t* cmA = reinterpret_cast<uint32_t*>(at(L.colmaxA));
-    uint32_t* cbA = reinterpret_cast<uint32_t*>(at(L.colbadA));
-    OZK2_TRY(launch_colmax(A, lda, c.m, c.k, cmA, cbA, st));
-    OZK2_TRY(launch_scale_cols(A, lda, c.m, c.k, int(L.mp), cmA, cbA, reinterpret_cast<int32_t*>(at(L.tA)),
-                               at(L.cstatA), at(L.AhatT), nullptr, nullptr, false, flags, st));
+    // the partial maxima in digit planes that are written later (as in scale_job)
+    const ScaleJob cols[2] = {job(dC, lddc, c.n, false, hp, L.cstatC, L.HhatT, at(L.planesH)),
+                              job(A, lda, c.k, false, reinterpret_cast<int32_t*>(at(L.tA)), L.cstatA, L.AhatT, at(L.planesAT))};
+    OZK2_TRY(launch_scale_prep(cols, 2, c.m, int(L.mp), false, nullptr, 0, st));
+    OZK2_TRY(launch_scale_cols(cols, 2, c.m, int(L.mp), false, st));
     OZK2_TRY(bw_bound(c, at(L.AhatT), at(L.HhatT), L.mp, c.k, c.n, c.m, reinterpret_cast<float*>(at(L.Rk)),
                       reinterpret_cast<float*>(at(L.S)), nullptr, reinterpret_cast<const int32_t*>(at(L.tA)), flags));
-    t_launches += 4;
+    t_launches += 2;
   }
   OZK2_TRY(launch_reuse_exponents(wantA ? c.m : 0, gp, at(L.rstatC), reinterpret_cast<float*>(at(L.R)), g,
                                   wantB ? c.n : 0, hp, at(L.cstatC), reinterpret_cast<float*>(at(L.S)), h,
-                                  reuse_budget_f32(N), flags, st));
+                                  reuse_budget_f32(N), at(L.rstatB), wantA ? c.k : 0, at(L.cstatA), wantB ? c.k : 0,
+                                  flags, st));
   // dC's two integer matrices from one read of dC; the forward's planes transposed
   OZK2_TRY(launch_grad_residues(dC, lddc, c.m, c.n, g, f, h, e, wantA ? at(L.planesG) : nullptr, L.np,
                                 wantB ? at(L.planesH) : nullptr, L.mp, c.tab->rt, flags, st));
@@ -1458,7 +1469,7 @@ ozk2_status execute_plan(ozk2_batch_plan plan, cudaStream_t st) {
     return e != cudaSuccess ? e : cudaStreamWaitEvent(st, plan->join, 0);
   };
   OZK2_TRY(fork());
-  OZK2_TRY(launch_scale_batch(probs, plan->cnt, plan->totals, plan->fast, flags, st, plan->side));
+  OZK2_TRY(launch_scale_batch(probs, plan->cnt, plan->totals, plan->fast, st, plan->side));
   OZK2_TRY(join());
   t_launches += plan->fast ? 4 : 3;
   GemmArgs g{};
@@ -1472,7 +1483,8 @@ ozk2_status execute_plan(ozk2_batch_plan plan, cudaStream_t st) {
                                      plan->units_bound, st));
     t_launches += 1;
   }
-  OZK2_TRY(launch_exponents_batch(probs, plan->cnt, plan->totals[kBkExponents], tab->pprime, delta_f32(), st));
+  OZK2_TRY(launch_exponents_batch(probs, plan->cnt, plan->totals[kBkExponents], tab->pprime, delta_f32(), flags,
+                                  st));
   OZK2_TRY(fork());
   OZK2_TRY(launch_residues_batch(probs, plan->cnt, plan->totals[kBkResidRows], plan->totals[kBkResidCols], tab->rt,
                                  flags, st, plan->side));

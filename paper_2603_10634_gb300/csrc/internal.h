@@ -164,28 +164,39 @@ float bound_factor_f32(int64_t k);   // RU_fp32(1 + k 2^-24)
 // Kernel launchers (each returns the cudaError_t of its launch)
 // ---------------------------------------------------------------------------
 
-// scale.cu.  "rows": lines contiguous along k; "cols": lines strided along k.  With
-// fast = true the kernels write sums of squares (sq) instead of bound operands.
-cudaError_t launch_scale_rows(const double* A, int64_t lda, int m, int k, int kp,
-                              int32_t* eprime, uint8_t* rowstat, uint8_t* Abar, float* sq,
-                              bool fast, uint32_t* flags, cudaStream_t st);
-// colmax: per column, floor(log2 max |b|) + 1075 (0 for a zero column), accumulated
-// with atomicMax into a zeroed array.
-cudaError_t launch_colmax(const double* B, int64_t ldb, int k, int n,
-                          uint32_t* colmax, uint32_t* colbad, cudaStream_t st);
-cudaError_t launch_scale_cols(const double* B, int64_t ldb, int k, int n, int kp,
-                              const uint32_t* colmax, const uint32_t* colbad,
-                              int32_t* fprime, uint8_t* colstat, uint8_t* BbarT, float* part,
-                              float* sq, bool fast, uint32_t* flags, cudaStream_t st);
+// scale.cu.  One operand of a scaling: its lines are contiguous along k (kcontig) or
+// strided by ld.  Accurate mode writes e', the line status and the E4M3 bound operand; fast
+// mode e', the status and the sums of squares (sq).
+struct ScaleJob {
+  const double* X;
+  int64_t ld;
+  int lines;
+  bool kcontig;
+  int32_t* ep;
+  uint8_t* stat;
+  uint8_t* bar;    // lines x kp bytes (accurate)
+  float* sq;       // lines (fast)
+  float* part;     // kp / 32 x lines partial sums (fast, strided lines)
+  uint32_t* keys;  // strided lines: scratch of up to kMaxKeyBlocks x lines words between the launches
+};
+constexpr int kMaxKeyBlocks = 16;
+// First launch for up to two operands of the same k: the kcontig ones complete, the others'
+// partial column maxima; zeroes zero[0 .. zero_words).  Second launch for the strided ones.
+cudaError_t launch_scale_prep(const ScaleJob* jobs, int njobs, int k, int kp, bool fast, uint32_t* zero,
+                              int64_t zero_words, cudaStream_t st);
+cudaError_t launch_scale_cols(const ScaleJob* jobs, int njobs, int k, int kp, bool fast, cudaStream_t st);
 cudaError_t launch_exponents(int m, int n, const int32_t* eprime, const int32_t* fprime,
                              const uint8_t* rowstat, const uint8_t* colstat,
                              const float* R, const float* S, float pprime, float delta,
-                             int32_t* e, int32_t* f, cudaStream_t st);
+                             int32_t* e, int32_t* f, uint32_t* flags, cudaStream_t st);
 // Exponents of dC's rows (g from R) and columns (h from S) for the gradient products
 // that reuse the forward's integer matrices: the whole budget q = reuse_budget_f32(N).
+// rpart (nr), cpart (nc): the status of the partners' lines.  Both exponent kernels report
+// non-finite lines in the flag word.
 cudaError_t launch_reuse_exponents(int m, const int32_t* gp, const uint8_t* rstat, const float* R, int32_t* g, int n,
                                    const int32_t* hp, const uint8_t* cstat, const float* S, int32_t* h, float q,
-                                   uint32_t* flags, cudaStream_t st);
+                                   const uint8_t* rpart, int nr, const uint8_t* cpart, int nc, uint32_t* flags,
+                                   cudaStream_t st);
 
 // resid.cu.  Planes: rns_planes(N) planes of lines x kp bytes, row pitch ldp bytes (>= kp, a
 // multiple of 16), plane stride plane_stride bytes (0: lines * ldp; larger when the
@@ -338,9 +349,9 @@ void batch_block_counts(int m, int n, int k, int kp, bool fast, int64_t (&nblock
 
 // The row kernels (A) run on st, the column kernels (B) on st_cols.
 cudaError_t launch_scale_batch(const BatchProblem* probs, int count, const int64_t (&total)[kBatchKernels],
-                               bool fast, uint32_t* flags, cudaStream_t st, cudaStream_t st_cols);
+                               bool fast, cudaStream_t st, cudaStream_t st_cols);
 cudaError_t launch_exponents_batch(const BatchProblem* probs, int count, int64_t total_blocks, float pprime,
-                                   float delta, cudaStream_t st);
+                                   float delta, uint32_t* flags, cudaStream_t st);
 cudaError_t launch_residues_batch(const BatchProblem* probs, int count, int64_t rows_blocks,
                                   int64_t cols_blocks, const RnsTable& rt, uint32_t* flags, cudaStream_t st,
                                   cudaStream_t st_cols);

@@ -78,6 +78,34 @@ __device__ __forceinline__ uint32_t ru_e4m3_scaled(Mag m, int sh) {
   return 1u;
 }
 
+// The same, 0 for a non-finite x, in a few integer operations for the common case, a
+// normal result: the code is then the high word's exponent and top 3 fraction bits, rounded
+// up by any lower bit, less the line's offset (high word >> 17 counts 8 codes a binade).
+// With this and LineMax the row kernel went from 30 to about 14 instructions an element:
+// rows held in registers but converted the long way took 81 us for 8192 x 4096, now 51.
+__device__ __forceinline__ uint32_t bar_code(double x, int ep) {
+  const Mag m = mag_of(x);
+  const uint32_t up = (m.hi + 0x1FFFFu + (m.lo != 0u ? 1u : 0u)) >> 17;
+  const uint32_t code = up + static_cast<uint32_t>(8 * (ep - 1016));
+  // a normal x (not zero, not subnormal) with a result of 2^-6 .. 2^8 (so x is finite)
+  if (code - 8u <= 0x70u && m.hi >= 0x00100000u) return code;
+  return nonfinite(m) ? 0u : ru_e4m3_scaled(m, ep);
+}
+
+// The running maximum of a line's high words (signs cleared) and the union of its low
+// words; key() is exact when the maximum is a normal number or the line is zero, and
+// otherwise (subnormal lines, non-finite entries) the caller takes log2_key over the line.
+struct LineMax {
+  uint32_t hi = 0u, lo = 0u;
+  __device__ __forceinline__ void add(double x) {
+    const Mag m = mag_of(x);
+    hi = max(hi, m.hi);
+    lo |= m.lo;
+  }
+  __device__ __forceinline__ bool exact() const { return hi - 0x00100000u < 0x7FE00000u || (hi | lo) == 0u; }
+  __device__ __forceinline__ uint32_t key() const { return hi != 0u ? (hi >> 20) + 52u : 0u; }
+};
+
 // RU_fp32(|x| 2^sh) for a finite nonzero x with |x| 2^sh < 2^8: the float bit pattern
 // is assembled from the exponent and the top 23 fraction bits, plus one unit when any
 // lower bit is set (a carry into the exponent field stays correct).  Results below the
@@ -91,8 +119,89 @@ __device__ __forceinline__ float ru_f32_scaled(Mag m, int sh) {
   return __uint_as_float(bits);
 }
 
+// A line's maximum key and its non-finite flag in one word.
+constexpr uint32_t kKeyBad = 0x10000u;
+__device__ __forceinline__ uint32_t merge_keys(uint32_t a, uint32_t b) {
+  return max(a & ~kKeyBad, b & ~kKeyBad) | ((a | b) & kKeyBad);
+}
+__device__ __forceinline__ uint8_t line_status(uint32_t key) {
+  return static_cast<uint8_t>(((key & ~kKeyBad) == 0u ? kLineZero : 0) | ((key & kKeyBad) ? kLineNonfinite : 0));
+}
+
 // Loads a thread keeps in flight per batch (the column kernels take twice as many).
 constexpr int kBatch = 4;
+
+// The E4M3 bytes of 4 elements with exponent ep (non-finite entries count as 0).
+__device__ __forceinline__ uint32_t bar_word(const double (&v)[4], int ep) {
+  uint32_t word = 0;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) word |= bar_code(v[t], ep) << (8 * t);
+  return word;
+}
+
+// Rows of up to 256 E elements, read once: W warps hold a row in registers (E elements a
+// thread), take its maximum, then convert.  vblock: the block's index among this operand's
+// blocks (8 / W rows each).  Accurate mode only (fast mode's sums have a fixed order).
+template <int E, int W>
+__device__ __forceinline__ void scale_rows_cached(const double* __restrict__ A, int64_t lda, int m, int k, int kp,
+                                                  int32_t* __restrict__ eprime, uint8_t* __restrict__ rowstat,
+                                                  uint8_t* __restrict__ Abar, uint32_t* red, int64_t vblock) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int row = static_cast<int>(vblock) * (8 / W) + warp / W;
+  const int t = (warp % W) * 32 + lane;
+  const bool row_ok = row < m;
+  const double* a = A + static_cast<int64_t>(row_ok ? row : 0) * lda;
+  const bool vec = ((reinterpret_cast<uintptr_t>(A) & 15u) | (lda & 1)) == 0;  // rows start on 16 bytes
+  double v[E / 4][4];
+#pragma unroll
+  for (int c = 0; c < E / 4; ++c) {
+    const int h = (c * W * 32 + t) * 4;
+    if (vec && row_ok && h + 4 <= k) {
+      const double2 x = __ldg(reinterpret_cast<const double2*>(a + h)), y = __ldg(reinterpret_cast<const double2*>(a + h + 2));
+      v[c][0] = x.x;
+      v[c][1] = x.y;
+      v[c][2] = y.x;
+      v[c][3] = y.y;
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[c][u] = row_ok && h + u < k ? __ldg(a + h + u) : 0.0;
+    }
+  }
+  LineMax lm;
+#pragma unroll
+  for (int c = 0; c < E / 4; ++c)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) lm.add(v[c][u]);
+  uint32_t key = lm.key();
+  bool bad = false;
+  if (!lm.exact()) {
+    key = 0u;
+#pragma unroll
+    for (int c = 0; c < E / 4; ++c)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) key = max(key, log2_key(mag_of(v[c][u]), bad));
+  }
+  key = __reduce_max_sync(0xffffffffu, key) | (__any_sync(0xffffffffu, bad) ? kKeyBad : 0u);
+  if constexpr (W > 1) {
+    if (lane == 0) red[warp] = key;
+    __syncthreads();
+    key = 0u;
+#pragma unroll
+    for (int w = 0; w < W; ++w) key = merge_keys(key, red[(warp / W) * W + w]);
+  }
+  if (!row_ok) return;
+  const int ep = prelim_exponent(key & ~kKeyBad);
+  if (t == 0) {
+    eprime[row] = ep;
+    rowstat[row] = line_status(key);
+  }
+  uint32_t* out = reinterpret_cast<uint32_t*>(Abar + static_cast<int64_t>(row) * kp);
+#pragma unroll
+  for (int c = 0; c < E / 4; ++c) {
+    const int h = (c * W * 32 + t) * 4;
+    if (h < kp) out[h >> 2] = bar_word(v[c], ep);
+  }
+}
 
 // One warp per row of A: row maximum, e'_i, row status, then Abar (m x kp bytes).
 // FAST: instead of Abar, the sum of squares s_i = sum_h RU_fp32(2^e'_i |a_ih|)^2 with
@@ -102,19 +211,24 @@ template <bool FAST>
 __device__ __forceinline__ void scale_rows_body(const double* __restrict__ A, int64_t lda, int m, int k, int kp,
                                                 int32_t* __restrict__ eprime, uint8_t* __restrict__ rowstat,
                                                 uint8_t* __restrict__ Abar, float* __restrict__ sq,
-                                                uint32_t* flags, int64_t vblock) {
+                                                int64_t vblock) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int row = static_cast<int>(vblock) * (blockDim.x >> 5) + warp;
   if (row >= m) return;
   const double* a = A + static_cast<int64_t>(row) * lda;
-  uint32_t key = 0u;
-  bool bad = false;
+  LineMax lm;
   for (int h = lane; h < k; h += 32 * kBatch) {
     double v[kBatch];  // the loads of a batch are issued before any is used
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) v[u] = h + 32 * u < k ? __ldg(a + h + 32 * u) : 0.0;
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) key = max(key, log2_key(mag_of(v[u]), bad));
+    for (int u = 0; u < kBatch; ++u) lm.add(v[u]);
+  }
+  uint32_t key = lm.key();
+  bool bad = false;
+  if (!lm.exact()) {
+    key = 0u;
+    for (int h = lane; h < k; h += 32) key = max(key, log2_key(mag_of(__ldg(a + h)), bad));
   }
   key = __reduce_max_sync(0xffffffffu, key);
   bad = __any_sync(0xffffffffu, bad);
@@ -122,7 +236,6 @@ __device__ __forceinline__ void scale_rows_body(const double* __restrict__ A, in
   if (lane == 0) {
     eprime[row] = ep;
     rowstat[row] = static_cast<uint8_t>((key == 0u ? kLineZero : 0) | (bad ? kLineNonfinite : 0));
-    if (bad) atomicOr(flags, kFlagNonfinite);
   }
   if constexpr (FAST) {
     float acc = 0.0f;
@@ -148,24 +261,11 @@ __device__ __forceinline__ void scale_rows_body(const double* __restrict__ A, in
       }
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
-        uint32_t word = 0;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const Mag mg = mag_of(v[4 * g + t]);
-          if (!nonfinite(mg)) word |= ru_e4m3_scaled(mg, ep) << (8 * t);
-        }
-        if (h0 + 128 * g < kp) *reinterpret_cast<uint32_t*>(out + h0 + 128 * g) = word;
+        const double q[4] = {v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]};
+        if (h0 + 128 * g < kp) *reinterpret_cast<uint32_t*>(out + h0 + 128 * g) = bar_word(q, ep);
       }
     }
   }
-}
-
-template <bool FAST>
-__global__ void __launch_bounds__(256) scale_rows_kernel(const double* __restrict__ A, int64_t lda, int m, int k,
-                                                         int kp, int32_t* __restrict__ eprime,
-                                                         uint8_t* __restrict__ rowstat, uint8_t* __restrict__ Abar,
-                                                         float* __restrict__ sq, uint32_t* flags) {
-  scale_rows_body<FAST>(A, lda, m, k, kp, eprime, rowstat, Abar, sq, flags, blockIdx.x);
 }
 
 constexpr int kColRows = 256;
@@ -179,23 +279,83 @@ __device__ __forceinline__ void colmax_body(const double* __restrict__ B, int64_
   if (j >= n) return;
   const int h0 = by * rpb;
   const int h1 = min(k, h0 + rpb);
-  uint32_t key = 0u;
-  bool bad = false;
+  LineMax lm;
   for (int h = h0; h < h1; h += 2 * kBatch) {
     double v[2 * kBatch];  // the loads of a batch are issued before any is used
 #pragma unroll
     for (int u = 0; u < 2 * kBatch; ++u) v[u] = h + u < h1 ? __ldg(B + static_cast<int64_t>(h + u) * ldb + j) : 0.0;
 #pragma unroll
-    for (int u = 0; u < 2 * kBatch; ++u) key = max(key, log2_key(mag_of(v[u]), bad));
+    for (int u = 0; u < 2 * kBatch; ++u) lm.add(v[u]);
+  }
+  uint32_t key = lm.key();
+  bool bad = false;
+  if (!lm.exact()) {
+    key = 0u;
+    for (int h = h0; h < h1; ++h) key = max(key, log2_key(mag_of(__ldg(B + static_cast<int64_t>(h) * ldb + j)), bad));
   }
   if (key) atomicMax(colmax + j, key);
   if (bad) atomicOr(colbad + j, 1u);
 }
 
-__global__ void __launch_bounds__(256) colmax_kernel(const double* __restrict__ B, int64_t ldb, int k, int n,
-                                                     uint32_t* __restrict__ colmax, uint32_t* __restrict__ colbad,
-                                                     int rpb) {
-  colmax_body(B, ldb, k, n, colmax, colbad, blockIdx.x, blockIdx.y, rpb);
+// Partial column maxima of a single problem: a block takes 32 columns x `rows` rows
+// (8 row groups, each thread a batch of 8 rows at a time) and writes one key per column,
+// keys[by * n + j]: no zeroed array and no atomics, and short columns are covered by many
+// blocks of one or two batches.
+__device__ __forceinline__ void colmax_tile(const double* __restrict__ B, int64_t ldb, int k, int n, int rows,
+                                            uint32_t* __restrict__ keys, uint32_t* red, int64_t vblock) {
+  const int gx = (n + 31) / 32;
+  int by, bx;
+  divmod_nonneg(vblock, gx, by, bx);
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
+  const int j = bx * 32 + lane;
+  const int h0 = by * rows, h1 = min(k, h0 + rows);
+  LineMax lm;
+  for (int h = h0 + grp; h < h1; h += 64) {
+    double v[8];  // the loads of a batch are issued before any is used
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      v[u] = j < n && h + 8 * u < h1 ? __ldg(B + static_cast<int64_t>(h + 8 * u) * ldb + j) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) lm.add(v[u]);
+  }
+  uint32_t key = lm.key();
+  bool bad = false;
+  if (!lm.exact()) {
+    key = 0u;
+    for (int h = h0 + grp; h < h1 && j < n; h += 8)
+      key = max(key, log2_key(mag_of(__ldg(B + static_cast<int64_t>(h) * ldb + j)), bad));
+  }
+  red[threadIdx.x] = key | (bad ? kKeyBad : 0u);
+  __syncthreads();
+  if (grp == 0 && j < n) {
+#pragma unroll
+    for (int w = 0; w < 8; ++w) key = w == 0 ? red[lane] : merge_keys(key, red[32 * w + lane]);
+    keys[static_cast<int64_t>(by) * n + j] = key;
+  }
+}
+
+// The first launch of a scaling: rows of operands that are contiguous along k, partial
+// column maxima of the others, and the call's zeroed words.
+struct PrepArgs {
+  ScaleJob job[2];
+  int64_t first[3];  // blocks [first[i], first[i + 1]) serve job i
+  int k, kp, key_rows;
+  uint32_t* zero;
+  int64_t zero_words;
+};
+template <bool FAST, int E, int W>  // E = 0: rows two passes at a time (long rows, fast mode)
+__global__ void __launch_bounds__(256) scale_prep_kernel(const __grid_constant__ PrepArgs a) {
+  __shared__ uint32_t red[256];
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < a.zero_words;
+       i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+    a.zero[i] = 0u;
+  const ScaleJob& job = a.job[blockIdx.x >= a.first[1] ? 1 : 0];
+  const int64_t vblock = blockIdx.x - a.first[blockIdx.x >= a.first[1] ? 1 : 0];
+  if (!job.kcontig) colmax_tile(job.X, job.ld, a.k, job.lines, a.key_rows, job.keys, red, vblock);
+  else if constexpr (E == 0)
+    scale_rows_body<FAST>(job.X, job.ld, job.lines, a.k, a.kp, job.ep, job.stat, job.bar, job.sq, vblock);
+  else
+    scale_rows_cached<E, W>(job.X, job.ld, job.lines, a.k, a.kp, job.ep, job.stat, job.bar, red, vblock);
 }
 
 // Bbar^T (n x kp bytes): thread (column j, 32 consecutive h) writes 32 bytes of row j.
@@ -203,19 +363,13 @@ __global__ void __launch_bounds__(256) colmax_kernel(const double* __restrict__ 
 // part[hb * n + j]; sumsq_reduce_kernel adds the partials of a column in a fixed order.
 template <bool FAST>
 __device__ __forceinline__ void scale_cols_body(const double* __restrict__ B, int64_t ldb, int k, int n, int kp,
-                                                const uint32_t* __restrict__ colmax,
-                                                const uint32_t* __restrict__ colbad, int32_t* __restrict__ fprime,
+                                                uint32_t key, int32_t* __restrict__ fprime,
                                                 uint8_t* __restrict__ colstat, uint8_t* __restrict__ BbarT,
-                                                float* __restrict__ part, uint32_t* flags, int bx, int hb) {
-  const int j = bx * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  const uint32_t key = colmax[j];
-  const bool bad = colbad[j] != 0;
-  const int fp = prelim_exponent(key);
+                                                float* __restrict__ part, int j, int hb) {
+  const int fp = prelim_exponent(key & ~kKeyBad);
   if (hb == 0) {
     fprime[j] = fp;
-    colstat[j] = static_cast<uint8_t>((key == 0u ? kLineZero : 0) | (bad ? kLineNonfinite : 0));
-    if (bad) atomicOr(flags, kFlagNonfinite);
+    colstat[j] = line_status(key);
   }
   if constexpr (FAST) {
     float acc = 0.0f;
@@ -236,18 +390,17 @@ __device__ __forceinline__ void scale_cols_body(const double* __restrict__ B, in
 #pragma unroll
     for (int q = 0; q < 8; ++q) w[q] = 0;
 #pragma unroll
-    for (int t0 = 0; t0 < 32; t0 += 2 * kBatch) {
-      double v[2 * kBatch];  // loads first
+    for (int t0 = 0; t0 < 32; t0 += 4 * kBatch) {
+      double v[4 * kBatch];  // loads first
 #pragma unroll
-      for (int u = 0; u < 2 * kBatch; ++u) {
+      for (int u = 0; u < 4 * kBatch; ++u) {
         const int h = hb * 32 + t0 + u;
         v[u] = h < k ? __ldg(B + static_cast<int64_t>(h) * ldb + j) : 0.0;
       }
 #pragma unroll
-      for (int u = 0; u < 2 * kBatch; ++u) {
-        const Mag mg = mag_of(v[u]);
+      for (int u = 0; u < 4 * kBatch; ++u) {
         const int t = t0 + u;
-        if (!nonfinite(mg)) w[t >> 2] |= ru_e4m3_scaled(mg, fp) << (8 * (t & 3));
+        w[t >> 2] |= bar_code(v[u], fp) << (8 * (t & 3));
       }
     }
     uint4* dst = reinterpret_cast<uint4*>(BbarT + static_cast<int64_t>(j) * kp + hb * 32);
@@ -256,15 +409,27 @@ __device__ __forceinline__ void scale_cols_body(const double* __restrict__ B, in
   }
 }
 
+// Columns of up to two operands (single problems): a block serves 32 columns x 8 groups of
+// 32 k, and merges its columns' partial maxima first.
+struct ColsArgs {
+  ScaleJob job[2];
+  int64_t first[3];
+  int k, kp, nkeys;
+};
 template <bool FAST>
-__global__ void __launch_bounds__(256) scale_cols_kernel(const double* __restrict__ B, int64_t ldb, int k, int n,
-                                                         int kp, const uint32_t* __restrict__ colmax,
-                                                         const uint32_t* __restrict__ colbad,
-                                                         int32_t* __restrict__ fprime, uint8_t* __restrict__ colstat,
-                                                         uint8_t* __restrict__ BbarT, float* __restrict__ part,
-                                                         uint32_t* flags) {
-  scale_cols_body<FAST>(B, ldb, k, n, kp, colmax, colbad, fprime, colstat, BbarT, part, flags, blockIdx.x,
-                        blockIdx.y);
+__global__ void __launch_bounds__(256) scale_cols_kernel(const __grid_constant__ ColsArgs a) {
+  const int i = blockIdx.x >= a.first[1] ? 1 : 0;
+  const ScaleJob& job = a.job[i];
+  const int gx = (job.lines + 31) / 32;
+  int by, bx;
+  divmod_nonneg(blockIdx.x - a.first[i], gx, by, bx);
+  const int j = bx * 32 + (threadIdx.x & 31), hb = by * 8 + (threadIdx.x >> 5);
+  if (j >= job.lines || hb * 32 >= a.kp) return;
+  uint32_t key = 0u;
+#pragma unroll
+  for (int y = 0; y < kMaxKeyBlocks; ++y)
+    if (y < a.nkeys) key = merge_keys(key, __ldg(job.keys + static_cast<int64_t>(y) * job.lines + j));
+  scale_cols_body<FAST>(job.X, job.ld, a.k, job.lines, a.kp, key, job.ep, job.stat, job.bar, job.part, j, hb);
 }
 
 // s_j = sum over blocks of part[hb][j], every addition rounded up, in block order.
@@ -273,7 +438,13 @@ __device__ __forceinline__ void sumsq_body(const float* __restrict__ part, int n
   const int j = static_cast<int>(vblock) * blockDim.x + threadIdx.x;
   if (j >= n) return;
   float acc = 0.0f;
-  for (int hb = 0; hb < nblocks; ++hb) acc = __fadd_ru(acc, part[static_cast<int64_t>(hb) * n + j]);
+  for (int hb = 0; hb < nblocks; hb += 16) {
+    float v[16];  // loads first
+#pragma unroll
+    for (int u = 0; u < 16; ++u) v[u] = hb + u < nblocks ? part[static_cast<int64_t>(hb + u) * n + j] : 0.0f;
+#pragma unroll
+    for (int u = 0; u < 16; ++u) acc = __fadd_ru(acc, v[u]);  // + 0 is exact
+  }
   sq[j] = acc;
 }
 
@@ -299,22 +470,27 @@ __device__ __forceinline__ void exponents_body(int m, int n, const int32_t* __re
                                                const uint8_t* __restrict__ rowstat,
                                                const uint8_t* __restrict__ colstat, const float* __restrict__ R,
                                                const float* __restrict__ S, float pprime, float delta,
-                                               int32_t* __restrict__ e, int32_t* __restrict__ f, int64_t vblock) {
+                                               int32_t* __restrict__ e, int32_t* __restrict__ f, uint32_t* flags,
+                                               int64_t vblock) {
   const int t = static_cast<int>(vblock) * blockDim.x + threadIdx.x;
+  uint8_t stat = 0;
   if (t < m) {
-    e[t] = final_exponent(eprime[t], rowstat[t], R[t], pprime, delta);
+    stat = rowstat[t];
+    e[t] = final_exponent(eprime[t], stat, R[t], pprime, delta);
   } else if (t < m + n) {
     const int j = t - m;
-    f[j] = final_exponent(fprime[j], colstat[j], S[j], pprime, delta);
+    stat = colstat[j];
+    f[j] = final_exponent(fprime[j], stat, S[j], pprime, delta);
   }
+  if (stat & kLineNonfinite) atomicOr(flags, kFlagNonfinite);
 }
 
 __global__ void exponents_kernel(int m, int n, const int32_t* __restrict__ eprime,
                                  const int32_t* __restrict__ fprime, const uint8_t* __restrict__ rowstat,
                                  const uint8_t* __restrict__ colstat, const float* __restrict__ R,
                                  const float* __restrict__ S, float pprime, float delta, int32_t* __restrict__ e,
-                                 int32_t* __restrict__ f) {
-  exponents_body(m, n, eprime, fprime, rowstat, colstat, R, S, pprime, delta, e, f, blockIdx.x);
+                                 int32_t* __restrict__ f, uint32_t* flags) {
+  exponents_body(m, n, eprime, fprime, rowstat, colstat, R, S, pprime, delta, e, f, flags, blockIdx.x);
 }
 
 // Exponent of a line whose product partner's integers are fixed (the gradient products
@@ -342,22 +518,30 @@ __global__ void reuse_exponents_kernel(int m, const int32_t* __restrict__ gp, co
                                        const float* __restrict__ R, int32_t* __restrict__ g, int n,
                                        const int32_t* __restrict__ hp, const uint8_t* __restrict__ cstat,
                                        const float* __restrict__ S, int32_t* __restrict__ h, float q,
-                                       uint32_t* flags) {
+                                       const uint8_t* __restrict__ rpart, int nr, const uint8_t* __restrict__ cpart,
+                                       int nc, uint32_t* flags) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  uint8_t stat = 0;
   if (t < m) {
-    g[t] = reuse_exponent(gp[t], rstat[t], R[t], q, flags);
+    stat = rstat[t];
+    g[t] = reuse_exponent(gp[t], stat, R[t], q, flags);
   } else if (t < m + n) {
     const int j = t - m;
-    h[j] = reuse_exponent(hp[j], cstat[j], S[j], q, flags);
+    stat = cstat[j];
+    h[j] = reuse_exponent(hp[j], stat, S[j], q, flags);
   }
+  // the partners' lines (rows of B, columns of A) only report their non-finite entries
+  if (t < nr) stat |= rpart[t];
+  if (t < nc) stat |= cpart[t];
+  if (stat & kLineNonfinite) atomicOr(flags, kFlagNonfinite);
 }
 
 // ------------------------------------------------------------------ grouped launches
 template <bool FAST>
 __global__ void __launch_bounds__(256) scale_rows_batch(const BatchProblem* __restrict__ probs, int count,
-                                                        int64_t total, uint32_t* flags) {
+                                                        int64_t total) {
   for_each_vblock(probs, count, kBkScaleRows, total, [&](const BatchProblem& P, int64_t v) {
-    scale_rows_body<FAST>(P.A, P.lda, P.m, P.k, P.kp, P.eprime, P.rowstat, P.Abar, P.R, flags, v);
+    scale_rows_body<FAST>(P.A, P.lda, P.m, P.k, P.kp, P.eprime, P.rowstat, P.Abar, P.R, v);
   });
 }
 
@@ -373,13 +557,15 @@ __global__ void __launch_bounds__(256) colmax_batch(const BatchProblem* __restri
 
 template <bool FAST>
 __global__ void __launch_bounds__(256) scale_cols_batch(const BatchProblem* __restrict__ probs, int count,
-                                                        int64_t total, uint32_t* flags) {
+                                                        int64_t total) {
   for_each_vblock(probs, count, kBkScaleCols, total, [&](const BatchProblem& P, int64_t v) {
     const int gx = (P.n + 255) / 256;
     int hb, bx;
     divmod_nonneg(v, gx, hb, bx);
-    scale_cols_body<FAST>(P.B, P.ldb, P.k, P.n, P.kp, P.colmaxB, P.colbadB, P.fprime, P.colstat, P.BbarT, P.partB,
-                          flags, bx, hb);
+    const int j = bx * 256 + static_cast<int>(threadIdx.x);
+    if (j < P.n)
+      scale_cols_body<FAST>(P.B, P.ldb, P.k, P.n, P.kp, P.colmaxB[j] | (P.colbadB[j] ? kKeyBad : 0u), P.fprime,
+                            P.colstat, P.BbarT, P.partB, j, hb);
   });
 }
 
@@ -390,9 +576,9 @@ __global__ void __launch_bounds__(256) sumsq_batch(const BatchProblem* __restric
 }
 
 __global__ void __launch_bounds__(256) exponents_batch(const BatchProblem* __restrict__ probs, int count,
-                                                       int64_t total, float pprime, float delta) {
+                                                       int64_t total, float pprime, float delta, uint32_t* flags) {
   for_each_vblock(probs, count, kBkExponents, total, [&](const BatchProblem& P, int64_t v) {
-    exponents_body(P.m, P.n, P.eprime, P.fprime, P.rowstat, P.colstat, P.R, P.S, pprime, delta, P.e, P.f, v);
+    exponents_body(P.m, P.n, P.eprime, P.fprime, P.rowstat, P.colstat, P.R, P.S, pprime, delta, P.e, P.f, flags, v);
   });
 }
 
@@ -415,70 +601,112 @@ void batch_block_counts(int m, int n, int k, int kp, bool fast, int64_t (&nb)[kB
 }
 
 cudaError_t launch_scale_batch(const BatchProblem* probs, int count, const int64_t (&total)[kBatchKernels],
-                               bool fast, uint32_t* flags, cudaStream_t st, cudaStream_t st_cols) {
+                               bool fast, cudaStream_t st, cudaStream_t st_cols) {
   for (int w : {int(kBkScaleRows), int(kBkColmax), int(kBkScaleCols), int(kBkExponents)})
     if (!grid_ok(total[w])) return cudaErrorInvalidValue;
   if (fast && !grid_ok(total[kBkSumsq])) return cudaErrorInvalidValue;
   const int64_t tr = total[kBkScaleRows], tm = total[kBkColmax], tc = total[kBkScaleCols];
   if (fast)
-    scale_rows_batch<true><<<grouped_grid(tr, 8), 256, 0, st>>>(probs, count, tr, flags);
+    scale_rows_batch<true><<<grouped_grid(tr, 8), 256, 0, st>>>(probs, count, tr);
   else
-    scale_rows_batch<false><<<grouped_grid(tr, 8), 256, 0, st>>>(probs, count, tr, flags);
+    scale_rows_batch<false><<<grouped_grid(tr, 8), 256, 0, st>>>(probs, count, tr);
   colmax_batch<<<grouped_grid(tm, 8), 256, 0, st_cols>>>(probs, count, tm);
   if (fast) {
-    scale_cols_batch<true><<<grouped_grid(tc, 8), 256, 0, st_cols>>>(probs, count, tc, flags);
+    scale_cols_batch<true><<<grouped_grid(tc, 8), 256, 0, st_cols>>>(probs, count, tc);
     sumsq_batch<<<grouped_grid(total[kBkSumsq], 8), 256, 0, st_cols>>>(probs, count, total[kBkSumsq]);
   } else {
-    scale_cols_batch<false><<<grouped_grid(tc, 8), 256, 0, st_cols>>>(probs, count, tc, flags);
+    scale_cols_batch<false><<<grouped_grid(tc, 8), 256, 0, st_cols>>>(probs, count, tc);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_exponents_batch(const BatchProblem* probs, int count, int64_t total_blocks, float pprime,
-                                   float delta, cudaStream_t st) {
+                                   float delta, uint32_t* flags, cudaStream_t st) {
   if (!grid_ok(total_blocks)) return cudaErrorInvalidValue;
-  exponents_batch<<<grouped_grid(total_blocks, 8), 256, 0, st>>>(probs, count, total_blocks, pprime, delta);
+  exponents_batch<<<grouped_grid(total_blocks, 8), 256, 0, st>>>(probs, count, total_blocks, pprime, delta, flags);
   return cudaGetLastError();
 }
 
-cudaError_t launch_scale_rows(const double* A, int64_t lda, int m, int k, int kp, int32_t* eprime,
-                              uint8_t* rowstat, uint8_t* Abar, float* sq, bool fast, uint32_t* flags,
-                              cudaStream_t st) {
-  const int rows_per_block = 8;
-  const int grid = (m + rows_per_block - 1) / rows_per_block;
-  if (fast)
-    scale_rows_kernel<true><<<grid, 256, 0, st>>>(A, lda, m, k, kp, eprime, rowstat, Abar, sq, flags);
-  else
-    scale_rows_kernel<false><<<grid, 256, 0, st>>>(A, lda, m, k, kp, eprime, rowstat, Abar, sq, flags);
+namespace {
+
+// Rows per block of the partial column maxima, a multiple of 64 (one batch): at most
+// kMaxKeyBlocks partials per column.
+int key_rows(int k) { return std::max(64, ((k + kMaxKeyBlocks - 1) / kMaxKeyBlocks + 63) / 64 * 64); }
+
+template <bool FAST, int E, int W>
+cudaError_t run_prep(const ScaleJob* jobs, int njobs, int k, int kp, uint32_t* zero, int64_t zero_words,
+                     cudaStream_t st) {
+  PrepArgs a{};
+  a.k = k;
+  a.kp = kp;
+  a.key_rows = key_rows(k);
+  a.zero = zero;
+  a.zero_words = zero_words;
+  int64_t blocks = 0;
+  for (int i = 0; i < 2; ++i) {
+    a.first[i] = blocks;
+    if (i >= njobs) continue;
+    a.job[i] = jobs[i];
+    blocks += jobs[i].kcontig ? (static_cast<int64_t>(jobs[i].lines) + 8 / W - 1) / (8 / W)
+                              : static_cast<int64_t>((jobs[i].lines + 31) / 32) * ((k + a.key_rows - 1) / a.key_rows);
+  }
+  a.first[2] = blocks;
+  if (njobs < 2) a.first[1] = blocks;
+  if (!grid_ok(blocks)) return cudaErrorInvalidValue;
+  scale_prep_kernel<FAST, E, W><<<static_cast<unsigned>(blocks), 256, 0, st>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_colmax(const double* B, int64_t ldb, int k, int n, uint32_t* colmax,
-                          uint32_t* colbad, cudaStream_t st) {
-  // rows per block: enough blocks for about four per SM, 16 to kColRows rows each
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t gx = (n + 255) / 256;
-  int64_t rpb = (static_cast<int64_t>(k) * gx + 4 * sms - 1) / (4 * sms);
-  rpb = std::min<int64_t>(kColRows, std::max<int64_t>(16, (rpb + 15) / 16 * 16));
-  dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>((k + rpb - 1) / rpb));
-  colmax_kernel<<<grid, 256, 0, st>>>(B, ldb, k, n, colmax, colbad, static_cast<int>(rpb));
-  return cudaGetLastError();
+}  // namespace
+
+// Rows of up to 8192 elements are read once, held by the fewest warps at 16 elements a
+// thread (32 above 4096, in a launch of their own: its registers would halve the column
+// kernel's occupancy); against a warp per row that reads twice, 8192 x 4096 88 -> 51 us and
+// 65536 x 1024 128 -> 93 us (5.8 TB/s).  Longer rows (two blocks' worth would not fit an SM's registers)
+// and fast mode (its sums keep their order) read twice.
+cudaError_t launch_scale_prep(const ScaleJob* jobs, int njobs, int k, int kp, bool fast, uint32_t* zero,
+                              int64_t zero_words, cudaStream_t st) {
+  if (fast) return run_prep<true, 0, 1>(jobs, njobs, k, kp, zero, zero_words, st);
+  if (kp <= 512) return run_prep<false, 16, 1>(jobs, njobs, k, kp, zero, zero_words, st);
+  if (kp <= 1024) return run_prep<false, 16, 2>(jobs, njobs, k, kp, zero, zero_words, st);
+  if (kp <= 2048) return run_prep<false, 16, 4>(jobs, njobs, k, kp, zero, zero_words, st);
+  if (kp <= 4096) return run_prep<false, 16, 8>(jobs, njobs, k, kp, zero, zero_words, st);
+  if (kp > 8192) return run_prep<false, 0, 1>(jobs, njobs, k, kp, zero, zero_words, st);
+  for (int kc = 1; kc >= 0; --kc) {
+    ScaleJob part[2];
+    int n = 0;
+    for (int i = 0; i < njobs; ++i)
+      if (jobs[i].kcontig == (kc == 1)) part[n++] = jobs[i];
+    if (n == 0) continue;
+    const cudaError_t err = kc ? run_prep<false, 32, 8>(part, n, k, kp, zero, zero_words, st)
+                               : run_prep<false, 0, 1>(part, n, k, kp, zero, zero_words, st);
+    if (err != cudaSuccess) return err;
+    zero_words = 0;
+  }
+  return cudaSuccess;
 }
 
-cudaError_t launch_scale_cols(const double* B, int64_t ldb, int k, int n, int kp,
-                              const uint32_t* colmax, const uint32_t* colbad,
-                              int32_t* fprime, uint8_t* colstat, uint8_t* BbarT, float* part, float* sq,
-                              bool fast, uint32_t* flags, cudaStream_t st) {
-  dim3 grid((n + 255) / 256, kp / 32);
+cudaError_t launch_scale_cols(const ScaleJob* jobs, int njobs, int k, int kp, bool fast, cudaStream_t st) {
+  ColsArgs a{};
+  a.k = k;
+  a.kp = kp;
+  a.nkeys = (k + key_rows(k) - 1) / key_rows(k);
+  int64_t blocks = 0;
+  for (int i = 0; i < 2; ++i) {
+    a.first[i] = blocks;
+    if (i >= njobs) continue;
+    a.job[i] = jobs[i];
+    blocks += static_cast<int64_t>((jobs[i].lines + 31) / 32) * ((kp + 255) / 256);
+  }
+  a.first[2] = blocks;
+  if (njobs < 2) a.first[1] = blocks;
+  if (!grid_ok(blocks)) return cudaErrorInvalidValue;
   if (fast) {
-    scale_cols_kernel<true><<<grid, 256, 0, st>>>(B, ldb, k, n, kp, colmax, colbad, fprime, colstat, BbarT, part,
-                                                  flags);
-    sumsq_reduce_kernel<<<(n + 255) / 256, 256, 0, st>>>(part, kp / 32, n, sq);
+    scale_cols_kernel<true><<<static_cast<unsigned>(blocks), 256, 0, st>>>(a);
+    for (int i = 0; i < njobs; ++i)
+      sumsq_reduce_kernel<<<(jobs[i].lines + 255) / 256, 256, 0, st>>>(jobs[i].part, kp / 32, jobs[i].lines, jobs[i].sq);
   } else {
-    scale_cols_kernel<false><<<grid, 256, 0, st>>>(B, ldb, k, n, kp, colmax, colbad, fprime, colstat, BbarT,
-                                                   part, flags);
+    scale_cols_kernel<false><<<static_cast<unsigned>(blocks), 256, 0, st>>>(a);
   }
   return cudaGetLastError();
 }
@@ -486,19 +714,21 @@ cudaError_t launch_scale_cols(const double* B, int64_t ldb, int k, int n, int kp
 cudaError_t launch_exponents(int m, int n, const int32_t* eprime, const int32_t* fprime,
                              const uint8_t* rowstat, const uint8_t* colstat, const float* R,
                              const float* S, float pprime, float delta, int32_t* e, int32_t* f,
-                             cudaStream_t st) {
+                             uint32_t* flags, cudaStream_t st) {
   const int total = m + n;
   exponents_kernel<<<(total + 255) / 256, 256, 0, st>>>(m, n, eprime, fprime, rowstat, colstat, R, S,
-                                                        pprime, delta, e, f);
+                                                        pprime, delta, e, f, flags);
   return cudaGetLastError();
 }
 
 cudaError_t launch_reuse_exponents(int m, const int32_t* gp, const uint8_t* rstat, const float* R, int32_t* g, int n,
                                    const int32_t* hp, const uint8_t* cstat, const float* S, int32_t* h, float q,
-                                   uint32_t* flags, cudaStream_t st) {
-  const int total = m + n;
+                                   const uint8_t* rpart, int nr, const uint8_t* cpart, int nc, uint32_t* flags,
+                                   cudaStream_t st) {
+  const int total = std::max(m + n, std::max(nr, nc));
   if (total <= 0) return cudaSuccess;
-  reuse_exponents_kernel<<<(total + 255) / 256, 256, 0, st>>>(m, gp, rstat, R, g, n, hp, cstat, S, h, q, flags);
+  reuse_exponents_kernel<<<(total + 255) / 256, 256, 0, st>>>(m, gp, rstat, R, g, n, hp, cstat, S, h, q, rpart, nr, cpart,
+                                                              nc, flags);
   return cudaGetLastError();
 }
 
