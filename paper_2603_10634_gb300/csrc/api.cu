@@ -458,24 +458,27 @@ ozk2_status phase_scales(Ctx& c, const Operand& a, const Operand& b, bool clear_
   return bound_and_exponents(c);
 }
 
-// plane_stride: bytes between the planes (0: lines * pitch; the whole operand's when
-// `op`, `ex` and `planes` point at a slice of its lines).
-cudaError_t residues_operand(Ctx& c, const Operand& op, int lines, const int32_t* ex, uint8_t* planes,
-                             int64_t plane_stride = 0) {
-  if (op.kcontig)
-    return launch_residues_rows(op.ptr, op.ld, lines, c.k, int(c.L.kp), c.L.ldp, ex, c.tab->rt, planes,
-                                c.at<uint32_t>(c.L.flags), c.st, plane_stride);
-  return launch_residues_cols(op.ptr, op.ld, c.k, lines, int(c.L.kp), c.L.ldp, ex, c.tab->rt, planes,
-                              c.at<uint32_t>(c.L.flags), c.st, plane_stride);
+// Lines [first, first + lines) of an operand (`op` points at line `first`) of `total`
+// lines for the residue kernels; ex, planes: of the whole operand.
+ResidArgs resid_args(const Ctx& c, const Operand& op, int64_t first, int lines, int64_t total, const int32_t* ex,
+                     uint8_t* planes) {
+  return ResidArgs{op.ptr, op.ld, lines, c.k, int(c.L.kp), c.L.ldp, ex + first, planes + first * c.L.ldp,
+                   total * c.L.ldp, c.at<uint32_t>(c.L.flags), op.kcontig};
+}
+ResidArgs resid_a(const Ctx& c, const Operand& a, int64_t first, int lines) {
+  return resid_args(c, a, first, lines, c.m, c.at<int32_t>(c.L.e), c.at<uint8_t>(c.L.planesA));
+}
+ResidArgs resid_b(const Ctx& c, const Operand& b) {
+  return resid_args(c, b, 0, c.n, c.n, c.at<int32_t>(c.L.f), c.at<uint8_t>(c.L.planesB));
 }
 
 // The hybrid list's digit planes of row-major A and B (parity hooks), packed.
 ozk2_status paper_planes(Ctx& c, const double* A, int64_t lda, const double* B, int64_t ldb, const int32_t* e,
                          const int32_t* f, uint8_t* planesA, uint8_t* planesB) {
-  uint32_t* flags = c.at<uint32_t>(c.L.flags);
-  OZK2_TRY(launch_paper_planes_rows(A, lda, c.m, c.k, int(c.L.kp), e, c.tab->mt, planesA, flags, c.st));
-  OZK2_TRY(launch_paper_planes_cols(B, ldb, c.k, c.n, int(c.L.kp), f, c.tab->mt, planesB, flags, c.st));
-  t_launches += 2;
+  const ResidArgs ops[2] = {resid_args(c, operand_a(OZK2_OP_N, A, lda), 0, c.m, c.m, e, planesA),
+                            resid_args(c, operand_b(OZK2_OP_N, B, ldb), 0, c.n, c.n, f, planesB)};
+  OZK2_TRY(launch_paper_planes(ops, c.tab->mt, c.st));
+  t_launches += 1;
   return OZK2_OK;
 }
 
@@ -617,22 +620,17 @@ int row_blocks(const Ctx& c, int64_t (&first)[kMaxRowBlocks + 1]) {
   return count;
 }
 
-// After the scaling, the exponents and B's residues (all on c.st): A's residues (unless
-// `a` is null: already converted), the residue products and the CRT, in order on c.st.
-// C (device, row-major, ldc) receives the result.  With cb the products and the CRT run
+// After the scaling, the exponents and the residues (all on c.st): the residue products
+// and the CRT, in order on c.st.  C (device, row-major, ldc) receives the result.  With cb the products and the CRT run
 // in output row blocks, and block b is copied to cb->hC on cb->cs while block b + 1 is
 // computed.  (Running the conversion kernels on a second stream beside the persistent
 // GEMM was measured and gains nothing: they get too little of an SM next to it.)
-ozk2_status products_and_crt(Ctx& c, const Operand* a, double* C, int64_t ldc, const CopyBack* cb) {
+ozk2_status products_and_crt(Ctx& c, double* C, int64_t ldc, const CopyBack* cb) {
   const Layout& L = c.L;
   const int32_t* e = c.at<int32_t>(L.e);
   const int32_t* f = c.at<int32_t>(L.f);
   const uint8_t* rs = c.at<uint8_t>(L.rowstat);
   const uint8_t* cs = c.at<uint8_t>(L.colstat);
-  if (a) {
-    OZK2_TRY(residues_operand(c, *a, c.m, e, c.at<uint8_t>(L.planesA)));
-    t_launches += 1;
-  }
   mark(c, 4);
   ozk2_status s;
   if (!cb) {
@@ -662,11 +660,11 @@ ozk2_status run_one(const Operand& a, const Operand& b, int64_t m, int64_t n, in
   ozk2_status s = setup(c, m, n, k, N, fast, ws, ws_bytes, st, 0, ws_trusted);
   if (s != OZK2_OK) return s;
   mark(c, 0);
-  const Layout& L = c.L;
   if ((s = phase_scales(c, a, b, first)) != OZK2_OK) return s;
-  OZK2_TRY(residues_operand(c, b, c.n, c.at<int32_t>(L.f), c.at<uint8_t>(L.planesB)));
+  const ResidArgs ops[2] = {resid_a(c, a, 0, c.m), resid_b(c, b)};
+  OZK2_TRY(launch_residues(ops, 2, c.tab->rt, c.st));
   t_launches += 1;
-  return products_and_crt(c, &a, C, ldc, nullptr);
+  return products_and_crt(c, C, ldc, nullptr);
 }
 
 int64_t block_or_all(int64_t b, int64_t total) { return (b <= 0 || b >= total) ? total : b; }
@@ -841,12 +839,12 @@ ozk2_status run_host(ozk2_op transa, ozk2_op transb, int64_t m, int64_t n, int64
   // bound), so B's residues need not wait for A
   auto residues_b = [&]() -> ozk2_status {
     OZK2_TRY(exponents_of(c, 0, 0, true));
-    OZK2_TRY(residues_operand(c, b, int(n), c.at<int32_t>(L.f), c.at<uint8_t>(L.planesB)));
+    const ResidArgs op = resid_b(c, b);
+    OZK2_TRY(launch_residues(&op, 1, c.tab->rt, st));
     t_launches += 1;
     return OZK2_OK;
   };
   if (fast && (s = residues_b()) != OZK2_OK) return s;
-  const int64_t planes_a_stride = int64_t(m) * L.ldp;
   for (int q = 0; q < kHostChunks; ++q) {
     const int64_t i0 = std::min(m, q * chunk), i1 = std::min(m, (q + 1) * chunk);
     const bool last = q == kHostChunks - 1;
@@ -860,8 +858,8 @@ ozk2_status run_host(ozk2_op transa, ozk2_op transb, int64_t m, int64_t n, int64
       if (!fast) OZK2_TRY(bound_rows(c, i0, rows));
       if (last) mark(c, 2);
       OZK2_TRY(exponents_of(c, i0, rows, false));
-      OZK2_TRY(residues_operand(c, ai, rows, c.at<int32_t>(L.e) + i0, c.at<uint8_t>(L.planesA) + i0 * L.ldp,
-                                planes_a_stride));
+      const ResidArgs op = resid_a(c, ai, i0, rows);
+      OZK2_TRY(launch_residues(&op, 1, c.tab->rt, st));
       t_launches += 1;
     } else if (last) {
       mark(c, 1);
@@ -877,7 +875,7 @@ ozk2_status run_host(ozk2_op transa, ozk2_op transb, int64_t m, int64_t n, int64
   ce->staged_bytes = G.total;
   // residue products and CRT in output row blocks; each finished block streams back
   const CopyBack cb{hC, ldc, ce->down, ev_blk};
-  if ((s = products_and_crt(c, nullptr, dC, n, &cb)) != OZK2_OK) return s;
+  if ((s = products_and_crt(c, dC, n, &cb)) != OZK2_OK) return s;
   mark(c, 5);
   // the call is complete on `st` once the last block is back on the host
   OZK2_TRY(cudaEventRecord(ev_done, ce->down));

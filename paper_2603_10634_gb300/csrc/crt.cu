@@ -334,6 +334,8 @@ __global__ void __launch_bounds__(256, 2)
                    int m, int n, const int32_t* __restrict__ e, const int32_t* __restrict__ f,
                    const uint8_t* __restrict__ rowstat, const uint8_t* __restrict__ colstat, double* __restrict__ C,
                    int64_t ldc, const __grid_constant__ RnsCrt ct) {
+  chain_wait();
+  chain_next();
   rns_crt_body<N>(cres, cres8, ldr, rstride, m, n, e, f, rowstat, colstat, C, ldc, ct, blockIdx.x, gridDim.x);
 }
 
@@ -353,6 +355,7 @@ __global__ void __launch_bounds__(256)
     paper_crt_kernel(const int16_t* __restrict__ cres, int64_t ldr, int64_t rstride, int m, int n,
                      const int32_t* __restrict__ e, const int32_t* __restrict__ f, double* __restrict__ C, int64_t ldc,
                      const __grid_constant__ CrtTable ct) {
+  chain_wait();
   const int64_t total = static_cast<int64_t>(m) * n;
   for (int64_t x = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; x < total;
        x += static_cast<int64_t>(gridDim.x) * blockDim.x) {
@@ -400,8 +403,7 @@ cudaError_t launch_N(const int16_t* cres, const int8_t* cres8, int64_t ldr, int6
                      const int32_t* f, const uint8_t* rowstat, const uint8_t* colstat, double* C, int64_t ldc,
                      const RnsCrt& ct, cudaStream_t st) {
   const int grid = crt_grid(static_cast<int64_t>(m) * ((n + crt_cols(N) - 1) / crt_cols(N)));
-  rns_crt_kernel<N><<<grid, 256, 0, st>>>(cres, cres8, ldr, rs, m, n, e, f, rowstat, colstat, C, ldc, ct);
-  return cudaGetLastError();
+  return launch_chained(rns_crt_kernel<N>, grid, 256, 0, st, cres, cres8, ldr, rs, m, n, e, f, rowstat, colstat, C, ldc, ct);
 }
 
 template <int N>

@@ -40,6 +40,16 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
+// ---------------------------------------------------------------- chained launches
+// The kernels of a call are launched with programmatic stream serialisation
+// (launch_chained): a kernel may start once every block of the one before has called
+// chain_next, runs its prologue, and then waits in chain_wait until that kernel is complete
+// and its writes visible.  Every kernel calls chain_wait before it touches global memory
+// that an earlier kernel may read or write, so completion is transitive.  Without the
+// launch attribute both are no-ops.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count)

@@ -517,6 +517,8 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
   if constexpr (PAIR) cluster_sync();  // both CTAs' barriers are ready
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  chain_wait();
+  chain_next();
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
@@ -885,12 +887,14 @@ cudaError_t launch_mode(const GemmParams& prm, const CUtensorMap& ta, const CUte
   cfg.blockDim = dim3(Epi<GROUPED>::kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = PAIR ? 2 : 1;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = PAIR ? 1 : 0;
+  cudaLaunchAttribute at[2]{};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_chained
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 2;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = GROUPED ? nullptr : at;
+  cfg.numAttrs = GROUPED ? 0 : (PAIR ? 2 : 1);
   return cudaLaunchKernelEx(&cfg, kernel, ta, tb, prm, probs, nprobs);
 }
 

@@ -151,18 +151,6 @@ __device__ __forceinline__ uint32_t e4m3x4(f2 lo, f2 hi) {
   return a | (b << 16);
 }
 
-struct ResidArgs {
-  const double* X;
-  int64_t ldx;
-  int lines;  // rows of A or columns of B
-  int k, kp;
-  int64_t ldp;  // row pitch of a plane (bytes)
-  const int32_t* exps;
-  uint8_t* planes;
-  int64_t plane_stride;  // lines * ldp
-  uint32_t* flags;
-};
-
 // The residue kernels' constants in shared memory (the modulus loops index them by a
 // loop counter): per modulus the FP32 pairs and the table of 2^t mod p.
 struct __align__(16) ModConsts {
@@ -771,22 +759,22 @@ __device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, con
   if (range_err) atomicOr(a.flags, kFlagRange);
 }
 
-// Both kernels stage the system's constants behind the column kernel's tile (rows: alone).
+// One or two operands: the first `split` blocks serve a, the rest b.  The constants come
+// first in shared memory, then the column tile (absent when both operands are rows).
 template <class Sys>
-__global__ void __launch_bounds__(256, 3) residues_cols_tiled_kernel(ResidArgs a,
-                                                                    const __grid_constant__ typename Sys::Table mt) {
+__global__ void __launch_bounds__(256, 3) residues_kernel(const __grid_constant__ ResidArgs a,
+                                                         const __grid_constant__ ResidArgs b, int split,
+                                                         const __grid_constant__ typename Sys::Table mt, int tables) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  Sys::load(mt, smem_raw + kTileBytes);
-  residues_cols_tiled_body<Sys>(a, mt, smem_raw + kTileBytes, reinterpret_cast<unsigned long long*>(smem_raw),
-                                blockIdx.x, gridDim.x);
-}
-
-template <class Sys>
-__global__ void __launch_bounds__(256, 3) residues_rows_kernel(ResidArgs a,
-                                                              const __grid_constant__ typename Sys::Table mt) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Sys::load(mt, smem_raw);
-  residues_rows_body<Sys>(a, mt, smem_raw, blockIdx.x, gridDim.x);
+  Sys::load(mt, smem_raw);  // constants only: before the wait
+  // no chain_next: the product kernel's blocks, which fill an SM each, would settle as these
+  // blocks leave and run the products unevenly (65536 x 1024 x 1024 2.57 instead of 2.52 ms)
+  chain_wait();
+  const bool second = static_cast<int>(blockIdx.x) >= split;
+  const ResidArgs& op = second ? b : a;
+  const int64_t v = second ? blockIdx.x - split : blockIdx.x, g = second ? gridDim.x - split : split;
+  if (op.kcontig) residues_rows_body<Sys>(op, mt, smem_raw, v, g);
+  else residues_cols_tiled_body<Sys>(op, mt, smem_raw, reinterpret_cast<unsigned long long*>(smem_raw + tables), v, g);
 }
 
 // Grouped: rows of every A; columns of every B (one virtual block per tile).
@@ -796,7 +784,7 @@ __global__ void __launch_bounds__(256, 2) residues_rows_batch(const BatchProblem
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RnsSys::load(mt, smem_raw);
   for_each_vblock(probs, count, kBkResidRows, total, [&](const BatchProblem& P, int64_t v) {
-    const ResidArgs a{P.A, P.lda, P.m, P.k, P.kp, P.ldp, P.e, P.planesA, static_cast<int64_t>(P.m) * P.ldp, flags};
+    const ResidArgs a{P.A, P.lda, P.m, P.k, P.kp, P.ldp, P.e, P.planesA, static_cast<int64_t>(P.m) * P.ldp, flags, true};
     residues_rows_body<RnsSys>(a, mt, smem_raw, v, P.nblocks[kBkResidRows]);
   });
 }
@@ -807,7 +795,7 @@ __global__ void __launch_bounds__(256, 3) residues_cols_batch(const BatchProblem
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RnsSys::load(mt, smem_raw + kTileBytes);
   for_each_vblock(probs, count, kBkResidCols, total, [&](const BatchProblem& P, int64_t v) {
-    const ResidArgs a{P.B, P.ldb, P.n, P.k, P.kp, P.ldp, P.f, P.planesB, static_cast<int64_t>(P.n) * P.ldp, flags};
+    const ResidArgs a{P.B, P.ldb, P.n, P.k, P.kp, P.ldp, P.f, P.planesB, static_cast<int64_t>(P.n) * P.ldp, flags, false};
     residues_cols_tiled_body<RnsSys>(a, mt, smem_raw + kTileBytes, reinterpret_cast<unsigned long long*>(smem_raw), v,
                                      P.nblocks[kBkResidCols]);
   });
@@ -846,6 +834,8 @@ __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const
   unsigned long long* tile = reinterpret_cast<unsigned long long*>(smem_raw);
   const unsigned char* tb = smem_raw + kTileBytes;
   RnsSys::load(mt, smem_raw + kTileBytes);
+  chain_wait();
+  chain_next();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tiles_n = (a.n + kTileCols - 1) / kTileCols, tiles_m = (a.m + kTileK - 1) / kTileK;
   const int64_t tiles = static_cast<int64_t>(tiles_n) * tiles_m;
@@ -934,6 +924,8 @@ __global__ void __launch_bounds__(256) transpose_planes_kernel(const uint8_t* __
                                                                uint8_t* __restrict__ dst, int64_t dst_pitch,
                                                                int64_t dst_stride, int planes) {
   __shared__ uint32_t tile[kTrTile * kTrPitchW];
+  chain_wait();
+  chain_next();
   const int tx = (len + kTrTile - 1) / kTrTile, ty = (lines + kTrTile - 1) / kTrTile;
   const int64_t total = static_cast<int64_t>(tx) * ty * planes;
   const int t = threadIdx.x;
@@ -1009,52 +1001,52 @@ int resident_grid(int64_t blocks, size_t smem) {
   return static_cast<int>(std::max<int64_t>(1, std::min(blocks, cap)));
 }
 
-template <class Sys>
-cudaError_t run_rows(const ResidArgs& a, const typename Sys::Table& t, cudaStream_t st) {
-  const size_t smem = Sys::smem_bytes(t);
-  static std::atomic<int> allowed[64];
-  allow_smem(residues_rows_kernel<Sys>, allowed, smem);
-  const int64_t items = resid_rows_items(a.lines, a.kp);
-  residues_rows_kernel<Sys><<<resident_grid((items + 7) / 8, smem), 256, smem, st>>>(a, t);
-  return cudaGetLastError();
+// Block iterations of an operand: 8 warps' items of 256 elements, or a tile.
+int64_t resid_blocks(const ResidArgs& a) {
+  if (a.kcontig) return (resid_rows_items(a.lines, a.kp) + 7) / 8;
+  return static_cast<int64_t>((a.lines + kTileCols - 1) / kTileCols) * ((a.kp + kTileK - 1) / kTileK);
 }
 
+// Two operands share a launch, its blocks in proportion to their elements, where they fit
+// one wave of blocks (about 900^2 entries each) or are both rows.  Otherwise each gets its
+// own: the row kernel reads through the L1 cache, which the column tile's shared memory
+// would take (8192 x 4096 rows beside 4096 x 100 columns: 268 us in two launches, 297 in
+// one).
 template <class Sys>
-cudaError_t run_cols(const ResidArgs& a, const typename Sys::Table& t, cudaStream_t st) {
-  const size_t smem = kTileBytes + Sys::smem_bytes(t);
+cudaError_t run_residues(const ResidArgs* ops, int nops, const typename Sys::Table& t, cudaStream_t st) {
+  const size_t tables = (Sys::smem_bytes(t) + 15) / 16 * 16;
+  auto need = [&](int n) {
+    bool cols = false;
+    for (int i = 0; i < n; ++i) cols |= !ops[i].kcontig;
+    return tables + (cols ? kTileBytes : 0);
+  };
+  const size_t smem = need(nops);
   static std::atomic<int> allowed[64];
-  allow_smem(residues_cols_tiled_kernel<Sys>, allowed, smem);
-  const int64_t tiles = static_cast<int64_t>((a.lines + kTileCols - 1) / kTileCols) * ((a.kp + kTileK - 1) / kTileK);
-  residues_cols_tiled_kernel<Sys><<<resident_grid(tiles, smem), 256, smem, st>>>(a, t);
-  return cudaGetLastError();
+  allow_smem(residues_kernel<Sys>, allowed, smem);
+  if (nops == 1) {
+    const int grid = resident_grid(resid_blocks(ops[0]), smem);
+    return launch_chained(residues_kernel<Sys>, grid, 256, smem, st, ops[0], ops[0], grid, t, static_cast<int>(tables));
+  }
+  const int64_t na = resid_blocks(ops[0]), nb = resid_blocks(ops[1]);
+  const int grid = resident_grid(na + nb, smem);
+  if (na + nb > 3 * static_cast<int64_t>(grid) && smem > tables) {
+    const cudaError_t err = run_residues<Sys>(ops, 1, t, st);
+    return err != cudaSuccess ? err : run_residues<Sys>(ops + 1, 1, t, st);
+  }
+  int split = grid == na + nb ? static_cast<int>(na)
+                              : static_cast<int>(static_cast<double>(grid) * ops[0].lines / (ops[0].lines + ops[1].lines) + 0.5);
+  split = std::max(1, std::min(split, grid - 1));
+  return launch_chained(residues_kernel<Sys>, grid, 256, smem, st, ops[0], ops[1], split, t, static_cast<int>(tables));
 }
 
 }  // namespace
 
-cudaError_t launch_residues_rows(const double* A, int64_t lda, int m, int k, int kp, int64_t ldp, const int32_t* e,
-                                 const RnsTable& rt, uint8_t* planes, uint32_t* flags, cudaStream_t st,
-                                 int64_t plane_stride) {
-  return run_rows<RnsSys>(
-      ResidArgs{A, lda, m, k, kp, ldp, e, planes, plane_stride ? plane_stride : static_cast<int64_t>(m) * ldp, flags},
-      rt, st);
+cudaError_t launch_residues(const ResidArgs* ops, int nops, const RnsTable& rt, cudaStream_t st) {
+  return run_residues<RnsSys>(ops, nops, rt, st);
 }
 
-cudaError_t launch_residues_cols(const double* B, int64_t ldb, int k, int n, int kp, int64_t ldp, const int32_t* f,
-                                 const RnsTable& rt, uint8_t* planes, uint32_t* flags, cudaStream_t st,
-                                 int64_t plane_stride) {
-  return run_cols<RnsSys>(
-      ResidArgs{B, ldb, n, k, kp, ldp, f, planes, plane_stride ? plane_stride : static_cast<int64_t>(n) * ldp, flags},
-      rt, st);
-}
-
-cudaError_t launch_paper_planes_rows(const double* A, int64_t lda, int m, int k, int kp, const int32_t* e,
-                                     const ModTable& mt, uint8_t* planes, uint32_t* flags, cudaStream_t st) {
-  return run_rows<PaperSys>(ResidArgs{A, lda, m, k, kp, kp, e, planes, static_cast<int64_t>(m) * kp, flags}, mt, st);
-}
-
-cudaError_t launch_paper_planes_cols(const double* B, int64_t ldb, int k, int n, int kp, const int32_t* f,
-                                     const ModTable& mt, uint8_t* planes, uint32_t* flags, cudaStream_t st) {
-  return run_cols<PaperSys>(ResidArgs{B, ldb, n, k, kp, kp, f, planes, static_cast<int64_t>(n) * kp, flags}, mt, st);
+cudaError_t launch_paper_planes(const ResidArgs* ops, const ModTable& mt, cudaStream_t st) {
+  return run_residues<PaperSys>(ops, 2, mt, st);
 }
 
 cudaError_t launch_residues_batch(const BatchProblem* probs, int count, int64_t rows_blocks, int64_t cols_blocks,
@@ -1078,8 +1070,7 @@ cudaError_t launch_grad_residues(const double* dC, int64_t lddc, int m, int n, c
   static std::atomic<int> allowed[64];
   allow_smem(grad_residues_kernel, allowed, smem);
   const int64_t tiles = static_cast<int64_t>((n + kTileCols - 1) / kTileCols) * ((m + kTileK - 1) / kTileK);
-  grad_residues_kernel<<<resident_grid(tiles, smem), 256, smem, st>>>(a, rt);
-  return cudaGetLastError();
+  return launch_chained(grad_residues_kernel, resident_grid(tiles, smem), 256, smem, st, a, rt);
 }
 
 cudaError_t launch_transpose_planes(const uint8_t* src, int64_t src_pitch, int64_t src_stride, int lines, int len,
@@ -1092,9 +1083,8 @@ cudaError_t launch_transpose_planes(const uint8_t* src, int64_t src_pitch, int64
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t total = static_cast<int64_t>((len + kTrTile - 1) / kTrTile) * ((lines + kTrTile - 1) / kTrTile) * planes;
   const int grid = static_cast<int>(std::min<int64_t>(total, 8 * static_cast<int64_t>(sms)));
-  transpose_planes_kernel<<<grid, 256, 0, st>>>(src, src_pitch, src_stride, lines, len, dst, dst_pitch, dst_stride,
-                                                planes);
-  return cudaGetLastError();
+  return launch_chained(transpose_planes_kernel, grid, 256, 0, st, src, src_pitch, src_stride, lines, len, dst, dst_pitch,
+                        dst_stride, planes);
 }
 
 }  // namespace ozk2

@@ -346,6 +346,8 @@ struct PrepArgs {
 template <bool FAST, int E, int W>  // E = 0: rows two passes at a time (long rows, fast mode)
 __global__ void __launch_bounds__(256) scale_prep_kernel(const __grid_constant__ PrepArgs a) {
   __shared__ uint32_t red[256];
+  chain_wait();
+  chain_next();
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < a.zero_words;
        i += static_cast<int64_t>(gridDim.x) * blockDim.x)
     a.zero[i] = 0u;
@@ -418,6 +420,8 @@ struct ColsArgs {
 };
 template <bool FAST>
 __global__ void __launch_bounds__(256) scale_cols_kernel(const __grid_constant__ ColsArgs a) {
+  chain_wait();
+  chain_next();
   const int i = blockIdx.x >= a.first[1] ? 1 : 0;
   const ScaleJob& job = a.job[i];
   const int gx = (job.lines + 31) / 32;
@@ -449,6 +453,8 @@ __device__ __forceinline__ void sumsq_body(const float* __restrict__ part, int n
 }
 
 __global__ void sumsq_reduce_kernel(const float* __restrict__ part, int nblocks, int n, float* __restrict__ sq) {
+  chain_wait();
+  chain_next();
   sumsq_body(part, nblocks, n, sq, blockIdx.x);
 }
 
@@ -490,6 +496,8 @@ __global__ void exponents_kernel(int m, int n, const int32_t* __restrict__ eprim
                                  const uint8_t* __restrict__ colstat, const float* __restrict__ R,
                                  const float* __restrict__ S, float pprime, float delta, int32_t* __restrict__ e,
                                  int32_t* __restrict__ f, uint32_t* flags) {
+  chain_wait();
+  chain_next();
   exponents_body(m, n, eprime, fprime, rowstat, colstat, R, S, pprime, delta, e, f, flags, blockIdx.x);
 }
 
@@ -520,6 +528,8 @@ __global__ void reuse_exponents_kernel(int m, const int32_t* __restrict__ gp, co
                                        const float* __restrict__ S, int32_t* __restrict__ h, float q,
                                        const uint8_t* __restrict__ rpart, int nr, const uint8_t* __restrict__ cpart,
                                        int nc, uint32_t* flags) {
+  chain_wait();
+  chain_next();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   uint8_t stat = 0;
   if (t < m) {
@@ -653,8 +663,7 @@ cudaError_t run_prep(const ScaleJob* jobs, int njobs, int k, int kp, uint32_t* z
   a.first[2] = blocks;
   if (njobs < 2) a.first[1] = blocks;
   if (!grid_ok(blocks)) return cudaErrorInvalidValue;
-  scale_prep_kernel<FAST, E, W><<<static_cast<unsigned>(blocks), 256, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(scale_prep_kernel<FAST, E, W>, static_cast<unsigned>(blocks), 256, 0, st, a);
 }
 
 }  // namespace
@@ -701,14 +710,12 @@ cudaError_t launch_scale_cols(const ScaleJob* jobs, int njobs, int k, int kp, bo
   a.first[2] = blocks;
   if (njobs < 2) a.first[1] = blocks;
   if (!grid_ok(blocks)) return cudaErrorInvalidValue;
-  if (fast) {
-    scale_cols_kernel<true><<<static_cast<unsigned>(blocks), 256, 0, st>>>(a);
-    for (int i = 0; i < njobs; ++i)
-      sumsq_reduce_kernel<<<(jobs[i].lines + 255) / 256, 256, 0, st>>>(jobs[i].part, kp / 32, jobs[i].lines, jobs[i].sq);
-  } else {
-    scale_cols_kernel<false><<<static_cast<unsigned>(blocks), 256, 0, st>>>(a);
-  }
-  return cudaGetLastError();
+  if (!fast) return launch_chained(scale_cols_kernel<false>, static_cast<unsigned>(blocks), 256, 0, st, a);
+  cudaError_t err = launch_chained(scale_cols_kernel<true>, static_cast<unsigned>(blocks), 256, 0, st, a);
+  for (int i = 0; i < njobs && err == cudaSuccess; ++i)
+    err = launch_chained(sumsq_reduce_kernel, (jobs[i].lines + 255) / 256, 256, 0, st, jobs[i].part, kp / 32,
+                         jobs[i].lines, jobs[i].sq);
+  return err;
 }
 
 cudaError_t launch_exponents(int m, int n, const int32_t* eprime, const int32_t* fprime,
@@ -716,9 +723,8 @@ cudaError_t launch_exponents(int m, int n, const int32_t* eprime, const int32_t*
                              const float* S, float pprime, float delta, int32_t* e, int32_t* f,
                              uint32_t* flags, cudaStream_t st) {
   const int total = m + n;
-  exponents_kernel<<<(total + 255) / 256, 256, 0, st>>>(m, n, eprime, fprime, rowstat, colstat, R, S,
-                                                        pprime, delta, e, f, flags);
-  return cudaGetLastError();
+  return launch_chained(exponents_kernel, (total + 255) / 256, 256, 0, st, m, n, eprime, fprime, rowstat, colstat, R, S,
+                        pprime, delta, e, f, flags);
 }
 
 cudaError_t launch_reuse_exponents(int m, const int32_t* gp, const uint8_t* rstat, const float* R, int32_t* g, int n,
@@ -727,9 +733,8 @@ cudaError_t launch_reuse_exponents(int m, const int32_t* gp, const uint8_t* rsta
                                    cudaStream_t st) {
   const int total = std::max(m + n, std::max(nr, nc));
   if (total <= 0) return cudaSuccess;
-  reuse_exponents_kernel<<<(total + 255) / 256, 256, 0, st>>>(m, gp, rstat, R, g, n, hp, cstat, S, h, q, rpart, nr, cpart,
-                                                              nc, flags);
-  return cudaGetLastError();
+  return launch_chained(reuse_exponents_kernel, (total + 255) / 256, 256, 0, st, m, gp, rstat, R, g, n, hp, cstat, S, h, q,
+                        rpart, nr, cpart, nc, flags);
 }
 
 }  // namespace ozk2
