@@ -46,12 +46,17 @@
 //   warp 0      TMA producer: 128-row A and 256-row B^T boxes (pairs: 128 rows) of 128
 //               bytes along K (K-major, 128-byte swizzle, zero fill past m, n, k) into a
 //               ring of 4 48-KiB stages (pairs: 6 of 32 KiB), mbarrier complete_tx.
-//   warp 1      TMEM allocation and the single MMA-issuing thread (pairs: the leader's):
+//   warp 1      TMEM allocation and the MMAs (pairs: the leader's warp issues them):
 //               tcgen05.mma.kind::f8f6f4, M = 128 (256), N = 256, K = 32; a pass starts
 //               once the epilogue has released the slot it writes.
 //   warps 2-9   epilogue (warps 2-17 in grouped launches): warp w reads TMEM lane
 //               quadrant w % 4, column half (quarter) (w - 2) / 4, with tcgen05.ld;
 //               FP32 math; global stores.
+// Warps 0 and 1 run their loops whole and put only the TMA, MMA and commit instructions under
+// elect_one: with one lane in the loop every operand had to be moved to a uniform register
+// (68 cycles an MMA), the issue of a k-step took as long as its products, and each pass
+// opened with the tensor cores idle for about 1000 cycles (4096^3 products 987 -> 950 us,
+// 65536 x 1024 x 1024 1188 -> 1133, 2048^3 145 -> 135).
 // Every wait is bounded (device.cuh; the limit is a launch parameter); a wait that gives
 // up raises a CTA-wide abort flag and the global timeout flag, drains the copies and
 // products this CTA has in flight, frees TMEM and returns.  Operands are read only with
@@ -80,7 +85,7 @@ struct Epi {
   static constexpr int kThreads = 64 + 32 * kWarps;
   static constexpr int kCW = GROUPED ? 16 : 32;  // columns per TMEM load of the residue epilogue
 };
-constexpr int kGroupM = 16;             // tile rasterisation: bands of 16 tile rows (2048 rows of A)
+constexpr int kBandLog = 4;             // tile rasterisation: bands of 16 tile rows (2048 rows of A)
 
 // Tile shapes: 128 x 256 (the default) or 128 x 128 (narrow or ragged products, where a
 // 256-wide tile would spend much of its tensor work on padding).  Both keep two TMEM
@@ -103,7 +108,7 @@ struct Tile {
 struct GemmParams {
   int mode;
   int m, n, k;
-  int tiles_m, tiles_n, tiles;
+  UnitGrid grid;
   int num_units;
   int16_t* cres;   // 16-bit residues (Karatsuba moduli; all of the paper mode)
   int8_t* cres8;   // 8-bit residues (single moduli)
@@ -125,18 +130,20 @@ struct GemmParams {
   uint32_t* pace;              // two zeroed words for the pacing of long reductions (Pace), or null
 };
 
-template <int GROUP_M>
-__device__ __forceinline__ void decode_unit(int tiles_m, int tiles_n, int tiles, int u, int& mod, int& tm,
-                                            int& tn) {
-  mod = u / tiles;
-  const int t = u - mod * tiles;
-  const int per_group = GROUP_M * tiles_n;
-  const int g = t / per_group;
-  const int first_m = g * GROUP_M;
-  const int gsz = min(tiles_m - first_m, GROUP_M);
-  const int r = t - g * per_group;
-  tm = first_m + r % gsz;
-  tn = r / gsz;
+// Tile row and column of tile t: bands of band tile rows, column by column within a band.
+// Every role of every CTA decodes every unit, between its waits, so the divisions are by
+// precomputed reciprocals (three integer divisions took 350 cycles a unit, a tenth of a
+// short pass).
+__device__ __forceinline__ void decode_tile(const UnitGrid& g, int t, int& tm, int& tn) {
+  const int band = static_cast<int>(g.per_band.quotient(static_cast<uint32_t>(t)));
+  const int r = t - band * static_cast<int>(g.per_band.d), first = band << g.band_log;
+  if (first + (1 << g.band_log) <= g.tiles_m) {
+    tn = r >> g.band_log;
+    tm = first + r - (tn << g.band_log);
+  } else {  // the last, narrower band
+    tn = static_cast<int>(g.last_band.quotient(static_cast<uint32_t>(r)));
+    tm = first + r - tn * static_cast<int>(g.last_band.d);
+  }
 }
 
 // Everything a role needs about one unit (a tile of one modulus of one problem).  A
@@ -147,9 +154,11 @@ struct UnitCtx {
   const CUtensorMap* tb;
   int m, n, k;
   int mod, tm, tn;
-  int prob = -1;  // grouped: problem of the fields below (-1: none yet)
-  int tiles_m, tiles_n, tiles;
-  int64_t unit_start, next_start;  // grouped: units [unit_start, next_start) are this problem's
+  int prob = -1;  // problem of the fields below (-1: none yet)
+  int tile;       // tile index within the modulus
+  int last_u;     // the unit of (mod, tile)
+  UnitGrid grid;
+  int64_t next_start;  // grouped: the next problem's first unit
   int16_t* cres;
   int8_t* cres8;
   int64_t ldr, res_stride;
@@ -158,24 +167,28 @@ struct UnitCtx {
   float* S;
 };
 
-template <bool GROUPED, bool PAIR>
+template <bool GROUPED>
 __device__ __forceinline__ void resolve_unit(const GemmParams& P, const CUtensorMap* tmA, const CUtensorMap* tmB,
                                              const GemmProblem* __restrict__ probs, int nprobs, int u, UnitCtx& c) {
   if constexpr (!GROUPED) {
-    c.ta = tmA;
-    c.tb = tmB;
-    c.m = P.m;
-    c.n = P.n;
-    c.k = P.k;
-    c.prob = 0;
-    decode_unit<PAIR ? kGroupM / 2 : kGroupM>(P.tiles_m, P.tiles_n, P.tiles, u, c.mod, c.tm, c.tn);
-    c.cres = P.cres;
-    c.cres8 = P.cres8;
-    c.ldr = P.ldr;
-    c.res_stride = P.res_stride;
-    c.factor = P.factor;
-    c.R = P.R;
-    c.S = P.S;
+    if (c.prob < 0) {
+      c.ta = tmA;
+      c.tb = tmB;
+      c.m = P.m;
+      c.n = P.n;
+      c.k = P.k;
+      c.prob = 0;
+      c.mod = 0;
+      c.tile = 0;
+      c.last_u = 0;
+      c.cres = P.cres;
+      c.cres8 = P.cres8;
+      c.ldr = P.ldr;
+      c.res_stride = P.res_stride;
+      c.factor = P.factor;
+      c.R = P.R;
+      c.S = P.S;
+    }
   } else {
     if (c.prob < 0 || u >= c.next_start) {
       // the last problem starting at or before u, searched above the current one
@@ -192,10 +205,10 @@ __device__ __forceinline__ void resolve_unit(const GemmParams& P, const CUtensor
       c.n = G.n;
       c.k = G.k;
       c.prob = lo;
-      c.tiles_m = G.tiles_m;
-      c.tiles_n = G.tiles_n;
-      c.tiles = G.tiles;
-      c.unit_start = G.unit_start;
+      c.grid = G.grid;
+      c.mod = 0;
+      c.tile = 0;
+      c.last_u = static_cast<int>(G.unit_start);
       c.next_start = lo + 1 < nprobs ? probs[lo + 1].unit_start : 0x7FFFFFFFFFFFFFFFll;
       c.cres = G.cres;
       c.cres8 = G.cres8;
@@ -205,9 +218,17 @@ __device__ __forceinline__ void resolve_unit(const GemmParams& P, const CUtensor
       c.R = G.R;
       c.S = G.S;
     }
-    decode_unit<PAIR ? kGroupM / 2 : kGroupM>(c.tiles_m, c.tiles_n, c.tiles, static_cast<int>(u - c.unit_start), c.mod,
-                                              c.tm, c.tn);
   }
+  // units are numbered modulus by modulus: step the tile, at most one modulus of the list
+  // at a time
+  const UnitGrid& g = GROUPED ? c.grid : P.grid;
+  c.tile += u - c.last_u;
+  c.last_u = u;
+  while (c.tile >= g.tiles) {
+    c.tile -= g.tiles;
+    ++c.mod;
+  }
+  decode_tile(g, c.tile, c.tm, c.tn);
 }
 
 // Tensor maps written to global memory before the launch: order the tensormap proxy's
@@ -230,7 +251,7 @@ __device__ __forceinline__ UnitPlan plan_of(const GemmParams& P, int k, int mod)
     u.chunk_len = P.mods.m[mod].chunk;
     if constexpr (MODE == kModeResidue) u.npasses = mod < P.mods.kars ? 3 : 1;
     else u.npasses = mod < kNumSquares ? 2 : 3;
-    u.nchunks = (k + u.chunk_len - 1) / u.chunk_len;
+    u.nchunks = k <= u.chunk_len ? 1 : (k + u.chunk_len - 1) / u.chunk_len;
   } else {
     u.chunk_len = ((k + BK - 1) / BK) * BK;
     u.npasses = 1;
@@ -297,13 +318,14 @@ struct Pace {
       return;
     }
     steps = 1;
-    atomicAdd(words, 1u);
+    if (elect_one()) atomicAdd(words, 1u);
+    __syncwarp();
     ++round;
     if (!on) return;
     const uint32_t want = pairs * round;
     const unsigned long long t0 = global_ns();
-    while (load_relaxed(words) < want) {
-      if (global_ns() - t0 > kPaceNs) {
+    while (__any_sync(0xffffffffu, load_relaxed(words) < want)) {
+      if (__any_sync(0xffffffffu, global_ns() - t0 > kPaceNs)) {
         on = false;
         break;
       }
@@ -311,11 +333,14 @@ struct Pace {
   }
   __device__ __forceinline__ void finish(uint32_t pairs) {
     if (words == nullptr) return;
-    atomicAdd(words, kPaceDone);
-    if (atomicAdd(words + 1, 1u) == pairs - 1u) {
-      words[0] = 0u;
-      words[1] = 0u;
+    if (elect_one()) {
+      atomicAdd(words, kPaceDone);
+      if (atomicAdd(words + 1, 1u) == pairs - 1u) {
+        words[0] = 0u;
+        words[1] = 0u;
+      }
     }
+    __syncwarp();
   }
   static __device__ __forceinline__ uint32_t load_relaxed(const uint32_t* p) {
     uint32_t v;
@@ -382,8 +407,15 @@ __device__ __forceinline__ uint32_t pack2(float2 r) {
   const float2 b = __fadd2_rn(r, dup2(kMagic));
   return __byte_perm(__float_as_uint(b.x), __float_as_uint(b.y), 0x5410);
 }
-__device__ __forceinline__ float2 unpack2(uint32_t w) {
-  return make_float2(static_cast<float>(static_cast<int16_t>(w & 0xFFFFu)), static_cast<float>(static_cast<int16_t>(w >> 16)));
+// Parked form: r + 2^15 as two unsigned 16-bit halves.  Unparking puts each under the
+// exponent of 2^23 (one byte permute) and takes 2^23 + 2^15 off; converting a signed half
+// instead needs the conversion unit, 16 lanes a cycle, which bound the Karatsuba passes.
+__device__ __forceinline__ uint32_t park2(float2 r) {
+  const float2 b = __fadd2_rn(r, dup2(kMagic + 32768.0f));
+  return __byte_perm(__float_as_uint(b.x), __float_as_uint(b.y), 0x5410);
+}
+__device__ __forceinline__ float2 unpark2(uint32_t w) {
+  return __fadd2_rn(bits2(__byte_perm(w, 0x4B00u, 0x5410), __byte_perm(w, 0x4B00u, 0x5432)), dup2(-8421376.0f));
 }
 
 // Store 8 int16 residues of one row at columns gc .. gc + 7 (gc < n), packed two per word,
@@ -522,7 +554,7 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    {
       int stage = 0;
       uint32_t phase = 0;
       uint32_t issued = 0, issued_phase = 0;
@@ -531,10 +563,13 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
       UnitCtx uc;
       Pace pace(PAIR && leader ? prm.pace : nullptr);
       for (int u = u_first; ok && u < prm.num_units; u += u_step) {
-        resolve_unit<GROUPED, PAIR>(prm, &tmA, &tmB, probs, nprobs, u, uc);
+        resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
         if (GROUPED && uc.prob != last_prob) {
-          tensormap_acquire(uc.ta);
-          tensormap_acquire(uc.tb);
+          if (elect_one()) {
+            tensormap_acquire(uc.ta);
+            tensormap_acquire(uc.tb);
+          }
+          __syncwarp();
           last_prob = uc.prob;
         }
         const int mod = uc.mod;
@@ -549,25 +584,28 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
                 pace.k_step(static_cast<uint32_t>(u_step));
               }
               for (int x = 0; x < np; ++x) {
-                if (!mbar_wait_bounded(empty + stage, phase ^ 1u, abort_flag, wait_ns)) {
+                if (!warp_wait(empty + stage, phase ^ 1u, abort_flag, wait_ns)) {
                   ok = false;
                   break;
                 }
                 int pa, pb;
                 product_of<MODE>(prm, mod, ps, x, pa, pb);
                 uint8_t* dst = tiles + stage * kStageBytes;
-                if constexpr (PAIR) {
-                  // both CTAs' bytes count on the leader's barrier
-                  const uint32_t bar = leader_addr(full + stage);
-                  if (leader) mbar_arrive_expect_tx(full + stage, 2 * kStageBytes);
-                  tma_load_3d_pair(dst, uc.ta, bar, k0 + s * BK, (uc.tm * 2 + static_cast<int>(rank)) * BM, pa);
-                  tma_load_3d_pair(dst + kATileBytes, uc.tb, bar, k0 + s * BK,
-                                   uc.tn * BN + static_cast<int>(rank) * T::kBRows, pb);
-                } else {
-                  mbar_arrive_expect_tx(full + stage, kStageBytes);
-                  tma_load_3d(dst, uc.ta, full + stage, k0 + s * BK, uc.tm * BM, pa);
-                  tma_load_3d(dst + kATileBytes, uc.tb, full + stage, k0 + s * BK, uc.tn * BN, pb);
+                if (elect_one()) {
+                  if constexpr (PAIR) {
+                    // both CTAs' bytes count on the leader's barrier
+                    const uint32_t bar = leader_addr(full + stage);
+                    if (leader) mbar_arrive_expect_tx(full + stage, 2 * kStageBytes);
+                    tma_load_3d_pair(dst, uc.ta, bar, k0 + s * BK, (uc.tm * 2 + static_cast<int>(rank)) * BM, pa);
+                    tma_load_3d_pair(dst + kATileBytes, uc.tb, bar, k0 + s * BK,
+                                     uc.tn * BN + static_cast<int>(rank) * T::kBRows, pb);
+                  } else {
+                    mbar_arrive_expect_tx(full + stage, kStageBytes);
+                    tma_load_3d(dst, uc.ta, full + stage, k0 + s * BK, uc.tm * BM, pa);
+                    tma_load_3d(dst + kATileBytes, uc.tb, full + stage, k0 + s * BK, uc.tn * BN, pb);
+                  }
                 }
+                __syncwarp();
                 issued |= 1u << stage;
                 issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
                 if (++stage == kStages) {
@@ -582,8 +620,8 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
       if constexpr (PAIR) pace.finish(static_cast<uint32_t>(u_step));
       if (!ok) {
         *abort_flag = 1;
-        atomicOr(prm.flags, kFlagTimeout);
-        int no_abort = 0;  // let this thread's copies in flight land before exiting
+        if (lane == 0) atomicOr(prm.flags, kFlagTimeout);
+        int no_abort = 0;  // let this warp's copies in flight land before exiting
         if constexpr (PAIR) {
           // the barriers count both CTAs' copies and the other CTA may have given up at
           // another stage: wait a fixed time, thousands of times a copy's
@@ -598,17 +636,17 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && leader) {
+    if (leader) {
       constexpr uint32_t idesc = fp8_idesc(G * BM, BN);
       int stage = 0;
       uint32_t phase = 0;
       Slots sl;
       // an injected stall (fault-injection tests): wait for a barrier nothing arrives at,
       // so this wait runs out and the kernel takes its timeout path
-      bool ok = prm.stall ? mbar_wait_bounded(never, 0u, abort_flag, wait_ns) : true;
+      bool ok = prm.stall ? warp_wait(never, 0u, abort_flag, wait_ns) : true;
       UnitCtx uc;
       for (int u = u_first; ok && u < prm.num_units; u += u_step) {
-        resolve_unit<GROUPED, PAIR>(prm, &tmA, &tmB, probs, nprobs, u, uc);
+        resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
         const int mod = uc.mod;
         const UnitPlan up = plan_of<MODE>(prm, uc.k, mod);
         for (int c = 0; ok && c < up.nchunks; ++c) {
@@ -616,40 +654,43 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
           const int ksteps = (min(uc.k, k0 + up.chunk_len) - k0 + BK - 1) / BK;
           for (int ps = 0; ok && ps < up.npasses; ++ps) {
             const uint32_t slot = sl.slot();
-            ok = mbar_wait_bounded(tempty + slot, (sl.uses() & 1u) ^ 1u, abort_flag, wait_ns);
+            ok = warp_wait(tempty + slot, (sl.uses() & 1u) ^ 1u, abort_flag, wait_ns);
             if (!ok) break;
             tc_fence_after();
             const uint32_t dtm = tmem_base + slot * static_cast<uint32_t>(BN);
             const int steps = ksteps * num_products<MODE>(mod, ps);
-            for (int s = 0; s < steps; ++s) {
-              if (!mbar_wait_bounded(full + stage, phase, abort_flag, wait_ns)) {
-                ok = false;
-                break;
-              }
+            for (int s = 0; ok && s < steps; ++s) {
+              ok = warp_wait(full + stage, phase, abort_flag, wait_ns);
+              if (!ok) break;
               tc_fence_after();
-              const uint32_t sa = smem_addr(tiles + stage * kStageBytes);
-              const uint64_t adesc = sw128_kmajor_desc(sa);
-              const uint64_t bdesc = sw128_kmajor_desc(sa + kATileBytes);
+              if (elect_one()) {
+                const uint32_t sa = smem_addr(tiles + stage * kStageBytes);
+                const uint64_t adesc = sw128_kmajor_desc(sa);
+                const uint64_t bdesc = sw128_kmajor_desc(sa + kATileBytes);
 #pragma unroll
-              for (int kk = 0; kk < BK / 32; ++kk)
-                mma_fp8<G>(dtm, adesc + 2ull * kk, bdesc + 2ull * kk, idesc, (s == 0 && kk == 0) ? 0u : 1u);
-              mma_commit<G>(empty + stage);
+                for (int kk = 0; kk < BK / 32; ++kk)
+                  mma_fp8<G>(dtm, adesc + 2ull * kk, bdesc + 2ull * kk, idesc, (s == 0 && kk == 0) ? 0u : 1u);
+                mma_commit<G>(empty + stage);
+                if (s == steps - 1) mma_commit<G>(tfull + slot);
+              }
+              __syncwarp();
               if (++stage == kStages) {
                 stage = 0;
                 phase ^= 1u;
               }
             }
-            if (ok) mma_commit<G>(tfull + slot);
             ++sl.t;
           }
         }
       }
-      mma_commit<G>(done);  // every product issued here completes before TMEM is freed
+      // every product issued here completes before TMEM is freed
+      if (elect_one()) mma_commit<G>(done);
+      __syncwarp();
       int no_abort = 0;
       mbar_wait_bounded(done, 0, &no_abort, kWaitLimitNs);
       if (!ok) {
         *abort_flag = 1;
-        atomicOr(prm.flags, kFlagTimeout);
+        if (lane == 0) atomicOr(prm.flags, kFlagTimeout);
       }
     }
   } else {
@@ -673,15 +714,14 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
     bool ok = true;
     UnitCtx uc;
     for (int u = u_first; ok && u < prm.num_units; u += u_step) {
-      resolve_unit<GROUPED, PAIR>(prm, &tmA, &tmB, probs, nprobs, u, uc);
+      resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
       const int mod = uc.mod, tn = uc.tn;
       const UnitPlan up = plan_of<MODE>(prm, uc.k, mod);
       const int gi = (uc.tm * G + static_cast<int>(rank)) * BM + row;
       for (int c = 0; ok && c < up.nchunks; ++c) {
         for (int ps = 0; ok && ps < up.npasses; ++ps) {
           const uint32_t slot = sl.slot();
-          ok = mbar_wait_bounded(tfull + slot, sl.uses() & 1u, abort_flag, wait_ns);
-          ok = __all_sync(0xffffffffu, ok);
+          ok = warp_wait(tfull + slot, sl.uses() & 1u, abort_flag, wait_ns);
           if (!ok) break;
           tc_fence_after();
           const uint32_t ts = tq + slot * static_cast<uint32_t>(BN);
@@ -753,7 +793,7 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
                   for (int w = 0; w < kCW / 8; ++w) {
                     uint32_t pk[4];
 #pragma unroll
-                    for (int z = 0; z < 4; ++z) pk[z] = pack2(mod_near2(bits2(v[8 * w + 2 * z], v[8 * w + 2 * z + 1]), mp));
+                    for (int z = 0; z < 4; ++z) pk[z] = park2(mod_near2(bits2(v[8 * w + 2 * z], v[8 * w + 2 * z + 1]), mp));
                     store4(sp, w, pk);
                   }
                 } else if (!last) {  // Karatsuba pass 2: park v = mod(c1 d1 + c2 D2, p); D2 mod p first
@@ -767,8 +807,8 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
                     for (int z = 0; z < 4; ++z) {
                       const int j = 8 * w + 2 * z;
                       const float2 d2 = mod_near2(bits2(v[j], v[j + 1]), mp);
-                      const float2 y = __ffma2_rn(dup2(c2), d2, __fmul2_rn(dup2(c1), unpack2(pr[z])));
-                      pk[z] = pack2(mod_near2(y, mp));
+                      const float2 y = __ffma2_rn(dup2(c2), d2, __fmul2_rn(dup2(c1), unpark2(pr[z])));
+                      pk[z] = park2(mod_near2(y, mp));
                     }
                     store4(sp, w, pk);
                   }
@@ -784,8 +824,8 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
                     for (int z = 0; z < 4; ++z) {
                       const int j = 8 * w + 2 * z;
                       const float2 d = bits2(v[j], v[j + 1]);
-                      if (square) pk[z] = pack2(smod2(__ffma2_rn(dup2(c1), unpack2(pr[z]), d), mp));
-                      else pk[z] = pack2(mod_near2(__ffma2_rn(dup2(c3), mod_near2(d, mp), unpack2(pr[z])), mp));
+                      if (square) pk[z] = pack2(smod2(__ffma2_rn(dup2(c1), unpark2(pr[z]), d), mp));
+                      else pk[z] = pack2(mod_near2(__ffma2_rn(dup2(c3), mod_near2(d, mp), unpark2(pr[z])), mp));
                     }
                     const int gc = gc0 + cb * kCW + 8 * w;
                     if (keep_row && gc < uc.n) store_residues8<MODE == kModePaper>(dst, gc, pk, c > 0, p, h, prm.flags);
@@ -926,6 +966,28 @@ bool use_pairs(const GemmArgs& g, int BN) {
   return rounds * ((g.k + BK - 1) / BK) >= 56;
 }
 
+// Reciprocal of d for numerators below 2^31: floor(n / d) = (n mul >> 32) >> shift.
+FastDiv fast_div(int d) {
+  FastDiv r{};
+  r.d = static_cast<uint32_t>(d);
+  int l = 0;
+  while ((int64_t(1) << l) < d) ++l;  // ceil(log2 d)
+  r.shift = l == 0 ? 0 : l - 1;
+  r.mul = l == 0 ? 0u : static_cast<uint32_t>(((uint64_t(1) << (31 + l)) + static_cast<uint64_t>(d) - 1) / static_cast<uint64_t>(d));
+  return r;
+}
+
+UnitGrid unit_grid(int tiles_m, int tiles_n, int band_log) {
+  UnitGrid g{};
+  g.tiles_m = tiles_m;
+  g.tiles = tiles_m * tiles_n;
+  g.band_log = band_log;
+  g.per_band = fast_div(tiles_n << band_log);
+  const int rest = tiles_m & ((1 << band_log) - 1);
+  g.last_band = fast_div(rest ? rest : 1);
+  return g;
+}
+
 int tile_width(int tile_n) { return tile_n == 128 ? 128 : 256; }
 
 }  // namespace
@@ -939,12 +1001,11 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
   prm.k = g.k;
   const int BN = g.mode == kModePaper ? 256 : tile_width(g.tile_n);
   const bool pair = use_pairs(g, BN);
-  prm.tiles_m = (g.m + (pair ? 2 : 1) * BM - 1) / ((pair ? 2 : 1) * BM);
-  prm.tiles_n = (g.n + BN - 1) / BN;
-  prm.tiles = prm.tiles_m * prm.tiles_n;
+  prm.grid = unit_grid((g.m + (pair ? 2 : 1) * BM - 1) / ((pair ? 2 : 1) * BM), (g.n + BN - 1) / BN,
+                       pair ? kBandLog - 1 : kBandLog);
   const bool residues = g.mode == kModeResidue || g.mode == kModePaper;
   if (residues) prm.mods = *g.mods;
-  prm.num_units = prm.tiles * (residues ? prm.mods.count : 1);
+  prm.num_units = prm.grid.tiles * (residues ? prm.mods.count : 1);
   prm.cres = g.cres;
   prm.cres8 = g.cres8;
   prm.ldr = g.ldr;
@@ -994,9 +1055,7 @@ bool encode_gemm_problem(GemmProblem* gp, const uint8_t* a, const uint8_t* b, in
   gp->m = m;
   gp->n = n;
   gp->k = k;
-  gp->tiles_m = (m + BM - 1) / BM;
-  gp->tiles_n = (n + BN - 1) / BN;
-  gp->tiles = gp->tiles_m * gp->tiles_n;
+  gp->grid = unit_grid((m + BM - 1) / BM, (n + BN - 1) / BN, kBandLog);
   return true;
 }
 

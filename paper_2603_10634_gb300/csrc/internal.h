@@ -250,6 +250,21 @@ cudaError_t launch_transpose_planes(const uint8_t* src, int64_t src_pitch, int64
                                     uint8_t* dst, int64_t dst_pitch, int64_t dst_stride, int planes, cudaStream_t st);
 
 // gemm.cu
+// Division by an invariant (numerators below 2^31).
+struct FastDiv {
+  uint32_t mul, d;
+  int shift;
+#ifdef __CUDACC__
+  __device__ __forceinline__ uint32_t quotient(uint32_t n) const { return mul == 0u ? n : __umulhi(n, mul) >> shift; }
+#endif
+};
+// Tiles of one modulus and their rasterisation.
+struct UnitGrid {
+  int tiles_m, tiles;
+  int band_log;       // bands of 2^band_log tile rows
+  FastDiv per_band;   // tiles per full band
+  FastDiv last_band;  // rows of the last band when it is narrower
+};
 enum GemmMode { kModeResidue = 0, kModeBound = 1, kModeRaw = 2, kModePaper = 3 };
 
 struct GemmArgs {
@@ -389,7 +404,7 @@ struct GemmProblem {  // CUtensorMap carries the 64-byte alignment TMA needs
   CUtensorMap ta;
   CUtensorMap tb;
   int m, n, k;
-  int tiles_m, tiles_n, tiles;
+  UnitGrid grid;
   int64_t unit_start;
   int16_t* cres;
   int8_t* cres8;
