@@ -41,17 +41,16 @@
 // barrier, and the leader's commits arrive on both CTAs' empty and tfull barriers; only
 // the release of an accumulator slot is a (relaxed) remote arrival, one per warp and pass.
 //
-// Roles (320 threads for single problems, 576 for grouped launches; one persistent CTA
-// per SM):
+// Roles (576 threads; 320 for pairs and 128-column tiles; one persistent CTA per SM):
 //   warp 0      TMA producer: 128-row A and 256-row B^T boxes (pairs: 128 rows) of 128
 //               bytes along K (K-major, 128-byte swizzle, zero fill past m, n, k) into a
 //               ring of 4 48-KiB stages (pairs: 6 of 32 KiB), mbarrier complete_tx.
 //   warp 1      TMEM allocation and the MMAs (pairs: the leader's warp issues them):
 //               tcgen05.mma.kind::f8f6f4, M = 128 (256), N = 256, K = 32; a pass starts
 //               once the epilogue has released the slot it writes.
-//   warps 2-9   epilogue (warps 2-17 in grouped launches): warp w reads TMEM lane
-//               quadrant w % 4, column half (quarter) (w - 2) / 4, with tcgen05.ld;
-//               FP32 math; global stores.
+//   warps 2-17  epilogue (pairs and 128-column tiles: 2-9): warp w reads TMEM lane
+//               quadrant w % 4, 64 (pairs: 128) columns from the (w - 2) / 4-th such group,
+//               with tcgen05.ld; FP32 math; global stores.
 // Warps 0 and 1 run their loops whole and put only the TMA, MMA and commit instructions under
 // elect_one: with one lane in the loop every operand had to be moved to a uniform register
 // (68 cycles an MMA), the issue of a k-step took as long as its products, and each pass
@@ -72,18 +71,19 @@ namespace {
 constexpr int BM = 128;
 constexpr int BK = 128;  // bytes = FP8 elements per k-step (one 128-byte swizzle row)
 constexpr int kATileBytes = BM * BK;  // 16 KiB
-// Epilogue warps: 8 for single problems, 16 for grouped launches.  Short reductions in
-// batches of small problems leave the tensor cores waiting for the epilogue (about 40%
-// of the MMA thread's time with 8 warps on the 512-product batch); twice the warps hide
-// more of its TMEM-load and store latency there (batch 14.8 -> 13.7 ms), while for
-// single problems the extra warps slowed the MMA and TMA threads that share their
-// schedulers (8192 x 8192 x 2048: 4.29 -> 4.53 ms).
-template <bool GROUPED>
+// Epilogue warps and the columns of a TMEM load.  Short reductions leave the tensor cores
+// waiting for the epilogue: a warp takes 64 columns of the tile, 16 warps for 256 columns,
+// which hides more of its TMEM-load and store latency than 8 warps (bound product of
+// 16384 x 16384 x 512: 0.358 -> 0.237 ms; whole calls 256^3 43.3 -> 40.9 us, 1024^3 106 ->
+// 99.9 us).  Pairs run long reductions, where 16 warps take issue slots from the MMA and TMA
+// threads on their schedulers (16384 x 16384 x 512 residue products: 3.84 ms with 16 warps,
+// 2.83 ms with 8), and keep 8 warps with 32-column loads.
+template <int TN, bool PAIR>
 struct Epi {
-  static constexpr int kWarps = GROUPED ? 16 : 8;
-  static constexpr int kColGroups = kWarps / 4;  // epilogue warps per TMEM lane quadrant
+  static constexpr int kWarps = PAIR ? 8 : 4 * TN / 64;
+  static constexpr int kCols = 4 * TN / kWarps;  // columns of a thread
+  static constexpr int kCW = PAIR ? 32 : 16;  // columns of a TMEM load
   static constexpr int kThreads = 64 + 32 * kWarps;
-  static constexpr int kCW = GROUPED ? 16 : 32;  // columns per TMEM load of the residue epilogue
 };
 constexpr int kBandLog = 4;             // tile rasterisation: bands of 16 tile rows (2048 rows of A)
 
@@ -452,9 +452,10 @@ __device__ __forceinline__ void store_residues8(int16_t* dst, int gc, uint32_t (
 }
 
 // The same for 16 int8 residues, packed four per word.
-__device__ __forceinline__ void store_residues16(int8_t* dst, int gc, uint32_t (&pk)[4], bool accumulate, int p, int h,
+__device__ __forceinline__ void store_residues16(int8_t* dst, int gc, uint4 x4, bool accumulate, int p, int h,
                                                  uint32_t* flags) {
   uint4* out = reinterpret_cast<uint4*>(dst + gc);
+  uint32_t pk[4] = {x4.x, x4.y, x4.z, x4.w};
   if (accumulate) {
     const uint4 prev = *out;
     const uint32_t pw[4] = {prev.x, prev.y, prev.z, prev.w};
@@ -483,6 +484,30 @@ __device__ __forceinline__ void store_residues16(int8_t* dst, int gc, uint32_t (
   *out = make_uint4(pk[0], pk[1], pk[2], pk[3]);
 }
 
+// 4 x 4 transpose of 16-byte items over groups of four lanes: lane i's item j comes from
+// lane j's item i.  Rows held one to a lane become 64-byte pieces of a row over four lanes,
+// so that a warp's store covers whole sectors of 8 rows instead of half sectors of 32
+// (16384 x 16384 x 512 residue products of a pair: 3.56 -> 2.83 ms).  The 16-bit planes keep
+// their row pieces: the items held over the pass cost more than the sectors gained (2.83 ->
+// 3.27 ms with them transposed too).
+__device__ __forceinline__ uint4 shfl_xor4(uint4 v, int mask) {
+  return make_uint4(__shfl_xor_sync(0xffffffffu, v.x, mask), __shfl_xor_sync(0xffffffffu, v.y, mask),
+                    __shfl_xor_sync(0xffffffffu, v.z, mask), __shfl_xor_sync(0xffffffffu, v.w, mask));
+}
+__device__ __forceinline__ void transpose4(uint4 (&x)[4], int lane) {
+#pragma unroll
+  for (int b = 1; b <= 2; b <<= 1) {
+    const bool up = (lane & b) != 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (j & b) continue;
+      const uint4 got = shfl_xor4(up ? x[j] : x[j | b], b);
+      if (up) x[j] = got;
+      else x[j | b] = got;
+    }
+  }
+}
+
 // Four exact-integer floats |r| < 2^7 as four int8 of one word, in order (the low bytes
 // of r + 1.5 2^23).
 __device__ __forceinline__ uint32_t pack4(float2 a, float2 b) {
@@ -494,7 +519,7 @@ __device__ __forceinline__ uint32_t pack4(float2 a, float2 b) {
 // GROUPED: the units of all `nprobs` problems of `probs` (tmA, tmB unused).  TN: tile width.
 // PAIR: launched in clusters of two CTAs.
 template <int MODE, bool GROUPED, int TN, bool PAIR>
-__global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
+__global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
     fp8_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ GemmParams prm, const GemmProblem* __restrict__ probs, int nprobs) {
   constexpr int BN = TN;
@@ -530,7 +555,7 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
     }
     for (int j = 0; j < 2; ++j) {
       mbar_init(tfull + j, 1);
-      mbar_init(tempty + j, PAIR ? 2 * Epi<GROUPED>::kWarps : 32 * Epi<GROUPED>::kWarps);  // per warp / per thread
+      mbar_init(tempty + j, PAIR ? 2 * Epi<TN, PAIR>::kWarps : 32 * Epi<TN, PAIR>::kWarps);  // per warp / per thread
     }
     mbar_init(done, 1);
     mbar_init(never, 1);
@@ -697,8 +722,8 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
     // ------------------------------------------------------------ epilogue
     const int q = warp & 3;                 // TMEM lane quadrant this warp may access
     const int cgrp = (warp - 2) >> 2;       // column group of the tile
-    constexpr int kCols = BN / Epi<GROUPED>::kColGroups;  // columns of this thread
-    constexpr int kCW = Epi<GROUPED>::kCW;
+    constexpr int kCols = Epi<TN, PAIR>::kCols;   // columns of this thread
+    constexpr int kCW = Epi<TN, PAIR>::kCW;
     constexpr int kChunks = kCols / kCW;
     const int row = q * 32 + lane;
     const uint32_t tq = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + static_cast<uint32_t>(cgrp * kCols);
@@ -761,22 +786,31 @@ __global__ void __launch_bounds__(Epi<GROUPED>::kThreads, 1)
             const int gc0 = tn * BN + cgrp * kCols;
             const int64_t off = static_cast<int64_t>(gi) * uc.ldr;
             if (MODE == kModeResidue && mod >= prm.mods.kars) {  // single modulus
-              int8_t* dst = uc.cres8 + static_cast<int64_t>(mod - prm.mods.kars) * uc.res_stride + off;
+              int8_t* plane = uc.cres8 + static_cast<int64_t>(mod - prm.mods.kars) * uc.res_stride;
 #pragma unroll
-              for (int cb = 0; cb < kChunks; ++cb) {
-                uint32_t v[kCW];
-                load(cb, v);
+              for (int g = 0; g < kCols / 64; ++g) {
+                uint4 px[4];  // this row's 64 columns, then four rows' 16 columns
 #pragma unroll
-                for (int w = 0; w < kCW / 16; ++w) {
-                  uint32_t pk[4];
+                for (int cb = 0; cb < 64 / kCW; ++cb) {
+                  uint32_t v[kCW];
+                  load(g * (64 / kCW) + cb, v);
 #pragma unroll
-                  for (int z = 0; z < 4; ++z) {
-                    const int j = 16 * w + 4 * z;
-                    pk[z] = pack4(mod_near2(bits2(v[j], v[j + 1]), mp), mod_near2(bits2(v[j + 2], v[j + 3]), mp));
+                  for (int w = 0; w < kCW / 16; ++w) {
+                    uint32_t pk[4];
+#pragma unroll
+                    for (int z = 0; z < 4; ++z) {
+                      const int j = 16 * w + 4 * z;
+                      pk[z] = pack4(mod_near2(bits2(v[j], v[j + 1]), mp), mod_near2(bits2(v[j + 2], v[j + 3]), mp));
+                    }
+                    px[cb * (kCW / 16) + w] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                   }
-                  const int gc = gc0 + cb * kCW + 16 * w;
-                  if (keep_row && gc < uc.n) store_residues16(dst, gc, pk, c > 0, p, h, prm.flags);
                 }
+                transpose4(px, lane);
+                const int gc = gc0 + 64 * g + 16 * (lane & 3), gr = gi - (lane & 3);
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                  if (gr + x < uc.m && gc < uc.n)
+                    store_residues16(plane + static_cast<int64_t>(gr + x) * uc.ldr, gc, px[x], c > 0, p, h, prm.flags);
               }
             } else {
               int16_t* dst = uc.cres + static_cast<int64_t>(mod) * uc.res_stride + off;
@@ -924,7 +958,7 @@ cudaError_t launch_mode(const GemmParams& prm, const CUtensorMap& ta, const CUte
   }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(grid));
-  cfg.blockDim = dim3(Epi<GROUPED>::kThreads);
+  cfg.blockDim = dim3(Epi<TN, PAIR>::kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[2]{};
