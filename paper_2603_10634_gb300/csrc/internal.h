@@ -47,17 +47,20 @@ struct ModTable {
 };
 
 // The product path's residue system (rns.h): constants of the residue kernels, per
-// remainder taken (groups of single moduli, then Karatsuba moduli).
+// remainder taken (groups of single moduli, then Karatsuba moduli), as duplicated FP32 pairs.
+struct alignas(16) RnsConsts {
+  float2 neg_m, inv_m;
+  float2 w[kRnsPieces - 1];                  // 2^22, 2^33, 2^44 mod M, symmetric
+  float2 scale, base;                        // table address of a remainder: entry size and byte offset of
+                                             // remainder 0, as multiples of 2^-149
+  float2 neg_p[kGroupMax], inv_p[kGroupMax]; // members of a group without a table: -p, RN(1/p)
+};
 struct RnsTable {
   int N;
   int singles, groups, kars;
   int pair_words, lut_words;                // 16-byte words of the pairs' digit tables, of all
-  float neg_m[kMaxVirtual], inv_m[kMaxVirtual];
-  float w[kMaxVirtual][kRnsPieces - 1];     // 2^22, 2^33, 2^44 mod M, symmetric
-  float neg_p[kMaxVirtual][kGroupMax];      // members of a group: -p, RN(1/p)
-  float inv_p[kMaxVirtual][kGroupMax];
+  RnsConsts c[kMaxVirtual];
   int16_t pow2[kMaxVirtual][kPow2Table];    // 2^t mod M, symmetric
-  int32_t lut_base[kMaxVirtual];            // byte offset of remainder 0 in the block's digit tables
 };
 
 // One modulus of the FP8 products' epilogue.
@@ -358,9 +361,8 @@ struct BatchProblem {
   int64_t nblocks[kBatchKernels];
 };
 
-// Tile of the column residue kernel: kResidTileCols columns x kResidTileK k per block
-// (one block per tile in a grouped launch).
-constexpr int kResidTileCols = 32, kResidTileK = 128;
+// Tile of the column residue kernel: kResidTileCols columns x kResidTileK k.
+constexpr int kResidTileCols = 16, kResidTileK = 128;
 
 // Items of the row residue kernel: a warp covers 2^s lanes x 8 k of 32 / 2^s rows, s = 4
 // (128 consecutive k of two rows) for kp > 64, else the smallest s with 2^s 8 >= kp (kp is

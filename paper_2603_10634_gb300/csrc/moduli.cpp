@@ -263,28 +263,37 @@ bool build_rns_table(int N, RnsTable* rt) {
   rt->groups = rns_groups(N);
   rt->kars = kRnsKars[N];
   const int pairs = rns_lut_pairs(N);
+  auto pair = [](float v) { return float2{v, v}; };
+  auto bits = [](int32_t i) {  // i 2^-149
+    float f;
+    std::memcpy(&f, &i, sizeof(f));
+    return f;
+  };
   rt->pair_words = pair_lut_offset(pairs) / 16;
   rt->lut_words = (pair_lut_offset(pairs) + kar_lut_offset(rt->kars)) / 16;
   for (int v = 0; v < rt->groups + rt->kars; ++v) {
     const bool kar = v >= rt->groups;
     const int M = kar ? kKarP[v - rt->groups] : group_modulus(v);
-    rt->neg_m[v] = -static_cast<float>(M);
-    rt->inv_m[v] = static_cast<float>(1.0 / M);
+    RnsConsts& c = rt->c[v];
+    c.neg_m = pair(-static_cast<float>(M));
+    c.inv_m = pair(static_cast<float>(1.0 / M));
     int x = 1;
     for (int t = 0; t < kPow2Table; ++t) {
       rt->pow2[v][t] = static_cast<int16_t>(symmetric(x, M));
       for (int j = 1; j < kRnsPieces; ++j)
-        if (t == kRnsPieceShift[j]) rt->w[v][j - 1] = static_cast<float>(symmetric(x, M));
+        if (t == kRnsPieceShift[j]) c.w[j - 1] = pair(static_cast<float>(symmetric(x, M)));
       x = 2 * x % M;
     }
     if (kar) {
-      rt->lut_base[v] = pair_lut_offset(pairs) + kar_lut_offset(v - rt->groups) + 4 * (M / 2 + 1);
+      c.scale = pair(bits(4));
+      c.base = pair(bits(pair_lut_offset(pairs) + kar_lut_offset(v - rt->groups) + 4 * (M / 2 + 1)));
     } else if (v < kLutPairs) {
-      rt->lut_base[v] = pair_lut_offset(v) + 2 * (M / 2 + 1);
+      c.scale = pair(bits(2));
+      c.base = pair(bits(pair_lut_offset(v) + 2 * (M / 2 + 1)));
     } else {
       for (int j = 0; j < (v == kGroups1 - 1 ? 3 : 2); ++j) {
-        rt->neg_p[v][j] = -static_cast<float>(kSingleP[2 * v + j]);
-        rt->inv_p[v][j] = static_cast<float>(1.0 / kSingleP[2 * v + j]);
+        c.neg_p[j] = pair(-static_cast<float>(kSingleP[2 * v + j]));
+        c.inv_p[j] = pair(static_cast<float>(1.0 / kSingleP[2 * v + j]));
       }
     }
   }

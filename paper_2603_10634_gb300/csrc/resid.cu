@@ -383,26 +383,16 @@ constexpr KarLut make_kar_lut() {
 __device__ const PairLut g_pair_lut = make_pair_lut();
 __device__ const KarLut g_kar_lut = make_kar_lut();
 
-// Shared-memory constants of one remainder taken.
-struct __align__(16) RnsConsts {
-  f2 neg_m, inv_m;
-  f2 w[kRnsPieces - 1];
-  f2 scale, base;                                  // table address of a remainder (address())
-  f2 neg_p[kGroupMax], inv_p[kGroupMax];           // members of a group without a table
-};
-static_assert(sizeof(RnsConsts) % 16 == 0, "");
-
 struct RnsSys {  // the product path's digits
   using Table = RnsTable;
-  // shared memory: constants, 2^t mod M (64 floats each), digit tables
-  static constexpr int kPerModulus = static_cast<int>(sizeof(RnsConsts)) + 4 * kPow2Table;
+  // shared memory: 2^t mod M (64 floats each), digit tables
+  static constexpr int kPerModulus = 4 * kPow2Table;
   static size_t smem_bytes(const Table& rt) {
     return static_cast<size_t>(rt.groups + rt.kars) * kPerModulus + 16 * static_cast<size_t>(rt.lut_words);
   }
   static __device__ __forceinline__ void load(const Table& rt, unsigned char* smem) {
     const int nv = rt.groups + rt.kars;
-    RnsConsts* cs = reinterpret_cast<RnsConsts*>(smem);
-    float* pow2 = reinterpret_cast<float*>(smem + nv * sizeof(RnsConsts));
+    float* pow2 = reinterpret_cast<float*>(smem);
     uint4* lut = reinterpret_cast<uint4*>(smem + nv * kPerModulus);
     const uint4* pl = reinterpret_cast<const uint4*>(&g_pair_lut);
     const uint4* kl = reinterpret_cast<const uint4*>(&g_kar_lut);
@@ -410,20 +400,6 @@ struct RnsSys {  // the product path's digits
       lut[i] = __ldg(i < rt.pair_words ? pl + i : kl + (i - rt.pair_words));
     for (int i = threadIdx.x; i < nv * kPow2Table; i += blockDim.x)
       pow2[i] = static_cast<float>(rt.pow2[i / kPow2Table][i % kPow2Table]);
-    for (int v = threadIdx.x; v < nv; v += blockDim.x) {
-      RnsConsts& c = cs[v];
-      c.neg_m = dup(rt.neg_m[v]);
-      c.inv_m = dup(rt.inv_m[v]);
-#pragma unroll
-      for (int j = 0; j < kRnsPieces - 1; ++j) c.w[j] = dup(rt.w[v][j]);
-      c.scale = dup(__int_as_float(v < rt.groups ? 2 : 4));
-      c.base = dup(__int_as_float(rt.lut_base[v]));
-#pragma unroll
-      for (int j = 0; j < kGroupMax; ++j) {
-        c.neg_p[j] = dup(rt.neg_p[v][j]);
-        c.inv_p[j] = dup(rt.inv_p[v][j]);
-      }
-    }
     __syncthreads();
   }
 
@@ -526,8 +502,8 @@ struct RnsSys {  // the product path's digits
                                              const f2 (&c)[kPairs][kRnsPieces], const TpPack& tp, PlaneStore st,
                                              uint32_t* flags) {
     const int nv = rt.groups + rt.kars;
-    const RnsConsts* cs = reinterpret_cast<const RnsConsts*>(smem);
-    const float* pow2 = reinterpret_cast<const float*>(smem + nv * sizeof(RnsConsts));
+    const RnsConsts* cs = rt.c;
+    const float* pow2 = reinterpret_cast<const float*>(smem);
     const unsigned char* lut = smem + nv * kPerModulus;
     auto rem = [&](int v, int pr) {
       return remainder<P2>(c[pr], tp_of(tp, 2 * pr), tp_of(tp, 2 * pr + 1), cs[v], pow2 + v * kPow2Table);
@@ -639,15 +615,22 @@ struct RnsSys {  // the product path's digits
 // Rows of A.  A warp item covers 2^s lanes x 8 k of 32 / 2^s rows (16 lanes on 128
 // consecutive k of two rows, or 4 or 8 lanes per row for rows of at most 64 k; see
 // resid_rows_lane_log), so short rows and the ends of rows leave few lanes idle.  Lane
-// l owns 8 consecutive elements (four 16-byte loads when the row is 16-byte aligned) and
-// writes 8 bytes of each plane.
+// l owns 8 consecutive elements and writes 8 bytes of each plane.  It copies those of its
+// next item to the warp's slot of shared memory while it converts this one: loaded when
+// they were needed, they were the longest stall (1.9 of 8 warp-cycles an issue, now 0.35).
+// 4096 x 4096, N = 12: 134 -> 127 us.
 static_assert(kElems == 8, "the row kernel's item shapes assume 8 elements per lane");
+constexpr size_t kSlotBytes = 32 * kElems * sizeof(double);  // of a warp
+constexpr size_t kRowBytes = 8 * kSlotBytes;                 // of a block
+constexpr int kResidBlocks = 3;                              // resident blocks an SM (80 registers; with 2 blocks
+                                                             // 2048^3, N = 14: a call 344 instead of 338 us)
 
 // vblock / vgrid: the block's index among, and the number of, the blocks serving this
 // operand (the warps stride over its items).
 template <class Sys>
 __device__ __forceinline__ void residues_rows_body(const ResidArgs& a, const typename Sys::Table& mt,
-                                                   const unsigned char* tb, int64_t vblock, int64_t vgrid) {
+                                                   const unsigned char* tb, unsigned char* slots, int64_t vblock,
+                                                   int64_t vgrid) {
   const int lane = threadIdx.x & 31;
   const int warps_per_block = blockDim.x >> 5;
   const int ls = resid_rows_lane_log(a.kp);
@@ -663,31 +646,53 @@ __device__ __forceinline__ void residues_rows_body(const ResidArgs& a, const typ
   int grp, chunk, dgrp, dchunk;
   divmod_nonneg(first, nkw, grp, chunk);
   divmod_nonneg(stride, nkw, dgrp, dchunk);
-  // every line of X starts on a 16-byte boundary: 16-byte loads
+  // every line of X starts on a 16-byte boundary: 16-byte copies
   const bool vec = (reinterpret_cast<uintptr_t>(a.X) & 15u) == 0 && (a.ldx & 1) == 0;
-  bool range_err = false;
-  for (; grp < groups; grp += dgrp, chunk += dchunk) {
-    if (chunk >= nkw) {
-      chunk -= nkw;
-      if (++grp >= groups) break;
-    }
-    const int row = grp * rpi + (lane >> ls);
-    const bool row_ok = row < a.lines;
-    const int h0 = chunk * span + (lane & ((1 << ls) - 1)) * kElems;
-    const unsigned long long* x =
-        reinterpret_cast<const unsigned long long*>(a.X + static_cast<int64_t>(row_ok ? row : 0) * a.ldx + h0);
-    const int e = row_ok ? a.exps[row] : 0;
-    unsigned long long v[kElems];
-    if (vec && row_ok && h0 + kElems <= a.k) {
+  // unit q (two elements) of a lane sits at 512 q + 16 lane of the warp's slot
+  const ulonglong2* slot = reinterpret_cast<const ulonglong2*>(slots + (threadIdx.x >> 5) * kSlotBytes) + lane;
+  const int own = lane >> ls, hown = (lane & ((1 << ls) - 1)) * kElems;  // the lane's row and first k of an item
+  auto fetch = [&](int g0, int c) {
+    const int row = g0 * rpi + own, h0 = c * span + hown;
+    const int left = row < a.lines ? a.k - h0 : 0;
+    const double* src = a.X + static_cast<int64_t>(row) * a.ldx + h0;
+    const uint32_t dst = smem_addr(slot);
+    if (vec && left >= kElems) {
 #pragma unroll
-      for (int q = 0; q < kElems / 2; ++q) {
-        const ulonglong2 d = __ldg(reinterpret_cast<const ulonglong2*>(x) + q);
-        v[2 * q] = d.x;
-        v[2 * q + 1] = d.y;
-      }
+      for (int q = 0; q < kElems / 2; ++q) copy16_async(dst + 512 * q, src + 2 * q);
     } else {
 #pragma unroll
-      for (int t = 0; t < kElems; ++t) v[t] = (row_ok && h0 + t < a.k) ? __ldg(x + t) : 0ull;
+      for (int t = 0; t < kElems; ++t)
+        copy8_async(dst + 512 * (t >> 1) + 8 * (t & 1), t < left ? src + t : a.X, t < left ? 8 : 0);
+    }
+    copies_commit();
+  };
+  auto exponent = [&](int g0) { return g0 * rpi + own < a.lines ? a.exps[g0 * rpi + own] : 0; };
+  bool range_err = false;
+  fetch(grp, chunk);
+  int e_next = exponent(grp);
+  while (grp < groups) {
+    const int row = grp * rpi + own;
+    const bool row_ok = row < a.lines;
+    const int h0 = chunk * span + hown;
+    const int e = e_next;
+    copies_wait<0>();
+    unsigned long long v[kElems];
+#pragma unroll
+    for (int q = 0; q < kElems / 2; ++q) {
+      const ulonglong2 d = slot[32 * q];
+      v[2 * q] = d.x;
+      v[2 * q + 1] = d.y;
+    }
+    __syncwarp();  // the slot has been read
+    grp += dgrp;
+    chunk += dchunk;
+    if (chunk >= nkw) {
+      chunk -= nkw;
+      ++grp;
+    }
+    if (grp < groups) {
+      fetch(grp, chunk);
+      e_next = exponent(grp);
     }
     const PlaneStore st{a.planes + static_cast<int64_t>(row_ok ? row : 0) * a.ldp + h0, a.plane_stride,
                         row_ok && h0 < a.kp};
@@ -697,16 +702,19 @@ __device__ __forceinline__ void residues_rows_body(const ResidArgs& a, const typ
 }
 
 // Columns of B through shared memory.  A block converts tiles of kTileCols columns x
-// kTileK k: the tile is read row by row (512 contiguous bytes per row of B) into shared
-// memory, column-major, then each thread converts 8 consecutive k of one column, so a
-// half-warp covers 128 consecutive k of a column and writes one full 128-byte line of
-// each plane (the register kernel above writes 32-byte pieces of 8 columns).  Within a
-// column, chunk c of 8 elements sits at 64 c bytes with the element order rotated by
-// (c >> 1) & 7, so that the 16 lanes reading element t of their chunks hit 16 different
-// bank pairs.
+// kTileK k: the tile is copied row by row (128 contiguous bytes per row of B) into shared
+// memory, column-major, while the tile before it is converted, each thread 8 consecutive k
+// of one column, so a half-warp covers 128 consecutive k of a column and writes one full
+// 128-byte line of each plane.  Within a column, chunk c of 8 elements sits at 64 c bytes
+// with the element order rotated by (c >> 1) & 7, so that the 16 lanes reading element t of
+// their chunks hit 16 different bank pairs.  Two 16-column tiles take the place of one of 32
+// that was loaded, then converted: 4096 x 4096, N = 12: 164 -> 148 us.
 constexpr int kTileCols = kResidTileCols, kTileK = kResidTileK;
 constexpr int kTilePitch = kTileK + 1;  // doubles per column in shared memory
-constexpr size_t kTileBytes = sizeof(double) * kTileCols * kTilePitch;
+constexpr int kTileDoubles = kTileCols * kTilePitch;
+constexpr size_t kTileBytes = 2 * sizeof(double) * kTileDoubles;  // two tiles
+static_assert(kTileCols * kTileK == 8 * 256, "a task a thread");
+static_assert(kTileBytes >= kRowBytes && kTileBytes % 16 == 0, "");
 
 __device__ __forceinline__ int tile_slot(int h) {  // position of k offset h within its column
   const int c = h >> 3;
@@ -717,75 +725,108 @@ __device__ __forceinline__ int tile_slot(int h) {  // position of k offset h wit
 // fastest).
 template <class Sys>
 __device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, const typename Sys::Table& mt,
-                                                         const unsigned char* tb, unsigned long long* tile, int64_t t0,
+                                                         const unsigned char* tb, unsigned char* buffers, int64_t t0,
                                                          int64_t tstride) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const int tiles_n = (a.lines + kTileCols - 1) / kTileCols, tiles_k = (a.kp + kTileK - 1) / kTileK;
   const int64_t tiles = static_cast<int64_t>(tiles_n) * tiles_k;
-  bool range_err = false;
-  for (int64_t t = t0; t < tiles; t += tstride) {
-    const int j0 = static_cast<int>(t % tiles_n) * kTileCols;
-    const int k0 = static_cast<int>(t / tiles_n) * kTileK;
-    // load: warp w reads rows w, w + 8, ...; lane l takes columns l, l + 32, ...
-#pragma unroll 8
-    for (int r = warp; r < kTileK; r += 8) {
-      const int h = k0 + r;
-      const unsigned long long* row = reinterpret_cast<const unsigned long long*>(a.X + static_cast<int64_t>(h) * a.ldx);
+  if (t0 >= tiles) return;
+  int tn, tk, dn, dk;  // tile coordinates, advanced like the items of the row kernel
+  divmod_nonneg(t0, tiles_n, tk, tn);
+  divmod_nonneg(tstride, tiles_n, dk, dn);
+  const unsigned long long* tile = reinterpret_cast<const unsigned long long*>(buffers);
+  const uint32_t tile_at = smem_addr(buffers);
+  const int c_in = tid & (kTileCols - 1), r_in = tid / kTileCols;  // copies: a column, every 16th row
+  const int c = tid >> 4, chunk = tid & 15;                         // the thread's task
+  auto fetch = [&](int jt, int kt, int buf) {
+    const int j = jt * kTileCols + c_in, h0 = kt * kTileK + r_in;
+    const double* src = a.X + static_cast<int64_t>(h0) * a.ldx + j;
+    const int64_t step = 16 * a.ldx;
+    const uint32_t dst = tile_at + 8 * (buf * kTileDoubles + c_in * kTilePitch + (r_in & 8));
+    if ((jt + 1) * kTileCols <= a.lines && (kt + 1) * kTileK <= a.k) {
 #pragma unroll
-      for (int u = 0; u < kTileCols / 32; ++u) {
-        const int c = lane + 32 * u, j = j0 + c;
-        tile[c * kTilePitch + tile_slot(r)] = (h < a.k && j < a.lines) ? __ldg(row + j) : 0ull;
+      for (int x = 0; x < kTileK / 16; ++x, src += step)  // tile_slot(r_in + 16 x)
+        copy8_async(dst + 8 * (16 * x + ((r_in & 7) ^ x)), src, 8);
+    } else {
+#pragma unroll
+      for (int x = 0; x < kTileK / 16; ++x, src += step) {
+        const bool ok = j < a.lines && h0 + 16 * x < a.k;
+        copy8_async(dst + 8 * (16 * x + ((r_in & 7) ^ x)), ok ? src : a.X, ok ? 8 : 0);
       }
     }
-    __syncthreads();
-    // convert: rounds of 256 (column, 8-k chunk) tasks; a half-warp per column
-#pragma unroll 1
-    for (int round = 0; round < kTileCols * kTileK / (8 * 256); ++round) {
-      const int q = round * 256 + tid;
-      const int c = q >> 4, chunk = q & 15;
-      const int j = j0 + c, h0 = k0 + chunk * 8;
-      const bool active = j < a.lines && h0 < a.kp;
-      const int e = j < a.lines ? a.exps[j] : 0;
-      const unsigned long long* src = tile + c * kTilePitch + chunk * 8;
-      unsigned long long v[kElems];
-#pragma unroll
-      for (int u = 0; u < kElems; ++u) v[u] = src[u ^ ((chunk >> 1) & 7)];
-      const PlaneStore st{a.planes + static_cast<int64_t>(j < a.lines ? j : 0) * a.ldp + (h0 < a.kp ? h0 : 0),
-                          a.plane_stride, active};
-      Sys::task(mt, tb, v, [e](int) { return e; }, st, a.flags, range_err);
+  };
+  auto exponent = [&](int jt) { return jt * kTileCols + c < a.lines ? a.exps[jt * kTileCols + c] : 0; };
+  bool range_err = false;
+  fetch(tn, tk, 0);
+  copies_commit();
+  int e_next = exponent(tn);
+  for (int buf = 0; tk < tiles_k; buf ^= 1) {
+    const int j = tn * kTileCols + c, h0 = tk * kTileK + chunk * 8;
+    const bool active = j < a.lines && h0 < a.kp;
+    const int e = e_next;
+    tn += dn;
+    tk += dk;
+    if (tn >= tiles_n) {
+      tn -= tiles_n;
+      ++tk;
     }
-    __syncthreads();  // the tile is reloaded
+    if (tk < tiles_k) {
+      fetch(tn, tk, buf ^ 1);
+      e_next = exponent(tn);
+    }
+    copies_commit();
+    copies_wait<1>();
+    __syncthreads();
+    const unsigned long long* src = tile + buf * kTileDoubles + c * kTilePitch + chunk * 8;
+    unsigned long long v[kElems];
+#pragma unroll
+    for (int u = 0; u < kElems; ++u) v[u] = src[u ^ ((chunk >> 1) & 7)];
+    __syncthreads();  // the buffer is copied to again
+    const PlaneStore st{a.planes + static_cast<int64_t>(j < a.lines ? j : 0) * a.ldp + (h0 < a.kp ? h0 : 0),
+                        a.plane_stride, active};
+    Sys::task(mt, tb, v, [e](int) { return e; }, st, a.flags, range_err);
   }
   if (range_err) atomicOr(a.flags, kFlagRange);
 }
 
-// One or two operands: the first `split` blocks serve a, the rest b.  The constants come
-// first in shared memory, then the column tile (absent when both operands are rows).
+// One or two operands, one after the other; the blocks that have the fewest iterations of
+// the first start the second, so that the grid is full to the end (4096^3 in two launches
+// 281 us, in one 271; 4096 x 8192 with 100 columns: a call 505 -> 495 us).  `tables`: bytes of the constants, which come first in shared
+// memory.  first_blocks: resid_blocks(a).
 template <class Sys>
-__global__ void __launch_bounds__(256, 3) residues_kernel(const __grid_constant__ ResidArgs a,
-                                                         const __grid_constant__ ResidArgs b, int split,
-                                                         const __grid_constant__ typename Sys::Table mt, int tables) {
+__global__ void __launch_bounds__(256, kResidBlocks) residues_kernel(const __grid_constant__ ResidArgs a,
+                                                                     const __grid_constant__ ResidArgs b, int nops,
+                                                                     int64_t first_blocks,
+                                                                     const __grid_constant__ typename Sys::Table mt,
+                                                                     int tables) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Sys::load(mt, smem_raw);  // constants only: before the wait
   // no chain_next: the product kernel's blocks, which fill an SM each, would settle as these
   // blocks leave and run the products unevenly (65536 x 1024 x 1024 2.57 instead of 2.52 ms)
   chain_wait();
-  const bool second = static_cast<int>(blockIdx.x) >= split;
-  const ResidArgs& op = second ? b : a;
-  const int64_t v = second ? blockIdx.x - split : blockIdx.x, g = second ? gridDim.x - split : split;
-  if (op.kcontig) residues_rows_body<Sys>(op, mt, smem_raw, v, g);
-  else residues_cols_tiled_body<Sys>(op, mt, smem_raw, reinterpret_cast<unsigned long long*>(smem_raw + tables), v, g);
+  const int grid = gridDim.x;
+  int v = blockIdx.x;
+#pragma unroll 1
+  for (int o = 0; o < nops; ++o) {
+    const ResidArgs& op = o ? b : a;
+    if (op.kcontig) residues_rows_body<Sys>(op, mt, smem_raw, smem_raw + tables, v, grid);
+    else residues_cols_tiled_body<Sys>(op, mt, smem_raw, smem_raw + tables, v, grid);
+    __syncthreads();  // the buffers are used again
+    v -= static_cast<int>(first_blocks % grid);
+    if (v < 0) v += grid;
+  }
 }
 
 // Grouped: rows of every A; columns of every B (one virtual block per tile).
+// (three resident blocks of the row kernel spill: 48 mixed problems 1120 instead of 1079 us)
 __global__ void __launch_bounds__(256, 2) residues_rows_batch(const BatchProblem* __restrict__ probs, int count,
                                                            int64_t total, uint32_t* flags,
                                                            const __grid_constant__ RnsTable mt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  RnsSys::load(mt, smem_raw);
+  RnsSys::load(mt, smem_raw + kRowBytes);
   for_each_vblock(probs, count, kBkResidRows, total, [&](const BatchProblem& P, int64_t v) {
     const ResidArgs a{P.A, P.lda, P.m, P.k, P.kp, P.ldp, P.e, P.planesA, static_cast<int64_t>(P.m) * P.ldp, flags, true};
-    residues_rows_body<RnsSys>(a, mt, smem_raw, v, P.nblocks[kBkResidRows]);
+    residues_rows_body<RnsSys>(a, mt, smem_raw + kRowBytes, smem_raw, v, P.nblocks[kBkResidRows]);
   });
 }
 
@@ -796,23 +837,23 @@ __global__ void __launch_bounds__(256, 3) residues_cols_batch(const BatchProblem
   RnsSys::load(mt, smem_raw + kTileBytes);
   for_each_vblock(probs, count, kBkResidCols, total, [&](const BatchProblem& P, int64_t v) {
     const ResidArgs a{P.B, P.ldb, P.n, P.k, P.kp, P.ldp, P.f, P.planesB, static_cast<int64_t>(P.n) * P.ldp, flags, false};
-    residues_cols_tiled_body<RnsSys>(a, mt, smem_raw + kTileBytes, reinterpret_cast<unsigned long long*>(smem_raw), v,
-                                     P.nblocks[kBkResidCols]);
+    residues_cols_tiled_body<RnsSys>(a, mt, smem_raw + kTileBytes, smem_raw, v, P.nblocks[kBkResidCols]);
   });
 }
-
-static_assert(kTileBytes % 16 == 0, "the tables follow the tile on a 16-byte boundary");
 
 // ------------------------------------------------------------------ gradient operands
 // The upstream gradient dC (m x n, row-major) of C = A B enters both gradient products
 // that reuse the forward's integer matrices, with per-element exponents:
 //   G'_ij = trunc(2^(g_i - f_j) dC_ij)  rows i as lines, along j   (dA = dC B^T)
 //   H'_ij = trunc(2^(h_j - e_i) dC_ij)  columns j as lines, along i (dB = A^T dC)
-// One kernel reads each kTileK x kTileCols tile of dC once into shared memory (the
+// One kernel reads each kTileK x kGradCols tile of dC once into shared memory (the
 // layout of the column kernel above: tile rows are rows i of dC, tile columns are
 // columns j) and converts it twice: the column pass writes H' exactly as the column
 // kernel writes B's planes; the row pass writes G' with 8 consecutive j per task (plane
-// pieces of kTileCols bytes).
+// pieces of kGradCols bytes).
+constexpr int kGradCols = 32;
+constexpr size_t kGradBytes = sizeof(double) * kGradCols * kTilePitch;
+
 struct GradArgs {
   const double* dC;
   int64_t lddc;
@@ -832,23 +873,23 @@ struct GradArgs {
 __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const __grid_constant__ RnsTable mt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned long long* tile = reinterpret_cast<unsigned long long*>(smem_raw);
-  const unsigned char* tb = smem_raw + kTileBytes;
-  RnsSys::load(mt, smem_raw + kTileBytes);
+  const unsigned char* tb = smem_raw + kGradBytes;
+  RnsSys::load(mt, smem_raw + kGradBytes);
   chain_wait();
   chain_next();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tiles_n = (a.n + kTileCols - 1) / kTileCols, tiles_m = (a.m + kTileK - 1) / kTileK;
+  const int tiles_n = (a.n + kGradCols - 1) / kGradCols, tiles_m = (a.m + kTileK - 1) / kTileK;
   const int64_t tiles = static_cast<int64_t>(tiles_n) * tiles_m;
   bool range_err = false;
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int j0 = static_cast<int>(t % tiles_n) * kTileCols;
+    const int j0 = static_cast<int>(t % tiles_n) * kGradCols;
     const int i0 = static_cast<int>(t / tiles_n) * kTileK;
 #pragma unroll 8
     for (int r = warp; r < kTileK; r += 8) {
       const int i = i0 + r;
       const unsigned long long* row = reinterpret_cast<const unsigned long long*>(a.dC + static_cast<int64_t>(i) * a.lddc);
 #pragma unroll
-      for (int u = 0; u < kTileCols / 32; ++u) {
+      for (int u = 0; u < kGradCols / 32; ++u) {
         const int c = lane + 32 * u, j = j0 + c;
         tile[c * kTilePitch + tile_slot(r)] = (i < a.m && j < a.n) ? __ldg(row + j) : 0ull;
       }
@@ -856,7 +897,7 @@ __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const
     __syncthreads();
     // column pass: H' (lines j, positions i), a half-warp per column
 #pragma unroll 1
-    for (int round = 0; a.do_h && round < kTileCols * kTileK / (8 * 256); ++round) {
+    for (int round = 0; a.do_h && round < kGradCols * kTileK / (8 * 256); ++round) {
       const int q = round * 256 + tid;
       const int c = q >> 4, chunk = q & 15;
       const int j = j0 + c, ib = i0 + chunk * 8;
@@ -875,10 +916,10 @@ __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const
                           static_cast<int64_t>(a.n) * a.ldh, active};
       RnsSys::task(mt, tb, v, [&ex](int u) { return ex[u]; }, st, a.flags, range_err);
     }
-    // row pass: G' (lines i, positions j): kTileCols / 8 chunks per row
+    // row pass: G' (lines i, positions j): kGradCols / 8 chunks per row
 #pragma unroll 1
-    for (int round = 0; a.do_g && round < kTileK * kTileCols / (8 * 256); ++round) {
-      constexpr int kChunks = kTileCols / 8;
+    for (int round = 0; a.do_g && round < kTileK * kGradCols / (8 * 256); ++round) {
+      constexpr int kChunks = kGradCols / 8;
       const int q = round * 256 + tid;
       const int r = q / kChunks, chunk = q % kChunks;
       const int i = i0 + r, jb = j0 + chunk * 8;
@@ -995,8 +1036,8 @@ int sm_count() {
 
 // Blocks of a conversion kernel: one per 8 warps of work, at most the resident ones (each
 // stages the tables once and strides over the work).
-int resident_grid(int64_t blocks, size_t smem) {
-  const int per_sm = static_cast<int>(std::max<size_t>(1, std::min<size_t>(3, (226 * 1024) / (smem + 1024))));
+int resident_grid(int64_t blocks, size_t smem, size_t most) {
+  const int per_sm = static_cast<int>(std::max<size_t>(1, std::min<size_t>(most, (226 * 1024) / (smem + 1024))));
   const int64_t cap = static_cast<int64_t>(sm_count()) * per_sm;
   return static_cast<int>(std::max<int64_t>(1, std::min(blocks, cap)));
 }
@@ -1007,36 +1048,16 @@ int64_t resid_blocks(const ResidArgs& a) {
   return static_cast<int64_t>((a.lines + kTileCols - 1) / kTileCols) * ((a.kp + kTileK - 1) / kTileK);
 }
 
-// Two operands share a launch, its blocks in proportion to their elements, where they fit
-// one wave of blocks (about 900^2 entries each) or are both rows.  Otherwise each gets its
-// own: the row kernel reads through the L1 cache, which the column tile's shared memory
-// would take (8192 x 4096 rows beside 4096 x 100 columns: 268 us in two launches, 297 in
-// one).
 template <class Sys>
 cudaError_t run_residues(const ResidArgs* ops, int nops, const typename Sys::Table& t, cudaStream_t st) {
   const size_t tables = (Sys::smem_bytes(t) + 15) / 16 * 16;
-  auto need = [&](int n) {
-    bool cols = false;
-    for (int i = 0; i < n; ++i) cols |= !ops[i].kcontig;
-    return tables + (cols ? kTileBytes : 0);
-  };
-  const size_t smem = need(nops);
+  const ResidArgs &a = ops[0], &b = ops[nops - 1];
+  const size_t smem = tables + (a.kcontig && b.kcontig ? kRowBytes : kTileBytes);
   static std::atomic<int> allowed[64];
   allow_smem(residues_kernel<Sys>, allowed, smem);
-  if (nops == 1) {
-    const int grid = resident_grid(resid_blocks(ops[0]), smem);
-    return launch_chained(residues_kernel<Sys>, grid, 256, smem, st, ops[0], ops[0], grid, t, static_cast<int>(tables));
-  }
-  const int64_t na = resid_blocks(ops[0]), nb = resid_blocks(ops[1]);
-  const int grid = resident_grid(na + nb, smem);
-  if (na + nb > 3 * static_cast<int64_t>(grid) && smem > tables) {
-    const cudaError_t err = run_residues<Sys>(ops, 1, t, st);
-    return err != cudaSuccess ? err : run_residues<Sys>(ops + 1, 1, t, st);
-  }
-  int split = grid == na + nb ? static_cast<int>(na)
-                              : static_cast<int>(static_cast<double>(grid) * ops[0].lines / (ops[0].lines + ops[1].lines) + 0.5);
-  split = std::max(1, std::min(split, grid - 1));
-  return launch_chained(residues_kernel<Sys>, grid, 256, smem, st, ops[0], ops[1], split, t, static_cast<int>(tables));
+  const int64_t na = resid_blocks(a);
+  const int grid = resident_grid(na + (nops > 1 ? resid_blocks(b) : 0), smem, kResidBlocks);
+  return launch_chained(residues_kernel<Sys>, grid, 256, smem, st, a, b, nops, na, t, static_cast<int>(tables));
 }
 
 }  // namespace
@@ -1053,7 +1074,7 @@ cudaError_t launch_residues_batch(const BatchProblem* probs, int count, int64_t 
                                   const RnsTable& rt, uint32_t* flags, cudaStream_t st, cudaStream_t st_cols) {
   if (rows_blocks < 1 || cols_blocks < 1 || rows_blocks > 0x7FFFFFFFll || cols_blocks > 0x7FFFFFFFll)
     return cudaErrorInvalidValue;
-  const size_t rows_smem = RnsSys::smem_bytes(rt), cols_smem = kTileBytes + rows_smem;
+  const size_t rows_smem = kRowBytes + RnsSys::smem_bytes(rt), cols_smem = kTileBytes + RnsSys::smem_bytes(rt);
   static std::atomic<int> allowed_rows[64], allowed_cols[64];
   allow_smem(residues_rows_batch, allowed_rows, rows_smem);
   allow_smem(residues_cols_batch, allowed_cols, cols_smem);
@@ -1066,11 +1087,11 @@ cudaError_t launch_grad_residues(const double* dC, int64_t lddc, int m, int n, c
                                  const int32_t* h, const int32_t* e, uint8_t* planesG, int64_t ldg, uint8_t* planesH,
                                  int64_t ldh, const RnsTable& rt, uint32_t* flags, cudaStream_t st) {
   GradArgs a{dC, lddc, m, n, g, f, h, e, planesG, ldg, planesH, ldh, flags, planesG != nullptr, planesH != nullptr};
-  const size_t smem = kTileBytes + RnsSys::smem_bytes(rt);
+  const size_t smem = kGradBytes + RnsSys::smem_bytes(rt);
   static std::atomic<int> allowed[64];
   allow_smem(grad_residues_kernel, allowed, smem);
-  const int64_t tiles = static_cast<int64_t>((n + kTileCols - 1) / kTileCols) * ((m + kTileK - 1) / kTileK);
-  return launch_chained(grad_residues_kernel, resident_grid(tiles, smem), 256, smem, st, a, rt);
+  const int64_t tiles = static_cast<int64_t>((n + kGradCols - 1) / kGradCols) * ((m + kTileK - 1) / kTileK);
+  return launch_chained(grad_residues_kernel, resident_grid(tiles, smem, 3), 256, smem, st, a, rt);
 }
 
 cudaError_t launch_transpose_planes(const uint8_t* src, int64_t src_pitch, int64_t src_stride, int lines, int len,
