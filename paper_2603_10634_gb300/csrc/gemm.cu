@@ -110,6 +110,8 @@ struct GemmParams {
   int m, n, k;
   UnitGrid grid;
   int num_units;
+  int kar_units;   // single problems: units of the Karatsuba moduli, which come first
+  int kar_rest;    // kar_units mod the CTAs (pairs) of the launch
   int16_t* cres;   // 16-bit residues (Karatsuba moduli; all of the paper mode)
   int8_t* cres8;   // 8-bit residues (single moduli)
   int64_t ldr;
@@ -165,6 +167,43 @@ struct UnitCtx {
   float factor;
   float* R;
   float* S;
+};
+
+// The units of one CTA (pair) i of G: i, i + G, ...  In a single problem with Karatsuba
+// moduli those come first and take three passes each, so after their last, incomplete round
+// of `rest` units the CTAs without one take three single units each before all go on in
+// turn.  Without that, CTAs had up to two passes more than the others: 1023 x 777 x 1501
+// with N = 14 8 passes instead of 7 (a call 139.0 -> 136.1 us), 4096^3 92 instead of 91
+// (1556 -> 1541 us), 300 x 700 x 500 52.5 -> 49.7 us.
+template <bool GROUPED>
+struct UnitWalk {
+  int u, first, step, catch_up;
+  __device__ __forceinline__ UnitWalk(int i, int G) : u(i), first(i), step(G), catch_up(-1) {}
+  __device__ __forceinline__ void start(const GemmParams& P) {
+    if (!GROUPED && P.kar_rest > 0 && u >= P.kar_units) catch_up = 2;
+  }
+  __device__ __forceinline__ void next(const GemmParams& P) {
+    if (GROUPED || P.kar_rest == 0) {
+      u += step;
+    } else if (u < P.kar_units) {
+      u += step;
+      if (u < P.kar_units) return;
+      if (first >= P.kar_rest) {  // u - step was in the last full round
+        u = P.kar_units + first - P.kar_rest;
+        catch_up = 2;
+      } else {
+        u = P.kar_units + 3 * (step - P.kar_rest) + first;
+      }
+    } else if (catch_up > 0) {
+      --catch_up;
+      u += step - P.kar_rest;
+    } else if (catch_up == 0) {
+      catch_up = -1;
+      u = P.kar_units + 3 * (step - P.kar_rest) + first;
+    } else {
+      u += step;
+    }
+  }
 };
 
 template <bool GROUPED>
@@ -423,9 +462,10 @@ __device__ __forceinline__ float2 unpark2(uint32_t w) {
 // padded to 16 columns, so the store stays inside the row.  The debug build checks that
 // every residue lies in [-h - 1, p - h] (paper mode: the symmetric range [-h, p - 1 - h]).
 template <bool EXACT>
-__device__ __forceinline__ void store_residues8(int16_t* dst, int gc, uint32_t (&pk)[4], bool accumulate, int p, int h,
+__device__ __forceinline__ void store_residues8(int16_t* dst, int gc, uint4 x4, bool accumulate, int p, int h,
                                                 uint32_t* flags) {
   uint4* out = reinterpret_cast<uint4*>(dst + gc);
+  uint32_t pk[4] = {x4.x, x4.y, x4.z, x4.w};
   if (accumulate) {
     const uint4 prev = *out;
     const uint32_t pw[4] = {prev.x, prev.y, prev.z, prev.w};
@@ -487,9 +527,7 @@ __device__ __forceinline__ void store_residues16(int8_t* dst, int gc, uint4 x4, 
 // 4 x 4 transpose of 16-byte items over groups of four lanes: lane i's item j comes from
 // lane j's item i.  Rows held one to a lane become 64-byte pieces of a row over four lanes,
 // so that a warp's store covers whole sectors of 8 rows instead of half sectors of 32
-// (16384 x 16384 x 512 residue products of a pair: 3.56 -> 2.83 ms).  The 16-bit planes keep
-// their row pieces: the items held over the pass cost more than the sectors gained (2.83 ->
-// 3.27 ms with them transposed too).
+// (16384 x 16384 x 512 residue products of a pair: 3.56 -> 2.83 ms).
 __device__ __forceinline__ uint4 shfl_xor4(uint4 v, int mask) {
   return make_uint4(__shfl_xor_sync(0xffffffffu, v.x, mask), __shfl_xor_sync(0xffffffffu, v.y, mask),
                     __shfl_xor_sync(0xffffffffu, v.z, mask), __shfl_xor_sync(0xffffffffu, v.w, mask));
@@ -506,6 +544,19 @@ __device__ __forceinline__ void transpose4(uint4 (&x)[4], int lane) {
       else x[j | b] = got;
     }
   }
+}
+
+// The same for pairs of lanes and the 16-bit residues: a row's 16 columns of a chunk fill one
+// sector of a store instead of two halves (2.83 -> 2.76 ms; calls 1024^3 94.9 -> 91.9 us,
+// 65536 x 1024 x 1024 2339 -> 2317, 4100 x 4100 x 1030 906 -> 856 with N = 16; 1023 x 777 x
+// 1501 with N = 14, the one slower of 15 shapes, 135.4 -> 138.2).  Wider pieces (four lanes, 32 columns) hold more over
+// the chunks and spill (3.27 ms); grouped launches (48 mixed problems 1084 -> 1090 us)
+// have nothing to gain.
+__device__ __forceinline__ void transpose2(uint4 (&x)[2], int lane) {
+  const bool up = (lane & 1) != 0;
+  const uint4 got = shfl_xor4(up ? x[0] : x[1], 1);
+  if (up) x[0] = got;
+  else x[1] = got;
 }
 
 // Four exact-integer floats |r| < 2^7 as four int8 of one word, in order (the low bytes
@@ -544,8 +595,9 @@ __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
   const int lane = threadIdx.x & 31;
   const uint32_t rank = PAIR ? cluster_rank() : 0u;
   const bool leader = rank == 0u;
-  const int u_first = static_cast<int>(blockIdx.x) / G;
   const int u_step = static_cast<int>(gridDim.x) / G;
+  UnitWalk<GROUPED> walk(static_cast<int>(blockIdx.x) / G, u_step);
+  walk.start(prm);
   const unsigned long long wait_ns = prm.wait_ns;
 
   if (threadIdx.x == 0) {
@@ -587,8 +639,8 @@ __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
       int last_prob = -1;
       UnitCtx uc;
       Pace pace(PAIR && leader ? prm.pace : nullptr);
-      for (int u = u_first; ok && u < prm.num_units; u += u_step) {
-        resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
+      for (UnitWalk<GROUPED> w = walk; ok && w.u < prm.num_units; w.next(prm)) {
+        resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, w.u, uc);
         if (GROUPED && uc.prob != last_prob) {
           if (elect_one()) {
             tensormap_acquire(uc.ta);
@@ -670,8 +722,8 @@ __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
       // so this wait runs out and the kernel takes its timeout path
       bool ok = prm.stall ? warp_wait(never, 0u, abort_flag, wait_ns) : true;
       UnitCtx uc;
-      for (int u = u_first; ok && u < prm.num_units; u += u_step) {
-        resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
+      for (UnitWalk<GROUPED> w = walk; ok && w.u < prm.num_units; w.next(prm)) {
+        resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, w.u, uc);
         const int mod = uc.mod;
         const UnitPlan up = plan_of<MODE>(prm, uc.k, mod);
         for (int c = 0; ok && c < up.nchunks; ++c) {
@@ -738,8 +790,8 @@ __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
     Slots sl;  // the MMA thread's pass sequence, replayed
     bool ok = true;
     UnitCtx uc;
-    for (int u = u_first; ok && u < prm.num_units; u += u_step) {
-      resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, u, uc);
+    for (UnitWalk<GROUPED> w = walk; ok && w.u < prm.num_units; w.next(prm)) {
+      resolve_unit<GROUPED>(prm, &tmA, &tmB, probs, nprobs, w.u, uc);
       const int mod = uc.mod, tn = uc.tn;
       const UnitPlan up = plan_of<MODE>(prm, uc.k, mod);
       const int gi = (uc.tm * G + static_cast<int>(rank)) * BM + row;
@@ -814,6 +866,8 @@ __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
               }
             } else {
               int16_t* dst = uc.cres + static_cast<int64_t>(mod) * uc.res_stride + off;
+              constexpr bool kSwap = TN == 256 && !GROUPED;
+              uint4 px[2];  // this row's 16 columns, then two rows' 8 columns
               const bool square = MODE == kModePaper && mod < kNumSquares;
               const bool last = ps == up.npasses - 1;
               const float c1 = gm.c1, c2 = gm.c2, c3 = gm.c3;
@@ -861,8 +915,22 @@ __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
                       if (square) pk[z] = pack2(smod2(__ffma2_rn(dup2(c1), unpark2(pr[z]), d), mp));
                       else pk[z] = pack2(mod_near2(__ffma2_rn(dup2(c3), mod_near2(d, mp), unpark2(pr[z])), mp));
                     }
-                    const int gc = gc0 + cb * kCW + 8 * w;
-                    if (keep_row && gc < uc.n) store_residues8<MODE == kModePaper>(dst, gc, pk, c > 0, p, h, prm.flags);
+                    if constexpr (kSwap) {
+                      px[w & 1] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                      if (w & 1) {
+                        transpose2(px, lane);
+                        const int odd = lane & 1, gc = gc0 + cb * kCW + 8 * (w - 1 + odd), gr = gi - odd;
+#pragma unroll
+                        for (int x = 0; x < 2; ++x)
+                          if (gr + x < uc.m && gc < uc.n)
+                            store_residues8<MODE == kModePaper>(dst + (x - odd) * uc.ldr, gc, px[x], c > 0, p, h, prm.flags);
+                      }
+                    } else {
+                      const int gc = gc0 + cb * kCW + 8 * w;
+                      if (keep_row && gc < uc.n)
+                        store_residues8<MODE == kModePaper>(dst, gc, make_uint4(pk[0], pk[1], pk[2], pk[3]), c > 0, p, h,
+                                                            prm.flags);
+                    }
                   }
                 }
               }
@@ -1062,6 +1130,10 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
     return cudaErrorInvalidValue;
   const int ctas = g.num_sms < kMaxGemmCtas ? g.num_sms : kMaxGemmCtas;
   const int grid = pair ? 2 * std::min(prm.num_units, ctas / 2) : std::min(prm.num_units, ctas);
+  if (g.mode == kModeResidue) {
+    prm.kar_units = prm.grid.tiles * prm.mods.kars;
+    prm.kar_rest = prm.kar_units % (pair ? grid / 2 : grid);
+  }
   switch (g.mode) {
     case kModeResidue:
       return pair ? launch_mode<kModeResidue, false, 256, true>(prm, ta, tb, grid, nullptr, 0, st)
