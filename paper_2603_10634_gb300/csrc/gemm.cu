@@ -811,6 +811,13 @@ __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
               mbar_arrive(tempty + slot);
             }
           };
+          // no entry of the matrix in this warp's rows and columns (48 mixed problems, whose
+          // tiles are 35% padding: 1082 -> 1071 us)
+          if (gi - lane >= uc.m || tn * BN + cgrp * kCols >= uc.n) {
+            release();
+            ++sl.t;
+            continue;
+          }
           if constexpr (kResidues) {
             const GemmMod& gm = prm.mods.m[mod];
             const int p = gm.p, h = gm.half;
