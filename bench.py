@@ -528,7 +528,7 @@ def run_ours(a, rank, world):
 def run_autograd(a, rank, world):
     """Forward + backward of the differentiable product: C = A B, then dA = W B^T and
     dB = A^T W for the upstream gradient W; three emulated products per step.  The
-    default backward reuses the forward's exponents and digit planes (one conversion of
+    default backward reuses the forward's exponents and integer matrices (one conversion of
     W for both gradients); the same step with fresh emulations of both gradients is
     timed beside it, and sampled entries of dA and dB of both are compared with the
     exact products next to native FP64."""
@@ -614,7 +614,7 @@ def run_autograd(a, rank, world):
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f8e4m3", "emulates": "f64",
             "data": "synthetic",
             "config": {"workload": f"autograd A {m}x{k} @ B {k}x{n}, W ~ N(0,1), phi={a.phi}, N={N}, {a.mode} mode, "
-                                   f"backward reusing the forward's exponents and digit planes",
+                                   f"backward reusing the forward's exponents and integer matrices",
                        "l2": "operands larger than L2, no flush"},
             "gpu_launches": launches * a.steps, "clocks": clk.summary(), "device_status": status,
             "gradient_error_vs_absAB": err_reuse,

@@ -412,7 +412,8 @@ int ozk2_debug_timeline(float *ms, int max);
  * g and h take the whole budget of P (Eq. condition: 2 sum |G'||B'| < P) from FP8 bound
  * products of |dC| with |B| and of |A| with |dC| (as accurate mode, Sec. III-E), so
  * as many FP8 products run per gradient as in a fresh emulation, but A and B are not
- * converted again (their planes are transposed), and one kernel converts dC for both.
+ * scaled again (their lines of the gradients are converted with the forward's exponents), and
+ * one kernel converts dC for both.
  *   forward_workspace  device memory of the current device, the workspace of the
  *                      ozk2_dgemm_ws / ozk2_dgemm_ex call (accurate mode, no blocking,
  *                      same m, n, k, num_moduli) that computed C = A B, unchanged since

@@ -2,10 +2,10 @@
 
 C = A B runs through the emulated DGEMM.  The backward pass needs two more products,
 dA = dC B^T and dB = A^T dC.  By default (``reuse=True``) they run through
-ozk2_dgemm_backward, which reuses the forward call's scaling exponents and digit planes
+ozk2_dgemm_backward, which reuses the forward call's scaling exponents and integer matrices
 of A' = trunc(diag(2^e) A) and B' = trunc(B diag(2^f)): the forward runs in a workspace
-kept in the autograd context, only dC is scaled and converted (once, for both
-gradients), and dC's exponents take the whole budget of P that A' and B' leave.  With
+kept in the autograd context, only dC is scaled, one conversion
+of it serves both gradients, and dC's exponents take the whole budget of P that A' and B' leave.  With
 ``reuse=False``, or where reuse does not apply (fast mode, operands that are transposed
 views), each gradient is an independent emulation with its own scaling (Sec. III-E) of
 operands read in place.
@@ -47,7 +47,7 @@ class OzakiMatmul(torch.autograd.Function):
             m, k = A.shape
             n = B.shape[1]
             ws = torch.empty(max(1, ozk2.workspace_size(m, n, k, num_moduli)), dtype=torch.uint8, device=A.device)
-            ctx.forward_workspace = ws  # the forward's exponents and digit planes, read by backward
+            ctx.forward_workspace = ws  # holds the forward's exponents, read by backward
             return ozk2.dgemm(A, B, num_moduli=num_moduli, workspace=ws)
         return ozk2.dgemm(_operand(A), _operand(B), num_moduli=num_moduli, mode=mode)
 

@@ -896,7 +896,8 @@ size_t host_workspace_bytes(int64_t m, int64_t n, int64_t k, int N, bool fast) {
 // The exponents g, h of dC's side come from FP8 bound products of |dC| with |B| (rows of
 // B as lines) and of |A| (columns as lines) with |dC|, whose maxima remove the lines'
 // own FP8 scalings (colshift / rowshift), under the budget Q = log2(P - 1) - 1 (B' and A'
-// are fixed).  The forward's planes are transposed into the layout the products read.
+// are fixed).  A' and B' are converted again, with the forward's exponents, into the layout
+// the products read.
 struct BwLayout {
   int64_t np, mp, ldrk, ldrn;
   int planes;
@@ -1028,10 +1029,7 @@ ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64
   const uint8_t* f8 = static_cast<const uint8_t*>(fws);
   const int32_t* e = reinterpret_cast<const int32_t*>(f8 + FL.e);
   const int32_t* f = reinterpret_cast<const int32_t*>(f8 + FL.f);
-  const uint8_t* planesA = f8 + FL.planesA;
-  const uint8_t* planesB = f8 + FL.planesB;
   uint32_t* flags = reinterpret_cast<uint32_t*>(at(L.flags));
-  const int P = rns_planes(N);
   int32_t* gp = reinterpret_cast<int32_t*>(at(L.gp));
   int32_t* hp = reinterpret_cast<int32_t*>(at(L.hp));
   int32_t* g = reinterpret_cast<int32_t*>(at(L.g));
@@ -1074,27 +1072,33 @@ ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64
                                   wantB ? c.n : 0, hp, at(L.cstatC), reinterpret_cast<float*>(at(L.S)), h,
                                   reuse_budget_f32(N), at(L.rstatB), wantA ? c.k : 0, at(L.cstatA), wantB ? c.k : 0,
                                   flags, st));
-  // dC's two integer matrices from one read of dC; the forward's planes transposed
+  // dC's two integer matrices from one read of dC; then the lines of A'^T and B'^T, which run
+  // across the forward's (their range flag, if any, was the forward's to report: its word
+  // here is a spare one)
   OZK2_TRY(launch_grad_residues(dC, lddc, c.m, c.n, g, f, h, e, wantA ? at(L.planesG) : nullptr, L.np,
                                 wantB ? at(L.planesH) : nullptr, L.mp, c.tab->rt, flags, st));
-  t_launches += 2;
+  const int np = int(L.np), mp = int(L.mp);
+  const ResidArgs bt{B, ldb, c.k, c.n, np, L.np, f, at(L.planesBT), int64_t(k) * L.np, flags + 1, true};
+  const ResidArgs at_{A, lda, c.k, c.m, mp, L.mp, e, at(L.planesAT), int64_t(k) * L.mp, flags + 1, false};
+  ResidArgs across[2];
+  int nacross = 0;
+  if (wantA) across[nacross++] = bt;
+  if (wantB) across[nacross++] = at_;
+  if (nacross) OZK2_TRY(launch_residues_across(across, nacross, c.tab->rt, st));
+  t_launches += 3;
   if (wantA) {
-    OZK2_TRY(launch_transpose_planes(planesB, FL.ldp, int64_t(n) * FL.ldp, c.n, c.k, at(L.planesBT), L.np,
-                                     int64_t(k) * L.np, P, st));
     OZK2_TRY(bw_products(c, at(L.planesG), at(L.planesBT), L.np, c.m, c.k, c.n, at(L.cresA), at(L.cresA8), L.ldrk,
                          flags));
     OZK2_TRY(launch_crt(reinterpret_cast<int16_t*>(at(L.cresA)), reinterpret_cast<int8_t*>(at(L.cresA8)), L.ldrk,
                         int64_t(m) * L.ldrk, c.m, c.k, g, zk, at(L.rstatC), at(L.rstatB), dA, ldda, c.tab->rc, st));
-    t_launches += 2;
+    t_launches += 1;
   }
   if (wantB) {
-    OZK2_TRY(launch_transpose_planes(planesA, FL.ldp, int64_t(m) * FL.ldp, c.m, c.k, at(L.planesAT), L.mp,
-                                     int64_t(k) * L.mp, P, st));
     OZK2_TRY(bw_products(c, at(L.planesAT), at(L.planesH), L.mp, c.k, c.n, c.m, at(L.cresB), at(L.cresB8), L.ldrn,
                          flags));
     OZK2_TRY(launch_crt(reinterpret_cast<int16_t*>(at(L.cresB)), reinterpret_cast<int8_t*>(at(L.cresB8)), L.ldrn,
                         int64_t(k) * L.ldrn, c.k, c.n, zk, h, at(L.cstatA), at(L.cstatC), dB, lddb, c.tab->rc, st));
-    t_launches += 2;
+    t_launches += 1;
   }
   return OZK2_OK;
 }

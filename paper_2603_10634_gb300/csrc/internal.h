@@ -238,6 +238,9 @@ struct ResidArgs {
 };
 // The planes of one or two operands.
 cudaError_t launch_residues(const ResidArgs* ops, int nops, const RnsTable& rt, cudaStream_t st);
+// The same with an exponent per position along k (exps[h] of the k entries of every line)
+// instead of one per line: the gradients' operands, whose lines run across the forward's.
+cudaError_t launch_residues_across(const ResidArgs* ops, int nops, const RnsTable& rt, cudaStream_t st);
 // The hybrid list's digit planes (parity hooks), packed.
 cudaError_t launch_paper_planes(const ResidArgs* ops /* two */, const ModTable& mt, cudaStream_t st);
 
@@ -247,11 +250,6 @@ cudaError_t launch_paper_planes(const ResidArgs* ops /* two */, const ModTable& 
 cudaError_t launch_grad_residues(const double* dC, int64_t lddc, int m, int n, const int32_t* g, const int32_t* f,
                                  const int32_t* h, const int32_t* e, uint8_t* planesG, int64_t ldg, uint8_t* planesH,
                                  int64_t ldh, const RnsTable& rt, uint32_t* flags, cudaStream_t st);
-// dst[p][x][y] = src[p][y][x], y < lines, x < len (pitches and strides multiples of 16;
-// src_pitch >= len and dst_pitch >= lines, both rounded up to 16).
-cudaError_t launch_transpose_planes(const uint8_t* src, int64_t src_pitch, int64_t src_stride, int lines, int len,
-                                    uint8_t* dst, int64_t dst_pitch, int64_t dst_stride, int planes, cudaStream_t st);
-
 // gemm.cu
 // Division by an invariant (numerators below 2^31).
 struct FastDiv {

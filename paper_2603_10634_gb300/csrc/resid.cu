@@ -625,9 +625,34 @@ constexpr size_t kRowBytes = 8 * kSlotBytes;                 // of a block
 constexpr int kResidBlocks = 3;                              // resident blocks an SM (80 registers; with 2 blocks
                                                              // 2048^3, N = 14: a call 344 instead of 338 us)
 
+// Exponents of the 8 positions from h on (a multiple of 8; the array is padded to 256 bytes).
+__device__ __forceinline__ void position_exponents(const ResidArgs& a, int h, int (&ex)[kElems]) {
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int4 x = h < a.k ? __ldg(reinterpret_cast<const int4*>(a.exps + h) + q) : make_int4(0, 0, 0, 0);
+    ex[4 * q] = x.x;
+    ex[4 * q + 1] = x.y;
+    ex[4 * q + 2] = x.z;
+    ex[4 * q + 3] = x.w;
+  }
+}
+// A task whose exponents are the line's (e) or, ACROSS, the positions'.
+template <class Sys, bool ACROSS>
+__device__ __forceinline__ void convert_task(const ResidArgs& a, const typename Sys::Table& mt, const unsigned char* tb,
+                                             const unsigned long long (&v)[kElems], int e, int h, const PlaneStore& st,
+                                             bool& range_err) {
+  if constexpr (ACROSS) {
+    int ex[kElems];
+    position_exponents(a, h, ex);
+    Sys::task(mt, tb, v, [&ex](int u) { return ex[u]; }, st, a.flags, range_err);
+  } else {
+    Sys::task(mt, tb, v, [e](int) { return e; }, st, a.flags, range_err);
+  }
+}
+
 // vblock / vgrid: the block's index among, and the number of, the blocks serving this
 // operand (the warps stride over its items).
-template <class Sys>
+template <class Sys, bool ACROSS = false>
 __device__ __forceinline__ void residues_rows_body(const ResidArgs& a, const typename Sys::Table& mt,
                                                    const unsigned char* tb, unsigned char* slots, int64_t vblock,
                                                    int64_t vgrid) {
@@ -666,7 +691,7 @@ __device__ __forceinline__ void residues_rows_body(const ResidArgs& a, const typ
     }
     copies_commit();
   };
-  auto exponent = [&](int g0) { return g0 * rpi + own < a.lines ? a.exps[g0 * rpi + own] : 0; };
+  auto exponent = [&](int g0) { return !ACROSS && g0 * rpi + own < a.lines ? a.exps[g0 * rpi + own] : 0; };
   bool range_err = false;
   fetch(grp, chunk);
   int e_next = exponent(grp);
@@ -696,7 +721,7 @@ __device__ __forceinline__ void residues_rows_body(const ResidArgs& a, const typ
     }
     const PlaneStore st{a.planes + static_cast<int64_t>(row_ok ? row : 0) * a.ldp + h0, a.plane_stride,
                         row_ok && h0 < a.kp};
-    Sys::task(mt, tb, v, [e](int) { return e; }, st, a.flags, range_err);
+    convert_task<Sys, ACROSS>(a, mt, tb, v, e, h0, st, range_err);
   }
   if (range_err) atomicOr(a.flags, kFlagRange);
 }
@@ -723,7 +748,7 @@ __device__ __forceinline__ int tile_slot(int h) {  // position of k offset h wit
 
 // Tiles t0, t0 + tstride, ... of the operand (tiles numbered with the column tile
 // fastest).
-template <class Sys>
+template <class Sys, bool ACROSS = false>
 __device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, const typename Sys::Table& mt,
                                                          const unsigned char* tb, unsigned char* buffers, int64_t t0,
                                                          int64_t tstride) {
@@ -755,7 +780,7 @@ __device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, con
       }
     }
   };
-  auto exponent = [&](int jt) { return jt * kTileCols + c < a.lines ? a.exps[jt * kTileCols + c] : 0; };
+  auto exponent = [&](int jt) { return !ACROSS && jt * kTileCols + c < a.lines ? a.exps[jt * kTileCols + c] : 0; };
   bool range_err = false;
   fetch(tn, tk, 0);
   copies_commit();
@@ -784,7 +809,7 @@ __device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, con
     __syncthreads();  // the buffer is copied to again
     const PlaneStore st{a.planes + static_cast<int64_t>(j < a.lines ? j : 0) * a.ldp + (h0 < a.kp ? h0 : 0),
                         a.plane_stride, active};
-    Sys::task(mt, tb, v, [e](int) { return e; }, st, a.flags, range_err);
+    convert_task<Sys, ACROSS>(a, mt, tb, v, e, h0, st, range_err);
   }
   if (range_err) atomicOr(a.flags, kFlagRange);
 }
@@ -793,7 +818,7 @@ __device__ __forceinline__ void residues_cols_tiled_body(const ResidArgs& a, con
 // the first start the second, so that the grid is full to the end (4096^3 in two launches
 // 281 us, in one 271; 4096 x 8192 with 100 columns: a call 505 -> 495 us).  `tables`: bytes of the constants, which come first in shared
 // memory.  first_blocks: resid_blocks(a).
-template <class Sys>
+template <class Sys, bool ACROSS>
 __global__ void __launch_bounds__(256, kResidBlocks) residues_kernel(const __grid_constant__ ResidArgs a,
                                                                      const __grid_constant__ ResidArgs b, int nops,
                                                                      int64_t first_blocks,
@@ -809,8 +834,8 @@ __global__ void __launch_bounds__(256, kResidBlocks) residues_kernel(const __gri
 #pragma unroll 1
   for (int o = 0; o < nops; ++o) {
     const ResidArgs& op = o ? b : a;
-    if (op.kcontig) residues_rows_body<Sys>(op, mt, smem_raw, smem_raw + tables, v, grid);
-    else residues_cols_tiled_body<Sys>(op, mt, smem_raw, smem_raw + tables, v, grid);
+    if (op.kcontig) residues_rows_body<Sys, ACROSS>(op, mt, smem_raw, smem_raw + tables, v, grid);
+    else residues_cols_tiled_body<Sys, ACROSS>(op, mt, smem_raw, smem_raw + tables, v, grid);
     __syncthreads();  // the buffers are used again
     v -= static_cast<int>(first_blocks % grid);
     if (v < 0) v += grid;
@@ -942,76 +967,6 @@ __global__ void __launch_bounds__(256, 3) grad_residues_kernel(GradArgs a, const
   if (range_err) atomicOr(a.flags, kFlagRange);
 }
 
-// dst[p][x][y] = src[p][y][x] for y < lines, x < len: the digit planes of an operand
-// (lines x len bytes, K-major) as the planes of its transpose.  A block moves 128 x 128
-// byte tiles through shared memory (row pitch 33 words: the words a warp reads along a
-// column fall in 32 different banks); each thread then reads a 16 x 4 byte block (16
-// rows, 4 columns) as 16 words, transposes it four 4 x 4 blocks at a time with byte
-// permutes, and writes 4 destination rows of 16 bytes.
-constexpr int kTrTile = 128, kTrPitchW = 33;
-
-// 4 x 4 byte block: in[r] holds bytes (r, 0..3); out[c] gets bytes (0..3, c).
-__device__ __forceinline__ void transpose4x4(const uint32_t (&in)[4], uint32_t (&out)[4]) {
-  const uint32_t t0 = __byte_perm(in[0], in[1], 0x5140), t1 = __byte_perm(in[0], in[1], 0x7362);
-  const uint32_t t2 = __byte_perm(in[2], in[3], 0x5140), t3 = __byte_perm(in[2], in[3], 0x7362);
-  out[0] = __byte_perm(t0, t2, 0x5410);
-  out[1] = __byte_perm(t0, t2, 0x7632);
-  out[2] = __byte_perm(t1, t3, 0x5410);
-  out[3] = __byte_perm(t1, t3, 0x7632);
-}
-
-__global__ void __launch_bounds__(256) transpose_planes_kernel(const uint8_t* __restrict__ src, int64_t src_pitch,
-                                                               int64_t src_stride, int lines, int len,
-                                                               uint8_t* __restrict__ dst, int64_t dst_pitch,
-                                                               int64_t dst_stride, int planes) {
-  __shared__ uint32_t tile[kTrTile * kTrPitchW];
-  chain_wait();
-  chain_next();
-  const int tx = (len + kTrTile - 1) / kTrTile, ty = (lines + kTrTile - 1) / kTrTile;
-  const int64_t total = static_cast<int64_t>(tx) * ty * planes;
-  const int t = threadIdx.x;
-  for (int64_t b = blockIdx.x; b < total; b += gridDim.x) {
-    const int p = static_cast<int>(b / (static_cast<int64_t>(tx) * ty));
-    const int rem = static_cast<int>(b - static_cast<int64_t>(p) * tx * ty);
-    const int y0 = (rem / tx) * kTrTile, x0 = (rem % tx) * kTrTile;
-    // load: 128 rows of 128 bytes, 16 bytes per thread and round (inside the source pitch)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = q * 32 + (t >> 3), c16 = (t & 7) * 16;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (y0 + r < lines && x0 + c16 < len)
-        v = *reinterpret_cast<const uint4*>(src + p * src_stride + static_cast<int64_t>(y0 + r) * src_pitch + x0 +
-                                            c16);
-      uint32_t* tw = tile + r * kTrPitchW + c16 / 4;
-      tw[0] = v.x;
-      tw[1] = v.y;
-      tw[2] = v.z;
-      tw[3] = v.w;
-    }
-    __syncthreads();
-    // store: destination rows x0 + 4 cw .. + 3, bytes y0 + 16 yb .. + 15
-    const int cw = t & 31, yb = t >> 5;
-    uint32_t out[4][4];  // out[c][w]: destination row 4 cw + c, word w (4 y's)
-#pragma unroll
-    for (int w = 0; w < 4; ++w) {
-      uint32_t in[4], o[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) in[r] = tile[(16 * yb + 4 * w + r) * kTrPitchW + cw];
-      transpose4x4(in, o);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) out[c][w] = o[c];
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int x = x0 + 4 * cw + c, y = y0 + 16 * yb;
-      if (x < len && y < lines)
-        *reinterpret_cast<uint4*>(dst + p * dst_stride + static_cast<int64_t>(x) * dst_pitch + y) =
-            make_uint4(out[c][0], out[c][1], out[c][2], out[c][3]);
-    }
-    __syncthreads();
-  }
-}
-
 // Opt a kernel into `bytes` of dynamic shared memory, raised when a later call needs more
 // (per device; a launch on a device where this failed reports the error itself).
 template <class K>
@@ -1048,22 +1003,29 @@ int64_t resid_blocks(const ResidArgs& a) {
   return static_cast<int64_t>((a.lines + kTileCols - 1) / kTileCols) * ((a.kp + kTileK - 1) / kTileK);
 }
 
-template <class Sys>
+template <class Sys, bool ACROSS = false>
 cudaError_t run_residues(const ResidArgs* ops, int nops, const typename Sys::Table& t, cudaStream_t st) {
   const size_t tables = (Sys::smem_bytes(t) + 15) / 16 * 16;
   const ResidArgs &a = ops[0], &b = ops[nops - 1];
   const size_t smem = tables + (a.kcontig && b.kcontig ? kRowBytes : kTileBytes);
   static std::atomic<int> allowed[64];
-  allow_smem(residues_kernel<Sys>, allowed, smem);
+  allow_smem(residues_kernel<Sys, ACROSS>, allowed, smem);
   const int64_t na = resid_blocks(a);
   const int grid = resident_grid(na + (nops > 1 ? resid_blocks(b) : 0), smem, kResidBlocks);
-  return launch_chained(residues_kernel<Sys>, grid, 256, smem, st, a, b, nops, na, t, static_cast<int>(tables));
+  return launch_chained(residues_kernel<Sys, ACROSS>, grid, 256, smem, st, a, b, nops, na, t, static_cast<int>(tables));
 }
 
 }  // namespace
 
 cudaError_t launch_residues(const ResidArgs* ops, int nops, const RnsTable& rt, cudaStream_t st) {
   return run_residues<RnsSys>(ops, nops, rt, st);
+}
+
+// Converting A and B again takes less than transposing the forward's planes: 8 bytes read and
+// 27 written an element (N = 12) instead of 27 and 27 (forward and both gradients of 8192 x
+// 4096 by 4096 x 4096: 8.90 -> 8.63 ms).
+cudaError_t launch_residues_across(const ResidArgs* ops, int nops, const RnsTable& rt, cudaStream_t st) {
+  return run_residues<RnsSys, true>(ops, nops, rt, st);
 }
 
 cudaError_t launch_paper_planes(const ResidArgs* ops, const ModTable& mt, cudaStream_t st) {
@@ -1092,20 +1054,6 @@ cudaError_t launch_grad_residues(const double* dC, int64_t lddc, int m, int n, c
   allow_smem(grad_residues_kernel, allowed, smem);
   const int64_t tiles = static_cast<int64_t>((n + kGradCols - 1) / kGradCols) * ((m + kTileK - 1) / kTileK);
   return launch_chained(grad_residues_kernel, resident_grid(tiles, smem, 3), 256, smem, st, a, rt);
-}
-
-cudaError_t launch_transpose_planes(const uint8_t* src, int64_t src_pitch, int64_t src_stride, int lines, int len,
-                                    uint8_t* dst, int64_t dst_pitch, int64_t dst_stride, int planes, cudaStream_t st) {
-  if ((src_pitch % 16) || (dst_pitch % 16) || (src_stride % 16) || (dst_stride % 16) || lines < 1 || len < 1 ||
-      planes < 1 || src_pitch < ((len + 15) / 16) * 16 || dst_pitch < ((lines + 15) / 16) * 16)
-    return cudaErrorInvalidValue;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t total = static_cast<int64_t>((len + kTrTile - 1) / kTrTile) * ((lines + kTrTile - 1) / kTrTile) * planes;
-  const int grid = static_cast<int>(std::min<int64_t>(total, 8 * static_cast<int64_t>(sms)));
-  return launch_chained(transpose_planes_kernel, grid, 256, 0, st, src, src_pitch, src_stride, lines, len, dst, dst_pitch,
-                        dst_stride, planes);
 }
 
 }  // namespace ozk2

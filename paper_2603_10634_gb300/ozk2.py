@@ -167,7 +167,7 @@ def workspace_size_backward(m, n, k, num_moduli=12):
 def dgemm_backward(A, B, dC, forward_workspace, num_moduli=12, need_dA=True, need_dB=True, workspace=None):
     """(dA, dB) = (dC @ B.T, A.T @ dC) for C = A @ B computed by ``dgemm(A, B, num_moduli,
     workspace=forward_workspace)`` (accurate mode, no blocking), reusing that call's
-    exponents and digit planes (ozk2_dgemm_backward).  A, B, dC: row-major float64 CUDA
+    exponents and integer matrices (ozk2_dgemm_backward).  A, B, dC: row-major float64 CUDA
     tensors; forward_workspace: the uint8 tensor the forward ran in, unchanged since.
     An output not needed is returned as None."""
     for x, name in ((A, "A"), (B, "B"), (dC, "dC")):
