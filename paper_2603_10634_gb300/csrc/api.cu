@@ -117,9 +117,25 @@ int tile_rule(int64_t padded256, int64_t padded128) { return 4 * padded256 >= 5 
 // results never depended on it.
 std::atomic<int64_t> g_split_kmax{0};
 
-int tile_for(int64_t n) {
-  const int t = g_tile_n.load();
-  return t ? t : tile_rule(padded(n, 256), padded(n, 128));
+// The tile of a single problem's product (g without its tile).  Residue and bound products
+// take the narrow one also where it keeps more SMs busy: its passes take about 0.72 of a
+// wide one's time (0.62 to 0.82 measured), so it pays while the CTA with the most of them has
+// less than 25 / 18 as many.  Narrow / wide, us: calls 256^3 34.9 / 36.9, 1024^3 (bound
+// product only) 90.6 / 92.3, 512 x 512 x 8192 197.7 / 216.4, 300 x 700 x 5000 151.8 / 157.2;
+// on the other side of the line 640 x 512 x 4096 with N = 14 158.4 / 155.2, 768 x 768 x 4096
+// 175.8 / 162.3.
+int tile_for(const GemmArgs& g) {
+  if (const int t = g_tile_n.load()) return t;
+  const int64_t n256 = padded(g.n, 256), n128 = padded(g.n, 128);
+  if (g.mode == kModeResidue || g.mode == kModeBound) {
+    const bool residue = g.mode == kModeResidue;
+    const int64_t passes = residue ? g.mods->planes : 1, longest = residue && g.mods->kars > 0 ? 3 : 1;
+    auto rounds = [&](int64_t tiles_n) {
+      return std::max<int64_t>(longest, (passes * ((g.m + 127) / 128) * tiles_n + g.num_sms - 1) / g.num_sms);
+    };
+    if (18 * rounds(n128 / 128) < 25 * rounds(n256 / 256)) return 128;
+  }
+  return tile_rule(n256, n128);
 }
 
 // ------------------------------------------------------------------ workspace checks
@@ -423,7 +439,7 @@ cudaError_t bound_rows(Ctx& c, int64_t i0, int rows) {
   g.R = c.at<float>(L.R) + i0;
   g.S = c.at<float>(L.S);
   g.flags = c.at<uint32_t>(L.flags);
-  g.tile_n = tile_for(c.n);
+  g.tile_n = tile_for(g);
   if (!launch_controls(g)) return cudaErrorLaunchFailure;
   t_launches += 1;
   return launch_fp8_gemm(g, c.at<uint8_t>(L.Abar) + i0 * L.kp, L.kp, 1, c.at<uint8_t>(L.BbarT), L.kp, 1, c.st);
@@ -500,7 +516,7 @@ ozk2_status products_rows(Ctx& c, int64_t i0, int rows, cudaStream_t st, int mod
   g.flags = c.at<uint32_t>(L.flags);
   g.plane_stride_a = int64_t(c.m) * L.ldp;
   g.plane_stride_b = int64_t(c.n) * L.ldp;
-  g.tile_n = tile_for(c.n);
+  g.tile_n = tile_for(g);
   if (!launch_controls(g)) return OZK2_ERR_CUDA;
   OZK2_TRY(launch_fp8_gemm(g, c.at<uint8_t>(L.planesA) + i0 * L.ldp, L.ldp, g.mods->planes,
                            c.at<uint8_t>(L.planesB), L.ldp, g.mods->planes, st));
@@ -967,7 +983,7 @@ cudaError_t bw_bound(const Ctx& c, const uint8_t* a, const uint8_t* b, int64_t p
   g.colshift = colshift;
   g.rowshift = rowshift;
   g.flags = flags;
-  g.tile_n = tile_for(cols);
+  g.tile_n = tile_for(g);
   if (!launch_controls(g)) return cudaErrorLaunchFailure;
   t_launches += 1;
   return launch_fp8_gemm(g, a, pitch, 1, b, pitch, 1, c.st);
@@ -991,7 +1007,7 @@ cudaError_t bw_products(const Ctx& c, const uint8_t* a, const uint8_t* b, int64_
   g.flags = flags;
   g.plane_stride_a = int64_t(rows) * pitch;
   g.plane_stride_b = int64_t(cols) * pitch;
-  g.tile_n = tile_for(cols);
+  g.tile_n = tile_for(g);
   if (!launch_controls(g)) return cudaErrorLaunchFailure;
   t_launches += 1;
   return launch_fp8_gemm(g, a, pitch, g.mods->planes, b, pitch, g.mods->planes, c.st);
@@ -1830,7 +1846,7 @@ ozk2_status ozk2_debug_fp8_gemm(int64_t m, int64_t n, int64_t k, const uint8_t* 
   uint8_t* ws = owned_workspace(256, &err);  // flag word only
   if (!ws) return err;
   g.flags = reinterpret_cast<uint32_t*>(ws);
-  g.tile_n = tile_for(n);
+  g.tile_n = tile_for(g);
   if (!launch_controls(g)) return OZK2_ERR_CUDA;
   OZK2_TRY(launch_fp8_gemm(g, A8, lda8, 1, B8, ldb8, 1, st));
   return OZK2_OK;
