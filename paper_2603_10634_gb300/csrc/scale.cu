@@ -206,21 +206,24 @@ __device__ __forceinline__ void scale_rows_cached(const double* __restrict__ A, 
 // One warp per row of A: row maximum, e'_i, row status, then Abar (m x kp bytes).
 // FAST: instead of Abar, the sum of squares s_i = sum_h RU_fp32(2^e'_i |a_ih|)^2 with
 // every addition rounded up (an upper bound of ||2^e'_i a_i||_2^2), written to sq[row].
-// vblock: the block's index among the blocks of this problem (8 rows each).
-template <bool FAST>
+// vblock: the block's index among the blocks of this problem (8 rows each).  W = 8: the
+// block's warps share a row (not FAST, whose sums keep a warp's order).
+template <bool FAST, int W = 1>
 __device__ __forceinline__ void scale_rows_body(const double* __restrict__ A, int64_t lda, int m, int k, int kp,
                                                 int32_t* __restrict__ eprime, uint8_t* __restrict__ rowstat,
                                                 uint8_t* __restrict__ Abar, float* __restrict__ sq,
-                                                int64_t vblock) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int row = static_cast<int>(vblock) * (blockDim.x >> 5) + warp;
+                                                int64_t vblock, uint32_t* red = nullptr) {
+  static_assert(W == 1 || (W == 8 && !FAST), "");
+  constexpr int T = 32 * W;  // threads of a row
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & (T - 1);
+  const int row = W == 8 ? static_cast<int>(vblock) : static_cast<int>(vblock) * (blockDim.x >> 5) + warp;
   if (row >= m) return;
   const double* a = A + static_cast<int64_t>(row) * lda;
   LineMax lm;
-  for (int h = lane; h < k; h += 32 * kBatch) {
+  for (int h = lane; h < k; h += T * kBatch) {
     double v[kBatch];  // the loads of a batch are issued before any is used
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) v[u] = h + 32 * u < k ? __ldg(a + h + 32 * u) : 0.0;
+    for (int u = 0; u < kBatch; ++u) v[u] = h + T * u < k ? __ldg(a + h + T * u) : 0.0;
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) lm.add(v[u]);
   }
@@ -228,10 +231,19 @@ __device__ __forceinline__ void scale_rows_body(const double* __restrict__ A, in
   bool bad = false;
   if (!lm.exact()) {
     key = 0u;
-    for (int h = lane; h < k; h += 32) key = max(key, log2_key(mag_of(__ldg(a + h)), bad));
+    for (int h = lane; h < k; h += T) key = max(key, log2_key(mag_of(__ldg(a + h)), bad));
   }
   key = __reduce_max_sync(0xffffffffu, key);
   bad = __any_sync(0xffffffffu, bad);
+  if constexpr (W == 8) {
+    red[threadIdx.x] = key | (bad ? kKeyBad : 0u);
+    __syncthreads();
+    key = red[0];
+#pragma unroll
+    for (int w = 1; w < W; ++w) key = merge_keys(key, red[32 * w]);
+    bad = (key & kKeyBad) != 0u;
+    key &= ~kKeyBad;
+  }
   const int ep = prelim_exponent(key);
   if (lane == 0) {
     eprime[row] = ep;
@@ -252,17 +264,17 @@ __device__ __forceinline__ void scale_rows_body(const double* __restrict__ A, in
     if (lane == 0) sq[row] = acc;
   } else {
     uint8_t* out = Abar + static_cast<int64_t>(row) * kp;
-    for (int h0 = lane * 4; h0 < kp; h0 += 256) {
-      double v[8];  // two words of 4 bytes, 128 bytes apart; loads first
+    for (int h0 = lane * 4; h0 < kp; h0 += 8 * T) {
+      double v[8];  // two words of 4 bytes, 4 T bytes apart; loads first
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
-        const int h = h0 + (t >> 2) * 128 + (t & 3);
+        const int h = h0 + (t >> 2) * 4 * T + (t & 3);
         v[t] = h < k ? __ldg(a + h) : 0.0;
       }
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
         const double q[4] = {v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]};
-        if (h0 + 128 * g < kp) *reinterpret_cast<uint32_t*>(out + h0 + 128 * g) = bar_word(q, ep);
+        if (h0 + 4 * T * g < kp) *reinterpret_cast<uint32_t*>(out + h0 + 4 * T * g) = bar_word(q, ep);
       }
     }
   }
@@ -355,7 +367,7 @@ __global__ void __launch_bounds__(256) scale_prep_kernel(const __grid_constant__
   const int64_t vblock = blockIdx.x - a.first[blockIdx.x >= a.first[1] ? 1 : 0];
   if (!job.kcontig) colmax_tile(job.X, job.ld, a.k, job.lines, a.key_rows, job.keys, red, vblock);
   else if constexpr (E == 0)
-    scale_rows_body<FAST>(job.X, job.ld, job.lines, a.k, a.kp, job.ep, job.stat, job.bar, job.sq, vblock);
+    scale_rows_body<FAST, W>(job.X, job.ld, job.lines, a.k, a.kp, job.ep, job.stat, job.bar, job.sq, vblock, red);
   else
     scale_rows_cached<E, W>(job.X, job.ld, job.lines, a.k, a.kp, job.ep, job.stat, job.bar, red, vblock);
 }
@@ -672,7 +684,10 @@ cudaError_t run_prep(const ScaleJob* jobs, int njobs, int k, int kp, uint32_t* z
 // thread (32 above 4096, in a launch of their own: its registers would halve the column
 // kernel's occupancy); against a warp per row that reads twice, 8192 x 4096 88 -> 51 us and
 // 65536 x 1024 128 -> 93 us (5.8 TB/s).  Longer rows (two blocks' worth would not fit an SM's registers)
-// and fast mode (its sums keep their order) read twice.
+// are read twice by a block each: a warp each left most of the chip idle when they are few
+// (calls 64 x 64 x 65536 1031 -> 664 us, 256 x 256 x 65536 1406 -> 923, 3000 x 200 x 20000
+// 1477 -> 1393; 4096 rows of 65536 are as fast either way).  Fast mode (its sums keep a warp's
+// order) reads twice by warps.  More than 16 partial keys a column gain nothing.
 cudaError_t launch_scale_prep(const ScaleJob* jobs, int njobs, int k, int kp, bool fast, uint32_t* zero,
                               int64_t zero_words, cudaStream_t st) {
   if (fast) return run_prep<true, 0, 1>(jobs, njobs, k, kp, zero, zero_words, st);
@@ -680,7 +695,7 @@ cudaError_t launch_scale_prep(const ScaleJob* jobs, int njobs, int k, int kp, bo
   if (kp <= 1024) return run_prep<false, 16, 2>(jobs, njobs, k, kp, zero, zero_words, st);
   if (kp <= 2048) return run_prep<false, 16, 4>(jobs, njobs, k, kp, zero, zero_words, st);
   if (kp <= 4096) return run_prep<false, 16, 8>(jobs, njobs, k, kp, zero, zero_words, st);
-  if (kp > 8192) return run_prep<false, 0, 1>(jobs, njobs, k, kp, zero, zero_words, st);
+  if (kp > 8192) return run_prep<false, 0, 8>(jobs, njobs, k, kp, zero, zero_words, st);
   for (int kc = 1; kc >= 0; --kc) {
     ScaleJob part[2];
     int n = 0;
