@@ -10,6 +10,13 @@ from paper_2603_10634_gb300 import _lib
 pytestmark = pytest.mark.gpu
 
 
+@pytest.fixture(autouse=True)
+def wide_tiles(cuda):
+    """Pairs run 256-wide tiles; the smaller shapes here would take the narrow ones."""
+    with ozk.tile_width(256):
+        yield
+
+
 def _integers(rows, cols, seed, device):
     g = torch.Generator(device=device).manual_seed(seed)
     return torch.randint(-1000, 1001, (rows, cols), generator=g, device=device).double()
