@@ -1059,11 +1059,14 @@ cudaError_t launch_tile(int tn, const GemmParams& prm, const CUtensorMap& ta, co
 constexpr int64_t kPaceBytes = int64_t(64) << 20;
 constexpr int kPaceWord = 32;  // offset of the pacing words in the zeroed 256-byte flag region
 
-// CTA pairs for the residue products of single problems in 256-wide tiles.  Their launch takes about 2 us longer
-// (clusters, the barriers between the CTAs) and their products 10-13% less time, so they
-// pay from about 16 us of products on: `rounds` (units per CTA, in passes) x k-steps of at
-// least 56 (single / pair: 512 x 512 x 4096 55 / 49 us, 1024^3 35 / 35, 768^3 27 / 29, 2048^3
-// 160 / 141, 4096^3 1067 / 956, 16384^3 70.9 / 64.5 ms).  A pair's tile is 256 rows high: not
+// CTA pairs for the residue products of single problems in 256-wide tiles.  Their products take
+// 10-13% less time, but their launch some 6 us more (clusters, the barriers between the CTAs),
+// and their 8 epilogue warps cannot hide the epilogue behind passes of three k-steps or
+// fewer: measured, a call gains about 0.12 us for each of `rounds` (units per CTA, in passes) x
+// (k-steps - 3), so they pay from 54 of these on.  Single / pairs, us: 1024^3 91.8 / 96.6, 1024
+// x 1024 x 1536 112.4 / 112.2, x 2048 133.8 / 127.9; 2048 x 2048 x 512 148 / 156, x 768 177 /
+// 172; 4096 x 4096 x 256 384 / 392, x 1024 586 / 527; 16384 x 16384 x 256 5182 / 5209, x 512
+// 5479 / 5394; products of 16384^3 70.9 / 64.5 ms.  A pair's tile is 256 rows high: not
 // where that pads the rows by over a third (384 x 4096 x 4096 145 / 137 us, 128 x 8192 x 4096
 // 160 / 166).  The bound product gains nothing (4096^3 55 / 55 us; at 16384^3 0.2 ms, which
 // the power cap takes back from the residue products).
@@ -1072,7 +1075,7 @@ bool use_pairs(const GemmArgs& g, int BN) {
   const int64_t rows1 = (g.m + BM - 1) / BM, rows2 = (g.m + 2 * BM - 1) / (2 * BM);
   if (6 * rows2 > 4 * rows1) return false;
   const int64_t rounds = (g.mods->planes * rows1 * ((g.n + BN - 1) / BN) + g.num_sms - 1) / g.num_sms;
-  return rounds * ((g.k + BK - 1) / BK) >= 56;
+  return rounds * ((g.k + BK - 1) / BK - 3) >= 54;
 }
 
 // Reciprocal of d for numerators below 2^31: floor(n / d) = (n mul >> 32) >> shift.
