@@ -362,15 +362,18 @@ cudaError_t copy_2d(void* dst, size_t dpitch, const void* src, size_t spitch, si
 }
 
 // ------------------------------------------------------------------ phases
-// Words a call's first scaling launch zeroes: the bound maxima and, with clear_flags (the
-// first block of a call; later blocks keep what earlier blocks recorded), the flag region.
+// Words a call's first scaling launch zeroes: the bound maxima (accurate mode) and, with
+// clear_flags (the first block of a call; later blocks keep what earlier blocks recorded),
+// the flag region.  Fast mode's R and S are left alone: they are sums that the scaling
+// launches store whole, some of them in the launch that does the zeroing, where nothing
+// orders the two.
 struct ZeroWords {
   uint32_t* at = nullptr;
   int64_t words = 0;
 };
 ZeroWords zero_words(const Ctx& c, bool clear_flags) {
-  const size_t from = clear_flags ? c.L.flags : c.L.R;
-  return ZeroWords{c.at<uint32_t>(from), int64_t(c.L.zero_end - from) / 4};
+  const size_t from = clear_flags ? c.L.flags : c.L.R, to = c.fast ? c.L.R : c.L.zero_end;
+  return ZeroWords{c.at<uint32_t>(from), int64_t(to - from) / 4};
 }
 
 // Which operand a scaling launch serves.

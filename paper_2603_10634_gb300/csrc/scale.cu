@@ -347,7 +347,8 @@ __device__ __forceinline__ void colmax_tile(const double* __restrict__ B, int64_
 }
 
 // The first launch of a scaling: rows of operands that are contiguous along k, partial
-// column maxima of the others, and the call's zeroed words.
+// column maxima of the others, and the call's zeroed words (which none of its blocks writes
+// otherwise: the blocks are not ordered).
 struct PrepArgs {
   ScaleJob job[2];
   int64_t first[3];  // blocks [first[i], first[i + 1]) serve job i
