@@ -87,8 +87,9 @@ __device__ __forceinline__ uint32_t bar_code(double x, int ep) {
   const Mag m = mag_of(x);
   const uint32_t up = (m.hi + 0x1FFFFu + (m.lo != 0u ? 1u : 0u)) >> 17;
   const uint32_t code = up + static_cast<uint32_t>(8 * (ep - 1016));
-  // a normal x (not zero, not subnormal) with a result of 2^-6 .. 2^8 (so x is finite)
-  if (code - 8u <= 0x70u && m.hi >= 0x00100000u) return code;
+  // a normal x (not zero, subnormal or non-finite) with a result of 2^-6 .. 2^8; an infinite
+  // one beside entries of 2^1023 and more would have the code of 2^8
+  if (code - 8u <= 0x70u && m.hi - 0x00100000u < 0x7FE00000u) return code;
   return nonfinite(m) ? 0u : ru_e4m3_scaled(m, ep);
 }
 
