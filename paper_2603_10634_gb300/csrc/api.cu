@@ -406,8 +406,7 @@ ScaleJob scale_job(const Ctx& c, const Operand& op, int64_t first, int lines, co
 // of up to two operands.
 ozk2_status scale_operands(Ctx& c, const ScaleJob* jobs, int njobs, ZeroWords z) {
   const int kp = int(c.L.kp);
-  OZK2_TRY(launch_scale_prep(jobs, njobs, c.k, kp, c.fast, z.at, z.words, c.st));
-  t_launches += 1;
+  OZK2_TRY(launch_scale_prep(jobs, njobs, c.k, kp, c.fast, z.at, z.words, &t_launches, c.st));
   ScaleJob cols[2];
   int ncols = 0;
   for (int i = 0; i < njobs; ++i)
@@ -1072,20 +1071,19 @@ ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64
   if (wantA) {
     const ScaleJob rows[2] = {job(dC, lddc, c.m, true, gp, L.rstatC, L.Gbar, nullptr),
                               job(B, ldb, c.k, true, reinterpret_cast<int32_t*>(at(L.t)), L.rstatB, L.Bhat, nullptr)};
-    OZK2_TRY(launch_scale_prep(rows, 2, c.n, int(L.np), false, nullptr, 0, st));
+    OZK2_TRY(launch_scale_prep(rows, 2, c.n, int(L.np), false, nullptr, 0, &t_launches, st));
     OZK2_TRY(bw_bound(c, at(L.Gbar), at(L.Bhat), L.np, c.m, c.k, c.n, reinterpret_cast<float*>(at(L.R)),
                       reinterpret_cast<float*>(at(L.Sk)), reinterpret_cast<const int32_t*>(at(L.t)), nullptr, flags));
-    t_launches += 1;
   }
   if (wantB) {
     // the partial maxima in digit planes that are written later (as in scale_job)
     const ScaleJob cols[2] = {job(dC, lddc, c.n, false, hp, L.cstatC, L.HhatT, at(L.planesH)),
                               job(A, lda, c.k, false, reinterpret_cast<int32_t*>(at(L.tA)), L.cstatA, L.AhatT, at(L.planesAT))};
-    OZK2_TRY(launch_scale_prep(cols, 2, c.m, int(L.mp), false, nullptr, 0, st));
+    OZK2_TRY(launch_scale_prep(cols, 2, c.m, int(L.mp), false, nullptr, 0, &t_launches, st));
     OZK2_TRY(launch_scale_cols(cols, 2, c.m, int(L.mp), false, st));
     OZK2_TRY(bw_bound(c, at(L.AhatT), at(L.HhatT), L.mp, c.k, c.n, c.m, reinterpret_cast<float*>(at(L.Rk)),
                       reinterpret_cast<float*>(at(L.S)), nullptr, reinterpret_cast<const int32_t*>(at(L.tA)), flags));
-    t_launches += 2;
+    t_launches += 1;
   }
   OZK2_TRY(launch_reuse_exponents(wantA ? c.m : 0, gp, at(L.rstatC), reinterpret_cast<float*>(at(L.R)), g,
                                   wantB ? c.n : 0, hp, at(L.cstatC), reinterpret_cast<float*>(at(L.S)), h,

@@ -204,9 +204,10 @@ struct ScaleJob {
 };
 constexpr int kMaxKeyBlocks = 16;
 // First launch for up to two operands of the same k: the kcontig ones complete, the others'
-// partial column maxima; zeroes zero[0 .. zero_words).  Second launch for the strided ones.
+// partial column maxima; zeroes zero[0 .. zero_words).  Two launches where the rows take one
+// of their own; their number is added to *launches.  Second launch for the strided ones.
 cudaError_t launch_scale_prep(const ScaleJob* jobs, int njobs, int k, int kp, bool fast, uint32_t* zero,
-                              int64_t zero_words, cudaStream_t st);
+                              int64_t zero_words, int* launches, cudaStream_t st);
 cudaError_t launch_scale_cols(const ScaleJob* jobs, int njobs, int k, int kp, bool fast, cudaStream_t st);
 cudaError_t launch_exponents(int m, int n, const int32_t* eprime, const int32_t* fprime,
                              const uint8_t* rowstat, const uint8_t* colstat,

@@ -691,19 +691,22 @@ cudaError_t run_prep(const ScaleJob* jobs, int njobs, int k, int kp, uint32_t* z
 // 1477 -> 1393; 4096 rows of 65536 are as fast either way).  Fast mode (its sums keep a warp's
 // order) reads twice by warps.  More than 16 partial keys a column gain nothing.
 cudaError_t launch_scale_prep(const ScaleJob* jobs, int njobs, int k, int kp, bool fast, uint32_t* zero,
-                              int64_t zero_words, cudaStream_t st) {
+                              int64_t zero_words, int* launches, cudaStream_t st) {
+  const bool split = !fast && kp > 4096 && kp <= 8192;
+  if (!split) *launches += 1;
   if (fast) return run_prep<true, 0, 1>(jobs, njobs, k, kp, zero, zero_words, st);
   if (kp <= 512) return run_prep<false, 16, 1>(jobs, njobs, k, kp, zero, zero_words, st);
   if (kp <= 1024) return run_prep<false, 16, 2>(jobs, njobs, k, kp, zero, zero_words, st);
   if (kp <= 2048) return run_prep<false, 16, 4>(jobs, njobs, k, kp, zero, zero_words, st);
   if (kp <= 4096) return run_prep<false, 16, 8>(jobs, njobs, k, kp, zero, zero_words, st);
-  if (kp > 8192) return run_prep<false, 0, 8>(jobs, njobs, k, kp, zero, zero_words, st);
+  if (!split) return run_prep<false, 0, 8>(jobs, njobs, k, kp, zero, zero_words, st);
   for (int kc = 1; kc >= 0; --kc) {
     ScaleJob part[2];
     int n = 0;
     for (int i = 0; i < njobs; ++i)
       if (jobs[i].kcontig == (kc == 1)) part[n++] = jobs[i];
     if (n == 0) continue;
+    *launches += 1;
     const cudaError_t err = kc ? run_prep<false, 32, 8>(part, n, k, kp, zero, zero_words, st)
                                : run_prep<false, 0, 1>(part, n, k, kp, zero, zero_words, st);
     if (err != cudaSuccess) return err;
