@@ -405,20 +405,20 @@ int ozk2_debug_timeline(float *ms, int max);
 /*
  * ozk2_dgemm_backward - the gradients dA = dC B^T (m x k) and dB = A^T dC (k x n) of
  * C = A B (row-major, as ozk2_dgemm) by the same emulation, reusing the forward call's
- * scaling exponents e, f and digit planes of A' = trunc(diag(2^e) A), B' = trunc(B diag(2^f))
+ * scaling exponents e, f and so A' = trunc(diag(2^e) A), B' = trunc(B diag(2^f))
  * (Eqs. def:A', def:B').  The paper treats the product only; the construction is its own:
  *   dA: G'_ij = trunc(2^(g_i - f_j) dC_ij) with B' fixed, dA_ih = 2^-g_i (G' B'^T)_ih;
  *   dB: H'_ij = trunc(2^(h_j - e_i) dC_ij) with A' fixed, dB_hj = 2^-h_j (A'^T H')_hj;
  * g and h take the whole budget of P (Eq. condition: 2 sum |G'||B'| < P) from FP8 bound
  * products of |dC| with |B| and of |A| with |dC| (as accurate mode, Sec. III-E), so
- * as many FP8 products run per gradient as in a fresh emulation, but A and B are not
- * scaled again (their lines of the gradients are converted with the forward's exponents), and
- * one kernel converts dC for both.
+ * as many FP8 products run per gradient as in a fresh emulation; one kernel converts dC for
+ * both.
  *   forward_workspace  device memory of the current device, the workspace of the
  *                      ozk2_dgemm_ws / ozk2_dgemm_ex call (accurate mode, no blocking,
  *                      same m, n, k, num_moduli) that computed C = A B, unchanged since
- *                      (at least ozk2_workspace_size bytes).  Read only.
- *   A, B, dC           device, row-major: A m x k (lda), B k x n (ldb), dC m x n (lddc).
+ *                      (at least ozk2_workspace_size bytes).  Only e and f are read.
+ *   A, B, dC           device, row-major: A m x k (lda), B k x n (ldb), with the forward's
+ *                      values (A' and B' are formed from them again), dC m x n (lddc).
  *   dA, dB             device outputs (ldda >= k, lddb >= n); either may be NULL (not
  *                      computed), not both.
  *   workspace          device, >= ozk2_workspace_size_backward bytes, 256-byte aligned,
@@ -438,7 +438,33 @@ ozk2_status ozk2_dgemm_backward(int64_t m, int64_t n, int64_t k,
                                 void *workspace, size_t workspace_bytes,
                                 ozk2_stream_t stream);
 
-/* ozk2_workspace_size_backward - bytes of one ozk2_dgemm_backward call's own workspace
+/*
+ * ozk2_dgemm_forward - ozk2_dgemm_ws (or, with workspace NULL, ozk2_dgemm) that leaves e and
+ * f in `state` instead of its workspace, which is free for other uses once the call is done:
+ * a training step keeps 4 (m + n) bytes for the gradients, not a workspace.  state: device
+ * memory of the current device, 256-byte aligned, >= ozk2_forward_state_size(m, n) bytes.
+ * ozk2_dgemm_backward_from - ozk2_dgemm_backward with that state (same m, n).
+ * Products with m, n or k = 0 neither write nor read a state.
+ */
+size_t ozk2_forward_state_size(int64_t m, int64_t n); /* 0 on invalid arguments */
+ozk2_status ozk2_dgemm_forward(int64_t m, int64_t n, int64_t k,
+                               const double *A, int64_t lda,
+                               const double *B, int64_t ldb,
+                               double *C, int64_t ldc, int num_moduli,
+                               void *state, size_t state_bytes,
+                               void *workspace, size_t workspace_bytes,
+                               ozk2_stream_t stream);
+ozk2_status ozk2_dgemm_backward_from(int64_t m, int64_t n, int64_t k,
+                                     const double *A, int64_t lda,
+                                     const double *B, int64_t ldb,
+                                     const double *dC, int64_t lddc,
+                                     double *dA, int64_t ldda,
+                                     double *dB, int64_t lddb,
+                                     int num_moduli, const void *state, size_t state_bytes,
+                                     void *workspace, size_t workspace_bytes,
+                                     ozk2_stream_t stream);
+
+/* ozk2_workspace_size_backward - bytes of one gradient call's own workspace
  * (bound operands, the digit planes of dC's two integer matrices and of the transposed
  * A', B', the residue products of both gradients); 0 on invalid arguments. */
 size_t ozk2_workspace_size_backward(int64_t m, int64_t n, int64_t k, int num_moduli);

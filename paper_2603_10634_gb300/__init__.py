@@ -17,9 +17,12 @@ from .ozk2 import (  # noqa: F401
     device_status,
     dgemm,
     dgemm_backward,
+    dgemm_backward_from,
+    dgemm_forward,
     backward_exponents,
     dgemm_host,
     fp8_gemm,
+    forward_state_size,
     get_timing,
     last_launch_count,
     moduli,

@@ -47,6 +47,12 @@ SIGNATURES = {
     "ozk2_dgemm_backward": (c_int, [c_i64, c_i64, c_i64, c_void_p, c_i64, c_void_p, c_i64, c_void_p, c_i64,
                                     c_void_p, c_i64, c_void_p, c_i64, c_int, c_void_p, c_size_t, c_void_p,
                                     c_size_t, c_void_p]),
+    "ozk2_forward_state_size": (c_size_t, [c_i64, c_i64]),
+    "ozk2_dgemm_forward": (c_int, [c_i64, c_i64, c_i64, c_void_p, c_i64, c_void_p, c_i64, c_void_p, c_i64, c_int,
+                                   c_void_p, c_size_t, c_void_p, c_size_t, c_void_p]),
+    "ozk2_dgemm_backward_from": (c_int, [c_i64, c_i64, c_i64, c_void_p, c_i64, c_void_p, c_i64, c_void_p, c_i64,
+                                         c_void_p, c_i64, c_void_p, c_i64, c_int, c_void_p, c_size_t, c_void_p,
+                                         c_size_t, c_void_p]),
     "ozk2_workspace_size_backward": (c_size_t, [c_i64, c_i64, c_i64, c_int]),
     "ozk2_debug_backward_exponents": (c_int, [c_i64, c_i64, c_i64, c_int, c_void_p, c_void_p, c_void_p, c_void_p]),
     "ozk2_set_wait_limit": (ctypes.c_uint64, [ctypes.c_uint64]),

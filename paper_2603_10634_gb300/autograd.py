@@ -2,10 +2,11 @@
 
 C = A B runs through the emulated DGEMM.  The backward pass needs two more products,
 dA = dC B^T and dB = A^T dC.  By default (``reuse=True``) they run through
-ozk2_dgemm_backward, which reuses the forward call's scaling exponents and integer matrices
-of A' = trunc(diag(2^e) A) and B' = trunc(B diag(2^f)): the forward runs in a workspace
-kept in the autograd context, only dC is scaled, one conversion
-of it serves both gradients, and dC's exponents take the whole budget of P that A' and B' leave.  With
+ozk2_dgemm_backward_from, which reuses the forward call's scaling exponents and so its integer
+matrices A' = trunc(diag(2^e) A) and B' = trunc(B diag(2^f)): the autograd context keeps
+the exponents (4 (m + n) bytes; the forward's workspace, a few GB for a large layer, is
+released at once), one conversion of dC serves both gradients, and dC's exponents take
+the whole budget of P that A' and B' leave.  With
 ``reuse=False``, or where reuse does not apply (fast mode, operands that are transposed
 views), each gradient is an independent emulation with its own scaling (Sec. III-E) of
 operands read in place.
@@ -47,8 +48,8 @@ class OzakiMatmul(torch.autograd.Function):
             m, k = A.shape
             n = B.shape[1]
             ws = torch.empty(max(1, ozk2.workspace_size(m, n, k, num_moduli)), dtype=torch.uint8, device=A.device)
-            ctx.forward_workspace = ws  # holds the forward's exponents, read by backward
-            return ozk2.dgemm(A, B, num_moduli=num_moduli, workspace=ws)
+            C, ctx.forward_state = ozk2.dgemm_forward(A, B, num_moduli, workspace=ws)
+            return C
         return ozk2.dgemm(_operand(A), _operand(B), num_moduli=num_moduli, mode=mode)
 
     @staticmethod
@@ -57,8 +58,8 @@ class OzakiMatmul(torch.autograd.Function):
         dA = dB = None
         if ctx.reuse:
             dC = dC.contiguous()
-            dA, dB = ozk2.dgemm_backward(A, B, dC, ctx.forward_workspace, ctx.num_moduli,
-                                         need_dA=ctx.needs_input_grad[0], need_dB=ctx.needs_input_grad[1])
+            dA, dB = ozk2.dgemm_backward_from(A, B, dC, ctx.forward_state, ctx.num_moduli,
+                                              need_dA=ctx.needs_input_grad[0], need_dB=ctx.needs_input_grad[1])
             return dA, dB, None, None, None
         dC = _operand(dC)
         if ctx.needs_input_grad[0]:

@@ -270,6 +270,7 @@ struct Ctx {
   uint64_t owned_use = 0;  // > 0: the call runs in the library-owned workspace, its use number
   Layout L;
   uint8_t* ws;
+  int32_t *e, *f;  // the exponents of the rows of A' and the columns of B'
   const Tables* tab;
   int num_sms;
   cudaStream_t st;
@@ -455,8 +456,8 @@ cudaError_t exponents_of(Ctx& c, int64_t i0, int rows, bool cols) {
   t_launches += 1;
   return launch_exponents(rows, cols ? c.n : 0, c.at<int32_t>(L.eprime) + i0, c.at<int32_t>(L.fprime),
                           c.at<uint8_t>(L.rowstat) + i0, c.at<uint8_t>(L.colstat), c.at<float>(L.R) + i0,
-                          c.at<float>(L.S), c.tab->pprime, delta_f32(), c.at<int32_t>(L.e) + i0,
-                          c.at<int32_t>(L.f), c.at<uint32_t>(L.flags), c.st);
+                          c.at<float>(L.S), c.tab->pprime, delta_f32(), c.e + i0, c.f, c.at<uint32_t>(L.flags),
+                          c.st);
 }
 
 // Bound product (accurate mode) and the exponents e, f.
@@ -484,10 +485,10 @@ ResidArgs resid_args(const Ctx& c, const Operand& op, int64_t first, int lines, 
                    total * c.L.ldp, c.at<uint32_t>(c.L.flags), op.kcontig};
 }
 ResidArgs resid_a(const Ctx& c, const Operand& a, int64_t first, int lines) {
-  return resid_args(c, a, first, lines, c.m, c.at<int32_t>(c.L.e), c.at<uint8_t>(c.L.planesA));
+  return resid_args(c, a, first, lines, c.m, c.e, c.at<uint8_t>(c.L.planesA));
 }
 ResidArgs resid_b(const Ctx& c, const Operand& b) {
-  return resid_args(c, b, 0, c.n, c.n, c.at<int32_t>(c.L.f), c.at<uint8_t>(c.L.planesB));
+  return resid_args(c, b, 0, c.n, c.n, c.f, c.at<uint8_t>(c.L.planesB));
 }
 
 // The hybrid list's digit planes of row-major A and B (parity hooks), packed.
@@ -606,6 +607,8 @@ ozk2_status setup(Ctx& c, int64_t m, int64_t n, int64_t k, int N, bool fast, voi
     c.ws = owned_workspace(c.L.total + extra, &err, &c.owned_use);
     if (!c.ws) return err;
   }
+  c.e = c.at<int32_t>(c.L.e);
+  c.f = c.at<int32_t>(c.L.f);
   return OZK2_OK;
 }
 
@@ -645,8 +648,7 @@ int row_blocks(const Ctx& c, int64_t (&first)[kMaxRowBlocks + 1]) {
 // GEMM was measured and gains nothing: they get too little of an SM next to it.)
 ozk2_status products_and_crt(Ctx& c, double* C, int64_t ldc, const CopyBack* cb) {
   const Layout& L = c.L;
-  const int32_t* e = c.at<int32_t>(L.e);
-  const int32_t* f = c.at<int32_t>(L.f);
+  const int32_t *e = c.e, *f = c.f;
   const uint8_t* rs = c.at<uint8_t>(L.rowstat);
   const uint8_t* cs = c.at<uint8_t>(L.colstat);
   mark(c, 4);
@@ -670,13 +672,31 @@ ozk2_status products_and_crt(Ctx& c, double* C, int64_t ldc, const CopyBack* cb)
   return OZK2_OK;
 }
 
+// What a forward call leaves for the gradients: the exponents e, then f, each on 256 bytes.
+struct ForwardState {
+  size_t f, total;  // e is at 0
+};
+ForwardState forward_state(int64_t m, int64_t n) {
+  const size_t f = align256(4 * size_t(m));
+  return ForwardState{f, f + align256(4 * size_t(n))};
+}
+bool valid_state(const void* state, size_t bytes, int64_t m, int64_t n) {
+  return state && bytes >= forward_state(m, n).total && (reinterpret_cast<uintptr_t>(state) & 255u) == 0 &&
+         device_memory_here(state);
+}
+
 // One emulated product over whole operands (no blocking); arguments already validated,
-// m, n, k > 0.
+// m, n, k > 0.  state: where the exponents go (null: the workspace).
 ozk2_status run_one(const Operand& a, const Operand& b, int64_t m, int64_t n, int64_t k, double* C, int64_t ldc,
-                    int N, bool fast, bool first, void* ws, size_t ws_bytes, cudaStream_t st, bool ws_trusted) {
+                    int N, bool fast, bool first, uint8_t* state, void* ws, size_t ws_bytes, cudaStream_t st,
+                    bool ws_trusted) {
   Ctx c;
   ozk2_status s = setup(c, m, n, k, N, fast, ws, ws_bytes, st, 0, ws_trusted);
   if (s != OZK2_OK) return s;
+  if (state) {
+    c.e = reinterpret_cast<int32_t*>(state);
+    c.f = reinterpret_cast<int32_t*>(state + forward_state(m, n).f);
+  }
   mark(c, 0);
   if ((s = phase_scales(c, a, b, first)) != OZK2_OK) return s;
   const ResidArgs ops[2] = {resid_a(c, a, 0, c.m), resid_b(c, b)};
@@ -712,7 +732,7 @@ ozk2_status dgemm_general(ozk2_op transa, ozk2_op transb, int64_t m, int64_t n, 
     for (int64_t j0 = 0; j0 < n; j0 += bn) {
       const int64_t mm = std::min(bm, m - i0), nn = std::min(bn, n - j0);
       s = run_one(shift_lines(a, i0), shift_lines(b, j0), mm, nn, k, C + i0 * ldc + j0, ldc, N, fast,
-                  i0 == 0 && j0 == 0, ws, ws_bytes, st, ws_trusted);
+                  i0 == 0 && j0 == 0, nullptr, ws, ws_bytes, st, ws_trusted);
       if (s != OZK2_OK) return s;
     }
   }
@@ -907,8 +927,8 @@ size_t host_workspace_bytes(int64_t m, int64_t n, int64_t k, int N, bool fast) {
 }
 
 // ------------------------------------------------------------------ gradients with reuse
-// dA = dC B^T and dB = A^T dC for C = A B computed in a caller workspace, reusing that
-// call's exponents e, f and digit planes of A' = trunc(diag(2^e) A), B' = trunc(B diag(2^f)):
+// dA = dC B^T and dB = A^T dC for C = A B, reusing that call's exponents e, f and with them
+// A' = trunc(diag(2^e) A), B' = trunc(B diag(2^f)):
 //   dA: G'_ij = trunc(2^(g_i - f_j) dC_ij); (G' B'^T)_ih = 2^g_i dA_ih (up to truncation)
 //   dB: H'_ij = trunc(2^(h_j - e_i) dC_ij); (A'^T H')_hj = 2^h_j dB_hj
 // The exponents g, h of dC's side come from FP8 bound products of |dC| with |B| (rows of
@@ -1017,7 +1037,7 @@ cudaError_t bw_products(const Ctx& c, const uint8_t* a, const uint8_t* b, int64_
 
 ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
                          int64_t ldb, const double* dC, int64_t lddc, double* dA, int64_t ldda, double* dB,
-                         int64_t lddb, int N, const void* fws, size_t fws_bytes, void* ws, size_t ws_bytes,
+                         int64_t lddb, int N, const int32_t* e, const int32_t* f, void* ws, size_t ws_bytes,
                          cudaStream_t st) {
   Ctx c;
   c.m = int(m);
@@ -1029,9 +1049,6 @@ ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64
   if (!encode_fn()) return OZK2_ERR_CUDA;
   c.tab = tables_for(N);
   if (!c.tab) return OZK2_ERR_INTERNAL;
-  const Layout FL = make_layout(m, n, k, N, false);
-  if (!fws || fws_bytes < FL.total || (reinterpret_cast<uintptr_t>(fws) & 255u) || !device_memory_here(fws))
-    return OZK2_ERR_INVALID_VALUE;
   const BwLayout L = make_bw_layout(m, n, k, N);
   uint8_t* w;
   if (ws) {
@@ -1044,9 +1061,6 @@ ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64
     if (!w) return err;
   }
   auto at = [w](size_t off) { return w + off; };
-  const uint8_t* f8 = static_cast<const uint8_t*>(fws);
-  const int32_t* e = reinterpret_cast<const int32_t*>(f8 + FL.e);
-  const int32_t* f = reinterpret_cast<const int32_t*>(f8 + FL.f);
   uint32_t* flags = reinterpret_cast<uint32_t*>(at(L.flags));
   int32_t* gp = reinterpret_cast<int32_t*>(at(L.gp));
   int32_t* hp = reinterpret_cast<int32_t*>(at(L.hp));
@@ -1118,6 +1132,42 @@ ozk2_status run_backward(int64_t m, int64_t n, int64_t k, const double* A, int64
     t_launches += 1;
   }
   return OZK2_OK;
+}
+
+// Checks of a gradient call, whose exponents come from the forward's workspace or (fws null) its state.
+ozk2_status backward(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B, int64_t ldb,
+                     const double* dC, int64_t lddc, double* dA, int64_t ldda, double* dB, int64_t lddb, int N,
+                     const void* fws, size_t fws_bytes, const void* state, size_t state_bytes, void* ws,
+                     size_t ws_bytes, cudaStream_t st) {
+  t_launches = 0;
+  const ozk2_status s = check_sizes(m, n, k, N);
+  if (s != OZK2_OK) return s;
+  if (lda < std::max<int64_t>(1, k) || ldb < std::max<int64_t>(1, n) || lddc < std::max<int64_t>(1, n) ||
+      (dA && ldda < std::max<int64_t>(1, k)) || (dB && lddb < std::max<int64_t>(1, n)))
+    return OZK2_ERR_INVALID_VALUE;
+  // empty shapes: dA (m x k) and dB (k x n) are zero where their reduction is empty
+  if (m == 0 || n == 0 || k == 0) {
+    if (dA && m > 0 && k > 0) OZK2_TRY(cudaMemset2DAsync(dA, size_t(ldda) * 8, 0, size_t(k) * 8, size_t(m), st));
+    if (dB && k > 0 && n > 0) OZK2_TRY(cudaMemset2DAsync(dB, size_t(lddb) * 8, 0, size_t(n) * 8, size_t(k), st));
+    return OZK2_OK;
+  }
+  if (!A || !B || !dC || (!dA && !dB)) return OZK2_ERR_INVALID_VALUE;
+  int sms = 0;
+  if (!device_info(&sms)) return OZK2_ERR_UNSUPPORTED;
+  const uint8_t *e, *f;
+  if (fws) {
+    const Layout L = make_layout(m, n, k, N, false);
+    if (fws_bytes < L.total || (reinterpret_cast<uintptr_t>(fws) & 255u) || !device_memory_here(fws))
+      return OZK2_ERR_INVALID_VALUE;
+    e = static_cast<const uint8_t*>(fws) + L.e;
+    f = static_cast<const uint8_t*>(fws) + L.f;
+  } else {
+    if (!valid_state(state, state_bytes, m, n)) return OZK2_ERR_INVALID_VALUE;
+    e = static_cast<const uint8_t*>(state);
+    f = e + forward_state(m, n).f;
+  }
+  return run_backward(m, n, k, A, lda, B, ldb, dC, lddc, dA, ldda, dB, lddb, N, reinterpret_cast<const int32_t*>(e),
+                      reinterpret_cast<const int32_t*>(f), ws, ws_bytes, st);
 }
 
 // ------------------------------------------------------------------ batches
@@ -1756,27 +1806,40 @@ size_t ozk2_workspace_size_backward(int64_t m, int64_t n, int64_t k, int num_mod
   return make_bw_layout(m, n, k, num_moduli).total;
 }
 
+size_t ozk2_forward_state_size(int64_t m, int64_t n) {
+  return check_sizes(m, n, 1, 1) == OZK2_OK ? forward_state(m, n).total : 0;
+}
+
+ozk2_status ozk2_dgemm_forward(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
+                               int64_t ldb, double* C, int64_t ldc, int num_moduli, void* state, size_t state_bytes,
+                               void* workspace, size_t workspace_bytes, ozk2_stream_t stream) {
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  const ozk2_status s = validate(OZK2_OP_N, OZK2_OP_N, m, n, k, A, lda, B, ldb, C, ldc, num_moduli);
+  if (s != OZK2_OK || m == 0 || n == 0 || k == 0)
+    return dgemm_general(OZK2_OP_N, OZK2_OP_N, m, n, k, A, lda, B, ldb, C, ldc, num_moduli, OZK2_MODE_ACCURATE, 0, 0,
+                         nullptr, 0, st);
+  t_launches = 0;
+  if (!valid_state(state, state_bytes, m, n)) return OZK2_ERR_INVALID_VALUE;
+  return run_one(operand_a(OZK2_OP_N, A, lda), operand_b(OZK2_OP_N, B, ldb), m, n, k, C, ldc, num_moduli, false, true,
+                 static_cast<uint8_t*>(state), workspace, workspace_bytes, st, false);
+}
+
 ozk2_status ozk2_dgemm_backward(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
                                 int64_t ldb, const double* dC, int64_t lddc, double* dA, int64_t ldda, double* dB,
                                 int64_t lddb, int num_moduli, const void* forward_workspace,
                                 size_t forward_workspace_bytes, void* workspace, size_t workspace_bytes,
                                 ozk2_stream_t stream) {
-  t_launches = 0;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  ozk2_status s = check_sizes(m, n, k, num_moduli);
-  if (s != OZK2_OK) return s;
-  if (lda < std::max<int64_t>(1, k) || ldb < std::max<int64_t>(1, n) || lddc < std::max<int64_t>(1, n) ||
-      (dA && ldda < std::max<int64_t>(1, k)) || (dB && lddb < std::max<int64_t>(1, n)))
-    return OZK2_ERR_INVALID_VALUE;
-  // empty shapes: dA (m x k) and dB (k x n) are zero where their reduction is empty
-  if (m == 0 || n == 0 || k == 0) {
-    if (dA && m > 0 && k > 0) OZK2_TRY(cudaMemset2DAsync(dA, size_t(ldda) * 8, 0, size_t(k) * 8, size_t(m), st));
-    if (dB && k > 0 && n > 0) OZK2_TRY(cudaMemset2DAsync(dB, size_t(lddb) * 8, 0, size_t(n) * 8, size_t(k), st));
-    return OZK2_OK;
-  }
-  if (!A || !B || !dC || (!dA && !dB)) return OZK2_ERR_INVALID_VALUE;
-  return run_backward(m, n, k, A, lda, B, ldb, dC, lddc, dA, ldda, dB, lddb, num_moduli, forward_workspace,
-                      forward_workspace_bytes, workspace, workspace_bytes, st);
+  return backward(m, n, k, A, lda, B, ldb, dC, lddc, dA, ldda, dB, lddb, num_moduli, forward_workspace,
+                  forward_workspace_bytes, nullptr, 0, workspace, workspace_bytes,
+                  reinterpret_cast<cudaStream_t>(stream));
+}
+
+ozk2_status ozk2_dgemm_backward_from(int64_t m, int64_t n, int64_t k, const double* A, int64_t lda, const double* B,
+                                     int64_t ldb, const double* dC, int64_t lddc, double* dA, int64_t ldda,
+                                     double* dB, int64_t lddb, int num_moduli, const void* state, size_t state_bytes,
+                                     void* workspace, size_t workspace_bytes, ozk2_stream_t stream) {
+  return backward(m, n, k, A, lda, B, ldb, dC, lddc, dA, ldda, dB, lddb, num_moduli, nullptr, 0, state, state_bytes,
+                  workspace, workspace_bytes, reinterpret_cast<cudaStream_t>(stream));
 }
 
 ozk2_status ozk2_debug_backward_exponents(int64_t m, int64_t n, int64_t k, int num_moduli, const void* workspace,

@@ -160,6 +160,40 @@ def dgemm(A, B, num_moduli=12, out=None, workspace=None, mode="accurate", block=
     return out
 
 
+def forward_state_size(m, n):
+    return int(_lib.load().ozk2_forward_state_size(m, n))
+
+
+def dgemm_forward(A, B, num_moduli=12, out=None, workspace=None):
+    """(C, state): C = A @ B as ``dgemm`` in accurate mode for row-major float64 CUDA tensors,
+    and the exponents that ``dgemm_backward_from`` needs, 4 (m + n) bytes.  The workspace is
+    not needed for the gradients."""
+    _check_matrix(A, "A")
+    _check_matrix(B, "B")
+    m, k = A.shape
+    k2, n = B.shape
+    if k != k2:
+        raise ValueError(f"inner dimensions differ: {tuple(A.shape)} @ {tuple(B.shape)}")
+    if A.device != B.device:
+        raise ValueError("A and B must be on the same device")
+    if out is None:
+        out = torch.empty((m, n), dtype=torch.float64, device=A.device)
+    else:
+        _check_matrix(out, "out")
+        if tuple(out.shape) != (m, n):
+            raise ValueError("out has the wrong shape")
+    if workspace is not None and (workspace.dtype != torch.uint8 or not workspace.is_cuda):
+        raise TypeError("workspace must be a uint8 CUDA tensor")
+    lib = _lib.load()
+    state = torch.empty(lib.ozk2_forward_state_size(m, n), dtype=torch.uint8, device=A.device)
+    with torch.cuda.device(A.device):
+        s = lib.ozk2_dgemm_forward(m, n, k, _ptr(A), _ld(A), _ptr(B), _ld(B), _ptr(out), _ld(out), num_moduli,
+                                   _ptr(state), state.numel(), _ptr(workspace),
+                                   0 if workspace is None else workspace.numel(), _stream(A.device))
+    _lib.check(s, "ozk2_dgemm_forward")
+    return out, state
+
+
 def workspace_size_backward(m, n, k, num_moduli=12):
     return int(_lib.load().ozk2_workspace_size_backward(m, n, k, num_moduli))
 
@@ -167,29 +201,38 @@ def workspace_size_backward(m, n, k, num_moduli=12):
 def dgemm_backward(A, B, dC, forward_workspace, num_moduli=12, need_dA=True, need_dB=True, workspace=None):
     """(dA, dB) = (dC @ B.T, A.T @ dC) for C = A @ B computed by ``dgemm(A, B, num_moduli,
     workspace=forward_workspace)`` (accurate mode, no blocking), reusing that call's
-    exponents and integer matrices (ozk2_dgemm_backward).  A, B, dC: row-major float64 CUDA
-    tensors; forward_workspace: the uint8 tensor the forward ran in, unchanged since.
-    An output not needed is returned as None."""
+    exponents and so its integer matrices (ozk2_dgemm_backward).  A, B, dC: row-major float64
+    CUDA tensors, A and B with the forward's values; forward_workspace: the uint8 tensor the
+    forward ran in, unchanged since.  An output not needed is returned as None."""
+    return _backward("ozk2_dgemm_backward", "forward_workspace", A, B, dC, forward_workspace, num_moduli, need_dA,
+                     need_dB, workspace)
+
+
+def dgemm_backward_from(A, B, dC, state, num_moduli=12, need_dA=True, need_dB=True, workspace=None):
+    """``dgemm_backward`` with the state of ``dgemm_forward`` in place of the workspace."""
+    return _backward("ozk2_dgemm_backward_from", "state", A, B, dC, state, num_moduli, need_dA, need_dB, workspace)
+
+
+def _backward(entry, kept_name, A, B, dC, kept, num_moduli, need_dA, need_dB, workspace):
     for x, name in ((A, "A"), (B, "B"), (dC, "dC")):
         _check_matrix(x, name)
     m, k = A.shape
     k2, n = B.shape
     if k != k2 or tuple(dC.shape) != (m, n):
         raise ValueError("shapes do not match C = A @ B")
-    if forward_workspace.dtype != torch.uint8 or not forward_workspace.is_cuda:
-        raise TypeError("forward_workspace must be a uint8 CUDA tensor")
+    if kept.dtype != torch.uint8 or not kept.is_cuda:
+        raise TypeError(f"{kept_name} must be a uint8 CUDA tensor")
     if workspace is not None and (workspace.dtype != torch.uint8 or not workspace.is_cuda):
         raise TypeError("workspace must be a uint8 CUDA tensor")
     dA = torch.empty((m, k), dtype=torch.float64, device=A.device) if need_dA else None
     dB = torch.empty((k, n), dtype=torch.float64, device=A.device) if need_dB else None
     lib = _lib.load()
     with torch.cuda.device(A.device):
-        s = lib.ozk2_dgemm_backward(m, n, k, _ptr(A), _ld(A), _ptr(B), _ld(B), _ptr(dC), _ld(dC), _ptr(dA),
-                                    _ld(dA) if dA is not None else max(1, k), _ptr(dB),
-                                    _ld(dB) if dB is not None else max(1, n), num_moduli, _ptr(forward_workspace),
-                                    forward_workspace.numel(), _ptr(workspace),
-                                    0 if workspace is None else workspace.numel(), _stream(A.device))
-    _lib.check(s, "ozk2_dgemm_backward")
+        s = getattr(lib, entry)(m, n, k, _ptr(A), _ld(A), _ptr(B), _ld(B), _ptr(dC), _ld(dC), _ptr(dA),
+                                _ld(dA) if dA is not None else max(1, k), _ptr(dB),
+                                _ld(dB) if dB is not None else max(1, n), num_moduli, _ptr(kept), kept.numel(),
+                                _ptr(workspace), 0 if workspace is None else workspace.numel(), _stream(A.device))
+    _lib.check(s, entry)
     return dA, dB
 
 
