@@ -202,39 +202,49 @@ Operand shift_lines(const Operand& o, int64_t first) {
 
 // ------------------------------------------------------------------ workspace layout
 struct Layout {
-  int64_t kp, ldp, ldr;  // kp: bytes of k per row; ldp: digit-plane row pitch
-  int planes;
+  int64_t kp, ldp, ldr;  // kp: bytes of k per row; ldp: digit-plane row pitch; ldr: columns of a residue row
   size_t flags, R, S, zero_end;
   size_t eprime, fprime, e, f, rowstat, colstat;
   size_t Abar, BbarT, partA, partB, planesA, planesB, cres, cres8, total;
 };
 
-// Residue rows hold a multiple of 16 columns (16-byte stores of 8-bit residues).
-int64_t residue_pitch(int64_t n) { return ((n + 15) / 16) * 16; }
-
-// Bytes of the residue region: the Karatsuba moduli's 16-bit planes, then the single
-// moduli's 8-bit planes.  Sized for at least N 16-bit planes with rows of a multiple of 8
-// columns, and the digit-plane regions for the hybrid list's M_N planes (which the parity
-// hooks write): the documented workspace, a few percent more than the product path uses.
-size_t residue_bytes(int64_t m, int64_t n, int N) {
-  const size_t own = size_t(kRnsSingles[N] + 2 * kRnsKars[N]) * size_t(m) * size_t(residue_pitch(n));
-  const size_t hybrid = 2 * size_t(N) * size_t(m) * size_t(((n + 7) / 8) * 8);
-  return std::max(own, hybrid);
-}
-// Offset of the 8-bit planes within it.
-size_t residue8_offset(int64_t m, int64_t n, int N) { return 2 * size_t(kRnsKars[N]) * size_t(m) * size_t(residue_pitch(n)); }
-
-// N 16-bit residue planes of the hybrid list (parity hooks, after the layout).
-size_t paper_residue_bytes(int64_t m, int64_t n, int N) { return 2 * size_t(N) * size_t(m) * size_t(residue_pitch(n)); }
-
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
-Layout make_layout(int64_t m, int64_t n, int64_t k, int N, bool fast) {
+// The documented workspace holds the hybrid list's M_N digit planes per operand and N 16-bit
+// residue planes with rows of a multiple of 8 columns (the parity hooks write them).  The
+// product path's rns_planes(N) planes and its residues, the Karatsuba moduli's 16-bit planes
+// and then the single moduli's 8-bit ones, take a few percent less.
+int hybrid_planes(int N) { return N <= kNumSquares ? 2 * N : 3 * N - kNumSquares; }
+int64_t residue_pitch(int64_t n) { return ((n + 7) / 8) * 8; }
+size_t hybrid_residue_bytes(int64_t m, int64_t n, int N) { return 2 * size_t(N) * size_t(m) * size_t(residue_pitch(n)); }
+size_t residue_bytes(int64_t m, int64_t ldr, int N) {
+  return size_t(kRnsSingles[N] + 2 * kRnsKars[N]) * size_t(m) * size_t(ldr);
+}
+constexpr bool residues_fit() {
+  for (int N = 1; N <= kMaxModuli; ++N)
+    if (kRnsSingles[N] + 2 * kRnsKars[N] > 2 * N) return false;
+  return true;
+}
+static_assert(residues_fit(), "the product path's residues fit in the hybrid list's space");
+// Offset of the 8-bit planes within the residues.
+size_t residue8_offset(int64_t m, int64_t ldr, int N) { return 2 * size_t(kRnsKars[N]) * size_t(m) * size_t(ldr); }
+
+// Columns of a residue row: a multiple of 16, which lets every 16 8-bit residues go out in one
+// store, where that fits in `room` bytes.  The documented space alone would be up to a fifth
+// too small for it at ragged n, so the residues start behind the digit planes in use and take
+// the unused ones and the bound operands (dead by then) as well; what does not fit even so
+// (N <= 6 or k of a few dozen) has rows of a multiple of 8.  Calls with rows on 8 / 16 bytes:
+// 4000 x 1000 x 500 166 / 152 us, 60000 x 200 x 300 641 / 605, 1500 x 2001 x 100 110 / 101.
+int64_t residue_pitch_in(size_t room, int64_t m, int64_t n, int N) {
+  const int64_t wide = (n + 15) / 16 * 16;
+  return residue_bytes(m, wide, N) <= room ? wide : residue_pitch(n);
+}
+
+// hybrid: the parity hooks' layout, with the hybrid list's planes and residues.
+Layout make_layout(int64_t m, int64_t n, int64_t k, int N, bool fast, bool hybrid = false) {
   Layout L;
   L.kp = ((k + 31) / 32) * 32;
   L.ldp = plane_pitch(L.kp);
-  L.ldr = residue_pitch(n);
-  L.planes = (N <= kNumSquares) ? 2 * N : 3 * N - kNumSquares;
   size_t o = 0;
   auto take = [&o](size_t bytes) {
     const size_t at = o;
@@ -251,15 +261,21 @@ Layout make_layout(int64_t m, int64_t n, int64_t k, int N, bool fast) {
   L.f = take(4 * size_t(n));
   L.rowstat = take(size_t(m));
   L.colstat = take(size_t(n));
+  // digit planes, then the residues, which overlap planes not in use and the bound operands
+  const int planes = hybrid ? hybrid_planes(N) : rns_planes(N);
+  L.planesA = o;
+  L.planesB = L.planesA + align256(size_t(planes) * m * L.ldp);
+  L.cres = L.planesB + align256(size_t(planes) * n * L.ldp);
+  take(size_t(hybrid_planes(N)) * m * L.ldp);
+  take(size_t(hybrid_planes(N)) * n * L.ldp);
   L.Abar = fast ? o : take(size_t(m) * L.kp);
   L.BbarT = fast ? o : take(size_t(n) * L.kp);
   L.partA = fast ? take(4 * size_t(m) * (L.kp / 32)) : o;
   L.partB = fast ? take(4 * size_t(n) * (L.kp / 32)) : o;
-  L.planesA = take(size_t(L.planes) * m * L.ldp);
-  L.planesB = take(size_t(L.planes) * n * L.ldp);
-  L.cres = take(residue_bytes(m, n, N));
-  L.cres8 = L.cres + residue8_offset(m, n, N);
+  take(hybrid_residue_bytes(m, n, N));
   L.total = o;
+  L.ldr = hybrid ? residue_pitch(n) : residue_pitch_in(o - L.cres, m, n, N);
+  L.cres8 = L.cres + residue8_offset(m, L.ldr, N);
   return L;
 }
 
@@ -584,9 +600,9 @@ ozk2_status validate_operands(ozk2_op transa, ozk2_op transb, int64_t m, int64_t
 
 // `extra`: bytes the caller needs after the layout (256-aligned, at offset L.total).
 // ws_trusted: `ws` is memory of this library (the static array of ozk2_dgemm_noalloc),
-// known to be device memory of the current device.
+// known to be device memory of the current device.  hybrid: see make_layout.
 ozk2_status setup(Ctx& c, int64_t m, int64_t n, int64_t k, int N, bool fast, void* ws, size_t ws_bytes,
-                  cudaStream_t st, size_t extra = 0, bool ws_trusted = false) {
+                  cudaStream_t st, size_t extra = 0, bool ws_trusted = false, bool hybrid = false) {
   c.m = int(m);
   c.n = int(n);
   c.k = int(k);
@@ -597,7 +613,7 @@ ozk2_status setup(Ctx& c, int64_t m, int64_t n, int64_t k, int N, bool fast, voi
   if (!encode_fn()) return OZK2_ERR_CUDA;
   c.tab = tables_for(N);
   if (!c.tab) return OZK2_ERR_INTERNAL;
-  c.L = make_layout(m, n, k, N, fast);
+  c.L = make_layout(m, n, k, N, fast, hybrid);
   if (ws) {
     if (ws_bytes < c.L.total + extra || (reinterpret_cast<uintptr_t>(ws) & 255u)) return OZK2_ERR_INVALID_VALUE;
     if (!ws_trusted && !device_memory_here(ws)) return OZK2_ERR_INVALID_VALUE;
@@ -938,7 +954,6 @@ size_t host_workspace_bytes(int64_t m, int64_t n, int64_t k, int N, bool fast) {
 // the products read.
 struct BwLayout {
   int64_t np, mp, ldrk, ldrn;
-  int planes;
   size_t flags, R, S, Rk, Sk, zk, zero_end;
   size_t gp, hp, g, h, t, tA, rstatC, cstatC, rstatB, cstatA;
   size_t Gbar, Bhat, AhatT, HhatT, planesG, planesBT, planesAT, planesH, cresA, cresA8, cresB, cresB8, total;
@@ -948,9 +963,6 @@ BwLayout make_bw_layout(int64_t m, int64_t n, int64_t k, int N) {
   BwLayout L;
   L.np = ((n + 31) / 32) * 32;
   L.mp = ((m + 31) / 32) * 32;
-  L.ldrk = residue_pitch(k);
-  L.ldrn = residue_pitch(n);
-  L.planes = (N <= kNumSquares) ? 2 * N : 3 * N - kNumSquares;
   size_t o = 0;
   auto take = [&o](size_t bytes) {
     const size_t at = o;
@@ -974,19 +986,29 @@ BwLayout make_bw_layout(int64_t m, int64_t n, int64_t k, int N) {
   L.cstatC = take(size_t(n));
   L.rstatB = take(size_t(k));
   L.cstatA = take(size_t(k));
+  // as make_layout: both gradients' residues behind the digit planes in use
+  const size_t planes = size_t(rns_planes(N)), documented = size_t(hybrid_planes(N));
+  L.planesG = o;
+  L.planesBT = L.planesG + align256(planes * m * L.np);
+  L.planesAT = L.planesBT + align256(planes * k * L.np);
+  L.planesH = L.planesAT + align256(planes * k * L.mp);
+  L.cresA = L.planesH + align256(planes * n * L.mp);
+  take(documented * m * L.np);
+  take(documented * k * L.np);
+  take(documented * k * L.mp);
+  take(documented * n * L.mp);
   L.Gbar = take(size_t(m) * L.np);
   L.Bhat = take(size_t(k) * L.np);
   L.AhatT = take(size_t(k) * L.mp);
   L.HhatT = take(size_t(n) * L.mp);
-  L.planesG = take(size_t(L.planes) * m * L.np);
-  L.planesBT = take(size_t(L.planes) * k * L.np);
-  L.planesAT = take(size_t(L.planes) * k * L.mp);
-  L.planesH = take(size_t(L.planes) * n * L.mp);
-  L.cresA = take(residue_bytes(m, k, N));
-  L.cresA8 = L.cresA + residue8_offset(m, k, N);
-  L.cresB = take(residue_bytes(k, n, N));
-  L.cresB8 = L.cresB + residue8_offset(k, n, N);
+  take(hybrid_residue_bytes(m, k, N));
+  take(hybrid_residue_bytes(k, n, N));
   L.total = o;
+  L.ldrk = residue_pitch_in(o - L.cresA - align256(residue_bytes(k, residue_pitch(n), N)), m, k, N);
+  L.cresA8 = L.cresA + residue8_offset(m, L.ldrk, N);
+  L.cresB = L.cresA + align256(residue_bytes(m, L.ldrk, N));
+  L.ldrn = residue_pitch_in(o - L.cresB, k, n, N);
+  L.cresB8 = L.cresB + residue8_offset(k, L.ldrn, N);
   return L;
 }
 
@@ -1203,6 +1225,7 @@ struct ozk2_batch_plan_st {
   // descriptors in 256-wide tiles, the next res_cnt[1] in 128-wide tiles.
   int res_cnt[2] = {0, 0};
   int64_t res_units[2] = {0, 0};
+  bool res_halves[2] = {false, false};  // some residue rows start on 8 bytes only
   int num_sms = 0;
   int tile_n = 256;      // tile width of the residue products (0: both widths)
   int bound_tile = 256;  // tile width of the bound products
@@ -1239,7 +1262,7 @@ bool active_problem(int64_t m, int64_t n, int64_t k) { return m > 0 && n > 0 && 
 BatchLayout batch_layout(int count, const int64_t* m, const int64_t* n, const int64_t* k, int N, bool fast,
                          std::vector<BatchProblem>* probs) {
   BatchLayout L{};
-  const int planes = (N <= kNumSquares) ? 2 * N : 3 * N - kNumSquares;
+  const size_t planes = size_t(rns_planes(N)), documented = size_t(hybrid_planes(N));
   int cnt = 0;
   for (int i = 0; i < count; ++i) cnt += active_problem(m[i], n[i], k[i]) ? 1 : 0;
   size_t o = 0;
@@ -1271,13 +1294,17 @@ BatchLayout batch_layout(int count, const int64_t* m, const int64_t* n, const in
   L.zero_end = o;
   for (int i = 0, j = 0; i < count; ++i) {
     if (!active_problem(m[i], n[i], k[i])) continue;
-    const int64_t mi = m[i], ni = n[i], kp = ((k[i] + 31) / 32) * 32, ldp = plane_pitch(kp), ldr = residue_pitch(ni);
+    const int64_t mi = m[i], ni = n[i], kp = ((k[i] + 31) / 32) * 32, ldp = plane_pitch(kp);
     const size_t ep = take(4 * size_t(mi)), fp = take(4 * size_t(ni)), e = take(4 * size_t(mi)),
                  f = take(4 * size_t(ni)), rs = take(size_t(mi)), cs = take(size_t(ni));
+    // as make_layout: the residues behind the digit planes in use
+    const size_t pa = o, pb = pa + align256(planes * mi * ldp), cres = pb + align256(planes * ni * ldp);
+    take(documented * mi * ldp);
+    take(documented * ni * ldp);
     const size_t abar = fast ? 0 : take(size_t(mi) * kp), bbar = fast ? 0 : take(size_t(ni) * kp);
     const size_t part = fast ? take(4 * size_t(ni) * size_t(kp / 32)) : 0;
-    const size_t pa = take(size_t(planes) * mi * ldp), pb = take(size_t(planes) * ni * ldp);
-    const size_t cres = take(residue_bytes(mi, ni, N));
+    take(hybrid_residue_bytes(mi, ni, N));
+    const int64_t ldr = residue_pitch_in(o - cres, mi, ni, N);
     if (probs) {
       BatchProblem& q = P(j);
       q.m = int(mi);
@@ -1298,7 +1325,7 @@ BatchLayout batch_layout(int count, const int64_t* m, const int64_t* n, const in
       q.planesA = at(pa);
       q.planesB = at(pb);
       q.cres = reinterpret_cast<int16_t*>(at(cres));
-      q.cres8 = reinterpret_cast<int8_t*>(at(cres + residue8_offset(mi, ni, N)));
+      q.cres8 = reinterpret_cast<int8_t*>(at(cres + residue8_offset(mi, ldr, N)));
     }
     ++j;
   }
@@ -1459,6 +1486,7 @@ ozk2_status create_plan(ozk2_batch_plan* out, int count, const int64_t* m, const
     g.res_stride = int64_t(q.m) * q.ldr;
     plan->res_units[grp] += fp8_gemm_units(kModeResidue, q.m, q.n, N, tile);
     plan->res_cnt[grp] += 1;
+    plan->res_halves[grp] = plan->res_halves[grp] || q.ldr % 16 != 0;
     if (!fast) {
       GemmProblem& b = gbound[r];
       std::memset(&b, 0, sizeof(b));
@@ -1564,6 +1592,7 @@ ozk2_status execute_plan(ozk2_batch_plan plan, cudaStream_t st) {
   for (int grp = 0, first = 0; grp < 2; first += plan->res_cnt[grp], ++grp) {
     if (plan->res_cnt[grp] == 0) continue;
     g.tile_n = grp ? 128 : 256;
+    g.halves = plan->res_halves[grp];
     if (!launch_controls(g)) return OZK2_ERR_CUDA;
     OZK2_TRY(launch_fp8_gemm_grouped(g, gres + first, plan->res_cnt[grp], plan->res_units[grp], st));
     t_launches += 1;
@@ -1963,7 +1992,7 @@ ozk2_status ozk2_debug_residue_planes(int64_t m, int64_t n, int64_t k, const dou
   if (m == 0 || n == 0 || k == 0 || !A || !B || !e || !f || !planesA || !planesB || lda < k || ldb < n)
     return OZK2_ERR_INVALID_VALUE;
   Ctx c;
-  if ((s = setup(c, m, n, k, num_moduli, false, nullptr, 0, st)) != OZK2_OK) return s;
+  if ((s = setup(c, m, n, k, num_moduli, false, nullptr, 0, st, 0, false, true)) != OZK2_OK) return s;
   return paper_planes(c, A, lda, B, ldb, e, f, planesA, planesB);
 }
 
@@ -1976,9 +2005,7 @@ ozk2_status ozk2_debug_residue_products(int64_t m, int64_t n, int64_t k, const d
   if (m == 0 || n == 0 || k == 0 || !A || !B || !e || !f || !Cres || lda < k || ldb < n)
     return OZK2_ERR_INVALID_VALUE;
   Ctx c;
-  if ((s = setup(c, m, n, k, num_moduli, false, nullptr, 0, st, paper_residue_bytes(m, n, num_moduli))) != OZK2_OK)
-    return s;
-  c.L.cres = c.L.total;
+  if ((s = setup(c, m, n, k, num_moduli, false, nullptr, 0, st, 0, false, true)) != OZK2_OK) return s;
   const Layout& L = c.L;
   if ((s = paper_planes(c, A, lda, B, ldb, e, f, c.at<uint8_t>(L.planesA), c.at<uint8_t>(L.planesB))) != OZK2_OK)
     return s;
@@ -1996,9 +2023,7 @@ ozk2_status ozk2_debug_crt(int64_t m, int64_t n, int num_moduli, const int16_t* 
   if (m == 0 || n == 0) return OZK2_OK;
   if (!Cres || !e || !f || !C || ldc < n) return OZK2_ERR_INVALID_VALUE;
   Ctx c;
-  if ((s = setup(c, m, n, 1, num_moduli, false, nullptr, 0, st, paper_residue_bytes(m, n, num_moduli))) != OZK2_OK)
-    return s;
-  c.L.cres = c.L.total;
+  if ((s = setup(c, m, n, 1, num_moduli, false, nullptr, 0, st, 0, false, true)) != OZK2_OK) return s;
   const Layout& L = c.L;
   OZK2_TRY(cudaMemcpy2DAsync(c.ws + L.cres, size_t(L.ldr) * 2, Cres, size_t(n) * 2, size_t(n) * 2,
                              size_t(num_moduli) * size_t(m), cudaMemcpyDeviceToDevice, st));

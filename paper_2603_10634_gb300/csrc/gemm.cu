@@ -459,7 +459,7 @@ __device__ __forceinline__ float2 unpark2(uint32_t w) {
 
 // Store 8 int16 residues of one row at columns gc .. gc + 7 (gc < n), packed two per word,
 // as one 16-byte store (adding the previous block's residues when `accumulate`): rows are
-// padded to 16 columns, so the store stays inside the row.  The debug build checks that
+// padded to 8 columns, so the store stays inside the row.  The debug build checks that
 // every residue lies in [-h - 1, p - h] (paper mode: the symmetric range [-h, p - 1 - h]).
 template <bool EXACT>
 __device__ __forceinline__ void store_residues8(int16_t* dst, int gc, uint4 x4, bool accumulate, int p, int h,
@@ -491,13 +491,24 @@ __device__ __forceinline__ void store_residues8(int16_t* dst, int gc, uint4 x4, 
   *out = make_uint4(pk[0], pk[1], pk[2], pk[3]);
 }
 
-// The same for 16 int8 residues, packed four per word.
-__device__ __forceinline__ void store_residues16(int8_t* dst, int gc, uint4 x4, bool accumulate, int p, int h,
-                                                 uint32_t* flags) {
+// The same for 16 int8 residues, packed four per word, of a row of ldr columns.  Where ldr is
+// an odd multiple of 8 (HALVES: possible), rows start on 8 bytes and the last 8 of a row's
+// final 16 columns are the next row's: two 8-byte stores, the second only inside the row.
+template <bool HALVES>
+__device__ __forceinline__ void store_residues16(int8_t* dst, int ldr, int gc, uint4 x4, bool accumulate, int p,
+                                                 int h, uint32_t* flags) {
+  const bool wide = !HALVES || (ldr & 8) == 0;
   uint4* out = reinterpret_cast<uint4*>(dst + gc);
+  uint2* half = reinterpret_cast<uint2*>(dst + gc);
   uint32_t pk[4] = {x4.x, x4.y, x4.z, x4.w};
   if (accumulate) {
-    const uint4 prev = *out;
+    uint4 prev;
+    if (wide) {
+      prev = *out;
+    } else {
+      const uint2 a = half[0], b = gc + 8 < ldr ? half[1] : make_uint2(0u, 0u);
+      prev = make_uint4(a.x, a.y, b.x, b.y);
+    }
     const uint32_t pw[4] = {prev.x, prev.y, prev.z, prev.w};
 #pragma unroll
     for (int z = 0; z < 4; ++z) {
@@ -521,7 +532,12 @@ __device__ __forceinline__ void store_residues16(int8_t* dst, int gc, uint4 x4, 
 #else
   (void)flags;
 #endif
-  *out = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+  if (wide) {
+    *out = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+  } else {
+    half[0] = make_uint2(pk[0], pk[1]);
+    if (gc + 8 < ldr) half[1] = make_uint2(pk[2], pk[3]);
+  }
 }
 
 // 4 x 4 transpose of 16-byte items over groups of four lanes: lane i's item j comes from
@@ -568,8 +584,10 @@ __device__ __forceinline__ uint32_t pack4(float2 a, float2 b) {
 }
 
 // GROUPED: the units of all `nprobs` problems of `probs` (tmA, tmB unused).  TN: tile width.
-// PAIR: launched in clusters of two CTAs.
-template <int MODE, bool GROUPED, int TN, bool PAIR>
+// PAIR: launched in clusters of two CTAs.  HALVES: rows of 8-bit residues may start on 8 bytes
+// (an instance of its own: one that decides at run time took 281 instead of 265 us for a call of
+// 65536 x 72 x 64 with rows on 16 bytes, and 1112 instead of 1072 us for 48 mixed problems).
+template <int MODE, bool GROUPED, int TN, bool PAIR, bool HALVES>
 __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
     fp8_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ GemmParams prm, const GemmProblem* __restrict__ probs, int nprobs) {
@@ -869,7 +887,8 @@ __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
 #pragma unroll
                 for (int x = 0; x < 4; ++x)
                   if (gr + x < uc.m && gc < uc.n)
-                    store_residues16(plane + static_cast<int64_t>(gr + x) * uc.ldr, gc, px[x], c > 0, p, h, prm.flags);
+                    store_residues16<HALVES>(plane + static_cast<int64_t>(gr + x) * uc.ldr, static_cast<int>(uc.ldr), gc, px[x], c > 0,
+                                             p, h, prm.flags);
               }
             } else {
               int16_t* dst = uc.cres + static_cast<int64_t>(mod) * uc.res_stride + off;
@@ -1018,12 +1037,12 @@ __global__ void __launch_bounds__(Epi<TN, PAIR>::kThreads, 1)
   }
 }
 
-template <int MODE, bool GROUPED, int TN, bool PAIR>
+template <int MODE, bool GROUPED, int TN, bool PAIR, bool HALVES = false>
 cudaError_t launch_mode(const GemmParams& prm, const CUtensorMap& ta, const CUtensorMap& tb, int grid,
                         const GemmProblem* probs, int nprobs, cudaStream_t st) {
   static bool configured[64] = {false};
   constexpr size_t smem = Tile<TN, PAIR>::kSmemBytes;
-  auto* kernel = fp8_gemm_kernel<MODE, GROUPED, TN, PAIR>;
+  auto* kernel = fp8_gemm_kernel<MODE, GROUPED, TN, PAIR, HALVES>;
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !configured[dev]) {
@@ -1047,11 +1066,11 @@ cudaError_t launch_mode(const GemmParams& prm, const CUtensorMap& ta, const CUte
   return cudaLaunchKernelEx(&cfg, kernel, ta, tb, prm, probs, nprobs);
 }
 
-template <int MODE, bool GROUPED>
+template <int MODE, bool GROUPED, bool HALVES = false>
 cudaError_t launch_tile(int tn, const GemmParams& prm, const CUtensorMap& ta, const CUtensorMap& tb, int grid,
                         const GemmProblem* probs, int nprobs, cudaStream_t st) {
-  if (tn == 128) return launch_mode<MODE, GROUPED, 128, false>(prm, ta, tb, grid, probs, nprobs, st);
-  return launch_mode<MODE, GROUPED, 256, false>(prm, ta, tb, grid, probs, nprobs, st);
+  if (tn == 128) return launch_mode<MODE, GROUPED, 128, false, HALVES>(prm, ta, tb, grid, probs, nprobs, st);
+  return launch_mode<MODE, GROUPED, 256, false, HALVES>(prm, ta, tb, grid, probs, nprobs, st);
 }
 
 // Single problems whose operand planes (one of A, one of B) exceed this are paced: smaller
@@ -1146,6 +1165,9 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
   }
   switch (g.mode) {
     case kModeResidue:
+      if (g.ldr % 16 != 0)
+        return pair ? launch_mode<kModeResidue, false, 256, true, true>(prm, ta, tb, grid, nullptr, 0, st)
+                    : launch_tile<kModeResidue, false, true>(BN, prm, ta, tb, grid, nullptr, 0, st);
       return pair ? launch_mode<kModeResidue, false, 256, true>(prm, ta, tb, grid, nullptr, 0, st)
                   : launch_tile<kModeResidue, false>(BN, prm, ta, tb, grid, nullptr, 0, st);
     case kModePaper:
@@ -1192,7 +1214,8 @@ cudaError_t launch_fp8_gemm_grouped(const GemmArgs& g, const GemmProblem* probs,
   const int grid = prm.num_units < ctas ? prm.num_units : ctas;
   const int BN = tile_width(g.tile_n);
   if (g.mode == kModeResidue)
-    return launch_tile<kModeResidue, true>(BN, prm, unused, unused, grid, probs, count, st);
+    return g.halves ? launch_tile<kModeResidue, true, true>(BN, prm, unused, unused, grid, probs, count, st)
+                    : launch_tile<kModeResidue, true>(BN, prm, unused, unused, grid, probs, count, st);
   return launch_tile<kModeBound, true>(BN, prm, unused, unused, grid, probs, count, st);
 }
 

@@ -277,7 +277,7 @@ struct GemmArgs {
   // moduli's; kModePaper: `cres` only)
   int16_t* cres;
   int8_t* cres8;
-  int64_t ldr;          // elements per row of a residue plane (a multiple of 16)
+  int64_t ldr;          // elements per row of a residue plane (a multiple of 8)
   int64_t res_stride;   // elements between residue planes
   const GemmMods* mods;
   // bound product
@@ -297,6 +297,7 @@ struct GemmArgs {
   unsigned long long wait_ns;  // limit of each device wait (wait_limit_ns())
   bool stall;                  // fault injection: the kernel's first MMA wait never completes
   int tile_n;                  // output tile width: 128, or 256 (any other value)
+  bool halves;                 // grouped launches: some problem's ldr is an odd multiple of 8
 };
 // A operand: `planes_a` digit planes (K-major, m x k bytes, row stride lda8 bytes, plane
 // stride plane_stride_a); B operand the same with n rows.
@@ -417,7 +418,7 @@ struct GemmProblem {  // CUtensorMap carries the 64-byte alignment TMA needs
 };
 // Units of one problem in a GEMM of mode `mode` with N moduli and tiles of width tile_n.
 int64_t fp8_gemm_units(int mode, int m, int n, int N, int tile_n);
-// g supplies mode, num_sms, mods and flags; the problems (device memory, built on
+// g supplies mode, num_sms, mods, flags and halves; the problems (device memory, built on
 // the host with encode_gemm_problem) supply everything else.
 cudaError_t launch_fp8_gemm_grouped(const GemmArgs& g, const GemmProblem* probs, int count, int64_t total_units,
                                     cudaStream_t st);
