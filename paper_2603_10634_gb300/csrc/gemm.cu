@@ -374,7 +374,9 @@ struct Pace {
     if (words == nullptr) return;
     if (elect_one()) {
       atomicAdd(words, kPaceDone);
+      __threadfence();  // every report is in before this pair counts as done, and before the zeros
       if (atomicAdd(words + 1, 1u) == pairs - 1u) {
+        __threadfence();
         words[0] = 0u;
         words[1] = 0u;
       }
