@@ -553,6 +553,17 @@ ozk2_status ozk2_debug_backward_exponents(int64_t m, int64_t n, int64_t k, int n
                                           ozk2_stream_t stream);
 
 /*
+ * ozk2_debug_workspace_layout - where an unblocked ozk2_dgemm_ws / ozk2_dgemm_ex call of these
+ * sizes leaves its integers in its workspace, all in bytes: out[0], out[1] the digit planes of
+ * A' and of B' transposed (ozk2_product_count planes of m, n rows: three per Karatsuba modulus,
+ * then one per single modulus), out[2] a row of a plane, out[3] the Karatsuba moduli's int16
+ * residues, out[4] the single moduli's int8 residues (m rows each), out[5] the columns of a
+ * residue row, out[6], out[7] the int32 exponents e, f.  Returns 8, or -1 on invalid arguments.
+ */
+int ozk2_debug_workspace_layout(int64_t m, int64_t n, int64_t k, int num_moduli, ozk2_mode mode,
+                                int64_t out[8]);
+
+/*
  * ozk2_debug_crt - C = diag(2^-e) mod(sum_l q_l P/p_l C'_l, P) diag(2^-f)
  * (Eqs. CRT_finalreduction, inversescaling) from given residue products
  * Cres (N x m x n int16, contiguous) and exponents; each entry correctly rounded.

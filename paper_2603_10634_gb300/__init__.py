@@ -34,6 +34,7 @@ from .ozk2 import (  # noqa: F401
     timeline,
     tile_width,
     workspace_size,
+    workspace_layout,
     workspace_size_backward,
     workspace_size_host,
 )

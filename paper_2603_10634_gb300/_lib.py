@@ -76,6 +76,7 @@ SIGNATURES = {
                                           c_void_p, c_void_p, c_void_p, c_void_p, c_void_p]),
     "ozk2_debug_residue_products": (c_int, [c_i64, c_i64, c_i64, c_void_p, c_i64, c_void_p, c_i64, c_int,
                                             c_void_p, c_void_p, c_void_p, c_void_p]),
+    "ozk2_debug_workspace_layout": (c_int, [c_i64, c_i64, c_i64, c_int, c_int, c_void_p]),
     "ozk2_debug_crt": (c_int, [c_i64, c_i64, c_int, c_void_p, c_void_p, c_void_p, c_void_p, c_i64, c_void_p]),
 }
 

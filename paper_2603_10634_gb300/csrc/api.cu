@@ -2015,6 +2015,14 @@ ozk2_status ozk2_debug_residue_products(int64_t m, int64_t n, int64_t k, const d
   return OZK2_OK;
 }
 
+int ozk2_debug_workspace_layout(int64_t m, int64_t n, int64_t k, int num_moduli, ozk2_mode mode, int64_t out[8]) {
+  if (check_sizes(m, n, k, num_moduli) != OZK2_OK || !valid_mode(mode) || !out) return -1;
+  const Layout L = make_layout(m, n, k, num_moduli, mode == OZK2_MODE_FAST);
+  const size_t at[8] = {L.planesA, L.planesB, size_t(L.ldp), L.cres, L.cres8, size_t(L.ldr), L.e, L.f};
+  for (int i = 0; i < 8; ++i) out[i] = int64_t(at[i]);
+  return 8;
+}
+
 ozk2_status ozk2_debug_crt(int64_t m, int64_t n, int num_moduli, const int16_t* Cres, const int32_t* e,
                            const int32_t* f, double* C, int64_t ldc, ozk2_stream_t stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

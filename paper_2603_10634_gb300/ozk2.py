@@ -160,6 +160,14 @@ def dgemm(A, B, num_moduli=12, out=None, workspace=None, mode="accurate", block=
     return out
 
 
+def workspace_layout(m, n, k, num_moduli=12, mode="accurate"):
+    """Where a call keeps its integers in its workspace (ozk2_debug_workspace_layout)."""
+    out = (ctypes.c_int64 * 8)()
+    if _lib.load().ozk2_debug_workspace_layout(m, n, k, num_moduli, _mode(mode), out) != 8:
+        raise ValueError("invalid sizes")
+    return dict(zip(("planesA", "planesB", "plane_row", "res16", "res8", "res_columns", "e", "f"), out))
+
+
 def forward_state_size(m, n):
     return int(_lib.load().ozk2_forward_state_size(m, n))
 
