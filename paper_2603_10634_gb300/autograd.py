@@ -6,7 +6,8 @@ ozk2_dgemm_backward_from, which reuses the forward call's scaling exponents and 
 matrices A' = trunc(diag(2^e) A) and B' = trunc(B diag(2^f)): the autograd context keeps
 the exponents (4 (m + n) bytes; the forward's workspace, a few GB for a large layer, is
 released at once), one conversion of dC serves both gradients, and dC's exponents take
-the whole budget of P that A' and B' leave.  With
+the whole budget of P that A' and B' leave: gradients 1.4 to 2 times more accurate than
+fresh emulations', in about their time (at 8192 x 4096 x 4096, see bench.py).  With
 ``reuse=False``, or where reuse does not apply (fast mode, operands that are transposed
 views), each gradient is an independent emulation with its own scaling (Sec. III-E) of
 operands read in place.

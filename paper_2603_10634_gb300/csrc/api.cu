@@ -1444,7 +1444,8 @@ ozk2_status create_plan(ozk2_batch_plan* out, int count, const int64_t* m, const
   }
   for (int w = 0; w < kBatchKernels; ++w) plan->totals[w] = running[w];
   // Tile widths.  The setting (ozk2_set_tile_n) fixes one for every product of the plan.
-  // Otherwise each problem's residue products take the rule of single calls (tile_for):
+  // Otherwise each problem's residue products take the padding rule (tile_rule; not the
+  // count of busy SMs that single calls add, since the problems fill the chip together):
   // narrow or ragged problems run in 128-wide tiles and the rest in 256-wide ones, in
   // two grouped launches (wide first), which spends less tensor work on padding than one
   // width for the whole batch.  The bound products (1-2% of a plan) run in one launch
@@ -1630,18 +1631,17 @@ int dgemm_library_ws(int64_t m, int64_t n, int64_t k, const double* A, int64_t l
 }
 
 bool encode_fp8_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int64_t planes,
-                    int64_t row_stride_bytes, int64_t plane_stride_bytes, int box_rows, int box_cols) {
+                    int64_t row_stride_bytes, int64_t plane_stride_bytes, int box_rows) {
   EncodeTiledFn fn = encode_fn();
-  if (!fn || cols < 1 || rows < 1 || planes < 1 || (box_cols != 128 && box_cols != 64)) return false;
+  if (!fn || cols < 1 || rows < 1 || planes < 1) return false;
   if (plane_stride_bytes == 0) plane_stride_bytes = row_stride_bytes * rows;
   if (planes > 1 && plane_stride_bytes < row_stride_bytes * rows) return false;
   const cuuint64_t dims[3] = {cuuint64_t(cols), cuuint64_t(rows), cuuint64_t(planes)};
   const cuuint64_t strides[2] = {cuuint64_t(row_stride_bytes), cuuint64_t(plane_stride_bytes)};
-  const cuuint32_t box[3] = {cuuint32_t(box_cols), cuuint32_t(box_rows), 1u};
+  const cuuint32_t box[3] = {128u, cuuint32_t(box_rows), 1u};
   const cuuint32_t estr[3] = {1u, 1u, 1u};
-  const CUtensorMapSwizzle sw = (box_cols == 128) ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

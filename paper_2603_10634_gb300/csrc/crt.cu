@@ -79,7 +79,6 @@ __device__ __forceinline__ void into_symmetric_range(uint32_t (&v)[L], const Crt
   }
 }
 
-// RN(v 2^-scale) of the two's complement integer v.
 // The double of (-1)^neg (top : mid : low : rest) 2^(32 (ti - 2) - scale), rounded to
 // nearest even, when it is a normal number or overflows and has more than 53 bits; ti is
 // the index of `top`, the leading nonzero limb, and `rest` is nonzero if any lower limb is.

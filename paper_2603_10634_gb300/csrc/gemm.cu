@@ -106,7 +106,6 @@ struct Tile {
 };
 
 struct GemmParams {
-  int mode;
   int m, n, k;
   UnitGrid grid;
   int num_units;
@@ -419,9 +418,11 @@ struct ModPair {
   bool is1024;  // p = 1024, the even modulus: the last step rounds (r + 1/2) / p
 };
 
-// x - p q for exact-integer floats |x| <= 2^24, q = RN(x RN(1/p)): x RN(1/p) is within
-// 0.003 of x / p for p >= 443, so the remainder, formed exactly by one FMA, lies in
-// (-0.51 p, 0.51 p) and is congruent to x.
+// x - p q for exact-integer floats |x| <= 2^24, q = RN(x RN(1/p)); the remainder, formed
+// exactly by one FMA, is congruent to x.  x RN(1/p) is within |x| 2^-24 / p of x / p.  For
+// p >= 443 that is at most 0.003 and the remainder lies in (-0.51 p, 0.51 p).  For the single
+// moduli |x| <= terms V^2 <= 2^24 (V the largest digit) gives at most 1 / p, so the remainder
+// is at most p / 2 + 1 in magnitude: one past the symmetric range, which the CRT allows for.
 __device__ __forceinline__ float2 mod_near2(float2 x, const ModPair& m) {
   const float2 q = __fadd2_rn(__ffma2_rn(x, m.inv_p, dup2(kMagic)), dup2(-kMagic));
   return __ffma2_rn(m.neg_p, q, x);
@@ -1128,7 +1129,6 @@ int tile_width(int tile_n) { return tile_n == 128 ? 128 : 256; }
 cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, int planes_a, const uint8_t* b,
                             int64_t ldb8, int planes_b, cudaStream_t st) {
   GemmParams prm{};
-  prm.mode = g.mode;
   prm.m = g.m;
   prm.n = g.n;
   prm.k = g.k;
@@ -1156,8 +1156,8 @@ cudaError_t launch_fp8_gemm(const GemmArgs& g, const uint8_t* a, int64_t lda8, i
   prm.pace = pair && static_cast<int64_t>(g.m + g.n) * g.k >= kPaceBytes ? g.flags + kPaceWord : nullptr;
 
   CUtensorMap ta, tb;
-  if (!encode_fp8_map(&ta, a, g.k, g.m, planes_a, lda8, g.plane_stride_a, BM, BK)) return cudaErrorInvalidValue;
-  if (!encode_fp8_map(&tb, b, g.k, g.n, planes_b, ldb8, g.plane_stride_b, pair ? BN / 2 : BN, BK))
+  if (!encode_fp8_map(&ta, a, g.k, g.m, planes_a, lda8, g.plane_stride_a, BM)) return cudaErrorInvalidValue;
+  if (!encode_fp8_map(&tb, b, g.k, g.n, planes_b, ldb8, g.plane_stride_b, pair ? BN / 2 : BN))
     return cudaErrorInvalidValue;
   const int ctas = g.num_sms < kMaxGemmCtas ? g.num_sms : kMaxGemmCtas;
   const int grid = pair ? 2 * std::min(prm.num_units, ctas / 2) : std::min(prm.num_units, ctas);
@@ -1190,8 +1190,8 @@ int64_t fp8_gemm_units(int mode, int m, int n, int N, int tile_n) {
 bool encode_gemm_problem(GemmProblem* gp, const uint8_t* a, const uint8_t* b, int64_t ld8, int planes, int m, int n,
                          int k, int tile_n) {
   const int BN = tile_width(tile_n);
-  if (!encode_fp8_map(&gp->ta, a, k, m, planes, ld8, 0, BM, BK)) return false;
-  if (!encode_fp8_map(&gp->tb, b, k, n, planes, ld8, 0, BN, BK)) return false;
+  if (!encode_fp8_map(&gp->ta, a, k, m, planes, ld8, 0, BM)) return false;
+  if (!encode_fp8_map(&gp->tb, b, k, n, planes, ld8, 0, BN)) return false;
   gp->m = m;
   gp->n = n;
   gp->k = k;
@@ -1204,7 +1204,6 @@ cudaError_t launch_fp8_gemm_grouped(const GemmArgs& g, const GemmProblem* probs,
   if (count < 1 || total_units < 1 || total_units > 0x7FFFFFFFll) return cudaErrorInvalidValue;
   if (g.mode != kModeResidue && g.mode != kModeBound) return cudaErrorInvalidValue;
   GemmParams prm{};
-  prm.mode = g.mode;
   prm.num_units = static_cast<int>(total_units);
   prm.flags = g.flags;
   prm.wait_ns = g.wait_ns;

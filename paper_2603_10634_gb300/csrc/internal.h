@@ -428,9 +428,8 @@ bool encode_gemm_problem(GemmProblem* gp, const uint8_t* a, const uint8_t* b, in
                          int n, int k, int tile_n);
 
 // tensor maps (api.cu)
-// Boxes of box_rows x box_cols bytes (box_cols 128 or 64, swizzled to match).
-bool encode_fp8_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows,
-                    int64_t planes, int64_t row_stride_bytes, int64_t plane_stride_bytes,
-                    int box_rows, int box_cols);
+// Boxes of box_rows x 128 bytes, 128-byte swizzle.
+bool encode_fp8_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int64_t planes,
+                    int64_t row_stride_bytes, int64_t plane_stride_bytes, int box_rows);
 
 }  // namespace ozk2
