@@ -111,7 +111,7 @@ ozk2_status ozk2_dgemm_ws(int64_t m, int64_t n, int64_t k,
  * Same arguments and result as ozk2_dgemm: argument errors, m or n = 0 (nothing written)
  * and k = 0 (C = 0) behave exactly as there.  Returns OZK2_ERR_UNSUPPORTED, touching no
  * memory, when ozk2_workspace_size(m, n, k, num_moduli) exceeds OZK2_NOALLOC_MAX_BYTES
- * (for N = 12 that is square sizes up to 1664).  The first call on a device looks
+ * (for N = 12 that is square sizes up to 1760).  The first call on a device looks
  * the array up (cudaGetSymbolAddress, which loads this part of the library on that
  * device and so reserves the array there); make that first call before any stream
  * capture.  On a device without room for the array that first call fails with

@@ -336,9 +336,9 @@ struct Slots {
 // still full, until all pairs have reported as often; a pair that is done reports for good.
 // Only a hint: a wait that takes longer than kPaceNs (the launch does not have the GPU to
 // itself, or the last round) ends the pacing for this pair.  words[0]: reports, words[1]:
-// pairs done; the last one zeroes both.  DRAM reads of a 16384^3 launch 331 -> 123 GB (the
-// single-CTA kernel, which the operand ring slowed into step: 128 GB), and with them the
-// power that the cap turns into clock: 72.4 -> 64.5 ms; 8192^3 8.55 -> 7.75 ms.  Waiting every
+// pairs done; the last one zeroes both.  The DRAM reads fall to
+// those of the single-CTA kernel, which the operand ring slows into step, and with them the
+// power that the cap turns into clock: products of 16384^3 72.4 -> 64.5 ms, 8192^3 8.55 -> 7.75.  Waiting every
 // 16 steps, or letting a pair run one round ahead, was slower (66.2, 66.9 ms).
 constexpr int kPaceSteps = 64;
 constexpr unsigned long long kPaceNs = 20000ull;
